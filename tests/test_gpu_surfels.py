@@ -74,3 +74,24 @@ def test_surfels_outside_every_window_are_removed_unchanged(ctx, smap):
     p, nr, keep, kept = ctx.surfel_correct(S.pos[:n], S.nrm[:n], t0, tu, S.T_old, S.T_new, S.t_kf, S.cam)
     assert kept == 0 and not keep.any()
     assert np.array_equal(p, S.pos[:n]) and np.array_equal(nr, S.nrm[:n])
+
+
+@gpu
+@pytest.mark.parametrize("n", [1, 31, 512, 513, 2051, 470_001])
+@pytest.mark.parametrize("m", [1, 2, 300, 600])
+def test_small_keyframe_tables_equal_the_general_kernel(ctx, n, m):
+    """A table of up to 600 keyframes takes the tile kernel. Keyframes stamped
+    after every surfel's window change nothing, but 601 and more rows take the
+    general kernel: the same bits, with surfels of empty windows among them."""
+    S = make_surfels(n, m, seed=31 + m)
+    t0, tu = S.t0.copy(), S.tu.copy()
+    tu[::7] = t0[::7]          # empty windows
+    t0[::11], tu[::11] = -5.0, 1e6
+    extra = 601
+    far = np.tile(np.eye(4), (extra, 1, 1))
+    a = ctx.surfel_correct(S.pos, S.nrm, t0, tu, S.T_old, S.T_new, S.t_kf, S.cam)
+    b = ctx.surfel_correct(S.pos, S.nrm, t0, tu, np.concatenate([S.T_old, far]), np.concatenate([S.T_new, far]),
+                           np.concatenate([S.t_kf, 2e6 + np.arange(extra, dtype=np.float32)]), S.cam)
+    assert a[3] == b[3]
+    for x, y in zip(a[:3], b[:3]):
+        assert np.array_equal(x, y)
