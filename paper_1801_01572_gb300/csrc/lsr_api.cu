@@ -214,9 +214,11 @@ struct CloudLayout {
   unsigned *mask_e = nullptr;
 };
 
+constexpr int kPairGrids = 3;  // grids a registration builds at once
+
 struct ScratchLayout {
-  int n_max = 0, cap_max = 0;
-  GridScratch g{};
+  int jobs = 0;
+  GridScratch g[kPairGrids];
 };
 
 void plan_cloud(Arena &a, int n, bool stage_src, bool features, bool eps_grid, CloudLayout &c) {
@@ -247,22 +249,25 @@ void plan_cloud(Arena &a, int n, bool stage_src, bool features, bool eps_grid, C
   }
 }
 
-void plan_scratch(Arena &a, int n_max, int cap_max, ScratchLayout &s) {
-  s.n_max = n_max;
-  s.cap_max = cap_max;
-  s.g.slot = a.take<int>(n_max);
-  s.g.tmp = a.take<int>(n_max);
-  s.g.counts = a.take<int>((size_t)cap_max + 1);
-  s.g.scan = a.take<int>((size_t)scan_scratch_ints(cap_max));
+// Scratch for `jobs` grids built at once.
+void plan_scratch(Arena &a, int n_max, int cap_max, ScratchLayout &s, int jobs = 1) {
+  s.jobs = jobs;
+  for (int j = 0; j < jobs; ++j) {
+    s.g[j].slot = a.take<int>(n_max);
+    s.g[j].rank = a.take<int>(n_max);
+    s.g[j].tmp = a.take<int>(n_max);
+    s.g[j].counts = a.take<int>((size_t)cap_max + 1);
+    s.g[j].scan = a.take<int>((size_t)scan_scratch_ints(cap_max));
+  }
 }
 
-// Coarse levels of the graduated refinement: subsampled copies of Q and their
-// grids (the finest level uses Q's eps grid).
+// Coarse levels of the graduated refinement: grids of Q's every sQ-th point
+// (the finest level uses Q's eps grid) and the subsampled copies of P.
 struct LevelLayout {
   int levels = 0;
   int sQ[kMaxLevels] = {}, nsub[kMaxLevels] = {}, cap[kMaxLevels] = {};
   int sP[kMaxLevels] = {}, nsubP[kMaxLevels] = {};
-  float4 *Qsub[kMaxLevels] = {}, *Xs[kMaxLevels] = {}, *Psub[kMaxLevels] = {};
+  float4 *Xs[kMaxLevels] = {}, *Psub[kMaxLevels] = {};
   int *start[kMaxLevels] = {};
   unsigned *mask[kMaxLevels] = {};
   GridParams *g[kMaxLevels] = {};
@@ -279,7 +284,6 @@ void plan_levels(Arena &a, int nP, int nQ, int levels, LevelLayout &V) {
     V.sQ[l] = gnc_stride(nQ, l, levels);
     V.nsub[l] = (int)lsr_div_up(nQ, V.sQ[l]);
     V.cap[l] = cap_cells_for(V.nsub[l]);
-    V.Qsub[l] = a.take<float4>(V.nsub[l]);
     V.Xs[l] = a.take<float4>(V.nsub[l]);
     V.start[l] = a.take<int>((size_t)V.cap[l] + 1);
     V.mask[l] = a.take<unsigned>((size_t)nbmask_words(V.cap[l]));
@@ -334,7 +338,7 @@ void plan_pair(Arena &a, int nP, int nQ, bool stP, bool stQ, int64_t H, int leve
   plan_cloud(a, nP, stP, true, false, L.P);
   plan_cloud(a, nQ, stQ, true, true, L.Q);
   plan_levels(a, nP, nQ, levels, L.lv);
-  plan_scratch(a, std::max(nP, nQ), std::max(L.P.cap_f, L.Q.cap_f), L.sc);
+  plan_scratch(a, std::max(nP, nQ), std::max(L.P.cap_f, L.Q.cap_f), L.sc, kPairGrids);
   L.nn = a.take<int>(nP);
   L.d1 = a.take<float>(nP);
   L.nb = hyp_blocks(H);
@@ -587,34 +591,84 @@ __global__ void k_sum_to_double(const unsigned long long *s, int n, double *d) {
 }
 int nblk(int64_t n, int t = 256) { return (int)std::max<int64_t>(1, std::min<int64_t>((n + t - 1) / t, kSms * 32)); }
 
-// Build the feature-radius grid (internal order) and, optionally, the
-// normal-radius and eps grids of one cloud.
-cudaError_t build_cloud(const float *xyz, CloudLayout &c, float r_f, float r_n, float eps, bool normal_grid,
-                        bool eps_grid, const ScratchLayout &sc, cudaStream_t s) {
-  LSR_CUDA_TRY(launch_bbox_xyz(xyz, c.n, c.box_part, bbox_blocks(c.n), c.box, s));
-  LSR_CUDA_TRY(launch_grid_params(c.box, r_f, c.n, c.cap_f, c.gf, s));
-  LSR_CUDA_TRY(build_grid_xyz(xyz, c.n, c.gf, c.cap_f, c.start_f, c.X, c.inv, sc.g, s));
-  if (normal_grid) {
-    LSR_CUDA_TRY(launch_grid_params(c.box, r_n, c.n, c.cap_n, c.gn, s));
-    LSR_CUDA_TRY(build_grid_f4(c.X, c.n, c.gn, c.cap_n, c.start_n, c.Xn, sc.g, s));
-  }
-  if (eps_grid) {
-    LSR_CUDA_TRY(launch_grid_params(c.box, eps, c.n, c.cap_e, c.ge, s));
-    LSR_CUDA_TRY(build_grid_f4(c.X, c.n, c.ge, c.cap_e, c.start_e, c.Xe, sc.g, s));
-    LSR_CUDA_TRY(build_nbmask(c.ge, c.start_e, c.cap_e, c.mask_e, s));
-  }
-  return cudaSuccess;
+// The feature-radius grid of a cloud (internal order) with its box.
+GridJob feature_grid(const float *xyz, const CloudLayout &c, float r_f, const GridScratch &sc) {
+  GridJob j;
+  j.xyz = xyz, j.n = c.n, j.cap = c.cap_f, j.radius = r_f;
+  j.box = c.box, j.box_part = c.box_part;
+  j.g = c.gf, j.start = c.start_f, j.out = c.X, j.inv = c.inv;
+  j.sc = sc;
+  return j;
+}
+
+// The normal-radius and eps grids over the internal order (w = internal index).
+GridJob normal_grid(const CloudLayout &c, float r_n, const GridScratch &sc) {
+  GridJob j;
+  j.x4 = c.X, j.n = c.n, j.cap = c.cap_n, j.radius = r_n;
+  j.box = c.box;
+  j.g = c.gn, j.start = c.start_n, j.out = c.Xn;
+  j.sc = sc;
+  return j;
+}
+GridJob eps_grid(const CloudLayout &c, float eps, const GridScratch &sc) {
+  GridJob j;
+  j.x4 = c.X, j.n = c.n, j.cap = c.cap_e, j.radius = eps;
+  j.box = c.box;
+  j.g = c.ge, j.start = c.start_e, j.out = c.Xe, j.mask = c.mask_e;
+  j.sc = sc;
+  return j;
+}
+
+// The eps grid alone, straight from the caller's xyz (w = caller index).
+GridJob eps_grid_xyz(const float *xyz, const CloudLayout &c, float eps, const GridScratch &sc) {
+  GridJob j;
+  j.xyz = xyz, j.n = c.n, j.cap = c.cap_e, j.radius = eps;
+  j.box = c.box, j.box_part = c.box_part;
+  j.g = c.ge, j.start = c.start_e, j.out = c.Xe, j.mask = c.mask_e;
+  j.sc = sc;
+  return j;
+}
+
+// A stage's cloud that needs one radius only: the eps grid with w = the sorted
+// index. It is the internal order of that radius too, so X is the same array.
+GridJob eps_cloud(const float *xyz, CloudLayout &c, float eps, const GridScratch &sc) {
+  GridJob j = eps_grid_xyz(xyz, c, eps, sc);
+  j.carry_pos = true;
+  c.X = c.Xe;
+  return j;
+}
+
+// The grids of a registration: both feature grids, then the grids over them.
+cudaError_t build_pair(const float *P, const float *Q, const CloudLayout &Pc, const CloudLayout &Qc, float r_f,
+                       float r_n, float eps, const ScratchLayout &sc, cudaStream_t s) {
+  const GridJob first[2] = {feature_grid(P, Pc, r_f, sc.g[0]), feature_grid(Q, Qc, r_f, sc.g[1])};
+  LSR_CUDA_TRY(build_grids(first, 2, s));
+  const GridJob then[3] = {normal_grid(Pc, r_n, sc.g[0]), normal_grid(Qc, r_n, sc.g[1]), eps_grid(Qc, eps, sc.g[2])};
+  return build_grids(then, 3, s);
 }
 
 // Graduated refinement (levels l = 0..L-1, radius eps * 2^(L-1-l)) from the
 // pose in st. XP: P in internal order with caller indices in w; Q: caller-order
 // xyz on the device; (ge, start_e, Xe): Q's eps grid for the finest level.
-cudaError_t enqueue_refine(const float4 *XP, const float *P, int nP, const float *Q, int nQ, const float *boxQ,
+cudaError_t enqueue_refine(const float4 *XP, const float *P, int nP, const float *Q, const float *boxQ,
                            const GridParams *ge, const int *start_e, const float4 *Xe, const LevelLayout &V, float eps,
                            float mu_scale, int iters, RansacState *st, double *part, int *seeds,
                            const ScratchLayout &sc, cudaStream_t s, bool chain) {
   int L = V.levels;
   LSR_CUDA_TRY(refine_reset_tickets(part, s));
+  // the coarse levels' grids, as many at once as there is scratch for
+  for (int l0 = 0; l0 + 1 < L; l0 += sc.jobs) {
+    GridJob jobs[kPairGrids];
+    int nj = 0;
+    for (int l = l0; l + 1 < L && nj < sc.jobs; ++l, ++nj) {
+      GridJob &j = jobs[nj];
+      j.xyz = Q, j.stride = V.sQ[l], j.n = V.nsub[l], j.cap = V.cap[l], j.radius = eps * (float)(1 << (L - 1 - l));
+      j.box = const_cast<float *>(boxQ);
+      j.g = V.g[l], j.start = V.start[l], j.out = V.Xs[l], j.mask = V.mask[l];
+      j.sc = sc.g[nj];
+    }
+    LSR_CUDA_TRY(build_grids(jobs, nj, s));
+  }
   for (int l = 0; l < L; ++l) {
     float e = eps * (float)(1 << (L - 1 - l));
     float mu = mu_scale * e * e;
@@ -628,13 +682,7 @@ cudaError_t enqueue_refine(const float4 *XP, const float *P, int nP, const float
     const GridParams *g = ge;
     const int *st0 = start_e;
     const float4 *xs = Xe;
-    if (l + 1 < L) {
-      LSR_CUDA_TRY(launch_subsample(Q, nQ, V.sQ[l], V.Qsub[l], s));
-      LSR_CUDA_TRY(launch_grid_params(boxQ, e, V.nsub[l], V.cap[l], V.g[l], s));
-      LSR_CUDA_TRY(build_grid_f4(V.Qsub[l], V.nsub[l], V.g[l], V.cap[l], V.start[l], V.Xs[l], sc.g, s));
-      LSR_CUDA_TRY(build_nbmask(V.g[l], V.start[l], V.cap[l], V.mask[l], s));
-      g = V.g[l], st0 = V.start[l], xs = V.Xs[l];
-    }
+    if (l + 1 < L) g = V.g[l], st0 = V.start[l], xs = V.Xs[l];
     LSR_CUDA_TRY(launch_refine_level_begin(st, s));
     LSR_CUDA_TRY(cudaMemsetAsync(seeds, 0xff, sizeof(int) * (size_t)np, s));  // no neighbour yet at this level
     for (int it = 0; it < iters; ++it)
@@ -676,8 +724,7 @@ int enqueue_pair(lsr_ctx *c, const PairLayout &L, const float *P, const float *Q
   tm.mark();
   TRY_CUDA(c, cudaMemsetAsync(L.st, 0, sizeof(RansacState), s), "memset state");
   CloudLayout Pc = L.P, Qc = L.Q;
-  TRY_CUDA(c, build_cloud(P, Pc, p.r_feature, p.r_normal, p.eps_inlier, true, false, L.sc, s), "grids P");
-  TRY_CUDA(c, build_cloud(Q, Qc, p.r_feature, p.r_normal, p.eps_inlier, true, true, L.sc, s), "grids Q");
+  TRY_CUDA(c, build_pair(P, Q, Pc, Qc, p.r_feature, p.r_normal, p.eps_inlier, L.sc, s), "grids");
   tm.mark();
   float3 vp_p = vpP ? make_float3(vpP[0], vpP[1], vpP[2]) : make_float3(0.f, 0.f, 0.f);
   float3 vp_q = vpQ ? make_float3(vpQ[0], vpQ[1], vpQ[2]) : make_float3(0.f, 0.f, 0.f);
@@ -723,7 +770,10 @@ int enqueue_pair(lsr_ctx *c, const PairLayout &L, const float *P, const float *Q
     const float4 *gx = Qc.Xe;
     if (single) {
       TRY_CUDA(c, launch_cell_grid_params(Qc.box, p.eps_inlier, nQ, L.cap_s, L.gs, s), "single-cell grid");
-      TRY_CUDA(c, build_grid_f4(Qc.X, nQ, L.gs, L.cap_s, L.start_s, L.Xs, L.sc.g, s), "single-cell grid");
+      GridJob j;
+      j.x4 = Qc.X, j.n = nQ, j.cap = L.cap_s, j.params_ready = true;
+      j.g = L.gs, j.start = L.start_s, j.out = L.Xs, j.sc = L.sc.g[0];
+      TRY_CUDA(c, build_grids(&j, 1, s), "single-cell grid");
       g = L.gs, gstart = L.start_s, gx = L.Xs;
     }
     TRY_CUDA(c, cudaMemsetAsync(L.count, 0, sizeof(int) * L.surv_cap, s), "memset count");
@@ -799,7 +849,7 @@ int enqueue_pair(lsr_ctx *c, const PairLayout &L, const float *P, const float *Q
   TRY_CUDA(c, launch_refine_init(L.st, Pc.box, nullptr, s), "refine init");
   float eps = p.eps_inlier;
   TRY_CUDA(c,
-           enqueue_refine(Pc.X, P, nP, Q, nQ, Qc.box, Qc.ge, Qc.start_e, Qc.Xe, L.lv, eps, p.mu_scale, p.refine_iters,
+           enqueue_refine(Pc.X, P, nP, Q, Qc.box, Qc.ge, Qc.start_e, Qc.Xe, L.lv, eps, p.mu_scale, p.refine_iters,
                           L.st, L.ref_part, L.seeds, L.sc, s, chain),
            "refine");
   TRY_CUDA(c, launch_final_pose(L.st, L.fpose, s), "final pose");
@@ -1501,9 +1551,10 @@ int lsr_stage_normals(lsr_ctx *c, const float *P, int64_t n, const float *vp, fl
   const float *src;
   if ((rc = stage_input(c, P, n, C.src, &src))) return rc;
   cudaStream_t s = c->stream;
-  TRY_CUDA(c, build_cloud(src, C, r, r, r, true, false, S, s), "grids");
+  const GridJob gj = feature_grid(src, C, r, S.g[0]);
+  TRY_CUDA(c, build_grids(&gj, 1, s), "grid");
   float3 v = vp ? make_float3(vp[0], vp[1], vp[2]) : make_float3(0.f, 0.f, 0.f);
-  TRY_CUDA(c, launch_normals(C.X, (int)n, C.gn, C.start_n, C.Xn, r, v, C.N, cnt, s), "normals");
+  TRY_CUDA(c, launch_normals(C.X, (int)n, C.gf, C.start_f, C.X, r, v, C.N, cnt, s), "normals");
   LSR_LAUNCH(k_scatter_normals<<<nblk(n), 256, 0, s>>>(C.N, cnt, C.X, (int)n, dn, dc, dv));
   TRY_CUDA(c, cudaGetLastError(), "scatter");
   if (normals && (rc = copy_out(c, normals, dn, sizeof(float) * 3 * n))) return rc;
@@ -1545,7 +1596,8 @@ static int stage_desc_common(lsr_ctx *c, const float *P, const float *normals, c
   const float *src;
   if ((rc = stage_input(c, P, n, C.src, &src))) return rc;
   TRY_CUDA(c, cudaMemcpyAsync(nrm, normals, sizeof(float) * 3 * n, cudaMemcpyDefault, s), "copy normals");
-  TRY_CUDA(c, build_cloud(src, C, r, r, r, false, false, S, s), "grids");
+  const GridJob gj = feature_grid(src, C, r, S.g[0]);
+  TRY_CUDA(c, build_grids(&gj, 1, s), "grid");
   LSR_LAUNCH(k_gather_normals<<<nblk(n), 256, 0, s>>>(nrm, C.X, (int)n, C.N));
   if (!spfh_in) {
     TRY_CUDA(c, launch_spfh(C.X, C.N, (int)n, C.gf, C.start_f, r, C.S, kk, C.F, s), "spfh");
@@ -1818,7 +1870,8 @@ int lsr_stage_consensus(lsr_ctx *c, const float *P, int64_t nP, const float *Q, 
   if ((rc = stage_input(c, Q, nQ, Cq.src, &qsrc))) return rc;
   TRY_CUDA(c, cudaMemcpyAsync(pose, Rt, sizeof(float) * 12 * nh, cudaMemcpyDefault, s), "copy Rt");
   LSR_LAUNCH(k_pack<<<nblk(nP), 256, 0, s>>>(p, (int)nP, XP));
-  TRY_CUDA(c, build_cloud(qsrc, Cq, eps, eps, eps, false, true, b.S, s), "grid Q");
+  const GridJob gj = eps_cloud(qsrc, Cq, eps, b.S.g[0]);
+  TRY_CUDA(c, build_grids(&gj, 1, s), "grid Q");
   TRY_CUDA(c, cudaMemsetAsync(cnt, 0, sizeof(int) * nh, s), "memset");
   TRY_CUDA(c, cudaMemsetAsync(b.cnt2, 0, sizeof(int) * nh, s), "memset");
   TRY_CUDA(c, cudaMemsetAsync(sum, 0, sizeof(unsigned long long) * nh, s), "memset");
@@ -1850,17 +1903,18 @@ int lsr_stage_refine(lsr_ctx *c, const float *P, int64_t nP, const float *Q, int
     return set_err(c, LSR_E_ARG, "bad argument");
   float *boxP = nullptr;
   double *boxP_part = nullptr;
-  int *seeds = nullptr;
+  int *seeds = nullptr, *ticketP = nullptr;
   auto plan = [&](Arena &a, float *&p, float4 *&XP, CloudLayout &Cq, LevelLayout &V, ScratchLayout &S, double *&part,
                   double *&Td, RansacState *&st) {
     seeds = a.take<int>(nP);
     p = a.take<float>(3 * nP);
     XP = a.take<float4>(nP);
     boxP = a.take<float>(kBox);
+    ticketP = a.take<int>(1);
     boxP_part = a.take<double>((size_t)kBoxPart * bbox_blocks((int)nP));
     plan_cloud(a, (int)nQ, true, false, true, Cq);
     plan_levels(a, (int)nP, (int)nQ, levels, V);
-    plan_scratch(a, (int)nQ, Cq.cap_f, S);
+    plan_scratch(a, (int)nQ, Cq.cap_f, S, kPairGrids);
     part = a.take<double>((size_t)refine_partial_doubles());
     Td = a.take<double>(16);
     st = a.take<RansacState>(1);
@@ -1891,11 +1945,13 @@ int lsr_stage_refine(lsr_ctx *c, const float *P, int64_t nP, const float *Q, int
   TRY_CUDA(c, cudaMemcpyAsync(Td, T_in, sizeof(double) * 16, cudaMemcpyDefault, s), "copy T");
   TRY_CUDA(c, cudaMemsetAsync(st, 0, sizeof(RansacState), s), "memset");
   LSR_LAUNCH(k_pack<<<nblk(nP), 256, 0, s>>>(p, (int)nP, XP));
-  TRY_CUDA(c, launch_bbox_xyz(p, (int)nP, boxP_part, bbox_blocks((int)nP), boxP, s), "bbox P");
-  TRY_CUDA(c, build_cloud(qsrc, Cq, eps, eps, eps, false, true, S, s), "grid Q");
+  // Q's eps grid and the box of P (its ticket: a spare word) together
+  GridJob gj[2] = {eps_cloud(qsrc, Cq, eps, S.g[0]), GridJob()};
+  gj[1].xyz = p, gj[1].n = (int)nP, gj[1].box = boxP, gj[1].box_part = boxP_part, gj[1].sc.counts = ticketP;
+  TRY_CUDA(c, build_grids(gj, 2, s), "grid Q, box P");
   TRY_CUDA(c, launch_refine_init(st, boxP, Td, s), "init");
   TRY_CUDA(c,
-           enqueue_refine(XP, p, (int)nP, qsrc, (int)nQ, Cq.box, Cq.ge, Cq.start_e, Cq.Xe, V, eps, mu_scale, iters, st,
+           enqueue_refine(XP, p, (int)nP, qsrc, Cq.box, Cq.ge, Cq.start_e, Cq.Xe, V, eps, mu_scale, iters, st,
                           part, seeds, S, s, true),
            "refine");
   RansacState h;
@@ -1939,7 +1995,8 @@ int lsr_information_matrix(lsr_ctx *c, const float *P, int64_t nP, const float *
   const float *psrc, *qsrc;
   if ((rc = stage_input(c, P, nP, b.p, &psrc))) return rc;
   if ((rc = stage_input(c, Q, nQ, b.Cq.src, &qsrc))) return rc;
-  TRY_CUDA(c, build_cloud(qsrc, b.Cq, eps, eps, eps, false, true, b.S, s), "grid Q");
+  const GridJob gj = eps_cloud(qsrc, b.Cq, eps, b.S.g[0]);
+  TRY_CUDA(c, build_grids(&gj, 1, s), "grid Q");
   float R[9], t[3];
   for (int r = 0; r < 3; ++r) {
     for (int q = 0; q < 3; ++q) R[3 * r + q] = (float)T[4 * r + q];
@@ -2017,13 +2074,13 @@ int lsr_stage_consensus_modes(lsr_ctx *c, const float *P, const float *NP, int64
     LSR_LAUNCH(k_gather_normals<<<nblk(nQ), 256, 0, s>>>(b.nq, b.XQ, (int)nQ, b.NQ4));
   }
   // Q's grid with caller indices in w (exact: cells of eps; single: the eps lattice through the centroid)
-  TRY_CUDA(c, launch_bbox_xyz(qsrc, Cq.n, Cq.box_part, bbox_blocks(Cq.n), Cq.box, s), "bbox");
-  if (single)
+  GridJob gj = eps_grid_xyz(qsrc, Cq, eps, b.S.g[0]);
+  if (single) {
+    TRY_CUDA(c, launch_bbox_xyz(qsrc, Cq.n, Cq.box_part, bbox_blocks(Cq.n), Cq.box, s), "bbox");
     TRY_CUDA(c, launch_cell_grid_params(Cq.box, eps, Cq.n, Cq.cap_e, Cq.ge, s), "grid params");
-  else
-    TRY_CUDA(c, launch_grid_params(Cq.box, eps, Cq.n, Cq.cap_e, Cq.ge, s), "grid params");
-  TRY_CUDA(c, build_grid_xyz(qsrc, Cq.n, Cq.ge, Cq.cap_e, Cq.start_e, Cq.Xe, Cq.inv, b.S.g, s), "grid");
-  if (!single) TRY_CUDA(c, build_nbmask(Cq.ge, Cq.start_e, Cq.cap_e, Cq.mask_e, s), "mask");
+    gj.box_part = nullptr, gj.mask = nullptr, gj.params_ready = true;
+  }
+  TRY_CUDA(c, build_grids(&gj, 1, s), "grid");
   TRY_CUDA(c, cudaMemsetAsync(b.cnt, 0, sizeof(int) * nh, s), "memset");
   TRY_CUDA(c, cudaMemsetAsync(b.sum, 0, sizeof(unsigned long long) * nh, s), "memset");
   const int nh32 = (int)nh;
@@ -2073,13 +2130,13 @@ int lsr_stage_nn(lsr_ctx *c, const float *Q, int64_t nQ, const float *X, int64_t
   if ((rc = stage_input(c, Q, nQ, b.Cq.src, &qsrc))) return rc;
   CloudLayout &Cq = b.Cq;
   const bool single = mode == LSR_NN_SINGLE_CELL;
-  TRY_CUDA(c, launch_bbox_xyz(qsrc, Cq.n, Cq.box_part, bbox_blocks(Cq.n), Cq.box, s), "bbox");
-  if (single)
+  GridJob gj = eps_grid_xyz(qsrc, Cq, r, b.S.g[0]);
+  if (single) {
+    TRY_CUDA(c, launch_bbox_xyz(qsrc, Cq.n, Cq.box_part, bbox_blocks(Cq.n), Cq.box, s), "bbox");
     TRY_CUDA(c, launch_cell_grid_params(Cq.box, r, Cq.n, Cq.cap_e, Cq.ge, s), "grid params");
-  else
-    TRY_CUDA(c, launch_grid_params(Cq.box, r, Cq.n, Cq.cap_e, Cq.ge, s), "grid params");
-  TRY_CUDA(c, build_grid_xyz(qsrc, Cq.n, Cq.ge, Cq.cap_e, Cq.start_e, Cq.Xe, Cq.inv, b.S.g, s), "grid");
-  if (!single) TRY_CUDA(c, build_nbmask(Cq.ge, Cq.start_e, Cq.cap_e, Cq.mask_e, s), "mask");
+    gj.box_part = nullptr, gj.mask = nullptr, gj.params_ready = true;
+  }
+  TRY_CUDA(c, build_grids(&gj, 1, s), "grid");
   TRY_CUDA(c, launch_nn_stage(xsrc, (int)nX, Cq.ge, Cq.start_e, Cq.Xe, r, single ? 1 : 0, b.nn, b.d2, s), "nn");
   if ((rc = copy_out(c, nn, b.nn, sizeof(int) * nX))) return rc;
   if (d2 && (rc = copy_out(c, d2, b.d2, sizeof(float) * nX))) return rc;
@@ -2137,15 +2194,12 @@ int lsr_pose_implicit_grad(lsr_ctx *c, const float *P, int64_t nP, const float *
   const float *psrc, *qsrc;
   if ((rc = stage_input(c, P, nP, b.p, &psrc))) return rc;
   if ((rc = stage_input(c, Q, nQ, b.Cq.src, &qsrc))) return rc;
-  // eps grid of Q with caller indices in w (build_grid_xyz carries the caller order), so dQ is in caller order
-  CloudLayout &Cq = b.Cq;
-  TRY_CUDA(c, launch_bbox_xyz(qsrc, Cq.n, Cq.box_part, bbox_blocks(Cq.n), Cq.box, s), "bbox");
-  TRY_CUDA(c, launch_grid_params(Cq.box, eps, Cq.n, Cq.cap_e, Cq.ge, s), "grid params");
-  TRY_CUDA(c, build_grid_xyz(qsrc, Cq.n, Cq.ge, Cq.cap_e, Cq.start_e, Cq.Xe, Cq.inv, b.S.g, s), "grid");
-  TRY_CUDA(c, build_nbmask(Cq.ge, Cq.start_e, Cq.cap_e, Cq.mask_e, s), "mask");
-  TRY_CUDA(c, cudaMemcpyAsync(b.dl, dl, sizeof(dl), cudaMemcpyHostToDevice, s), "H2D");
+  // eps grid of Q with caller indices in w, so dQ is in caller order; its build clears dQ too
   float *gp = dev_out ? dP : b.gp, *gq = dev_out ? dQ : b.gq;
-  TRY_CUDA(c, cudaMemsetAsync(gq, 0, sizeof(float) * 3 * nQ, s), "memset dQ");
+  GridJob gj = eps_grid_xyz(qsrc, b.Cq, eps, b.S.g[0]);
+  gj.zero = gq, gj.zero_words = 3 * nQ;
+  TRY_CUDA(c, build_grids(&gj, 1, s), "grid");
+  TRY_CUDA(c, cudaMemcpyAsync(b.dl, dl, sizeof(dl), cudaMemcpyHostToDevice, s), "H2D");
   TRY_CUDA(c,
            launch_implicit(psrc, (int)nP, b.Cq.ge, b.Cq.start_e, b.Cq.Xe, (int)nQ, T, eps, (double)mu, b.dl, b.part,
                            b.out, gp, gq, s),
@@ -2403,12 +2457,10 @@ static int objective_impl(lsr_ctx *c, int32_t n, const float *const *P, const in
         Tm[4 * r + q] = acc;
       }
     const double vd[3] = {w[3], w[4], w[5]};
-    // eps grid of Q with caller indices (build_grid_xyz carries caller order)
-    TRY_CUDA(c, launch_bbox_xyz(Q[i], Cq.n, Cq.box_part, bbox_blocks(Cq.n), Cq.box, s), "bbox");
-    TRY_CUDA(c, launch_grid_params(Cq.box, eps, Cq.n, Cq.cap_e, Cq.ge, s), "grid params");
-    TRY_CUDA(c, build_grid_xyz(Q[i], Cq.n, Cq.ge, Cq.cap_e, Cq.start_e, Cq.Xe, Cq.inv, Sc.g, s), "grid");
-    TRY_CUDA(c, build_nbmask(Cq.ge, Cq.start_e, Cq.cap_e, Cq.mask_e, s), "mask");
-    if (grad) TRY_CUDA(c, cudaMemsetAsync(dQ[i], 0, sizeof(float) * 3 * nQ[i], s), "memset dQ");
+    // eps grid of Q with caller indices; its build clears dQ too
+    GridJob gj = eps_grid_xyz(Q[i], Cq, eps, Sc.g[0]);
+    if (grad) gj.zero = dQ[i], gj.zero_words = 3 * nQ[i];
+    TRY_CUDA(c, build_grids(&gj, 1, s), "grid");
     TRY_CUDA(c,
              launch_objective(P[i], (int)nP[i], Cq.ge, Cq.start_e, Cq.Xe, Tm, vd, eps, mu,
                               grad ? dE[i] : 1.0, grad ? 1 : 0, part, out7 + 7 * i, grad ? dP[i] : nullptr,

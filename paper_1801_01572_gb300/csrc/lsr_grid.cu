@@ -8,6 +8,8 @@
 // reads at most nine contiguous ranges.
 #include <float.h>
 
+#include <algorithm>
+
 #include "lsr_internal.cuh"
 
 namespace lsr {
@@ -21,24 +23,17 @@ __device__ __forceinline__ float3 load_xyz(const float *xyz, int i) {
   return make_float3(xyz[3 * i], xyz[3 * i + 1], xyz[3 * i + 2]);
 }
 
-// Per block: min (3), max (3), non-finite flag, count and coordinate sums (3)
-// of the finite points, as kBoxPart doubles.
-template <bool kF4>
-__global__ void __launch_bounds__(kBoxThreads) k_bbox_partial(const void *src, int n, double *partials) {
+// The partial of one block of points: min (3), max (3), non-finite flag, count
+// and coordinate sums (3) of the finite ones, as kBoxPart doubles.
+__device__ __forceinline__ void bbox_partial(const float *__restrict__ xyz, int n, int block, double *out) {
   float lo[3] = {FLT_MAX, FLT_MAX, FLT_MAX}, hi[3] = {-FLT_MAX, -FLT_MAX, -FLT_MAX};
   float bad = 0.f, cnt = 0.f;
   float sum[3] = {0.f, 0.f, 0.f};
-  int base = blockIdx.x * kBoxThreads * kBoxItems;
+  int base = block * kBoxThreads * kBoxItems;
   for (int k = 0; k < kBoxItems; ++k) {
     int i = base + k * kBoxThreads + threadIdx.x;
     if (i >= n) break;
-    float3 p;
-    if (kF4) {
-      float4 q = reinterpret_cast<const float4 *>(src)[i];
-      p = make_float3(q.x, q.y, q.z);
-    } else {
-      p = load_xyz(reinterpret_cast<const float *>(src), i);
-    }
+    const float3 p = load_xyz(xyz, i);
     if (!(isfinite(p.x) && isfinite(p.y) && isfinite(p.z))) {
       bad = 1.f;
       continue;
@@ -72,30 +67,50 @@ __global__ void __launch_bounds__(kBoxThreads) k_bbox_partial(const void *src, i
       double u = sm[k][t];
       v = t < 3 ? fmin(v, u) : (t < 7 ? fmax(v, u) : v + u);
     }
-    partials[(size_t)kBoxPart * blockIdx.x + t] = v;
+    out[t] = v;
   }
 }
 
-// box: min (3), max (3), non-finite flag, number of finite points, centroid (3).
-__global__ void k_bbox_final(const double *partials, int nblk, float *box) {
-  __shared__ double acc[kBoxPart];
-  int t = threadIdx.x;
-  if (t < kBoxPart) {
-    double v = partials[t];
-    for (int b = 1; b < nblk; ++b) {
-      double u = partials[(size_t)kBoxPart * b + t];
-      v = t < 3 ? fmin(v, u) : (t < 7 ? fmax(v, u) : v + u);
+// box from the nblk partials, combined in block order (a block of kBoxThreads
+// stages them in shared memory; combining straight from global memory was a
+// chain of 74 loads at 150k points, 14 to 25 us): min (3), max (3), non-finite
+// flag, number of finite points, centroid (3). Ends with a barrier.
+__device__ __forceinline__ void bbox_combine(const double *partials, int nblk, float *box) {
+  constexpr int kStage = 64;
+  __shared__ double st[kStage * kBoxPart], acc[kBoxPart];
+  const int t = threadIdx.x;
+  double v = 0.0;
+  for (int b0 = 0; b0 < nblk; b0 += kStage) {
+    const int nb = min(kStage, nblk - b0);
+    for (int k = t; k < nb * kBoxPart; k += kBoxThreads) st[k] = __ldcg(partials + (size_t)b0 * kBoxPart + k);
+    __syncthreads();
+    if (t < kBoxPart) {
+      if (b0 == 0) v = st[t];
+      for (int b = b0 == 0 ? 1 : 0; b < nb; ++b) {
+        const double u = st[b * kBoxPart + t];
+        v = t < 3 ? fmin(v, u) : (t < 7 ? fmax(v, u) : v + u);
+      }
     }
-    acc[t] = v;
+    __syncthreads();
   }
+  if (t < kBoxPart) acc[t] = v;
   __syncthreads();
   if (t < 8) box[t] = (float)acc[t];
   if (t >= 8 && t < 11) box[t] = acc[7] > 0.0 ? (float)(acc[t] / acc[7]) : 0.f;
   if (t == 11) box[t] = 0.f;
+  __threadfence_block();
+  __syncthreads();
 }
 
-__global__ void k_grid_params(const float *box, float radius, int npts, int cap, GridParams *g) {
-  if (threadIdx.x != 0) return;
+__global__ void __launch_bounds__(kBoxThreads) k_bbox_partial(const float *xyz, int n, double *partials) {
+  bbox_partial(xyz, n, blockIdx.x, partials + (size_t)kBoxPart * blockIdx.x);
+}
+
+__global__ void __launch_bounds__(kBoxThreads) k_bbox_final(const double *partials, int nblk, float *box) {
+  bbox_combine(partials, nblk, box);
+}
+
+__device__ void grid_params(const float *box, float radius, int npts, int cap, const unsigned *mask, GridParams *g) {
   GridParams q;
   float ext[3] = {box[3] - box[0], box[4] - box[1], box[5] - box[2]};
   // Cell coordinates (x - origin) / cell are computed in FP32 with a relative
@@ -138,48 +153,48 @@ __global__ void k_grid_params(const float *box, float radius, int npts, int cap,
   q.ncells = (int)(wx * wy * wz);
   q.npts = npts;
   q.pad_ = 0;
-  q.nbmask = nullptr;
+  q.nbmask = mask;
   *g = q;
 }
 
-// Dilate the occupied storage cells into their 3 x 3 x 3 neighbourhoods
+// Dilate the occupied storage cell c into its 3 x 3 x 3 neighbourhood
 // (neighbourhoods are symmetric, so a query cell's bit is set iff some point
 // lies in the block around it; wrapped axes dilate modulo the stored extent,
-// which can only add bits).
-__global__ void k_nbmask(const GridParams *gp, const int *start, unsigned *mask) {
-  const GridParams g = *gp;
-  bool wx = g.wx != g.nx, wy = g.wy != g.ny, wz = g.wz != g.nz;
-  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < g.ncells; c += gridDim.x * blockDim.x) {
-    if (start[c + 1] == start[c]) continue;
-    int sx = c % g.wx, sy = (c / g.wx) % g.wy, sz = c / (g.wx * g.wy);
-    for (int dz = -1; dz <= 1; ++dz) {
-      int z = sz + dz;
-      if (z < 0 || z >= g.wz) {
-        if (!wz) continue;
-        z = (z + g.wz) % g.wz;
+// which can only add bits). The x-adjacent bits of a row are set at once.
+__device__ __forceinline__ void dilate_cell(const GridParams &g, int c, unsigned *mask) {
+  const bool wx = g.wx != g.nx, wy = g.wy != g.ny, wz = g.wz != g.nz;
+  const int sx = c % g.wx, sy = (c / g.wx) % g.wy, sz = c / (g.wx * g.wy);
+  for (int dz = -1; dz <= 1; ++dz) {
+    int z = sz + dz;
+    if (z < 0 || z >= g.wz) {
+      if (!wz) continue;
+      z = (z + g.wz) % g.wz;
+    }
+    for (int dy = -1; dy <= 1; ++dy) {
+      int y = sy + dy;
+      if (y < 0 || y >= g.wy) {
+        if (!wy) continue;
+        y = (y + g.wy) % g.wy;
       }
-      for (int dy = -1; dy <= 1; ++dy) {
-        int y = sy + dy;
-        if (y < 0 || y >= g.wy) {
-          if (!wy) continue;
-          y = (y + g.wy) % g.wy;
+      const int row = (z * g.wy + y) * g.wx;
+      int word = -1;
+      unsigned bits = 0u;
+      for (int dx = -1; dx <= 1; ++dx) {
+        int x = sx + dx;
+        if (x < 0 || x >= g.wx) {
+          if (!wx) continue;
+          x = (x + g.wx) % g.wx;
         }
-        for (int dx = -1; dx <= 1; ++dx) {
-          int x = sx + dx;
-          if (x < 0 || x >= g.wx) {
-            if (!wx) continue;
-            x = (x + g.wx) % g.wx;
-          }
-          int s = (z * g.wy + y) * g.wx + x;
-          atomicOr(&mask[s >> 5], 1u << (s & 31));
+        const int t = row + x;
+        if ((t >> 5) != word) {
+          if (bits) atomicOr(mask + word, bits);
+          word = t >> 5, bits = 0u;
         }
+        bits |= 1u << (t & 31);
       }
+      if (bits) atomicOr(mask + word, bits);
     }
   }
-}
-
-__global__ void k_set_mask(GridParams *g, const unsigned *mask) {
-  if (threadIdx.x == 0) g->nbmask = mask;
 }
 
 __device__ __forceinline__ int clampi(int v, int lo, int hi) { return v < lo ? lo : (v > hi ? hi : v); }
@@ -191,57 +206,105 @@ __device__ __forceinline__ int cell_slot(const GridParams &g, float x, float y, 
   return ((cz % g.wz) * g.wy + (cy % g.wy)) * g.wx + (cx % g.wx);
 }
 
-template <bool kF4>
-__global__ void k_slots(const void *src, int n, const GridParams *gp, int *slot, int *counts) {
-  GridParams g = *gp;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+// Grids are built for up to kGridJobs clouds at once: blockIdx.y is the job.
+// At the library's sizes (5k to 200k points) every step is a launch of a few
+// microseconds, so what a build costs is the number of launches: six for any
+// number of grids, seven with a bounding box to find, where each grid used to
+// take twelve kernels and three memsets of its own.
+struct GridJobs {
+  GridJob j[kGridJobs];
+};
+
+// Clears the counts, the neighbourhood mask and the caller's array, and fills
+// the grid's parameters from a known box.
+__global__ void k_grid_begin(const __grid_constant__ GridJobs J) {
+  const GridJob &job = J.j[blockIdx.y];
+  const int t = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
+  auto zero = [&](void *p, int64_t words) {
+    if (!p) return;
+    int *w = static_cast<int *>(p);
+    // word by word up to a 16-byte boundary (a caller's array may start anywhere), then vectors
+    const int64_t head = min(words, (int64_t)(((16 - ((uintptr_t)p & 15)) & 15) >> 2)), vec = (words - head) / 4;
+    for (int64_t k = t; k < vec; k += step) reinterpret_cast<int4 *>(w + head)[k] = make_int4(0, 0, 0, 0);
+    for (int64_t k = t; k < words - 4 * vec; k += step) w[k < head ? k : k + 4 * vec] = 0;
+  };
+  zero(job.sc.counts, (int64_t)job.cap + 1);
+  zero(job.mask, job.mask ? job.cap / 32 + 2 : 0);
+  zero(job.zero, job.zero_words);
+  if (t == 0 && !job.box_part && !job.params_ready) grid_params(job.box, job.radius, job.n, job.cap, job.mask, job.g);
+}
+
+// Bounding box of the jobs that need one; the last block of a job to finish
+// (a ticket in the spare word after the counts) combines the partials in
+// block order and fills the grid's parameters.
+__global__ void __launch_bounds__(kBoxThreads) k_grid_bbox(const __grid_constant__ GridJobs J) {
+  const GridJob &job = J.j[blockIdx.y];
+  const int nblk = (job.n + kBoxThreads * kBoxItems - 1) / (kBoxThreads * kBoxItems);
+  if (!job.box_part || (int)blockIdx.x >= nblk) return;
+  __shared__ int s_last;
+  bbox_partial(job.xyz, job.n, blockIdx.x, job.box_part + (size_t)kBoxPart * blockIdx.x);
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(job.sc.counts + job.cap, 1) == nblk - 1;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  bbox_combine(job.box_part, nblk, job.box);
+  if (threadIdx.x == 0 && job.g) grid_params(job.box, job.radius, job.n, job.cap, job.mask, job.g);
+}
+
+// The cell of every point and its arrival number there.
+__global__ void k_grid_slots(const __grid_constant__ GridJobs J) {
+  const GridJob &job = J.j[blockIdx.y];
+  if (!job.out) return;
+  const GridParams g = *job.g;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < job.n; i += gridDim.x * blockDim.x) {
     float3 p;
-    if (kF4) {
-      float4 q = reinterpret_cast<const float4 *>(src)[i];
+    if (job.x4) {
+      const float4 q = job.x4[i];
       p = make_float3(q.x, q.y, q.z);
     } else {
-      p = load_xyz(reinterpret_cast<const float *>(src), i);
+      p = load_xyz(job.xyz, i * job.stride);
     }
-    int s = cell_slot(g, p.x, p.y, p.z);
-    slot[i] = s;
-    atomicAdd(&counts[s], 1);
+    const int s = cell_slot(g, p.x, p.y, p.z);
+    job.sc.slot[i] = s;
+    job.sc.rank[i] = atomicAdd(job.sc.counts + s, 1);
   }
 }
 
-__global__ void k_scatter(int n, const int *slot, const int *start, int *cursor, int *tmp) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    int s = slot[i];
-    tmp[start[s] + atomicAdd(&cursor[s], 1)] = i;
-  }
+__global__ void k_grid_scatter(const __grid_constant__ GridJobs J) {
+  const GridJob &job = J.j[blockIdx.y];
+  if (!job.out) return;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < job.n; i += gridDim.x * blockDim.x)
+    job.sc.tmp[job.start[job.sc.slot[i]] + job.sc.rank[i]] = i;
 }
 
-// One warp per cell: order the cell's entries by source index (rank = number
-// of smaller indices in the cell) and write the sorted points.
-template <bool kF4>
-__global__ void k_cell_order(const void *src, const GridParams *gp, const int *start, const int *tmp, float4 *out,
-                             int *inv_out) {
-  int ncells = gp->ncells;
-  int lane = threadIdx.x & 31;
-  int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  int nwarps = (gridDim.x * blockDim.x) >> 5;
-  for (int c = warp; c < ncells; c += nwarps) {
-    int b = start[c], e = start[c + 1];
-    for (int t = b + lane; t < e; t += 32) {
-      int v = tmp[t];
-      int rank = 0;
-      for (int u = b; u < e; ++u) rank += tmp[u] < v;
-      int k = b + rank;
-      float4 o;
-      if (kF4) {
-        o = reinterpret_cast<const float4 *>(src)[v];
-      } else {
-        float3 p = load_xyz(reinterpret_cast<const float *>(src), v);
-        o = make_float4(p.x, p.y, p.z, 0.f);
-      }
-      o.w = __int_as_float(v);
-      out[k] = o;
-      if (inv_out) inv_out[v] = k;
+// A thread per point, in cell order: its place among the cell's points by
+// source index (the arrival order is arbitrary, the result is not), and, once
+// per occupied cell, the neighbourhood mask. (A warp per cell walked mostly
+// empty cells: two dependent loads for each of up to 400k cells.)
+__global__ void k_grid_order(const __grid_constant__ GridJobs J) {
+  const GridJob &job = J.j[blockIdx.y];
+  if (!job.out) return;
+  const int *__restrict__ tmp = job.sc.tmp;
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < job.n; t += gridDim.x * blockDim.x) {
+    const int v = tmp[t];
+    const int c = job.sc.slot[v];
+    const int b = job.start[c], e = job.start[c + 1];
+    float4 o;
+    if (job.x4) {
+      o = job.x4[v];
+    } else {
+      const float3 p = load_xyz(job.xyz, v * job.stride);
+      o = make_float4(p.x, p.y, p.z, 0.f);
     }
+    int rank = 0;
+#pragma unroll 4
+    for (int u = b; u < e; ++u) rank += tmp[u] < v;
+    o.w = __int_as_float(job.carry_pos ? b + rank : v);
+    job.out[b + rank] = o;
+    if (job.inv) job.inv[v] = b + rank;
+    if (job.mask && t == b) dilate_cell(*job.g, c, job.mask);
   }
 }
 
@@ -274,64 +337,101 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int *sm_warp, int *to
   return warp_off + x - v;
 }
 
-// Scans in[0..n] with in[n] taken as 0, so out[n] is the total.
-__global__ void __launch_bounds__(kScanThreads) k_scan_local(const int *in, int *out, const int *n_dev, int *block_sums) {
+// Exclusive scans in two launches: the sum of every tile, then each tile adds
+// up the sums before its own (at most kScanTiles of them) and scans itself.
+// Tiles grow with the capacity so that there are never more.
+constexpr int kScanTiles = 1024;
+__host__ __device__ __forceinline__ int64_t scan_tile_size(int64_t cap) {
+  const int64_t parts = (cap + kScanTile) / kScanTile;  // of kScanTile entries, cap + 1 in all
+  return (parts + kScanTiles - 1) / kScanTiles * kScanTile;
+}
+
+__device__ __forceinline__ int block_sum(int v, int *sm_warp) {
+  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+  if ((threadIdx.x & 31) == 0) sm_warp[threadIdx.x >> 5] = v;
+  __syncthreads();
+  int t = 0;
+  for (int w = 0; w < kScanThreads / 32; ++w) t += sm_warp[w];
+  __syncthreads();
+  return t;
+}
+
+// in (256-byte aligned): n entries; sums[tile] for the tiles that begin before n.
+__device__ __forceinline__ void scan_tile_sum(const int *__restrict__ in, int n, int64_t tile, int *__restrict__ sums) {
   __shared__ int sm[kScanThreads / 32];
-  int n1 = *n_dev + 1;
-  int base = blockIdx.x * kScanTile;
-  if (base >= n1) {
-    if (threadIdx.x == 0) block_sums[blockIdx.x] = 0;
-    return;
-  }
-  int v[kScanItems];
+  const int64_t base = (int64_t)blockIdx.x * tile;
+  if (base >= n) return;
+  const int64_t end = base + tile < n ? base + tile : n;
   int sum = 0;
-  int i0 = base + threadIdx.x * kScanItems;
-  for (int k = 0; k < kScanItems; ++k) {
-    int i = i0 + k;
-    v[k] = (i < n1 - 1) ? in[i] : 0;
-    sum += v[k];
+  for (int64_t i = base + 4 * (int)threadIdx.x; i < end; i += 4 * kScanThreads) {
+    if (i + 3 < end) {
+      const int4 q = *reinterpret_cast<const int4 *>(in + i);
+      sum += q.x + q.y + q.z + q.w;
+    } else {
+      for (int64_t k = i; k < end; ++k) sum += in[k];
+    }
   }
-  int total;
-  int pre = block_exclusive_scan(sum, sm, &total);
-  for (int k = 0; k < kScanItems; ++k) {
-    int i = i0 + k;
-    if (i < n1) out[i] = pre;
-    pre += v[k];
-  }
-  if (threadIdx.x == 0) block_sums[blockIdx.x] = total;
+  sum = block_sum(sum, sm);
+  if (threadIdx.x == 0) sums[blockIdx.x] = sum;
 }
 
-__global__ void __launch_bounds__(kScanThreads) k_scan_blocks(int *block_sums, int nblocks) {
+// out[0..n] = exclusive scan of in[0..n), out[n] = the total.
+__device__ __forceinline__ void scan_tile_write(const int *__restrict__ in, int n, int64_t tile,
+                                                const int *__restrict__ sums, int *__restrict__ out) {
   __shared__ int sm[kScanThreads / 32];
+  const int64_t base = (int64_t)blockIdx.x * tile;
+  if (base > n) return;
   int carry = 0;
-  for (int base = 0; base < nblocks; base += kScanThreads) {
-    int i = base + threadIdx.x;
-    int v = i < nblocks ? block_sums[i] : 0;
+  for (int k = threadIdx.x; k < (int)blockIdx.x; k += kScanThreads) carry += sums[k];
+  carry = block_sum(carry, sm);
+  const int64_t end = base + tile < (int64_t)n + 1 ? base + tile : (int64_t)n + 1;
+  for (int64_t b = base; b < end; b += kScanTile) {
+    const int64_t i0 = b + threadIdx.x * kScanItems;
+    int v[kScanItems];
+    int sum = 0;
+    if (i0 + kScanItems <= n) {
+      const int4 q0 = reinterpret_cast<const int4 *>(in + i0)[0], q1 = reinterpret_cast<const int4 *>(in + i0)[1];
+      v[0] = q0.x, v[1] = q0.y, v[2] = q0.z, v[3] = q0.w, v[4] = q1.x, v[5] = q1.y, v[6] = q1.z, v[7] = q1.w;
+    } else {
+#pragma unroll
+      for (int k = 0; k < kScanItems; ++k) v[k] = i0 + k < n ? in[i0 + k] : 0;
+    }
+#pragma unroll
+    for (int k = 0; k < kScanItems; ++k) sum += v[k];
     int total;
-    int pre = block_exclusive_scan(v, sm, &total);
-    if (i < nblocks) block_sums[i] = carry + pre;
+    int pre = carry + block_exclusive_scan(sum, sm, &total);
     carry += total;
+#pragma unroll
+    for (int k = 0; k < kScanItems; ++k) {
+      const int c = v[k];
+      v[k] = pre;
+      pre += c;
+    }
+    if (i0 + kScanItems <= end) {
+      reinterpret_cast<int4 *>(out + i0)[0] = make_int4(v[0], v[1], v[2], v[3]);
+      reinterpret_cast<int4 *>(out + i0)[1] = make_int4(v[4], v[5], v[6], v[7]);
+    } else {
+#pragma unroll
+      for (int k = 0; k < kScanItems; ++k)
+        if (i0 + k < end) out[i0 + k] = v[k];
+    }
   }
 }
 
-__global__ void __launch_bounds__(kScanThreads) k_scan_add(int *out, const int *n_dev, const int *block_sums) {
-  int n1 = *n_dev + 1;
-  int base = blockIdx.x * kScanTile;
-  if (base >= n1 || blockIdx.x == 0) return;
-  int add = block_sums[blockIdx.x];
-  for (int k = threadIdx.x; k < kScanTile; k += kScanThreads) {
-    int i = base + k;
-    if (i < n1) out[i] += add;
-  }
+__global__ void __launch_bounds__(kScanThreads) k_scan_sums(const int *in, const int *n_dev, int64_t tile, int *sums) {
+  scan_tile_sum(in, *n_dev, tile, sums);
 }
-
-__global__ void k_ncells_ptr(const GridParams *g, int *dst) {
-  if (threadIdx.x == 0) *dst = g->ncells;
+__global__ void __launch_bounds__(kScanThreads) k_scan_write(const int *in, const int *n_dev, int64_t tile,
+                                                             const int *sums, int *out) {
+  scan_tile_write(in, *n_dev, tile, sums, out);
 }
-
-inline int grid_blocks(int n, int threads = 256) {
-  int b = (int)lsr_div_up(n, threads);
-  return b < 1 ? 1 : (b > 65535 * 8 ? 65535 * 8 : b);
+__global__ void __launch_bounds__(kScanThreads) k_grid_sums(const __grid_constant__ GridJobs J) {
+  const GridJob &job = J.j[blockIdx.y];
+  if (job.out) scan_tile_sum(job.sc.counts, job.g->ncells, scan_tile_size(job.cap), job.sc.scan);
+}
+__global__ void __launch_bounds__(kScanThreads) k_grid_starts(const __grid_constant__ GridJobs J) {
+  const GridJob &job = J.j[blockIdx.y];
+  if (job.out) scan_tile_write(job.sc.counts, job.g->ncells, scan_tile_size(job.cap), job.sc.scan, job.start);
 }
 
 }  // namespace
@@ -341,70 +441,50 @@ int bbox_blocks(int n) { return (int)lsr_div_up(n > 0 ? n : 1, kBoxThreads * kBo
 cudaError_t launch_bbox_xyz(const float *xyz, int n, double *partials, int nblk_cap, float *box, cudaStream_t s) {
   int nb = bbox_blocks(n);
   if (nb > nblk_cap) return cudaErrorInvalidValue;
-  LSR_LAUNCH(k_bbox_partial<false><<<nb, kBoxThreads, 0, s>>>(xyz, n, partials));
-  LSR_LAUNCH(k_bbox_final<<<1, 32, 0, s>>>(partials, nb, box));
-  return cudaGetLastError();
-}
-
-cudaError_t launch_bbox_f4(const float4 *x, int n, double *partials, int nblk_cap, float *box, cudaStream_t s) {
-  int nb = bbox_blocks(n);
-  if (nb > nblk_cap) return cudaErrorInvalidValue;
-  LSR_LAUNCH(k_bbox_partial<true><<<nb, kBoxThreads, 0, s>>>(x, n, partials));
-  LSR_LAUNCH(k_bbox_final<<<1, 32, 0, s>>>(partials, nb, box));
-  return cudaGetLastError();
-}
-
-cudaError_t launch_grid_params(const float *box, float radius, int npts, int cap_cells, GridParams *g, cudaStream_t s) {
-  LSR_LAUNCH(k_grid_params<<<1, 32, 0, s>>>(box, radius, npts, cap_cells, g));
+  LSR_LAUNCH(k_bbox_partial<<<nb, kBoxThreads, 0, s>>>(xyz, n, partials));
+  LSR_LAUNCH(k_bbox_final<<<1, kBoxThreads, 0, s>>>(partials, nb, box));
   return cudaGetLastError();
 }
 
 int64_t nbmask_words(int cap_cells) { return cap_cells / 32 + 2; }
 
-cudaError_t build_nbmask(GridParams *g, const int *start, int cap_cells, unsigned *mask, cudaStream_t s) {
-  LSR_CUDA_TRY(cudaMemsetAsync(mask, 0, sizeof(unsigned) * (size_t)nbmask_words(cap_cells), s));
-  int b = (int)lsr_div_up(cap_cells, 256);
-  LSR_LAUNCH(k_nbmask<<<b < kSms * 16 ? b : kSms * 16, 256, 0, s>>>(g, start, mask));
-  LSR_LAUNCH(k_set_mask<<<1, 32, 0, s>>>(g, mask));
-  return cudaGetLastError();
-}
-
 int64_t scan_scratch_ints(int64_t n) { return lsr_div_up(n + 1, kScanTile) + 64; }
 
 cudaError_t scan_exclusive(const int *in, int *out, const int *n_dev, int cap, int *scratch, cudaStream_t s) {
-  int nblocks = (int)lsr_div_up((int64_t)cap + 1, kScanTile);
-  LSR_LAUNCH(k_scan_local<<<nblocks, kScanThreads, 0, s>>>(in, out, n_dev, scratch));
-  LSR_LAUNCH(k_scan_blocks<<<1, kScanThreads, 0, s>>>(scratch, nblocks));
-  LSR_LAUNCH(k_scan_add<<<nblocks, kScanThreads, 0, s>>>(out, n_dev, scratch));
+  const int64_t tile = scan_tile_size(cap);
+  const int nb = (int)lsr_div_up((int64_t)cap + 1, tile);
+  LSR_LAUNCH(k_scan_sums<<<nb, kScanThreads, 0, s>>>(in, n_dev, tile, scratch));
+  LSR_LAUNCH(k_scan_write<<<nb, kScanThreads, 0, s>>>(in, n_dev, tile, scratch, out));
   return cudaGetLastError();
 }
 
-template <bool kF4>
-static cudaError_t build_grid_impl(const void *src, int n, const GridParams *g, int cap_cells, int *start, float4 *out,
-                                   int *inv_out, GridScratch sc, cudaStream_t s) {
-  LSR_CUDA_TRY(cudaMemsetAsync(sc.counts, 0, sizeof(int) * ((size_t)cap_cells + 1), s));
-  LSR_LAUNCH(k_slots<kF4><<<grid_blocks(n), 256, 0, s>>>(src, n, g, sc.slot, sc.counts));
-  // the cell count lives in device memory; keep a copy next to the counts
-  int *ncells_dev = sc.counts + cap_cells;  // counts[cap] is never used as a cell
-  LSR_LAUNCH(k_ncells_ptr<<<1, 32, 0, s>>>(g, ncells_dev));
-  LSR_CUDA_TRY(scan_exclusive(sc.counts, start, ncells_dev, cap_cells, sc.scan, s));
-  LSR_CUDA_TRY(cudaMemsetAsync(sc.counts, 0, sizeof(int) * (size_t)cap_cells, s));
-  LSR_LAUNCH(k_scatter<<<grid_blocks(n), 256, 0, s>>>(n, sc.slot, start, sc.counts, sc.tmp));
-  // warps stride over the cells (most are empty: a block per cell would spend
-  // the kernel on scheduling blocks)
-  const int cells_warps = cap_cells < kSms * 16 * 8 ? cap_cells : kSms * 16 * 8;
-  LSR_LAUNCH(k_cell_order<kF4><<<grid_blocks(cells_warps * 32, 256), 256, 0, s>>>(src, g, start, sc.tmp, out, inv_out));
+cudaError_t build_grids(const GridJob *jobs, int count, cudaStream_t s) {
+  for (int j0 = 0; j0 < count; j0 += kGridJobs) {
+    GridJobs J{};
+    const int nj = count - j0 < kGridJobs ? count - j0 : kGridJobs;
+    int64_t words = 1, npts = 1, tiles = 1;
+    int boxes = 0, grids = 0;
+    for (int j = 0; j < nj; ++j) {
+      const GridJob &q = J.j[j] = jobs[j0 + j];
+      words = std::max(words, std::max((int64_t)q.cap + 1, q.zero_words));
+      if (q.box_part) boxes = std::max(boxes, bbox_blocks(q.n));
+      if (!q.out) continue;
+      ++grids;
+      npts = std::max(npts, (int64_t)q.n);
+      tiles = std::max(tiles, lsr_div_up((int64_t)q.cap + 1, scan_tile_size(q.cap)));
+    }
+    const int zb = (int)std::min<int64_t>(lsr_div_up(words, 4 * 256), kSms * 8);
+    const int pb = (int)lsr_div_up(npts, 256);
+    LSR_LAUNCH(k_grid_begin<<<dim3(zb, nj), 256, 0, s>>>(J));
+    if (boxes) LSR_LAUNCH(k_grid_bbox<<<dim3(boxes, nj), kBoxThreads, 0, s>>>(J));
+    if (!grids) continue;
+    LSR_LAUNCH(k_grid_slots<<<dim3(pb, nj), 256, 0, s>>>(J));
+    LSR_LAUNCH(k_grid_sums<<<dim3((int)tiles, nj), kScanThreads, 0, s>>>(J));
+    LSR_LAUNCH(k_grid_starts<<<dim3((int)tiles, nj), kScanThreads, 0, s>>>(J));
+    LSR_LAUNCH(k_grid_scatter<<<dim3(pb, nj), 256, 0, s>>>(J));
+    LSR_LAUNCH(k_grid_order<<<dim3(pb, nj), 256, 0, s>>>(J));
+  }
   return cudaGetLastError();
-}
-
-cudaError_t build_grid_xyz(const float *xyz, int n, const GridParams *g, int cap_cells, int *start, float4 *out,
-                           int *inv_out, GridScratch sc, cudaStream_t s) {
-  return build_grid_impl<false>(xyz, n, g, cap_cells, start, out, inv_out, sc, s);
-}
-
-cudaError_t build_grid_f4(const float4 *x, int n, const GridParams *g, int cap_cells, int *start, float4 *out,
-                          GridScratch sc, cudaStream_t s) {
-  return build_grid_impl<true>(x, n, g, cap_cells, start, out, nullptr, sc, s);
 }
 
 }  // namespace lsr

@@ -440,39 +440,57 @@ __device__ __forceinline__ int warp_sum(int v) {
 }
 
 // ----------------------------------------------------------------- grid build (lsr_grid.cu)
-// Bounding box and centroid of a float32 xyz array (AoS) or a float4 array,
-// reduced through kBoxPart doubles per block into box[kBox] = (min xyz, max
-// xyz, non-finite flag, finite count, centroid xyz, 0).
+// Bounding box and centroid of a float32 xyz array, reduced through kBoxPart
+// doubles per block into box[kBox] = (min xyz, max xyz, non-finite flag,
+// finite count, centroid xyz, 0).
 constexpr int kBox = 12;
 constexpr int kBoxPart = 11;
 cudaError_t launch_bbox_xyz(const float *xyz, int n, double *partials, int nblk_cap, float *box, cudaStream_t s);
-cudaError_t launch_bbox_f4(const float4 *x, int n, double *partials, int nblk_cap, float *box, cudaStream_t s);
 int bbox_blocks(int n);
 
-// Fill a GridParams from a bounding box on the device (no neighbourhood mask).
-cudaError_t launch_grid_params(const float *box, float radius, int npts, int cap_cells, GridParams *g, cudaStream_t s);
-// Build the neighbourhood bitmap of a built grid (nbmask_words(cap) words)
-// and attach it to g.
+// Words of a neighbourhood mask: a bit per storage cell, set if the 3 x 3 x 3
+// block around the cell holds a point.
 int64_t nbmask_words(int cap_cells);
-cudaError_t build_nbmask(GridParams *g, const int *start, int cap_cells, unsigned *mask, cudaStream_t s);
 
-// Counting sort of points into the grid: out[k] = point sorted k-th by (cell,
-// source index) with w replaced by the carried index (source index if
-// carry == nullptr). start gets the exclusive cell offsets (ncells + 1).
-// Scratch: slot (n ints), counts (cap + 1 ints), scan scratch (scan_scratch_ints(cap)).
+// Scratch of one grid build: slot, rank and tmp of n ints, counts of cap + 1,
+// scan of scan_scratch_ints(cap).
 struct GridScratch {
   int *slot;
+  int *rank;
   int *counts;
-  int *tmp;       // n ints
-  int *scan;      // scan_scratch_ints(cap + 1)
+  int *tmp;
+  int *scan;
 };
 int64_t scan_scratch_ints(int64_t n);
-cudaError_t build_grid_xyz(const float *xyz, int n, const GridParams *g, int cap_cells, int *start, float4 *out,
-                           int *inv_out, GridScratch sc, cudaStream_t s);
-cudaError_t build_grid_f4(const float4 *x, int n, const GridParams *g, int cap_cells, int *start, float4 *out,
-                          GridScratch sc, cudaStream_t s);
 
-// Exclusive scan of in[0..*n_dev) into out[0..*n_dev] (out[n] = total).
+// One grid to build: a counting sort of the source points into cells of the
+// radius (out[k] = the point sorted k-th by (cell, source index), w = its
+// source index; start: the exclusive cell offsets, ncells + 1).
+struct GridJob {
+  const float *xyz = nullptr;      // source: n xyz triples,
+  const float4 *x4 = nullptr;      // or n packed points
+  int stride = 1;                  // point i is xyz[i * stride]
+  int n = 0, cap = 0;              // cap: capacity in cells of start, counts and the mask
+  float radius = 0.f;
+  float *box = nullptr;            // the source's box: read, or found from xyz when box_part is given
+  double *box_part = nullptr;      // kBoxPart doubles per bbox_blocks(n)
+  bool params_ready = false;       // *g is filled already (box is not needed)
+  GridParams *g = nullptr;
+  int *start = nullptr;
+  float4 *out = nullptr;           // null: the box only (g may then be null too)
+  bool carry_pos = false;          // w = the sorted index itself instead of the source index
+  int *inv = nullptr;              // optional: source index -> sorted index
+  unsigned *mask = nullptr;        // optional: nbmask_words(cap) words, attached to g (not with params_ready)
+  float *zero = nullptr;           // optional: another array to clear, zero_words of it
+  int64_t zero_words = 0;
+  GridScratch sc{};
+};
+constexpr int kGridJobs = 16;      // jobs of one launch (kernel parameters)
+// Builds the grids together, kGridJobs at a time; the jobs' buffers must not overlap.
+cudaError_t build_grids(const GridJob *jobs, int count, cudaStream_t s);
+
+// Exclusive scan of in[0..*n_dev) into out[0..*n_dev] (out[n] = total); in and
+// out are 16-byte aligned, *n_dev <= cap, scratch: scan_scratch_ints(cap).
 cudaError_t scan_exclusive(const int *in, int *out, const int *n_dev, int cap, int *scratch, cudaStream_t s);
 
 // ----------------------------------------------------------------- features (lsr_features.cu)

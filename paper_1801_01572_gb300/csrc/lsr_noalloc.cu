@@ -125,6 +125,7 @@ extern "C" int lsr_consensus_static(const float *P, int64_t nP, const float *Q, 
   unsigned *mask = a.take<unsigned>((size_t)nbmask_words(kStaticCapCells));
   GridScratch sc;
   sc.slot = a.take<int>(nQ);
+  sc.rank = a.take<int>(nQ);
   sc.tmp = a.take<int>(nQ);
   sc.counts = a.take<int>((size_t)kStaticCapCells + 1);
   sc.scan = a.take<int>((size_t)scan_scratch_ints(kStaticCapCells));
@@ -148,10 +149,11 @@ extern "C" int lsr_consensus_static(const float *P, int64_t nP, const float *Q, 
   LSR_LAUNCH(k_pack_static<<<blocks_for(nP), 256, 0, s>>>(p, (int)nP, XP));
   // the eps grid of Q (the array keeps the previous call's contents: every
   // piece below is fully rewritten, and the sums are cleared)
-  LSR_STATIC_TRY(launch_bbox_xyz(q, (int)nQ, box_part, bbox_blocks((int)nQ), box, s));
-  LSR_STATIC_TRY(launch_grid_params(box, eps, (int)nQ, kStaticCapCells, ge, s));
-  LSR_STATIC_TRY(build_grid_xyz(q, (int)nQ, ge, kStaticCapCells, start, Xe, inv, sc, s));
-  LSR_STATIC_TRY(build_nbmask(ge, start, kStaticCapCells, mask, s));
+  GridJob gj;
+  gj.xyz = q, gj.n = (int)nQ, gj.cap = kStaticCapCells, gj.radius = eps;
+  gj.box = box, gj.box_part = box_part;
+  gj.g = ge, gj.start = start, gj.out = Xe, gj.inv = inv, gj.mask = mask, gj.sc = sc;
+  LSR_STATIC_TRY(build_grids(&gj, 1, s));
   LSR_STATIC_TRY(cudaMemsetAsync(cnt, 0, sizeof(int) * nh, s));
   LSR_STATIC_TRY(cudaMemsetAsync(sum, 0, sizeof(unsigned long long) * nh, s));
   LSR_STATIC_TRY(launch_consensus(XP, (int)nP, ge, start, Xe, pose, nullptr, nullptr, (int)nh, eps, cnt, sum, s));
