@@ -638,6 +638,17 @@ GridJob eps_cloud(const float *xyz, CloudLayout &c, float eps, const GridScratch
   return j;
 }
 
+// Neighbours in a cloud's eps grid of P moved by T (rounded to FP32).
+PoseNnJob pose_nn_job(const float *P, int64_t nP, const CloudLayout &c, const double *T, float eps, int *nn) {
+  PoseNnJob j{};
+  j.P = P, j.nP = (int)nP, j.g = c.ge, j.start = c.start_e, j.Xe = c.Xe, j.eps2 = eps * eps, j.nn = nn;
+  for (int r = 0; r < 3; ++r) {
+    for (int q = 0; q < 3; ++q) j.R[3 * r + q] = (float)T[4 * r + q];
+    j.t[r] = (float)T[4 * r + 3];
+  }
+  return j;
+}
+
 // The grids of a registration: both feature grids, then the grids over them.
 cudaError_t build_pair(const float *P, const float *Q, const CloudLayout &Pc, const CloudLayout &Qc, float r_f,
                        float r_n, float eps, const ScratchLayout &sc, cudaStream_t s) {
@@ -2170,6 +2181,7 @@ int lsr_pose_implicit_grad(lsr_ctx *c, const float *P, int64_t nP, const float *
     CloudLayout Cq;
     ScratchLayout S;
     double *part, *out, *dl;
+    int *nn;
   };
   const bool dev_out = is_device_ptr(dP);
   if (dev_out != is_device_ptr(dQ)) return set_err(c, LSR_E_ARG, "dP and dQ must both be device or both host");
@@ -2182,6 +2194,7 @@ int lsr_pose_implicit_grad(lsr_ctx *c, const float *P, int64_t nP, const float *
     b.part = a.take<double>((size_t)implicit_partials((int)nP));
     b.out = a.take<double>(50);
     b.dl = a.take<double>(6);
+    b.nn = a.take<int>(nP);
   };
   Arena m(nullptr);
   Bufs bm;
@@ -2200,9 +2213,10 @@ int lsr_pose_implicit_grad(lsr_ctx *c, const float *P, int64_t nP, const float *
   gj.zero = gq, gj.zero_words = 3 * nQ;
   TRY_CUDA(c, build_grids(&gj, 1, s), "grid");
   TRY_CUDA(c, cudaMemcpyAsync(b.dl, dl, sizeof(dl), cudaMemcpyHostToDevice, s), "H2D");
+  const PoseNnJob nj = pose_nn_job(psrc, nP, b.Cq, T, eps, b.nn);
+  TRY_CUDA(c, launch_pose_nn(&nj, 1, s), "neighbours");
   TRY_CUDA(c,
-           launch_implicit(psrc, (int)nP, b.Cq.ge, b.Cq.start_e, b.Cq.Xe, (int)nQ, T, eps, (double)mu, b.dl, b.part,
-                           b.out, gp, gq, s),
+           launch_implicit(psrc, (int)nP, b.nn, b.Cq.Xe, (int)nQ, T, (double)mu, b.dl, b.part, b.out, gp, gq, s),
            "implicit");
   double host[50];
   TRY_CUDA(c, cudaMemcpyAsync(host, b.out, sizeof(host), cudaMemcpyDeviceToHost, s), "D2H");
@@ -2407,69 +2421,90 @@ static int objective_impl(lsr_ctx *c, int32_t n, const float *const *P, const in
   if (n < 0 || (n > 0 && (!P || !nP || !Q || !nQ || !xi || !T0)) || !(eps > 0.f && eps <= 10.f) || !(mu > 0.f) ||
       (!grad && !E) || (grad && (!dP || !dQ || !dxi)))
     return set_err(c, LSR_E_ARG, "bad argument");
-  int64_t maxP = 0, maxQ = 0;
   for (int i = 0; i < n; ++i) {
     if (!P[i] || !Q[i] || nP[i] < 1 || nQ[i] < 1 || nP[i] > kMaxPoints || nQ[i] > kMaxPoints)
       return set_err(c, LSR_E_ARG, "bad cloud");
     if (!is_device_ptr(P[i]) || !is_device_ptr(Q[i])) return set_err(c, LSR_E_ARG, "objective clouds must be on the device");
     if (grad && (!dP[i] || !dQ[i] || !is_device_ptr(dP[i]) || !is_device_ptr(dQ[i])))
       return set_err(c, LSR_E_ARG, "objective gradients must be device arrays");
-    maxP = std::max(maxP, nP[i]);
-    maxQ = std::max(maxQ, nQ[i]);
   }
   if (n == 0) return LSR_OK;
-  // pairs round-robin over S lanes (own stream and workspace each): at these
-  // sizes every pair is a chain of short launches, and the lanes overlap them
-  const int nl = std::max(1, std::min((int)n, c->prm.batch_streams > 0 ? c->prm.batch_streams : 4));
-  auto plan = [&](Arena &a, CloudLayout &Cq, ScratchLayout &Sc, double *&part) {
-    plan_cloud(a, (int)maxQ, false, false, true, Cq);
-    plan_scratch(a, (int)maxQ, Cq.cap_f, Sc);
-    part = a.take<double>((size_t)7 * objective_blocks((int)maxP));
+  // Up to kPoseJobs pairs go through every step together (a pair's step at
+  // these sizes is a launch of a few microseconds): as many as their workspace
+  // allows, one at least.
+  auto plan = [&](Arena &a, int i, CloudLayout &Cq, ScratchLayout &Sc, double *&part, int *&nn) {
+    plan_cloud(a, (int)nQ[i], false, false, true, Cq);
+    plan_scratch(a, (int)nQ[i], Cq.cap_e, Sc);
+    part = a.take<double>((size_t)7 * objective_blocks((int)nP[i]));
+    nn = a.take<int>(nP[i]);
   };
-  Arena m(nullptr);
-  CloudLayout q1;
-  ScratchLayout q2;
-  double *q3;
-  plan(m, q1, q2, q3);
-  if ((rc = ensure_lanes(c, nl, m.off))) return rc;
-  if ((rc = ensure_ws(c, sizeof(double) * 7 * (size_t)n))) return rc;
-  double *out7 = reinterpret_cast<double *>(c->ws);
-  TRY_CUDA(c, cudaEventRecord(c->fork, c->stream), "fork");
-  for (int l = 0; l < nl; ++l) TRY_CUDA(c, cudaStreamWaitEvent(c->lanes[l], c->fork, 0), "fork");
-  std::vector<double> host7((size_t)7 * n);
-  for (int i = 0; i < n; ++i) {
-    const int l = i % nl;
-    cudaStream_t s = c->lanes[l];
-    Arena a(c->lane_ws[l]);
-    CloudLayout Cq;
-    ScratchLayout Sc;
-    double *part;
-    plan(a, Cq, Sc, part);
-    Cq.n = (int)nQ[i];
-    const double *w = xi + 6 * i, *T = T0 + 16 * i;
-    double Rw[9], Tm[16];
-    host_exp_so3(w, Rw);
-    double M[16] = {Rw[0], Rw[1], Rw[2], w[3], Rw[3], Rw[4], Rw[5], w[4], Rw[6], Rw[7], Rw[8], w[5], 0, 0, 0, 1};
-    for (int r = 0; r < 4; ++r)
-      for (int q = 0; q < 4; ++q) {
-        double acc = 0.0;
-        for (int k = 0; k < 4; ++k) acc += M[4 * r + k] * T[4 * k + q];
-        Tm[4 * r + q] = acc;
+  constexpr size_t kChunkBytes = (size_t)1 << 30;
+  const size_t out_bytes = sizeof(double) * 7 * (size_t)n + kAlign;
+  std::vector<int> first{0};  // chunks of consecutive pairs
+  size_t most = 0;
+  {
+    Arena m(nullptr);
+    for (int i = 0; i < n; ++i) {
+      CloudLayout q1;
+      ScratchLayout q2;
+      double *q3;
+      int *q4;
+      const size_t before = m.off;
+      plan(m, i, q1, q2, q3, q4);
+      if (i > first.back() && (i - first.back() == kPoseJobs || m.off > kChunkBytes)) {
+        first.push_back(i);
+        m.off = m.off - before + kAlign;
       }
-    const double vd[3] = {w[3], w[4], w[5]};
-    // eps grid of Q with caller indices; its build clears dQ too
-    GridJob gj = eps_grid_xyz(Q[i], Cq, eps, Sc.g[0]);
-    if (grad) gj.zero = dQ[i], gj.zero_words = 3 * nQ[i];
-    TRY_CUDA(c, build_grids(&gj, 1, s), "grid");
-    TRY_CUDA(c,
-             launch_objective(P[i], (int)nP[i], Cq.ge, Cq.start_e, Cq.Xe, Tm, vd, eps, mu,
-                              grad ? dE[i] : 1.0, grad ? 1 : 0, part, out7 + 7 * i, grad ? dP[i] : nullptr,
-                              grad ? dQ[i] : nullptr, s),
-             "objective");
+      most = std::max(most, m.off);
+    }
+    first.push_back(n);
   }
-  for (int l = 0; l < nl; ++l) {
-    TRY_CUDA(c, cudaEventRecord(c->lane_done[l], c->lanes[l]), "join");
-    TRY_CUDA(c, cudaStreamWaitEvent(c->stream, c->lane_done[l], 0), "join");
+  if ((rc = ensure_ws(c, out_bytes + most))) return rc;
+  double *out7 = reinterpret_cast<double *>(c->ws);
+  cudaStream_t s = c->stream;
+  std::vector<double> host7((size_t)7 * n);
+  for (size_t k = 0; k + 1 < first.size(); ++k) {
+    Arena a(c->ws);
+    a.off = out_bytes;
+    GridJob gj[kPoseJobs];
+    PoseNnJob nj[kPoseJobs];
+    ObjJob oj[kPoseJobs];
+    const int i0 = first[k], m = first[k + 1] - i0;
+    for (int u = 0; u < m; ++u) {
+      const int i = i0 + u;
+      CloudLayout Cq;
+      ScratchLayout Sc;
+      double *part;
+      int *nn;
+      plan(a, i, Cq, Sc, part, nn);
+      const double *w = xi + 6 * i, *T = T0 + 16 * i;
+      double Rw[9], Tm[16];
+      host_exp_so3(w, Rw);
+      double M[16] = {Rw[0], Rw[1], Rw[2], w[3], Rw[3], Rw[4], Rw[5], w[4], Rw[6], Rw[7], Rw[8], w[5], 0, 0, 0, 1};
+      for (int r = 0; r < 4; ++r)
+        for (int q = 0; q < 4; ++q) {
+          double acc = 0.0;
+          for (int d = 0; d < 4; ++d) acc += M[4 * r + d] * T[4 * d + q];
+          Tm[4 * r + q] = acc;
+        }
+      // eps grid of Q with caller indices; its build clears dQ too
+      gj[u] = eps_grid_xyz(Q[i], Cq, eps, Sc.g[0]);
+      if (grad) gj[u].zero = dQ[i], gj[u].zero_words = 3 * nQ[i];
+      nj[u] = pose_nn_job(P[i], nP[i], Cq, Tm, eps, nn);
+      ObjJob &o = oj[u] = ObjJob{};
+      o.P = P[i], o.nP = (int)nP[i], o.nn = nn, o.Xe = Cq.Xe;
+      for (int r = 0; r < 3; ++r) {
+        for (int q = 0; q < 3; ++q) o.R[3 * r + q] = Tm[4 * r + q];
+        o.t[r] = Tm[4 * r + 3], o.v[r] = w[3 + r];
+      }
+      const double e2 = (double)eps * (double)eps;
+      o.mu = mu, o.rho_eps = o.mu * e2 / (o.mu + e2), o.scale = grad ? dE[i] : 1.0;
+      o.partials = part, o.out = out7 + 7 * i;
+      o.dP = grad ? dP[i] : nullptr, o.dQ = grad ? dQ[i] : nullptr;
+    }
+    TRY_CUDA(c, build_grids(gj, m, s), "grids");
+    TRY_CUDA(c, launch_pose_nn(nj, m, s), "neighbours");
+    TRY_CUDA(c, launch_objective(oj, m, grad ? 1 : 0, s), "objective");
   }
   TRY_CUDA(c, cudaMemcpyAsync(host7.data(), out7, sizeof(double) * 7 * n, cudaMemcpyDeviceToHost, c->stream), "D2H");
   SYNC_CHECKED(c, c->stream);

@@ -430,6 +430,38 @@ __device__ __forceinline__ void block_sum_partials(const double *__restrict__ pa
   __syncthreads();
 }
 
+// Sums of N per-thread FP64 quantities over a block of kThreads, in a fixed
+// order: out[k] = the sum of v[k]. Each warp lays its 32 values of a quantity
+// out as a row in shared memory and a lane adds a row: 32 FP64 instructions a
+// warp for up to 32 quantities, where a butterfly takes 5 for each.
+template <int N, int kThreads>
+__device__ __forceinline__ void block_sum_rows(const double (&v)[N], double *out) {
+  static_assert(N <= 32, "a lane per quantity");
+  constexpr int kWarps = kThreads / 32;
+  __shared__ double row[kWarps][N][33];
+  __shared__ double part[kWarps][N];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+  for (int k = 0; k < N; ++k) row[w][k][lane] = v[k];
+  __syncwarp();
+  if (lane < N) {
+    // four interleaved chains: the adds' latency overlaps
+    double s[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+    for (int l = 0; l < 32; l += 4)
+#pragma unroll
+      for (int u = 0; u < 4; ++u) s[u] += row[w][lane][l + u];
+    part[w][lane] = (s[0] + s[1]) + (s[2] + s[3]);
+  }
+  __syncthreads();
+  if (threadIdx.x < N) {
+    double s = part[0][threadIdx.x];
+#pragma unroll
+    for (int k = 1; k < kWarps; ++k) s += part[k][threadIdx.x];
+    out[threadIdx.x] = s;
+  }
+}
+
 __device__ __forceinline__ float warp_sum(float v) {
   for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
   return v;
@@ -682,11 +714,41 @@ cudaError_t launch_subsample(const float *xyz, int n, int stride, float4 *out, c
 cudaError_t launch_final_pose(RansacState *st, float *pose, cudaStream_t s);
 cudaError_t launch_final_count(const int *count, const unsigned long long *sum, RansacState *st, cudaStream_t s);
 
-// Objective forward / backward for one pair (lsr_refine.cu). P: caller-order
-// float32 xyz; the eps grid of Q carries caller indices in Xe.w. out7 (device):
-// E, g_v[3], g_w[3]. dP / dQ (device, caller order) are written when want_grad
-// (dQ must be zeroed by the caller), scaled by `scale`.
-int objective_blocks(int nP);
+// Neighbours of a cloud under a pose (lsr_refine.cu): nn[i] = the position in
+// Xe of the nearest Q point of R p_i + t within eps, -1 if none. P: caller-order
+// float32 xyz. Up to kPoseJobs clouds at once.
+constexpr int kPoseJobs = 8;
+struct PoseNnJob {
+  const float *P;
+  int nP;
+  const GridParams *g;
+  const int *start;
+  const float4 *Xe;
+  float R[9], t[3], eps2;
+  int *nn;
+};
+cudaError_t launch_pose_nn(const PoseNnJob *jobs, int n, cudaStream_t s);
+
+// Objective forward / backward of up to kPoseJobs pairs (lsr_refine.cu), after
+// launch_pose_nn for the same poses; the eps grid of Q carries caller indices
+// in Xe.w. out (device): E, g_v[3], g_w[3]. dP / dQ (device, caller order) are
+// written when want_grad (dQ must be zeroed by the caller), scaled by `scale`.
+// partials: 7 x objective_blocks(nP) doubles.
+struct ObjJob {
+  const float *P;
+  int nP;
+  const int *nn;
+  const float4 *Xe;
+  double R[9], t[3], v[3];
+  double mu, rho_eps, scale;
+  double *partials, *out;
+  float *dP, *dQ;
+};
+__host__ __device__ inline int objective_blocks(int nP) {
+  const int64_t b = lsr_div_up(nP > 0 ? nP : 1, 128);
+  return (int)(b > kSms * 2 ? kSms * 2 : b);
+}
+cudaError_t launch_objective(const ObjJob *jobs, int n, int want_grad, cudaStream_t s);
 // Voxel downsampling (Algorithm 1, first line; lsr_voxel.cu). kb: 6 ints (key
 // minima, maxima). launch_vox_cells needs kb's box on the host (ncells) and on
 // the device (ncells_dev); cnt, flag: ncells ints, pos: ncells + 1 ints, sums:
@@ -731,15 +793,13 @@ cudaError_t launch_consensus_variant(const float4 *XP, int nP, const float4 *NP,
                                      const uint8_t *ok, const int *n_dev, float eps, bool single, bool normals,
                                      float cos_normal, int *count, unsigned long long *sum, cudaStream_t s);
 
-// Implicit gradient of the refined pose (lsr_implicit.cu): partials holds
-// implicit_partials(nP) doubles; out 50 doubles (g 6, H 36, lambda 6, count,
-// singular flag); dl_dev: dL/dxi (6 doubles, device); dQ must be zeroed.
+// Implicit gradient of the refined pose (lsr_implicit.cu), after launch_pose_nn
+// for the same pose (nn): partials holds implicit_partials(nP) doubles; out 50
+// doubles (g 6, H 36, lambda 6, count, singular flag); dl_dev: dL/dxi (6
+// doubles, device); dQ must be zeroed.
 int implicit_partials(int nP);
-cudaError_t launch_implicit(const float *P, int nP, const GridParams *ge, const int *start_e, const float4 *Xe,
-                            int nQ, const double T[16], float eps, double mu, const double *dl_dev,
-                            double *partials, double *out, float *dP, float *dQ, cudaStream_t s);
-cudaError_t launch_objective(const float *P, int nP, const GridParams *ge, const int *start_e, const float4 *Xe,
-                             const double T[16], const double v[3], float eps, float mu, double scale,
-                             int want_grad, double *partials, double *out7, float *dP, float *dQ, cudaStream_t s);
+cudaError_t launch_implicit(const float *P, int nP, const int *nn, const float4 *Xe, int nQ, const double T[16],
+                            double mu, const double *dl_dev, double *partials, double *out, float *dP, float *dQ,
+                            cudaStream_t s);
 
 }  // namespace lsr

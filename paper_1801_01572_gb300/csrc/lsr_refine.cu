@@ -23,7 +23,6 @@ constexpr int kRefBlocksPerSm = 4;  // resident refinement blocks per SM (64 reg
 constexpr int kRefMaxBlocks = kSms * kRefBlocksPerSm;  // refine_blocks' cap
 constexpr int kRefGroup = 16;                           // blocks per first-level closing sum
 constexpr int kRefMaxGroups = (kRefMaxBlocks + kRefGroup - 1) / kRefGroup;
-constexpr int kObjG = 8;   // lanes per query in the objective
 // 21 (upper triangle of A) + 6 (b) + count + sum w + sum w x (3)
 constexpr int kNAcc = kRefAcc;
 static_assert(kNAcc == 32, "refinement partial layout");
@@ -453,55 +452,69 @@ __global__ void k_info_final(const double *__restrict__ partials, int nb, const 
   out[36] = n;
 }
 
+// ---------------------------------------------------------------- neighbours under a pose
+// The nearest Q point of every moved point of P, for the kernels that then
+// evaluate their terms in FP64: nn[i] = its position in the sorted array, -1
+// if none lies within eps. Searching and evaluating in one kernel left the
+// FP64 unit (2 lanes a clock on an SM, a warp instruction every 16 clocks
+// however many of its lanes live) to the one lane in four or eight that held a
+// point: 59 to 75% of its cycles for an eighth to a quarter of the work, and
+// the registers of the FP64 terms kept the search at 16 warps an SM. As a pass
+// of its own it runs at full occupancy, writes 4 bytes a point, and the terms
+// run a point per lane.
+struct PoseNnJobs {
+  PoseNnJob j[kPoseJobs];
+};
+constexpr int kPoseNnG = 4;  // lanes per query
+
+__global__ void __launch_bounds__(kRefThreads, 5) k_pose_nn(const __grid_constant__ PoseNnJobs J) {
+  const PoseNnJob &a = J.j[blockIdx.y];
+  constexpr int GPB = kRefThreads / kPoseNnG;
+  const int i = blockIdx.x * GPB + threadIdx.x / kPoseNnG;
+  if ((int)blockIdx.x * GPB >= a.nP) return;
+  const bool valid = i < a.nP;
+  const GridParams g = *a.g;
+  const float px = valid ? a.P[3 * i] : __int_as_float(0x7fc00000), py = valid ? a.P[3 * i + 1] : 0.f,
+              pz = valid ? a.P[3 * i + 2] : 0.f;  // NaN: the query visits no cell
+  const float x = fmaf(a.R[0], px, fmaf(a.R[1], py, fmaf(a.R[2], pz, a.t[0])));
+  const float y = fmaf(a.R[3], px, fmaf(a.R[4], py, fmaf(a.R[5], pz, a.t[1])));
+  const float z = fmaf(a.R[6], px, fmaf(a.R[7], py, fmaf(a.R[8], pz, a.t[2])));
+  float best;
+  int bt, bidx;
+  group_nn<kPoseNnG>(g, a.start, a.Xe, x, y, z, a.eps2, best, bt, bidx);
+  if (valid && (threadIdx.x & (kPoseNnG - 1)) == 0) a.nn[i] = bt;
+}
+
 // ---------------------------------------------------------------- objective
 // E = sum_i rho(s_i) - rho(eps^2) over points with an NN closer than eps.
 // Forward and backward share this kernel; the backward also writes
 // dP_i = 2 rho'(s) R^T r_i, scatters dQ_j -= 2 rho'(s) r_i, and reduces
 // g_v = sum 2 rho' r_i and g_w = sum z_i x (2 rho' r_i) with z_i = x_i - v.
 // dxi = (J_l(w)^T g_w, g_v) is finished on the host. The nearest neighbour is
-// found in FP32 (the pose rounded to FP32); the residual of the pair, the
+// found in FP32 (k_pose_nn, the pose rounded to FP32); the residual of the pair, the
 // terms and their sums are evaluated in FP64 from the FP32 coordinates: a
 // residual of a few millimetres between points metres from the origin would
 // otherwise carry the 2^-24 rounding of the coordinates (about 1e-7 m).
-struct ObjArgs {
-  float Rf[9], tf[3];    // the pose in FP32, for the neighbour search
-  double R[9], t[3], v[3];
-  float eps2;
-  double mu, rho_eps, scale;
+// A thread per point; blockIdx.y is the pair. Bound by FP64 issue (about 110
+// instructions a point backward); 8 pairs of 50k points took 8 x 57 us.
+struct ObjJobs {
+  ObjJob j[kPoseJobs];
 };
+constexpr int kObjThreads = 128;
 
-__device__ __forceinline__ double warp_sum_dbl(double v) {
-  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-  return v;
-}
-
-__global__ void __launch_bounds__(kRefThreads) k_objective(const float *__restrict__ P, int nP, const GridParams *gep,
-                                                           const int *__restrict__ start,
-                                                           const float4 *__restrict__ Xe, ObjArgs a, int want_grad,
-                                                           double *partials, float *__restrict__ dP,
-                                                           float *__restrict__ dQ) {
-  const GridParams g = *gep;
+__global__ void __launch_bounds__(kObjThreads) k_objective(const __grid_constant__ ObjJobs J, int want_grad) {
+  const ObjJob &a = J.j[blockIdx.y];
+  if ((int)blockIdx.x >= objective_blocks(a.nP)) return;
+  const int nblk = objective_blocks(a.nP);
   double acc[7] = {0, 0, 0, 0, 0, 0, 0};  // E, g_v (3), g_w (3)
-  constexpr int G = kObjG, GPB = kRefThreads / G;
-  int grp = threadIdx.x / G, sub = threadIdx.x & (G - 1);
-  for (int rb = blockIdx.x * GPB; rb < nP; rb += gridDim.x * GPB) {
-    int i = rb + grp;
-    bool valid = i < nP;
-    float px = valid ? P[3 * i] : __int_as_float(0x7fc00000), py = valid ? P[3 * i + 1] : 0.f,
-          pz = valid ? P[3 * i + 2] : 0.f;
-    float x = fmaf(a.Rf[0], px, fmaf(a.Rf[1], py, fmaf(a.Rf[2], pz, a.tf[0])));
-    float y = fmaf(a.Rf[3], px, fmaf(a.Rf[4], py, fmaf(a.Rf[5], pz, a.tf[1])));
-    float z = fmaf(a.Rf[6], px, fmaf(a.Rf[7], py, fmaf(a.Rf[8], pz, a.tf[2])));
-    float best;
-    int bt, bidx;
-    group_nn<G>(g, start, Xe, x, y, z, a.eps2, best, bt, bidx);
-    if (!valid || sub != 0) continue;
+  for (int i = blockIdx.x * kObjThreads + threadIdx.x; i < a.nP; i += nblk * kObjThreads) {
+    const int bt = a.nn[i];
     if (bt < 0) {
-      if (want_grad) dP[3 * i] = dP[3 * i + 1] = dP[3 * i + 2] = 0.f;
+      if (want_grad) a.dP[3 * i] = a.dP[3 * i + 1] = a.dP[3 * i + 2] = 0.f;
       continue;
     }
-    const float4 q = Xe[bt];
-    const double p[3] = {px, py, pz};
+    const float4 q = a.Xe[bt];
+    const double p[3] = {a.P[3 * i], a.P[3 * i + 1], a.P[3 * i + 2]};
     double zd[3], r[3];
     for (int k = 0; k < 3; ++k) {
       zd[k] = a.R[3 * k] * p[0] + a.R[3 * k + 1] * p[1] + a.R[3 * k + 2] * p[2] + a.t[k];
@@ -513,13 +526,13 @@ __global__ void __launch_bounds__(kRefThreads) k_objective(const float *__restri
     if (want_grad) {
       const double k2 = 2.0 * a.mu * a.mu / (den * den);
       const double g0 = k2 * r[0], g1 = k2 * r[1], g2 = k2 * r[2];
-      dP[3 * i + 0] = (float)(a.scale * (a.R[0] * g0 + a.R[3] * g1 + a.R[6] * g2));
-      dP[3 * i + 1] = (float)(a.scale * (a.R[1] * g0 + a.R[4] * g1 + a.R[7] * g2));
-      dP[3 * i + 2] = (float)(a.scale * (a.R[2] * g0 + a.R[5] * g1 + a.R[8] * g2));
+      a.dP[3 * i + 0] = (float)(a.scale * (a.R[0] * g0 + a.R[3] * g1 + a.R[6] * g2));
+      a.dP[3 * i + 1] = (float)(a.scale * (a.R[1] * g0 + a.R[4] * g1 + a.R[7] * g2));
+      a.dP[3 * i + 2] = (float)(a.scale * (a.R[2] * g0 + a.R[5] * g1 + a.R[8] * g2));
       const int j = __float_as_int(q.w);
-      atomicAdd(&dQ[3 * j + 0], (float)(-a.scale * g0));
-      atomicAdd(&dQ[3 * j + 1], (float)(-a.scale * g1));
-      atomicAdd(&dQ[3 * j + 2], (float)(-a.scale * g2));
+      atomicAdd(&a.dQ[3 * j + 0], (float)(-a.scale * g0));
+      atomicAdd(&a.dQ[3 * j + 1], (float)(-a.scale * g1));
+      atomicAdd(&a.dQ[3 * j + 2], (float)(-a.scale * g2));
       const double zx = zd[0] - a.v[0], zy = zd[1] - a.v[1], zz = zd[2] - a.v[2];
       acc[1] += g0, acc[2] += g1, acc[3] += g2;
       acc[4] += zy * g2 - zz * g1;
@@ -527,25 +540,14 @@ __global__ void __launch_bounds__(kRefThreads) k_objective(const float *__restri
       acc[6] += zx * g1 - zy * g0;
     }
   }
-  __shared__ double sm[kRefThreads / 32][7];
-  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-#pragma unroll
-  for (int k = 0; k < 7; ++k) {
-    const double v = warp_sum_dbl(acc[k]);
-    if (lane == 0) sm[wp][k] = v;
-  }
-  __syncthreads();
-  if (threadIdx.x < 7) {
-    double t = 0.0;
-    for (int k = 0; k < kRefThreads / 32; ++k) t += sm[k][threadIdx.x];
-    partials[(size_t)blockIdx.x * 7 + threadIdx.x] = t;
-  }
+  block_sum_rows<7, kObjThreads>(acc, a.partials + (size_t)blockIdx.x * 7);
 }
 
-__global__ void k_objective_sum(const double *partials, int nblocks, double *out) {
+__global__ void k_objective_sum(const __grid_constant__ ObjJobs J) {
+  const ObjJob &a = J.j[blockIdx.y];
   __shared__ double seg[256], tot[7];
-  block_sum_partials(partials, nblocks, 7, 7, seg, tot);
-  if (threadIdx.x < 7) out[threadIdx.x] = tot[threadIdx.x];
+  block_sum_partials(a.partials, objective_blocks(a.nP), 7, 7, seg, tot);
+  if (threadIdx.x < 7) a.out[threadIdx.x] = tot[threadIdx.x];
 }
 
 }  // namespace
@@ -634,27 +636,27 @@ cudaError_t launch_information(const float *P, int nP, const GridParams *ge, con
   return cudaGetLastError();
 }
 
-int objective_blocks(int nP) {
-  int64_t b = lsr_div_up((int64_t)(nP > 0 ? nP : 1) * kObjG, kRefThreads);
-  return (int)(b < 1 ? 1 : (b > kSms * 2 ? kSms * 2 : b));
+cudaError_t launch_pose_nn(const PoseNnJob *jobs, int n, cudaStream_t s) {
+  if (n < 1 || n > kPoseJobs) return cudaErrorInvalidValue;
+  PoseNnJobs J{};
+  int64_t most = 1;
+  for (int k = 0; k < n; ++k) J.j[k] = jobs[k], most = jobs[k].nP > most ? jobs[k].nP : most;
+  const int nb = (int)lsr_div_up(most * kPoseNnG, kRefThreads);
+  LSR_LAUNCH(k_pose_nn<<<dim3(nb, n), kRefThreads, 0, s>>>(J));
+  return cudaGetLastError();
 }
 
-cudaError_t launch_objective(const float *P, int nP, const GridParams *ge, const int *start_e, const float4 *Xe,
-                             const double T[16], const double v[3], float eps, float mu, double scale,
-                             int want_grad, double *partials, double *out7, float *dP, float *dQ, cudaStream_t s) {
-  ObjArgs a;
-  for (int r = 0; r < 3; ++r) {
-    for (int q = 0; q < 3; ++q) a.R[3 * r + q] = T[4 * r + q], a.Rf[3 * r + q] = (float)T[4 * r + q];
-    a.t[r] = T[4 * r + 3], a.tf[r] = (float)T[4 * r + 3], a.v[r] = v[r];
+cudaError_t launch_objective(const ObjJob *jobs, int n, int want_grad, cudaStream_t s) {
+  if (n < 1 || n > kPoseJobs) return cudaErrorInvalidValue;
+  ObjJobs J{};
+  int most = 1;
+  for (int k = 0; k < n; ++k) {
+    J.j[k] = jobs[k];
+    const int nb = objective_blocks(jobs[k].nP);
+    most = nb > most ? nb : most;
   }
-  a.eps2 = eps * eps;
-  a.mu = mu;
-  const double e2 = (double)eps * (double)eps;
-  a.rho_eps = a.mu * e2 / (a.mu + e2);
-  a.scale = scale;
-  int nb = objective_blocks(nP);
-  LSR_LAUNCH(k_objective<<<nb, kRefThreads, 0, s>>>(P, nP, ge, start_e, Xe, a, want_grad, partials, dP, dQ));
-  LSR_LAUNCH(k_objective_sum<<<1, 256, 0, s>>>(partials, nb, out7));
+  LSR_LAUNCH(k_objective<<<dim3(most, n), kObjThreads, 0, s>>>(J, want_grad));
+  LSR_LAUNCH(k_objective_sum<<<dim3(1, n), 256, 0, s>>>(J));
   return cudaGetLastError();
 }
 

@@ -1,0 +1,50 @@
+"""The objective of several pairs at once: pairs go through every step
+together, eight at a time, so batches around that number and of very uneven
+sizes (one point to thousands) must give what single-pair calls give. Sums are
+FP64 in a fixed order per pair and do not depend on the batch: energies and
+pose gradients equal bit for bit; dP is written once per point, so equal too;
+dQ adds FP32 atomics in any order (a point closes at most a few pairs): 1e-6.
+"""
+import numpy as np
+import pytest
+
+gpu = pytest.mark.gpu
+EPS = 0.0375
+
+
+@gpu
+@pytest.mark.parametrize("sizes", [[(1, 1)], [(5, 4), (3000, 1), (1, 2500), (127, 129)],
+                                   [(64 * k + 1, 97 * k + 3) for k in range(8)],
+                                   [(33 * k + 7, 511 + k) for k in range(19)]])
+def test_objective_batches_equal_single_pairs(sizes):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1801_01572_gb300 as lsr
+    rng = np.random.default_rng(len(sizes))
+    P, Q = [], []
+    for a, b in sizes:
+        q = rng.uniform(0, 0.4, (b, 3))
+        p = q[rng.integers(0, b, a)] + rng.normal(0, 0.01, (a, 3))
+        p[::5] += 2.0  # no neighbour
+        P.append(torch.from_numpy(p.astype(np.float32)).cuda())
+        Q.append(torch.from_numpy(q.astype(np.float32)).cuda())
+    n = len(sizes)
+    xi = rng.normal(0, 2e-3, (n, 6))
+    T0 = np.tile(np.eye(4), (n, 1, 1))
+    dE = rng.uniform(0.5, 2.0, n)
+    with lsr.Context(0) as ctx:
+        def bwd(i):
+            dP = [torch.full_like(P[k], 7.0) for k in i]
+            dQ = [torch.full_like(Q[k], 7.0) for k in i]
+            dx = ctx.objective_bwd([P[k] for k in i], [Q[k] for k in i], xi[i], T0[i], dE[i], dP, dQ, EPS)
+            return dx, dP, dQ
+        E = ctx.objective_fwd(P, Q, xi, T0, EPS)
+        dxi, dP, dQ = bwd(list(range(n)))
+        assert np.isfinite(E).all()
+        for k in range(n):
+            assert ctx.objective_fwd(P[k:k + 1], Q[k:k + 1], xi[k:k + 1], T0[k:k + 1], EPS)[0] == E[k]
+            dx1, dP1, dQ1 = bwd([k])
+            assert np.array_equal(dx1[0], dxi[k])
+            assert torch.equal(dP1[0], dP[k])
+            assert torch.allclose(dQ1[0], dQ[k], rtol=1e-6, atol=1e-6 * float(dQ[k].abs().max()) + 1e-12)
