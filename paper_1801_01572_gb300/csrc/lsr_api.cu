@@ -408,9 +408,10 @@ int check_report(lsr_ctx *c) {
   static cudaError_t (*const readers[])(CheckReport *) = {check_read_features, check_read_match,
                                                           check_read_match_tc, check_read_ransac,
                                                           check_read_classify, check_read_refine,
-                                                          check_read_nn,       check_read_implicit};
+                                                          check_read_nn,       check_read_implicit,
+                                                          check_read_order};
   static const char *const units[] = {"features", "match", "match_tc", "ransac",
-                                      "classify", "refine", "nn",       "implicit"};
+                                      "classify", "refine", "nn",       "implicit", "order"};
   constexpr int kUnits = (int)(sizeof(units) / sizeof(units[0]));
   static const char *const sites[] = {"?", "grid row", "grid cell", "grid point", "hypothesis sample",
                                       "hypothesis match", "matcher row", "matcher query", "probe"};

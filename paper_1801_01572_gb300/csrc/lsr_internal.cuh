@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 namespace lsr {
 
 constexpr int kD = 33;       // FPFH length: 3 features x 11 bins
@@ -128,6 +130,7 @@ __device__ __forceinline__ bool check_in_bounds(long long i, long long n, int si
 // Readers of the units that hold checks.
 cudaError_t check_read_features(CheckReport *r);
 cudaError_t check_read_match(CheckReport *r);
+cudaError_t check_read_order(CheckReport *r);
 cudaError_t check_read_match_tc(CheckReport *r);
 cudaError_t check_read_ransac(CheckReport *r);
 cudaError_t check_read_classify(CheckReport *r);
@@ -534,6 +537,41 @@ cudaError_t launch_spfh(const float4 *X, const float4 *N, int n, const GridParam
                         float *spfh, int *k, void *scratch, cudaStream_t s);
 cudaError_t launch_fpfh(const float4 *X, const float4 *N, const float *spfh, int n, const GridParams *gf,
                         const int *start_f, float r, float *fpfh, cudaStream_t s);
+
+// ----------------------------------------------------------------- descriptor order (lsr_order.cu)
+constexpr int kAx = 8;           // projection axes
+constexpr int kOrdTile = 32;     // rows of a tile (a leaf of the k-d splits; a query group)
+constexpr int kOrdLeaf = 128;    // rows of a leaf box: four tiles
+constexpr int kOrdSlab = 4096;   // rows split by one block
+struct OrderParams {
+  float u[kD][kAx];              // the axes, a row per bin
+  float fac;                     // lower-bound factor of a sum of squared projection gaps
+  unsigned key_min, key_max;     // range of the first projection (ordered keys)
+  int ntot;                      // nQ + nP (read by the scan)
+};
+// Elements: the nQ database rows, then the nP queries. Positions: the final order.
+struct DescOrder {
+  OrderParams *pp;
+  float4 *pq;                    // per element: its kAx projections
+  float *pe;                     // per element: their error bound
+  int *slot, *rank, *counts, *start, *order1, *order, *scan;
+  float *FQs;                    // database rows in the final order, chunk-major per tile
+  int *dorig;                    // their original indices
+  float4 *tbox, *lbox;           // boxes of the database's tiles and leaves (lo 0..3, 4..7, hi 0..3, 4..7)
+  float *FPs;                    // queries in the final order (desc_order rows)
+  int *qorig;                    // their original indices
+  float4 *qp;                    // per query position: projections
+  float *qe;                     // and their error bound
+  float4 *gbox, *qbox;           // boxes of the query groups (tiles) and of their leaves
+};
+// Places o's arrays at base (null: measures); returns their bytes.
+size_t desc_order_layout(char *base, int nP, int nQ, DescOrder &o);
+cudaError_t launch_desc_order(const float *FP, int nP, const float *FQ, int nQ, const DescOrder &o, cudaStream_t s);
+
+// Adds the square of a projection gap (rounded down; not above zero: none) to
+// a lower bound, rounded down. Gaps below 1e-18 count as 0 (subnormal terms of
+// a distance lose their relative rounding bound).
+__device__ __forceinline__ float gap_add(float s, float gap) { return gap > 1e-18f ? __fmaf_rd(gap, gap, s) : s; }
 
 // ----------------------------------------------------------------- matching (lsr_match.cu)
 // ws: fp32_workspace_bytes(nP, nQ) of device memory, 256-byte aligned (the
