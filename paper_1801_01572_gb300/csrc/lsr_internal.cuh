@@ -567,6 +567,8 @@ struct DescOrder {
 // Places o's arrays at base (null: measures); returns their bytes.
 size_t desc_order_layout(char *base, int nP, int nQ, DescOrder &o);
 cudaError_t launch_desc_order(const float *FP, int nP, const float *FQ, int nQ, const DescOrder &o, cudaStream_t s);
+// The rows and indices alone (FQs, dorig, FPs, qorig), in the caller's order.
+cudaError_t launch_desc_rows(const float *FP, int nP, const float *FQ, int nQ, const DescOrder &o, cudaStream_t s);
 
 // Adds the square of a projection gap (rounded down; not above zero: none) to
 // a lower bound, rounded down. Gaps below 1e-18 count as 0 (subnormal terms of
@@ -582,6 +584,17 @@ size_t fp32_workspace_bytes(int nP, int nQ);
 int device_sm_count();
 cudaError_t launch_match_fp32(const float *FP, int nP, const float *FQ, int nQ, void *ws, int *nn, float *d1,
                               cudaStream_t s, unsigned long long *terms = nullptr);
+// The FP32 matcher's passes over an order: packed (per query position, ~0
+// before) gets (distance bits << 32 | original index) minima. launch_match_seed:
+// of the two nearest leaves. launch_match_listed: of all rows, for the
+// positions with flag set in the groups of 32 listed (counts on the device;
+// work: a zeroed word). launch_match_finish: nn / d1 from packed.
+cudaError_t launch_match_seed(const DescOrder &o, int nP, int nQ, unsigned long long *packed, cudaStream_t s);
+cudaError_t launch_match_listed(const DescOrder &o, int nP, int nQ, const int *groups, const int *ngroups,
+                                const int *flag, unsigned long long *packed, unsigned long long *work,
+                                cudaStream_t s);
+cudaError_t launch_match_finish(const unsigned long long *packed, const int *qorig, int nP, int *nn, float *d1,
+                                cudaStream_t s);
 // Exact FP32 scan of the queries rows[0..*nrows) (count read on the device),
 // split over database chunks; packed: scratch of nP 64-bit words.
 cudaError_t launch_match_fp32_rows(const float *FP, int nP, const float *FQ, int nQ, const int *rows,

@@ -226,9 +226,10 @@ struct QueryLane {
 };
 
 __device__ __forceinline__ void load_query(QueryLane &q, const DescOrder &o, int g, int nP,
-                                           const unsigned long long *packed, float (*sp)[32]) {
+                                           const unsigned long long *packed, float (*sp)[32],
+                                           const int *flag = nullptr) {
   const int lane = threadIdx.x & 31, k = g * 32 + lane;
-  q.valid = k < nP;
+  q.valid = k < nP && (!flag || flag[k]);
   const int kq = q.valid ? k : 0;
   const float4 *row = reinterpret_cast<const float4 *>(o.FPs + (size_t)kq * kDS);
 #pragma unroll
@@ -400,16 +401,22 @@ __global__ void __launch_bounds__(kMT, kMatchBlocks) k_match_seed(DescOrder o, i
 // groups read the same tiles, so they share L2). Small sets take blocks of 8
 // tiles so that there are items for every warp. kCount: also add the number of
 // terms (a_k - b_k)^2 evaluated for the valid queries to *terms (a separate
-// instantiation, used when profiling).
+// instantiation, used when profiling). list: only its groups, and of those the
+// queries with flag set.
+struct MatchList {
+  const int *groups, *count, *flag;
+};
 template <int kTpi, bool kCount>
 __global__ void __launch_bounds__(kMT, kMatchBlocks) k_match_win(DescOrder o, int nP, int nQ, int run,
-                                                                 unsigned long long *packed, unsigned long long *work,
+                                                                 MatchList list, unsigned long long *packed,
+                                                                 unsigned long long *work,
                                                                  unsigned long long *__restrict__ terms) {
   __shared__ MatchWarp sm[kMT / 32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int nt = (int)lsr_div_up(nQ, kTile);
-  const int G = (int)lsr_div_up(nP, 32);
+  const int G = list.groups ? *list.count : (int)lsr_div_up(nP, 32);
   const long long nitems = lsr_div_up(nt, kTpi) * (long long)G;
+  if (nitems <= 0) return;
   const float fac = o.pp->fac;
   unsigned long long nterm = 0;
   for (;;) {
@@ -417,14 +424,15 @@ __global__ void __launch_bounds__(kMT, kMatchBlocks) k_match_win(DescOrder o, in
     if (lane == 0) u0 = (long long)atomicAdd(work, (unsigned long long)run);
     u0 = __shfl_sync(0xffffffffu, u0, 0);
     if (u0 >= nitems) break;
-    int b = (int)(u0 / G), g = (int)(u0 - (long long)b * G);
+    int b = (int)(u0 / G), at = (int)(u0 - (long long)b * G);
 #pragma unroll 1
-    for (int r = 0; r < run && u0 + r < nitems; ++r, ++g) {
-      if (g == G) g = 0, ++b;
+    for (int r = 0; r < run && u0 + r < nitems; ++r, ++at) {
+      if (at == G) at = 0, ++b;
+      const int g = list.groups ? list.groups[at] : at;
       // the group's largest published distance against this lane's tile
       const int k = g * 32 + lane, t = b * kTpi + lane;
       unsigned far = 0u;
-      if (k < nP) {
+      if (k < nP && (!list.flag || list.flag[k])) {
         const unsigned long long pv = __ldcg(packed + k);
         far = pv == ~0ull ? __float_as_uint(FLT_MAX) : (unsigned)(pv >> 32);
       }
@@ -446,7 +454,7 @@ __global__ void __launch_bounds__(kMT, kMatchBlocks) k_match_win(DescOrder o, in
       const unsigned todo = __ballot_sync(0xffffffffu, open);
       if (!todo) continue;
       QueryLane q;
-      load_query(q, o, g, nP, packed, sm[w].sp);
+      load_query(q, o, g, nP, packed, sm[w].sp, list.flag);
       unsigned uterm = 0;  // terms of this item (at most 33 per database row)
       visit_tiles<kCount>(q, o, b * kTpi, todo, nQ, sm[w], fac, uterm);
       publish(q, g, nP, packed);
@@ -599,15 +607,37 @@ cudaError_t launch_match_fp32(const float *FP, int nP, const float *FQ, int nQ, 
     const int run = (int)std::max(1ll, std::min(8ll, items / (8 * warps)));
     const int blocks = (int)std::min(resident, (long long)lsr_div_up(lsr_div_up(items, run), kMT / 32));
     if (small && terms)
-      LSR_LAUNCH(k_match_win<8, true><<<blocks, kMT, 0, s>>>(L.o, nP, nQ, run, L.packed, L.work, terms));
+      LSR_LAUNCH(k_match_win<8, true><<<blocks, kMT, 0, s>>>(L.o, nP, nQ, run, MatchList{}, L.packed, L.work, terms));
     else if (small)
-      LSR_LAUNCH(k_match_win<8, false><<<blocks, kMT, 0, s>>>(L.o, nP, nQ, run, L.packed, L.work, nullptr));
+      LSR_LAUNCH(k_match_win<8, false><<<blocks, kMT, 0, s>>>(L.o, nP, nQ, run, MatchList{}, L.packed, L.work, nullptr));
     else if (terms)
-      LSR_LAUNCH(k_match_win<32, true><<<blocks, kMT, 0, s>>>(L.o, nP, nQ, run, L.packed, L.work, terms));
+      LSR_LAUNCH(k_match_win<32, true><<<blocks, kMT, 0, s>>>(L.o, nP, nQ, run, MatchList{}, L.packed, L.work, terms));
     else
-      LSR_LAUNCH(k_match_win<32, false><<<blocks, kMT, 0, s>>>(L.o, nP, nQ, run, L.packed, L.work, nullptr));
+      LSR_LAUNCH(k_match_win<32, false><<<blocks, kMT, 0, s>>>(L.o, nP, nQ, run, MatchList{}, L.packed, L.work, nullptr));
   }
-  LSR_LAUNCH(k_win_finish<<<(int)lsr_div_up(nP, 256), 256, 0, s>>>(L.packed, L.o.qorig, nP, nn, d1));
+  return launch_match_finish(L.packed, L.o.qorig, nP, nn, d1, s);
+}
+
+cudaError_t launch_match_seed(const DescOrder &o, int nP, int nQ, unsigned long long *packed, cudaStream_t s) {
+  LSR_CUDA_TRY(prefer_shared());
+  const int blocks = (int)lsr_div_up(lsr_div_up(nP, 32), kMT / 32);
+  LSR_LAUNCH(k_match_seed<false><<<blocks, kMT, 0, s>>>(o, nP, nQ, packed, nullptr));
+  return cudaGetLastError();
+}
+
+cudaError_t launch_match_listed(const DescOrder &o, int nP, int nQ, const int *groups, const int *ngroups,
+                                const int *flag, unsigned long long *packed, unsigned long long *work,
+                                cudaStream_t s) {
+  LSR_CUDA_TRY(prefer_shared());
+  const int blocks = kMatchBlocks * device_sm_count();
+  LSR_LAUNCH(k_match_win<8, false><<<blocks, kMT, 0, s>>>(o, nP, nQ, 1, MatchList{groups, ngroups, flag}, packed, work,
+                                                          nullptr));
+  return cudaGetLastError();
+}
+
+cudaError_t launch_match_finish(const unsigned long long *packed, const int *qorig, int nP, int *nn, float *d1,
+                                cudaStream_t s) {
+  LSR_LAUNCH(k_win_finish<<<(int)lsr_div_up(nP, 256), 256, 0, s>>>(packed, qorig, nP, nn, d1));
   return cudaGetLastError();
 }
 

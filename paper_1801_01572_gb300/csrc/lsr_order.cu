@@ -400,7 +400,9 @@ __global__ void __launch_bounds__(kKdThreads) k_kd(const float4 *__restrict__ pq
 // boxes of the projection intervals [p - pe, p + pe]. Database rows go
 // chunk-major per tile of 32 (float4 chunk c of row j at c * 32 + j), query
 // rows one after another, both with bins in desc_order and zeros in slots
-// 33..35; a box is (lo 0..3, lo 4..7, hi 0..3, hi 4..7).
+// 33..35; a box is (lo 0..3, lo 4..7, hi 0..3, hi 4..7). Without kBoxes: the
+// rows alone, in the caller's order.
+template <bool kBoxes>
 __global__ void __launch_bounds__(kGatherThreads) k_gather(const float *__restrict__ FP, int nP,
                                                            const float *__restrict__ FQ, int nQ, int leaves_db,
                                                            DescOrder o) {
@@ -412,7 +414,7 @@ __global__ void __launch_bounds__(kGatherThreads) k_gather(const float *__restri
 #pragma unroll
   for (int d = 0; d < kAx; ++d) lo[d] = INFINITY, hi[d] = -INFINITY;
   if (pos < n) {
-    int e = o.order[(db ? 0 : nQ) + pos];
+    int e = kBoxes ? o.order[(db ? 0 : nQ) + pos] : (db ? 0 : nQ) + pos;
     if (!LSR_IN_BOUNDS(db ? e : e - nQ, n, db ? kSiteMatchRow : kSiteMatchQuery)) e = db ? 0 : nQ;
     const int i = db ? e : e - nQ;
     const float *src = (db ? FQ : FP) + (size_t)i * kDS;
@@ -426,12 +428,11 @@ __global__ void __launch_bounds__(kGatherThreads) k_gather(const float *__restri
       for (int k = 0; k < 4; ++k) v[k] = 4 * c + k < kD ? src[desc_order(4 * c + k)] : 0.f;
       dst[c * step] = make_float4(v[0], v[1], v[2], v[3]);
     }
+    (db ? o.dorig : o.qorig)[pos] = i;
+    if (!kBoxes) return;
     const float4 p0 = o.pq[2 * (size_t)e], p1 = o.pq[2 * (size_t)e + 1];
     const float err = o.pe[e];
-    if (db) {
-      o.dorig[pos] = i;
-    } else {
-      o.qorig[pos] = i;
+    if (!db) {
       o.qp[2 * (size_t)pos] = p0, o.qp[2 * (size_t)pos + 1] = p1;
       o.qe[pos] = err;
     }
@@ -439,6 +440,7 @@ __global__ void __launch_bounds__(kGatherThreads) k_gather(const float *__restri
 #pragma unroll
     for (int d = 0; d < kAx; ++d) lo[d] = __fsub_rd(p[d], err), hi[d] = __fadd_ru(p[d], err);
   }
+  if (!kBoxes) return;
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1)
 #pragma unroll
@@ -525,7 +527,13 @@ cudaError_t launch_desc_order(const float *FP, int nP, const float *FQ, int nQ, 
   const int slabs_db = (int)lsr_div_up(nQ, kOrdSlab), slabs_q = (int)lsr_div_up(nP, kOrdSlab);
   LSR_LAUNCH(k_kd<<<slabs_db + slabs_q, kKdThreads, kKdSmem, s>>>(o.pq, o.order1, nQ, nP, slabs_db, o.order));
   const int leaves_db = (int)lsr_div_up(nQ, kOrdLeaf), leaves_q = (int)lsr_div_up(nP, kOrdLeaf);
-  LSR_LAUNCH(k_gather<<<leaves_db + leaves_q, kGatherThreads, 0, s>>>(FP, nP, FQ, nQ, leaves_db, o));
+  LSR_LAUNCH(k_gather<true><<<leaves_db + leaves_q, kGatherThreads, 0, s>>>(FP, nP, FQ, nQ, leaves_db, o));
+  return cudaGetLastError();
+}
+
+cudaError_t launch_desc_rows(const float *FP, int nP, const float *FQ, int nQ, const DescOrder &o, cudaStream_t s) {
+  const int leaves_db = (int)lsr_div_up(nQ, kOrdLeaf), leaves_q = (int)lsr_div_up(nP, kOrdLeaf);
+  LSR_LAUNCH(k_gather<false><<<leaves_db + leaves_q, kGatherThreads, 0, s>>>(FP, nP, FQ, nQ, leaves_db, o));
   return cudaGetLastError();
 }
 
