@@ -83,6 +83,48 @@ __device__ __forceinline__ bool hyp_pass(const HypIn &in, uint32_t h, int ii[4],
   return true;
 }
 
+// What a hypothesis needs of a sampled point, by the caller's index: the point
+// (w: 1 if it, its match and both normals are valid, else 0), then its match.
+// A sample is one 32-byte sector; through the index, the validity flags and the
+// match it was six sectors and three dependent loads (310 us for 4M hypotheses
+// of 150k points, 180 us of 5k).
+__global__ void k_hyp_records(HypIn in, float4 *__restrict__ rec) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < in.nP; i += gridDim.x * blockDim.x) {
+    float4 p = in.XP[i], q = make_float4(0.f, 0.f, 0.f, 0.f);
+    const int c = __float_as_int(p.w), j = in.nn[i];
+    if (!LSR_IN_BOUNDS(c, in.nP, kSiteHypSample)) continue;
+    p.w = 0.f;
+    if (in.NP[i].w >= 0.f && j >= 0 && j < in.nQ && in.NQ[j].w >= 0.f) {
+      q = in.XQ[j];
+      p.w = 1.f;
+    }
+    rec[2 * (size_t)c] = p;
+    rec[2 * (size_t)c + 1] = q;
+  }
+}
+
+// hyp_pass from the records (the same test).
+__device__ __forceinline__ bool hyp_test(const HypIn &in, const float4 *__restrict__ rec, uint32_t h) {
+  int idx[4];
+  sample4(in.seed, in.pair, h, in.nP, idx);
+  float4 p[4], q[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    if (!LSR_IN_BOUNDS(idx[k], in.nP, kSiteHypSample)) return false;
+    p[k] = __ldg(rec + 2 * (size_t)idx[k]);
+    q[k] = __ldg(rec + 2 * (size_t)idx[k] + 1);
+  }
+  bool ok = idx[0] != idx[1] && idx[0] != idx[2] && idx[0] != idx[3] && idx[1] != idx[2] && idx[1] != idx[3] &&
+            idx[2] != idx[3];
+#pragma unroll
+  for (int a = 0; a < 4; ++a) {
+    const int b = (a + 1) & 3;
+    const float ep = d2f(p[a], p[b]), eq = d2f(q[a], q[b]);
+    ok = ok && p[a].w > 0.f && !(ep < 1e-12f || eq < 1e-12f) && !(ep < in.tau2 * eq || eq < in.tau2 * ep);
+  }
+  return ok;
+}
+
 constexpr int kHypThreads = 256;
 constexpr int kHypIters = 16;
 constexpr int kHypPerBlock = kHypThreads * kHypIters;
@@ -99,7 +141,8 @@ static __device__ int g_check_probe;
 // block prefix per iteration) to the block's own region of local
 // (kHypPerBlock ints a block), so that one gather after the scan places them
 // in order without testing the hypotheses again.
-__global__ void __launch_bounds__(kHypThreads) k_hyp_count(HypIn in, int64_t H, int *block_counts, int *local) {
+__global__ void __launch_bounds__(kHypThreads) k_hyp_count(HypIn in, const float4 *__restrict__ rec, int64_t H,
+                                                           int *block_counts, int *local) {
 #ifdef LSR_CHECKED
   if (blockIdx.x == 0 && threadIdx.x == 0 && g_check_probe) {
     g_check_probe = 0;
@@ -113,8 +156,7 @@ __global__ void __launch_bounds__(kHypThreads) k_hyp_count(HypIn in, int64_t H, 
   int64_t base = (int64_t)blockIdx.x * kHypPerBlock;
   for (int it = 0; it < kHypIters; ++it) {
     int64_t h = base + it * kHypThreads + threadIdx.x;
-    int ii[4], jj[4];
-    const bool ok = h < H && hyp_pass(in, (uint32_t)h, ii, jj);
+    const bool ok = h < H && hyp_test(in, rec, (uint32_t)h);
     const unsigned m = __ballot_sync(0xffffffffu, ok);
     if (lane == 0) warp_cnt[w] = __popc(m);
     __syncthreads();
@@ -463,10 +505,11 @@ cudaError_t launch_hypotheses(const float4 *XP, const int *invP, const float4 *N
                               const float4 *NQ, int nQ, const int *nn, const uint8_t *, const uint8_t *, int64_t H,
                               uint64_t seed, uint64_t pair, float tau, int *block_counts, int *block_offsets,
                               int *scan_scratch, int *surv, int surv_cap, RansacState *st, int *local,
-                              cudaStream_t s) {
+                              float4 *rec, cudaStream_t s) {
   HypIn in{XP, invP, NP, nP, XQ, NQ, nQ, nn, seed, pair, tau * tau};
   int nb = hyp_blocks(H);
-  LSR_LAUNCH(k_hyp_count<<<nb, kHypThreads, 0, s>>>(in, H, block_counts, local));
+  LSR_LAUNCH(k_hyp_records<<<(int)lsr_div_up(nP, 256), 256, 0, s>>>(in, rec));
+  LSR_LAUNCH(k_hyp_count<<<nb, kHypThreads, 0, s>>>(in, rec, H, block_counts, local));
   int *nb_dev = block_counts + nb;  // one spare int after the counts holds nb
   LSR_LAUNCH(k_set_int<<<1, 32, 0, s>>>(nb_dev, nb));
   LSR_CUDA_TRY(scan_exclusive(block_counts, block_offsets, nb_dev, nb, scan_scratch, s));
