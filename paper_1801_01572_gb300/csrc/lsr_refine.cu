@@ -193,22 +193,151 @@ __device__ void refine_solve(const double *S, const StepState &ss, RansacState *
   }
 }
 
+// group_nn<kRefG, true> for few queries (grids without wrapped storage): half a
+// warp a query, its lanes read the nine rows' ranges at once and then walk the
+// candidates of all of them together, so that a search is three or four
+// dependent loads long instead of two or more for each row.
+constexpr int kRefH = 16;
+__device__ __forceinline__ void half_nn(const GridParams &g, const int *__restrict__ start,
+                                        const float4 *__restrict__ Xe, float x, float y, float z, float eps2,
+                                        int seed, float guard, int &bt, float &apart) {
+  const int sub = threadIdx.x & (kRefH - 1);
+  float best = eps2, m1 = 3e38f, m2 = 3e38f, reach2 = 3e38f;
+  int bidx = 0x7fffffff;
+  bt = -1;
+  if (seed >= 0 && LSR_IN_BOUNDS(seed, g.npts, kSiteGridPoint)) {
+    const float4 q = Xe[seed];
+    const float d2 = nn_d2(q, x, y, z);
+    if (d2 < eps2) best = d2, bt = seed, bidx = __float_as_int(q.w);
+  }
+  const float fx = (x - g.ox) * g.inv_cell, fy = (y - g.oy) * g.inv_cell, fz = (z - g.oz) * g.inv_cell;
+  bool go = fx >= -1.f && fx < (float)g.nx + 1.f && fy >= -1.f && fy < (float)g.ny + 1.f && fz >= -1.f &&
+            fz < (float)g.nz + 1.f;
+  const int cx = go ? __float2int_rd(fx) : 0, cy = go ? __float2int_rd(fy) : 0, cz = go ? __float2int_rd(fz) : 0;
+  const int x0 = cx - 1 < 0 ? 0 : cx - 1, x1 = cx + 1 > g.nx - 1 ? g.nx - 1 : cx + 1;
+  go = go && x0 <= x1;
+  if (go && g.nbmask && cx >= 0 && cx < g.nx && cy >= 0 && cy < g.ny && cz >= 0 && cz < g.nz) {
+    const int slot = (cz * g.wy + cy) * g.wx + cx;
+    go = (__ldg(g.nbmask + (slot >> 5)) >> (slot & 31)) & 1u;
+  }
+  constexpr float kShrink = 1.f - 1e-6f;  // the FP32 rounding of d^2 itself
+  int b = 0, len = 0;
+  if (go) {
+    const float r = sqrtf(best) + guard, gb = r * r;
+    reach2 = gb * kShrink;
+    // lane sub < 9: a row of cells and the part of it within reach
+    const int dy = sub % 3 - 1, dz = sub / 3 - 1, iy = cy + dy, iz = cz + dz;
+    if (sub < 9 && iy >= 0 && iy < g.ny && iz >= 0 && iz < g.nz) {
+      const float mg = 2e-4f * g.cell;
+      auto gsq = [&](float d) {
+        const float t = fmaxf(d - mg, 0.f);
+        return t * t;
+      };
+      const float ux = fx - (float)cx, uy = fy - (float)cy, uz = fz - (float)cz;
+      const float r2 = (dy < 0 ? gsq(uy * g.cell) : dy > 0 ? gsq((1.f - uy) * g.cell) : 0.f) +
+                       (dz < 0 ? gsq(uz * g.cell) : dz > 0 ? gsq((1.f - uz) * g.cell) : 0.f);
+      int a = x0, e = x1;
+      if (a < cx && (r2 + gsq(ux * g.cell)) * kShrink > gb) a = cx;
+      if (e > cx && (r2 + gsq((1.f - ux) * g.cell)) * kShrink > gb) e = cx;
+      const int row = (iz * g.wy + iy) * g.wx;
+      if (!(r2 * kShrink > gb) && a <= e && LSR_IN_BOUNDS(row + e + 1, g.ncells + 1, kSiteGridRow) &&
+          LSR_IN_BOUNDS(row + a, g.ncells + 1, kSiteGridRow)) {
+        b = start[row + a], len = start[row + e + 1] - b;
+        if (len > 0 && (!LSR_IN_BOUNDS(b + len - 1, g.npts, kSiteGridPoint) || !LSR_IN_BOUNDS(b, g.npts, kSiteGridPoint)))
+          len = 0;
+      }
+    }
+  }
+  // the rows' candidates numbered through: row k's begin at its first
+  int end = len;
+#pragma unroll
+  for (int off = 1; off < kRefH; off <<= 1) {
+    const int o = __shfl_up_sync(0xffffffffu, end, off, kRefH);
+    if (sub >= off) end += o;
+  }
+  const int total = __shfl_sync(0xffffffffu, end, kRefH - 1, kRefH), shift = b - (end - len);
+  const int most = max(total, __shfl_xor_sync(0xffffffffu, total, kRefH));
+  for (int t = sub; t - sub < most; t += kRefH) {
+    int row = 0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) row += t >= __shfl_sync(0xffffffffu, end, k, kRefH);
+    const int at = t + __shfl_sync(0xffffffffu, shift, row, kRefH);
+    if (t < total) {
+      const float4 q = Xe[at];
+      const float d2 = nn_d2(q, x, y, z);
+      m2 = fminf(m2, fmaxf(m1, d2)), m1 = fminf(m1, d2);
+      const int qi = __float_as_int(q.w);
+      if (d2 < best || (d2 == best && qi < bidx)) best = d2, bt = at, bidx = qi;
+    }
+  }
+#pragma unroll
+  for (int off = kRefH / 2; off > 0; off >>= 1) {
+    const float ob = __shfl_xor_sync(0xffffffffu, best, off);
+    const int ot = __shfl_xor_sync(0xffffffffu, bt, off);
+    const int oi = __shfl_xor_sync(0xffffffffu, bidx, off);
+    if (ob < best || (ob == best && oi < bidx)) best = ob, bt = ot, bidx = oi;
+    const float o1 = __shfl_xor_sync(0xffffffffu, m1, off), o2 = __shfl_xor_sync(0xffffffffu, m2, off);
+    m2 = fminf(fmaxf(m1, o1), fminf(m2, o2)), m1 = fminf(m1, o1);
+  }
+  // (as group_nn)
+  const float other = bt >= 0 && m1 <= best ? m2 : m1;
+  apart = fminf(sqrtf(fminf(other, reach2)), nn_border(g, fx, fy, fz)) * (1.f - 4e-6f);
+}
+
 // One IRLS step. Every block accumulates its points; the last block to
 // finish (atomic ticket, no waiting) sums all block partials and solves.
-__global__ void __launch_bounds__(kRefThreads, kRefBlocksPerSm) k_refine_step(const float4 *__restrict__ XP, int nP, int strideP,
+//
+// Most steps move the points by far less than the gap between their nearest
+// and second nearest Q point, so most searches would find what the last one
+// found. A search therefore also leaves where it was made and a distance that
+// no other point is closer than (group_nn, kApart); by the triangle inequality
+// the neighbour stands while its distance now is below that distance less the
+// way moved since, and there is still none while eps is. A block first decides
+// that with a point per thread, lists the points that need a search, searches
+// those with kRefG lanes each, and a point per thread then lays out the values
+// whose products the sums take. The neighbours are those of a search of every
+// point. With a search of every point each step was bound by the latency of
+// the grid walks (42 us of 55 at 150k points).
+// seeds[i]: the neighbour, kSeedNone or kSeedFresh (no search yet at this level).
+//
+// A block's points are the runs of kRefSlots points numbered blockIdx.x,
+// + gridDim.x, ..., kRefRuns of them at a time; the 17 sums of each slot go
+// through the runs in order (four lanes a slot, every fourth sum each), then
+// over the slots.
+constexpr int kSeedFresh = -1, kSeedNone = -2;
+// Cells are visited up to this part of eps beyond the nearest point (a refinement
+// of 50k points took 3.31 ms with 0.06, 3.26 with 0.125, 3.47 with 0.25).
+constexpr float kRefGuard = 0.125f;
+// Up to this many searches of a block take half a warp each (a refinement of 50k
+// points: 3.64 ms with none, 3.26 with 64, 3.28 with all).
+constexpr int kRefFew = 64;
+constexpr int kRefSlots = 64, kRefRuns = kRefThreads / kRefSlots;
+// The values of a point: 1, w, w xc (3), xc (3), xc x e (3), e (3), or all 0
+// without a neighbour; sum k takes the products of kTermA[k] and kTermB[k].
+constexpr int kNVal = 14;
+__constant__ const unsigned char kTermA[20] = {0, 1, 2, 3, 4, 2, 2, 2, 3, 3, 4, 1, 1, 1, 1, 1, 1, 0, 0, 0};
+__constant__ const unsigned char kTermB[20] = {0, 0, 0, 0, 0, 5, 6, 7, 6, 7, 7, 8, 9, 10, 11, 12, 13, 0, 0, 0};
+
+__global__ void __launch_bounds__(kRefThreads, kRefBlocksPerSm) k_refine_step(const float4 *__restrict__ XP, int nP,
                                                              const GridParams *gep, const int *__restrict__ start,
-                                                             const float4 *__restrict__ Xe, float eps2, float mu,
+                                                             const float4 *__restrict__ Xe, float eps, float mu,
                                                              RansacState *st, double *partials, int max_iters,
-                                                             double tol, int *__restrict__ seeds) {
-  __shared__ int s_last;
+                                                             double tol, int *__restrict__ seeds,
+                                                             float4 *__restrict__ certs) {
+  __shared__ int s_last, s_need;
   __shared__ double tot[kNSum];
+  __shared__ float4 s_query[kRefThreads];  // the points to search: position, thread
+  __shared__ int s_found[kRefThreads];     // per thread: its seed, then its neighbour
+  __shared__ float s_val[kNVal][kRefThreads + 8];
   // the next step may be scheduled now (launched as a programmatic dependent,
   // it waits below for this one to finish); this step reads the pose, the
   // state and the seeds the previous step wrote
   asm volatile("griddepcontrol.launch_dependents;");
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  const int run = gridDim.x * kRefSlots;  // points from one run of this block to its next
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (!st->active) return;
-  const GridParams g = *gep;
+  const float eps2 = eps * eps;
   const double *T = st->T;
   float R[9], tc[3], c[3];
   for (int r = 0; r < 3; ++r) {
@@ -216,53 +345,114 @@ __global__ void __launch_bounds__(kRefThreads, kRefBlocksPerSm) k_refine_step(co
     c[r] = (float)st->center[r];
     tc[r] = (float)(T[4 * r + 3] - st->center[r]);
   }
-  constexpr int G = kRefG, GPB = kRefThreads / G;
-  const int grp = threadIdx.x / G, sub = threadIdx.x & (G - 1);
-  float acc[kNSum];
+  if (threadIdx.x == 0) s_need = 0;
+  // sums lane % 4, + 4, ... of the slot threadIdx.x / 4
+  constexpr int kMine = (kNSum + 3) / 4;
+  float acc[kMine];
 #pragma unroll
-  for (int u = 0; u < kNSum; ++u) acc[u] = 0.f;
-  // block-uniform trip count: every lane reaches the group shuffles
-  for (int r0 = blockIdx.x * GPB; r0 < nP; r0 += gridDim.x * GPB) {
-    int i = r0 + grp;
-    bool valid = i < nP;
-    float4 p = valid ? XP[i] : make_float4(0.f, 0.f, 0.f, 0.f);
-    if (valid && strideP > 1 && __float_as_int(p.w) % strideP != 0) valid = false;
-    if (!valid) p.x = __int_as_float(0x7fc00000);  // NaN: the query visits no cell
-    const float xc0 = fmaf(R[0], p.x, fmaf(R[1], p.y, fmaf(R[2], p.z, tc[0])));
-    const float xc1 = fmaf(R[3], p.x, fmaf(R[4], p.y, fmaf(R[5], p.z, tc[1])));
-    const float xc2 = fmaf(R[6], p.x, fmaf(R[7], p.y, fmaf(R[8], p.z, tc[2])));
-    const float x = xc0 + c[0], y = xc1 + c[1], z = xc2 + c[2];
-    float best;
-    int bt, bidx;
-    // the previous step's neighbour of this point starts the search (an exact
-    // search either way)
-    const int seed = valid ? seeds[i] : -1;
-    group_nn<G>(g, start, Xe, x, y, z, eps2, best, bt, bidx, seed);
-    if (valid && sub == 0) seeds[i] = bt;
-    if (!valid || bt < 0 || sub != 0) continue;
-    const float4 q = Xe[bt];
-    const float e0 = x - q.x, e1 = y - q.y, e2 = z - q.z;  // the residual
-    const float s = e0 * e0 + e1 * e1 + e2 * e2;
-    const float l = mu / (mu + s);
-    const float w = l * l;
-    const float w0 = w * xc0, w1 = w * xc1, w2 = w * xc2;
-    acc[0] += 1.f;
-    acc[1] += w;
-    acc[2] += w0, acc[3] += w1, acc[4] += w2;
-    acc[5] += w0 * xc0, acc[6] += w0 * xc1, acc[7] += w0 * xc2;
-    acc[8] += w1 * xc1, acc[9] += w1 * xc2, acc[10] += w2 * xc2;
-    acc[11] += w * (xc1 * e2 - xc2 * e1);
-    acc[12] += w * (xc2 * e0 - xc0 * e2);
-    acc[13] += w * (xc0 * e1 - xc1 * e0);
-    acc[14] += w * e0, acc[15] += w * e1, acc[16] += w * e2;
+  for (int u = 0; u < kMine; ++u) acc[u] = 0.f;
+  for (int r0 = blockIdx.x * kRefSlots; r0 < nP; r0 += kRefRuns * run) {
+    const int i = r0 + (threadIdx.x / kRefSlots) * run + (threadIdx.x % kRefSlots);
+    const bool valid = i < nP;
+    float xc0 = 0.f, xc1 = 0.f, xc2 = 0.f, x = 0.f, y = 0.f, z = 0.f;
+    int bt = kSeedNone;
+    bool search = false;
+    __syncthreads();  // s_need is 0; the previous round's s_found and s_val have been read
+    if (valid) {
+      const float4 p = XP[i], at = certs[i];
+      const int seed = seeds[i];
+      xc0 = fmaf(R[0], p.x, fmaf(R[1], p.y, fmaf(R[2], p.z, tc[0])));
+      xc1 = fmaf(R[3], p.x, fmaf(R[4], p.y, fmaf(R[5], p.z, tc[1])));
+      xc2 = fmaf(R[6], p.x, fmaf(R[7], p.y, fmaf(R[8], p.z, tc[2])));
+      x = xc0 + c[0], y = xc1 + c[1], z = xc2 + c[2];
+      bt = seed;
+      search = true;
+      if (seed != kSeedFresh) {
+        float d = eps;
+        if (seed >= 0 && LSR_IN_BOUNDS(seed, gep->npts, kSiteGridPoint)) d = sqrtf(nn_d2(Xe[seed], x, y, z));
+        // (4e-6: above the FP32 rounding of both distances; a NaN searches)
+        search = !((d + sqrtf(nn_d2(at, x, y, z))) * (1.f + 4e-6f) < at.w);
+      }
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, search);
+    if (m) {
+      int base = 0;
+      if (lane == 0) base = atomicAdd(&s_need, __popc(m));
+      base = __shfl_sync(0xffffffffu, base, 0);
+      if (search) {
+        s_query[base + __popc(m & ((1u << lane) - 1u))] = make_float4(x, y, z, __int_as_float(threadIdx.x));
+        s_found[threadIdx.x] = bt;
+      }
+    }
+    __syncthreads();
+    const int need = s_need;
+    if (need) {
+      constexpr int kWarps = kRefThreads / 32;
+      const GridParams g = *gep;
+      const bool few = need <= kRefFew && g.wx == g.nx && g.wy == g.ny && g.wz == g.nz;
+      const int G = few ? kRefH : kRefG;  // lanes a query
+      // consecutive queries go to different warps; whole warps reach the shuffles
+      for (int q0 = wp; q0 < need; q0 += kRefThreads / G) {
+        const int k = q0 + kWarps * (lane / G);
+        float4 w = make_float4(__int_as_float(0x7fc00000), 0.f, 0.f, 0.f);  // NaN: the query visits no cell
+        int thread = 0, seed = -1;
+        if (k < need) w = s_query[k], thread = __float_as_int(w.w), seed = s_found[thread];
+        float best, apart;
+        int nn, bidx;
+        if (few)
+          half_nn(g, start, Xe, w.x, w.y, w.z, eps2, seed, kRefGuard * eps, nn, apart);
+        else
+          group_nn<kRefG, true>(g, start, Xe, w.x, w.y, w.z, eps2, best, nn, bidx, seed, kRefGuard * eps, &apart);
+        if (k < need && (lane & (G - 1)) == 0) {
+          nn = nn < 0 ? kSeedNone : nn;
+          s_found[thread] = nn;
+          const int j = r0 + (thread / kRefSlots) * run + (thread % kRefSlots);
+          seeds[j] = nn;
+          certs[j] = make_float4(w.x, w.y, w.z, apart);
+        }
+      }
+      __syncthreads();
+      if (threadIdx.x == 0) s_need = 0;
+      if (search) bt = s_found[threadIdx.x];
+    }
+    const float4 q = bt >= 0 ? Xe[bt] : make_float4(__int_as_float(0x7fc00000), 0.f, 0.f, 0.f);
+    float v[kNVal];
+#pragma unroll
+    for (int u = 0; u < kNVal; ++u) v[u] = 0.f;
+    if (nn_d2(q, x, y, z) < eps2) {
+      const float e0 = x - q.x, e1 = y - q.y, e2 = z - q.z;  // the residual
+      const float s = e0 * e0 + e1 * e1 + e2 * e2;
+      const float l = mu / (mu + s);
+      const float w = l * l;
+      v[0] = 1.f, v[1] = w;
+      v[2] = w * xc0, v[3] = w * xc1, v[4] = w * xc2;
+      v[5] = xc0, v[6] = xc1, v[7] = xc2;
+      v[8] = xc1 * e2 - xc2 * e1;
+      v[9] = xc2 * e0 - xc0 * e2;
+      v[10] = xc0 * e1 - xc1 * e0;
+      v[11] = e0, v[12] = e1, v[13] = e2;
+    }
+#pragma unroll
+    for (int u = 0; u < kNVal; ++u) s_val[u][threadIdx.x] = v[u];
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < kMine; ++u) {
+      const float *A = s_val[kTermA[4 * u + (lane & 3)]], *B = s_val[kTermB[4 * u + (lane & 3)]];
+#pragma unroll
+      for (int k = 0; k < kRefRuns; ++k) {
+        const int t = k * kRefSlots + threadIdx.x / 4;
+        acc[u] = fmaf(A[t], B[t], acc[u]);
+      }
+    }
   }
   {
-    __shared__ float sm[kRefThreads / 32][kNSum];
-    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+    __shared__ float sm[kRefThreads / 32][4 * kMine];
 #pragma unroll
-    for (int u = 0; u < kNSum; ++u) {
-      const float v = warp_sum(acc[u]);
-      if (lane == 0) sm[wp][u] = v;
+    for (int u = 0; u < kMine; ++u) {
+      // over the warp's eight slots
+#pragma unroll
+      for (int off = 16; off >= 4; off >>= 1) acc[u] += __shfl_xor_sync(0xffffffffu, acc[u], off);
+      if (lane < 4) sm[wp][4 * u + lane] = acc[u];
     }
     __syncthreads();
     if (threadIdx.x < kNSum) {
@@ -591,19 +781,19 @@ cudaError_t launch_subsample(const float *xyz, int n, int stride, float4 *out, c
   return cudaGetLastError();
 }
 
-cudaError_t launch_refine_step(const float4 *XP, int nP, int strideP, const GridParams *ge, const int *start_e,
-                               const float4 *Xe, float eps_r, float mu, int max_iters, RansacState *st,
-                               double *partials, int *seeds, bool chained, cudaStream_t s) {
-  int nb = refine_blocks((int)lsr_div_up(nP, strideP));
+cudaError_t launch_refine_step(const float4 *XP, int nP, const GridParams *ge, const int *start_e, const float4 *Xe,
+                               float eps_r, float mu, int max_iters, RansacState *st, double *partials, int *seeds,
+                               float4 *certs, bool chained, cudaStream_t s) {
+  const int nb = refine_blocks(nP);
   if (chained) {
     // directly after the previous step: scheduled while it closes
     cudaError_t e = cudaSuccess;
-    LSR_LAUNCH(e = pdl_launch(k_refine_step, dim3(nb), dim3(kRefThreads), s, XP, nP, strideP, ge, start_e, Xe,
-                              eps_r * eps_r, mu, st, partials, max_iters, 1e-6, seeds));
+    LSR_LAUNCH(e = pdl_launch(k_refine_step, dim3(nb), dim3(kRefThreads), s, XP, nP, ge, start_e, Xe, eps_r, mu, st,
+                              partials, max_iters, 1e-6, seeds, certs));
     LSR_CUDA_TRY(e);
   } else {
-    LSR_LAUNCH(k_refine_step<<<nb, kRefThreads, 0, s>>>(XP, nP, strideP, ge, start_e, Xe, eps_r * eps_r, mu, st,
-                                                        partials, max_iters, 1e-6, seeds));
+    LSR_LAUNCH(k_refine_step<<<nb, kRefThreads, 0, s>>>(XP, nP, ge, start_e, Xe, eps_r, mu, st, partials, max_iters,
+                                                        1e-6, seeds, certs));
   }
   return cudaGetLastError();
 }
