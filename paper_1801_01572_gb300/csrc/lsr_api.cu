@@ -211,6 +211,8 @@ struct CloudLayout {
   float4 *X = nullptr, *Xn = nullptr, *Xe = nullptr, *N = nullptr;
   int *inv = nullptr;
   float *S = nullptr, *F = nullptr;
+  int2 *win = nullptr;  // FPFH windows
+  int *win_ctl = nullptr;
   unsigned *mask_e = nullptr;
 };
 
@@ -241,6 +243,8 @@ void plan_cloud(Arena &a, int n, bool stage_src, bool features, bool eps_grid, C
     c.N = a.take<float4>(n);
     c.S = a.take<float>((size_t)n * kDS);
     c.F = a.take<float>((size_t)n * kDS);
+    c.win = a.take<int2>(n);
+    c.win_ctl = a.take<int>(kWinCtl);
   }
   if (eps_grid) {
     c.start_e = a.take<int>((size_t)c.cap_e + 1);
@@ -749,8 +753,8 @@ int enqueue_pair(lsr_ctx *c, const PairLayout &L, const float *P, const float *Q
   tm.mark();
   TRY_CUDA(c, launch_spfh(Pc.X, Pc.N, nP, Pc.gf, Pc.start_f, p.r_feature, Pc.S, nullptr, Pc.F, s), "spfh P");
   TRY_CUDA(c, launch_spfh(Qc.X, Qc.N, nQ, Qc.gf, Qc.start_f, p.r_feature, Qc.S, nullptr, Qc.F, s), "spfh Q");
-  TRY_CUDA(c, launch_fpfh(Pc.X, Pc.N, Pc.S, nP, Pc.gf, Pc.start_f, p.r_feature, Pc.F, s), "fpfh P");
-  TRY_CUDA(c, launch_fpfh(Qc.X, Qc.N, Qc.S, nQ, Qc.gf, Qc.start_f, p.r_feature, Qc.F, s), "fpfh Q");
+  TRY_CUDA(c, launch_fpfh(Pc.X, Pc.N, Pc.S, nP, Pc.gf, Pc.start_f, p.r_feature, Pc.win, Pc.win_ctl, Pc.F, s), "fpfh P");
+  TRY_CUDA(c, launch_fpfh(Qc.X, Qc.N, Qc.S, nQ, Qc.gf, Qc.start_f, p.r_feature, Qc.win, Qc.win_ctl, Qc.F, s), "fpfh Q");
   tm.mark();
   if (p.match_precision != LSR_MATCH_FP32)
     TRY_CUDA(c,
@@ -1622,7 +1626,7 @@ static int stage_desc_common(lsr_ctx *c, const float *P, const float *normals, c
   } else {
     TRY_CUDA(c, cudaMemcpyAsync(sp, spfh_in, sizeof(float) * kD * n, cudaMemcpyDefault, s), "copy spfh");
     LSR_LAUNCH(k_gather_rows<<<nblk(n * kDS), 256, 0, s>>>(sp, kD, C.X, (int)n, C.S));
-    TRY_CUDA(c, launch_fpfh(C.X, C.N, C.S, (int)n, C.gf, C.start_f, r, C.F, s), "fpfh");
+    TRY_CUDA(c, launch_fpfh(C.X, C.N, C.S, (int)n, C.gf, C.start_f, r, C.win, C.win_ctl, C.F, s), "fpfh");
     LSR_LAUNCH(k_scatter_rows<<<nblk(n * kD), 256, 0, s>>>(C.F, C.X, (int)n, o));
   }
   TRY_CUDA(c, cudaGetLastError(), "stage kernels");

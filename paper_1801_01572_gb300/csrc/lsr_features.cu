@@ -4,7 +4,7 @@
 // Normals and SPFH are warp-per-point: the 32 lanes of a warp stride over the
 // contiguous sorted ranges of the neighbouring grid cells, so the neighbour
 // loads of a warp are coalesced and the work per point is split evenly. FPFH
-// is lane-per-point over candidates staged in shared memory (see k_fpfh).
+// is lane-per-point over candidates staged in shared memory (fpfh_window).
 #include <math_constants.h>
 
 #include "lsr_internal.cuh"
@@ -15,6 +15,7 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
+constexpr int kWin = 64;  // points of a window
 
 __device__ __forceinline__ float3 f3(float4 a) { return make_float3(a.x, a.y, a.z); }
 __device__ __forceinline__ float dot3(float3 a, float3 b) { return a.x * b.x + a.y * b.y + a.z * b.z; }
@@ -302,48 +303,114 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait_group() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-// FPFH: one query per lane. A window of 32 consecutive points of the
-// cell-sorted array is taken by kFpParts warps of one block; the lanes whose
-// queries lie in the same grid cell (most of a window: a cell holds dozens of
-// points) walk that cell's 3 x 3 x 3 neighbourhood together. The cell's
+// Windows: runs of at most kWin consecutive points of the cell-sorted array that
+// share a storage cell (first point, number of points), in no particular order.
+// ctl[0]: their number; ctl[1]: the next one to take (the blocks take them one by
+// one, so that long ones do not queue up behind each other).
+__global__ void k_windows(const GridParams *gfp, const int *__restrict__ start, int2 *__restrict__ win,
+                          int *__restrict__ ctl) {
+  const int ncells = gfp->ncells, lane = threadIdx.x & 31;
+  for (int c0 = (blockIdx.x * blockDim.x + threadIdx.x) & ~31; c0 < ncells; c0 += gridDim.x * blockDim.x) {
+    const int c = c0 + lane;
+    int b = 0, m = 0;
+    if (c < ncells) b = start[c], m = start[c + 1] - b;
+    const int k = (m + kWin - 1) / kWin;
+    if (!__any_sync(0xffffffffu, k > 0)) continue;
+    int end = k;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const int o = __shfl_up_sync(0xffffffffu, end, off);
+      if (lane >= off) end += o;
+    }
+    int base = 0;
+    if (lane == 31) base = atomicAdd(ctl, end);
+    base = __shfl_sync(0xffffffffu, base, 31) + end - k;
+    for (int u = 0; u < k; ++u) win[base + u] = make_int2(b + u * kWin, min(kWin, m - u * kWin));
+  }
+}
+
+// The candidate ranges of the cell of (x, y, z), in the order of grid_ranges
+// without the empty ones, listed by a warp as (begin, end) pairs in rl (27 at
+// most); their number is returned. Without wrapped storage the nine rows are
+// read at once, a lane each.
+__device__ __forceinline__ int cell_ranges(const GridParams &g, const int *__restrict__ start, float x, float y,
+                                           float z, int *rl) {
+  const int lane = threadIdx.x & 31;
+  int nr = 0;
+  if ((g.wx != g.nx) | (g.wy != g.ny) | (g.wz != g.nz)) {
+    grid_ranges(g, start, x, y, z, [&](int b, int e) {
+      if (b >= e) return;
+      if (lane == 0) rl[2 * nr] = b, rl[2 * nr + 1] = e;
+      ++nr;
+    });
+    __syncwarp();
+    return nr;
+  }
+  const int cx = __float2int_rd((x - g.ox) * g.inv_cell), cy = __float2int_rd((y - g.oy) * g.inv_cell),
+            cz = __float2int_rd((z - g.oz) * g.inv_cell);
+  const int x0 = max(cx - 1, 0), x1 = min(cx + 1, g.nx - 1), iy = cy + lane % 3 - 1, iz = cz + lane / 3 - 1;
+  int b = 0, e = 0;
+  if (lane < 9 && x0 <= x1 && iy >= 0 && iy < g.ny && iz >= 0 && iz < g.nz) {
+    const int row = (iz * g.wy + iy) * g.wx;
+    if (LSR_IN_BOUNDS(row + x1 + 1, g.ncells + 1, kSiteGridRow) && LSR_IN_BOUNDS(row + x0, g.ncells + 1, kSiteGridRow))
+      b = start[row + x0], e = start[row + x1 + 1];
+    if (e > b && (!LSR_IN_BOUNDS(e - 1, g.npts, kSiteGridPoint) || !LSR_IN_BOUNDS(b, g.npts, kSiteGridPoint))) b = e;
+  }
+  const unsigned m = __ballot_sync(0xffffffffu, b < e);
+  if (b < e) {
+    nr = __popc(m & ((1u << lane) - 1u));
+    rl[2 * nr] = b, rl[2 * nr + 1] = e;
+  }
+  __syncwarp();
+  return __popc(m);
+}
+
+// FPFH: one or two queries per lane. A window is taken by kFpParts warps, a
+// block; its queries walk their cell's 3 x 3 x 3 neighbourhood together
+// (wrapped storage: once per distinct cell). The cell's
 // candidate ranges are listed, cut into chunks of 32 candidates and dealt out
 // to the window's warps round robin; a warp copies its next chunk's positions,
 // normal flags and SPFH rows (contiguous in the sorted array) to shared memory
 // with coalesced asynchronous copies while it sums the current one, every lane
 // reading each candidate from there (a broadcast) and adding its row weighted
 // by 1/d when the candidate is its neighbour (0 < d <= r, not itself, valid
-// normal). A window spanning several cells walks once per distinct cell. The
-// parts' sums are then added in part order (the window's warps meet at a named
-// barrier of their own), SPFH(p) added and each lane's three sub-histograms
-// rescaled. Every sum runs in a fixed order, so the result is deterministic.
+// normal). The parts' sums are then added in part order, SPFH(p) added and each
+// query's three sub-histograms rescaled. Every sum runs in a fixed order, so
+// the result is deterministic.
+// Bound by instruction issue (63% of the cycles; ~70 instructions a candidate and
+// window, of them 34 packed multiply-adds and 10 loads) and its latency at 15
+// warps an SM. Windows of 32 consecutive points whatever their cells walked 1.5
+// neighbourhoods each with a query per lane (9 loads and 33 multiply-adds for
+// 11 neighbours); two queries a lane without the cut at cells walked 1.9 and
+// gained nothing. 120k points: 790 us under ncu, 1131 without the cut.
 constexpr int kFpParts = 3;                      // warps per window
-constexpr int kFpWin = 2;                        // windows per block
-constexpr int kFpThreads = 32 * kFpParts * kFpWin;
+constexpr int kFpThreads = 32 * kFpParts;        // a block is a window
 constexpr int kFpRowV = kDS / 4;                 // float4 per SPFH row
+constexpr int kFpAcc = (kD + 1) / 2;             // sums of a query, two to a register pair
 // one staging buffer: 32 rows, 32 positions, 32 normal flags (float4 units)
 constexpr int kFpBufV = 32 * kFpRowV + 32 + 8;
 constexpr int kFpWarpV = 2 * kFpBufV + 14;    // two buffers and the range list (27 pairs) a warp
-constexpr int kFpSmem = kFpParts * kFpWin * kFpWarpV * 16;
-static_assert(kFpRowV * 32 * 4 >= (kD + 1) * 32, "the staging buffer holds a part's sums");
+constexpr int kFpSmem = kFpParts * kFpWarpV * 16;
+static_assert(2 * kFpBufV * 4 >= 2 * (kD + 1) * 32, "the staging buffers hold a part's sums");
+static_assert(kWin == 64, "two queries a lane");
 
-// barrier of the kFpParts warps of one window (named barrier 1 + window slot)
-__device__ __forceinline__ void window_sync(int wslot) {
-  static_assert(kFpWin == 2, "one named barrier per window slot");
-  if (wslot == 0)
-    asm volatile("bar.sync 1, %0;" ::"n"(32 * kFpParts) : "memory");
-  else
-    asm volatile("bar.sync 2, %0;" ::"n"(32 * kFpParts) : "memory");
+// acc += w v on two FP32 lanes at once (each rounded as fmaf rounds)
+__device__ __forceinline__ void fma2(unsigned long long &acc, unsigned long long w, unsigned long long v) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(w), "l"(v));
+}
+__device__ __forceinline__ float2 unpack2(unsigned long long v) {
+  return make_float2(__uint_as_float((unsigned)v), __uint_as_float((unsigned)(v >> 32)));
 }
 
-__global__ void __launch_bounds__(kFpThreads, 3) k_fpfh(const float4 *__restrict__ X, const float4 *__restrict__ N,
-                                                        const float *__restrict__ S, int n, const GridParams *gfp,
-                                                        const int *__restrict__ start, float r2,
-                                                        float *__restrict__ F) {
-  extern __shared__ float4 fp_smem[];
-  const GridParams g = *gfp;
-  const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
-  const int part = wl % kFpParts, wslot = wl / kFpParts;
-  float4 *const wbuf = fp_smem + (size_t)wl * kFpWarpV;
+// kQ queries a lane: a window of `count` points from `first` on.
+template <int kQ>
+__device__ __forceinline__ void fpfh_window(const float4 *__restrict__ X, const float4 *__restrict__ N,
+                                            const float *__restrict__ S, const GridParams &g,
+                                            const int *__restrict__ start, float r2, float *__restrict__ F, int first,
+                                            int count, float4 *fp_smem) {
+  const int lane = threadIdx.x & 31, part = threadIdx.x >> 5;
+  const int n = first + count;
+  float4 *const wbuf = fp_smem + (size_t)part * kFpWarpV;
   // stage candidates c0 .. c0 + m - 1 into buffer bi
   auto stage = [&](int c0, int m, int bi) {
     float4 *bb = wbuf + bi * kFpBufV;
@@ -359,43 +426,56 @@ __global__ void __launch_bounds__(kFpThreads, 3) k_fpfh(const float4 *__restrict
     }
     cp_async_commit();
   };
-  const int nwin = (n + 31) / 32;
-  // the window's warps meet at its barrier twice a window (the trip count is
-  // the same for the whole block)
-  for (int wb = blockIdx.x * kFpWin; wb < nwin; wb += gridDim.x * kFpWin) {
-    const int i0 = (wb + wslot) * 32;
-    const int i = i0 + lane;
-    const bool in = i < n;
-    const float4 p4 = in ? X[i] : make_float4(0.f, 0.f, 0.f, 0.f);
-    const bool valid = in && N[i].w >= 0.f;
-    // the cell as the grid walk computes it (the grouping key)
-    const int cx = __float2int_rd((p4.x - g.ox) * g.inv_cell), cy = __float2int_rd((p4.y - g.oy) * g.inv_cell),
-              cz = __float2int_rd((p4.z - g.oz) * g.inv_cell);
-    float acc[kD];
+  {
+    const int i0 = first + lane;  // query q of this lane: i0 + 32 q
+    float3 p[kQ];
+    unsigned todo[kQ];
 #pragma unroll
-    for (int b = 0; b < kD; ++b) acc[b] = 0.f;
-    int kk = 0;
-    unsigned todo = __ballot_sync(0xffffffffu, valid);
-    while (todo) {
-      const int lead = __ffs(todo) - 1;
-      const int lx = __shfl_sync(0xffffffffu, cx, lead), ly = __shfl_sync(0xffffffffu, cy, lead),
-                lz = __shfl_sync(0xffffffffu, cz, lead);
-      const bool mine = valid && cx == lx && cy == ly && cz == lz && ((todo >> lane) & 1u);
-      todo &= ~__ballot_sync(0xffffffffu, mine);
-      // the leader's position gives the cell's ranges (the same for every
-      // lane of the group and every part); every lane runs the uniform loop
-      const float px = __shfl_sync(0xffffffffu, p4.x, lead), py = __shfl_sync(0xffffffffu, p4.y, lead),
-                  pz = __shfl_sync(0xffffffffu, p4.z, lead);
+    for (int q = 0; q < kQ; ++q) {
+      const int i = i0 + 32 * q;
+      p[q] = i < n ? f3(X[i]) : make_float3(0.f, 0.f, 0.f);
+      todo[q] = __ballot_sync(0xffffffffu, i < n && N[i].w >= 0.f);
+    }
+    const auto valid = [&](int q) { return i0 + 32 * q < n && N[i0 + 32 * q].w >= 0.f; };
+    // the cell as the grid walk computes it (the grouping key)
+    const auto cell = [&](float3 v) {
+      return make_int3(__float2int_rd((v.x - g.ox) * g.inv_cell), __float2int_rd((v.y - g.oy) * g.inv_cell),
+                       __float2int_rd((v.z - g.oz) * g.inv_cell));
+    };
+    unsigned long long acc[kQ][kFpAcc];
+    int kk[kQ];
+#pragma unroll
+    for (int q = 0; q < kQ; ++q) {
+      kk[q] = 0;
+#pragma unroll
+      for (int b = 0; b < kFpAcc; ++b) acc[q][b] = 0ull;
+    }
+    while (true) {
+      // the first query left leads: those in its cell walk the cell's ranges together
+      float3 l = make_float3(0.f, 0.f, 0.f);
+      bool left = false;
+#pragma unroll
+      for (int q = kQ - 1; q >= 0; --q) {
+        if (!todo[q]) continue;
+        const int lead = __ffs(todo[q]) - 1;
+        l = make_float3(__shfl_sync(0xffffffffu, p[q].x, lead), __shfl_sync(0xffffffffu, p[q].y, lead),
+                        __shfl_sync(0xffffffffu, p[q].z, lead));
+        left = true;
+      }
+      if (!left) break;
+      const int3 lc = cell(l);
+      float rr[kQ];  // r^2 for the queries of this walk, a negative bound for the others
+#pragma unroll
+      for (int q = 0; q < kQ; ++q) {
+        const int3 c = cell(p[q]);
+        const bool mine = ((todo[q] >> lane) & 1u) && c.x == lc.x && c.y == lc.y && c.z == lc.z;
+        todo[q] &= ~__ballot_sync(0xffffffffu, mine);
+        rr[q] = mine ? r2 : -1.f;
+      }
       // the cell's candidate ranges, listed first (uniform), then dealt out
       // to the window's warps 32 candidates at a time, round robin
       int *rl = reinterpret_cast<int *>(wbuf + 2 * kFpBufV);
-      int nr = 0;
-      grid_ranges(g, start, px, py, pz, [&](int b, int e) {
-        if (b >= e) return;
-        if (lane == 0) rl[2 * nr] = b, rl[2 * nr + 1] = e;
-        ++nr;
-      });
-      __syncwarp();
+      const int nr = cell_ranges(g, start, l.x, l.y, l.z, rl);
       // (r, k): chunk k of range r; advance past the ends of ranges
       auto settle = [&](int &r, int &k) {
         while (r < nr) {
@@ -437,49 +517,72 @@ __global__ void __launch_bounds__(kFpThreads, 3) k_fpfh(const float4 *__restrict
         const float *nw = reinterpret_cast<const float *>(pos + 32);
 #pragma unroll 1
         for (int j = 0; j < m; ++j) {
-          const float4 q4 = pos[j];
-          const float dx = q4.x - p4.x, dy = q4.y - p4.y, dz = q4.z - p4.z;
-          const float d2 = dx * dx + dy * dy + dz * dz;
-          const bool acc_t = mine && c0 + j != i && d2 <= r2 && d2 != 0.f && nw[j] >= 0.f;
-          if (!__any_sync(0xffffffffu, acc_t)) continue;
-          const float w = acc_t ? rsqrtf(d2) : 0.f;
-          kk += acc_t ? 1 : 0;
-          const float4 *rj = rows + kFpRowV * j;
+          const float4 c4 = pos[j];
+          const bool cv = nw[j] >= 0.f;
+          float w[kQ];
+          bool any = false;
 #pragma unroll
-          for (int q = 0; q < 8; ++q) {
-            const float4 v = rj[q];
-            acc[4 * q + 0] += w * v.x;
-            acc[4 * q + 1] += w * v.y;
-            acc[4 * q + 2] += w * v.z;
-            acc[4 * q + 3] += w * v.w;
+          for (int q = 0; q < kQ; ++q) {
+            const float dx = c4.x - p[q].x, dy = c4.y - p[q].y, dz = c4.z - p[q].z;
+            const float d2 = dx * dx + dy * dy + dz * dz;
+            const bool take = cv && c0 + j != i0 + 32 * q && d2 <= rr[q] && d2 != 0.f;
+            w[q] = take ? rsqrtf(d2) : 0.f;
+            kk[q] += take ? 1 : 0;
+            any |= take;
           }
-          acc[32] += w * rj[8].x;
+          if (!__any_sync(0xffffffffu, any)) continue;
+          unsigned long long ww[kQ];
+#pragma unroll
+          for (int q = 0; q < kQ; ++q) asm("mov.b64 %0, {%1, %1};" : "=l"(ww[q]) : "f"(w[q]));
+          const ulonglong2 *rj = reinterpret_cast<const ulonglong2 *>(rows + kFpRowV * j);
+#pragma unroll
+          for (int u = 0; u < kFpAcc / 2; ++u) {
+            const ulonglong2 v = rj[u];
+#pragma unroll
+            for (int q = 0; q < kQ; ++q) {
+              fma2(acc[q][2 * u], ww[q], v.x);
+              fma2(acc[q][2 * u + 1], ww[q], v.y);
+            }
+          }
+          const unsigned long long v = rj[kFpAcc / 2].x;
+#pragma unroll
+          for (int q = 0; q < kQ; ++q) fma2(acc[q][kFpAcc - 1], ww[q], v);
         }
         __syncwarp();  // this buffer is refilled two chunks on
         r = rn, k = kn, bi ^= 1;
       }
     }
-    // the parts' sums meet in the staging buffers ([bin][lane], then counts)
+    // the parts' sums meet in the staging buffers (per query [bin][lane], then counts)
     float *cb = reinterpret_cast<float *>(wbuf);
 #pragma unroll
-    for (int b = 0; b < kD; ++b) cb[b * 32 + lane] = acc[b];
-    cb[kD * 32 + lane] = __int_as_float(kk);
-    window_sync(wslot);
-    if (part == 0 && in) {
-      kk = 0;
+    for (int q = 0; q < kQ; ++q) {
 #pragma unroll
-      for (int b = 0; b < kD; ++b) acc[b] = 0.f;
-      for (int pp = 0; pp < kFpParts; ++pp) {
-        const float *ob = reinterpret_cast<const float *>(fp_smem + (size_t)(wslot * kFpParts + pp) * kFpWarpV);
-#pragma unroll
-        for (int b = 0; b < kD; ++b) acc[b] += ob[b * 32 + lane];
-        kk += __float_as_int(ob[kD * 32 + lane]);
+      for (int b = 0; b < kD; ++b) {
+        const float2 v = unpack2(acc[q][b / 2]);
+        cb[(q * (kD + 1) + b) * 32 + lane] = (b & 1) ? v.y : v.x;
       }
+      cb[(q * (kD + 1) + kD) * 32 + lane] = __int_as_float(kk[q]);
+    }
+    __syncthreads();
+    // part q finishes the queries q of the lanes
+    const int i = i0 + 32 * part;
+    if (part < kQ && i < n) {
+      int cnt = 0;
       float f[kD];
-      const float ik = kk > 0 ? 1.f / (float)kk : 0.f;
+#pragma unroll
+      for (int b = 0; b < kD; ++b) f[b] = 0.f;
+      for (int pp = 0; pp < kFpParts; ++pp) {
+        const float *ob = reinterpret_cast<const float *>(fp_smem + (size_t)pp * kFpWarpV) +
+                          part * (kD + 1) * 32;
+#pragma unroll
+        for (int b = 0; b < kD; ++b) f[b] += ob[b * 32 + lane];
+        cnt += __float_as_int(ob[kD * 32 + lane]);
+      }
+      const bool ok = valid(part);
+      const float ik = cnt > 0 ? 1.f / (float)cnt : 0.f;
       const float *srow_i = S + (size_t)i * kDS;
 #pragma unroll
-      for (int b = 0; b < kD; ++b) f[b] = valid ? srow_i[b] + acc[b] * ik : 0.f;
+      for (int b = 0; b < kD; ++b) f[b] = ok ? srow_i[b] + f[b] * ik : 0.f;
       // sub-histograms: bins 0..10, 11..21, 22..32
       float gs[3];
 #pragma unroll
@@ -495,7 +598,28 @@ __global__ void __launch_bounds__(kFpThreads, 3) k_fpfh(const float4 *__restrict
 #pragma unroll
       for (int b = kD; b < kDS; ++b) row[b] = 0.f;
     }
-    window_sync(wslot);  // the buffers are reused by the next window
+    __syncthreads();  // the buffers are reused by the next window
+  }
+}
+
+__global__ void __launch_bounds__(kFpThreads, 5) k_fpfh(const float4 *__restrict__ X, const float4 *__restrict__ N,
+                                                        const float *__restrict__ S, const GridParams *gfp,
+                                                        const int *__restrict__ start, float r2,
+                                                        const int2 *__restrict__ win, int *__restrict__ ctl,
+                                                        float *__restrict__ F) {
+  extern __shared__ float4 fp_smem[];
+  __shared__ int s_w;
+  const GridParams g = *gfp;
+  const int nwin = ctl[0];
+  while (true) {
+    if (threadIdx.x == 0) s_w = atomicAdd(ctl + 1, 1);
+    __syncthreads();
+    if (s_w >= nwin) break;
+    const int2 w = win[s_w];
+    if (w.y > 32)
+      fpfh_window<2>(X, N, S, g, start, r2, F, w.x, w.y, fp_smem);
+    else
+      fpfh_window<1>(X, N, S, g, start, r2, F, w.x, w.y, fp_smem);
   }
 }
 
@@ -525,12 +649,12 @@ cudaError_t launch_spfh(const float4 *X, const float4 *N, int n, const GridParam
 }
 
 cudaError_t launch_fpfh(const float4 *X, const float4 *N, const float *spfh, int n, const GridParams *gf,
-                        const int *start_f, float r, float *fpfh, cudaStream_t s) {
-  const int64_t nb = lsr_div_up(lsr_div_up(n > 0 ? n : 1, 32), kFpWin);
-  // dynamic shared memory above the default 48 KB
-  LSR_CUDA_TRY(cudaFuncSetAttribute(k_fpfh, cudaFuncAttributeMaxDynamicSharedMemorySize, kFpSmem));
-  LSR_LAUNCH(k_fpfh<<<(int)(nb < kSms * 64 ? nb : kSms * 64), kFpThreads, kFpSmem, s>>>(X, N, spfh, n, gf, start_f,
-                                                                                        r * r, fpfh));
+                        const int *start_f, float r, int2 *win, int *ctl, float *fpfh, cudaStream_t s) {
+  LSR_CUDA_TRY(cudaMemsetAsync(ctl, 0, sizeof(int) * kWinCtl, s));
+  const int64_t nb = lsr_div_up(n > 0 ? n : 1, 64);
+  LSR_LAUNCH(k_windows<<<(int)(nb < kSms * 4 ? nb : kSms * 4), 256, 0, s>>>(gf, start_f, win, ctl));
+  LSR_LAUNCH(k_fpfh<<<n < kSms * 5 ? n : kSms * 5, kFpThreads, kFpSmem, s>>>(X, N, spfh, gf, start_f, r * r, win, ctl,
+                                                                             fpfh));
   return cudaGetLastError();
 }
 

@@ -575,8 +575,10 @@ cudaError_t launch_normals(const float4 *X, int n, const GridParams *gn, const i
 // buffer may serve, as SPFH comes first).
 cudaError_t launch_spfh(const float4 *X, const float4 *N, int n, const GridParams *gf, const int *start_f, float r,
                         float *spfh, int *k, void *scratch, cudaStream_t s);
+// win (n) and ctl (kWinCtl ints): scratch for the list of windows.
+constexpr int kWinCtl = 2;
 cudaError_t launch_fpfh(const float4 *X, const float4 *N, const float *spfh, int n, const GridParams *gf,
-                        const int *start_f, float r, float *fpfh, cudaStream_t s);
+                        const int *start_f, float r, int2 *win, int *ctl, float *fpfh, cudaStream_t s);
 
 // ----------------------------------------------------------------- descriptor order (lsr_order.cu)
 constexpr int kAx = 8;           // projection axes
