@@ -1848,29 +1848,21 @@ int lsr_stage_consensus(lsr_ctx *c, const float *P, int64_t nP, const float *Q, 
       nh > ((int64_t)1 << 26) || !(eps > 0.f && eps <= 10.f))
     return set_err(c, LSR_E_ARG, "bad argument");
   struct Bufs {
-    float *p, *pose;
-    float4 *XP;
-    CloudLayout Cq;
+    float *pose;
+    CloudLayout Cp, Cq;
     ScratchLayout S;
-    int *cnt, *cnt2;
+    int *cnt;
     unsigned long long *sum;
     double *sd;
-    ClsParams *cls;
-    unsigned *in_bits, *near_bits;
   };
   auto plan = [&](Arena &a, Bufs &b) {
-    b.p = a.take<float>(3 * nP);
-    b.XP = a.take<float4>(nP);
+    plan_cloud(a, (int)nP, true, false, true, b.Cp);
     plan_cloud(a, (int)nQ, true, false, true, b.Cq);
-    plan_scratch(a, (int)nQ, b.Cq.cap_f, b.S);
+    plan_scratch(a, (int)std::max(nP, nQ), std::max(b.Cp.cap_e, b.Cq.cap_e), b.S, 2);
     b.pose = a.take<float>(12 * nh);
     b.cnt = a.take<int>(nh);
-    b.cnt2 = a.take<int>(nh);
     b.sum = a.take<unsigned long long>(nh);
     b.sd = a.take<double>(nh);
-    b.cls = a.take<ClsParams>(1);
-    b.in_bits = a.take<unsigned>(kClsCapWords);
-    b.near_bits = a.take<unsigned>(kClsCapWords);
   };
   Arena m(nullptr);
   Bufs bm;
@@ -1879,34 +1871,27 @@ int lsr_stage_consensus(lsr_ctx *c, const float *P, int64_t nP, const float *Q, 
   Arena a(c->ws);
   Bufs b;
   plan(a, b);
-  float *p = b.p, *pose = b.pose;
-  float4 *XP = b.XP;
+  float *pose = b.pose;
   CloudLayout &Cq = b.Cq;
   int *cnt = b.cnt;
   unsigned long long *sum = b.sum;
   double *sd = b.sd;
   cudaStream_t s = c->stream;
-  TRY_CUDA(c, cudaMemcpyAsync(p, P, sizeof(float) * 3 * nP, cudaMemcpyDefault, s), "copy P");
-  const float *qsrc;
+  const float *psrc, *qsrc;
+  if ((rc = stage_input(c, P, nP, b.Cp.src, &psrc))) return rc;
   if ((rc = stage_input(c, Q, nQ, Cq.src, &qsrc))) return rc;
   TRY_CUDA(c, cudaMemcpyAsync(pose, Rt, sizeof(float) * 12 * nh, cudaMemcpyDefault, s), "copy Rt");
-  LSR_LAUNCH(k_pack<<<nblk(nP), 256, 0, s>>>(p, (int)nP, XP));
-  const GridJob gj = eps_cloud(qsrc, Cq, eps, b.S.g[0]);
-  TRY_CUDA(c, build_grids(&gj, 1, s), "grid Q");
+  // P is read in the order of a grid of its own, built beside Q's: the points
+  // of a warp then walk the same cells (counts and fixed-point sums do not
+  // depend on the order)
+  const GridJob gj[2] = {eps_cloud(qsrc, Cq, eps, b.S.g[0]), eps_cloud(psrc, b.Cp, eps, b.S.g[1])};
+  TRY_CUDA(c, build_grids(gj, 2, s), "grids");
   TRY_CUDA(c, cudaMemsetAsync(cnt, 0, sizeof(int) * nh, s), "memset");
-  TRY_CUDA(c, cudaMemsetAsync(b.cnt2, 0, sizeof(int) * nh, s), "memset");
   TRY_CUDA(c, cudaMemsetAsync(sum, 0, sizeof(unsigned long long) * nh, s), "memset");
-  // counts as the registration pipeline takes them (voxel classification),
-  // sums from the exact kernel
-  TRY_CUDA(c, launch_cls_build(Cq.box, eps, Cq.X, (int)nQ, b.cls, b.in_bits, b.near_bits, s), "classify");
   TRY_CUDA(c,
-           launch_consensus_count(XP, (int)nP, b.cls, b.in_bits, b.near_bits, Cq.ge, Cq.start_e, Cq.Xe, pose, nullptr,
-                                  nullptr, (int)nh, eps, cnt, s),
-           "consensus");
-  TRY_CUDA(c,
-           launch_consensus(XP, (int)nP, Cq.ge, Cq.start_e, Cq.Xe, pose, nullptr, nullptr, (int)nh, eps, b.cnt2, sum, s,
+           launch_consensus(b.Cp.Xe, (int)nP, Cq.ge, Cq.start_e, Cq.Xe, pose, nullptr, nullptr, (int)nh, eps, cnt, sum, s,
                             c->cons_lanes),
-           "consensus sums");
+           "consensus");
   LSR_LAUNCH(k_sum_to_double<<<nblk(nh), 256, 0, s>>>(sum, (int)nh, sd));
   if ((rc = copy_out(c, count, cnt, sizeof(int) * nh))) return rc;
   if ((rc = copy_out(c, sumd2, sd, sizeof(double) * nh))) return rc;

@@ -352,14 +352,17 @@ constexpr int kConsChunk = 2048;
 
 
 // Minimum squared distance below eps2 by a group of G lanes (no index needed).
+// The query's own row of cells first; a row of cells, and the x-neighbour
+// cells of a row, that the best so far does not reach is left out (as in
+// group_nn, with its margins).
 template <int G>
 __device__ __forceinline__ float group_min_d2(const GridParams &g, const int *__restrict__ start,
                                               const float4 *__restrict__ Xe, float x, float y, float z, float eps2) {
-  int sub = threadIdx.x & (G - 1);
+  const int sub = threadIdx.x & (G - 1);
   float best = eps2;
   int next = sub, base = 0;
-  grid_ranges(g, start, x, y, z, [&](int b, int e) {
-    int len = e - b;
+  auto scan = [&](int b, int e) {
+    const int len = e - b;
     // four independent loads in flight per lane, then the remainder
     for (; next + 3 * G < base + len; next += 4 * G) {
       int t = b + next - base;
@@ -369,7 +372,58 @@ __device__ __forceinline__ float group_min_d2(const GridParams &g, const int *__
     }
     for (; next < base + len; next += G) best = fminf(best, dist2(Xe[b + next - base], x, y, z));
     base += len;
-  });
+  };
+  if ((g.wx != g.nx) | (g.wy != g.ny) | (g.wz != g.nz)) {
+    grid_ranges(g, start, x, y, z, scan);
+  } else {
+    const float fx = (x - g.ox) * g.inv_cell, fy = (y - g.oy) * g.inv_cell, fz = (z - g.oz) * g.inv_cell;
+    bool go = fx >= -1.f && fx < (float)g.nx + 1.f && fy >= -1.f && fy < (float)g.ny + 1.f && fz >= -1.f &&
+              fz < (float)g.nz + 1.f;
+    const int cx = go ? __float2int_rd(fx) : 0, cy = go ? __float2int_rd(fy) : 0, cz = go ? __float2int_rd(fz) : 0;
+    const int x0 = cx - 1 < 0 ? 0 : cx - 1, x1 = cx + 1 > g.nx - 1 ? g.nx - 1 : cx + 1;
+    go = go && x0 <= x1;
+    if (go && g.nbmask && cx >= 0 && cx < g.nx && cy >= 0 && cy < g.ny && cz >= 0 && cz < g.nz) {
+      const int slot = (cz * g.wy + cy) * g.wx + cx;
+      go = (__ldg(g.nbmask + (slot >> 5)) >> (slot & 31)) & 1u;
+    }
+    if (go) {
+      const unsigned gmask = ((1u << G) - 1u) << ((threadIdx.x & 31) & ~(G - 1));
+      const float mg = 2e-4f * g.cell;
+      auto gsq = [&](float d) {
+        const float t = fmaxf(d - mg, 0.f);
+        return t * t;
+      };
+      const float gxl = gsq((fx - (float)cx) * g.cell), gxh = gsq(((float)cx + 1.f - fx) * g.cell);
+      const float gyl = gsq((fy - (float)cy) * g.cell), gyh = gsq(((float)cy + 1.f - fy) * g.cell);
+      const float gzl = gsq((fz - (float)cz) * g.cell), gzh = gsq(((float)cz + 1.f - fz) * g.cell);
+      constexpr float kShrink = 1.f - 1e-6f;  // the FP32 rounding of d^2 itself
+      float gb = eps2;
+#pragma unroll 1
+      for (int k = 0; k < 9; ++k) {
+        // rows: own, then the four edge neighbours, then the four corners
+        const int dy = k == 1 ? -1 : k == 2 ? 1 : (k >= 5 ? ((k & 1) ? -1 : 1) : 0);
+        const int dz = k == 3 ? -1 : k == 4 ? 1 : (k >= 5 ? (k < 7 ? -1 : 1) : 0);
+        const int iy = cy + dy, iz = cz + dz;
+        if (iy < 0 || iy >= g.ny || iz < 0 || iz >= g.nz) continue;
+        const float r2 = (dy < 0 ? gyl : dy > 0 ? gyh : 0.f) + (dz < 0 ? gzl : dz > 0 ? gzh : 0.f);
+        if (r2 * kShrink > gb) continue;
+        int a = x0, e = x1;
+        if (a < cx && (r2 + gxl) * kShrink > gb) a = cx;
+        if (e > cx && (r2 + gxh) * kShrink > gb) e = cx;
+        if (a > e) continue;
+        const int row = (iz * g.wy + iy) * g.wx;
+        if (!LSR_IN_BOUNDS(row + e + 1, g.ncells + 1, kSiteGridRow) || !LSR_IN_BOUNDS(row + a, g.ncells + 1, kSiteGridRow))
+          continue;
+        const int b = start[row + a], end = start[row + e + 1];
+        if (end > b && (!LSR_IN_BOUNDS(end - 1, g.npts, kSiteGridPoint) || !LSR_IN_BOUNDS(b, g.npts, kSiteGridPoint)))
+          continue;
+        scan(b, end);
+        gb = best;
+#pragma unroll
+        for (int off = G / 2; off > 0; off >>= 1) gb = fminf(gb, __shfl_xor_sync(gmask, gb, off));
+      }
+    }
+  }
 #pragma unroll
   for (int off = G / 2; off > 0; off >>= 1) best = fminf(best, __shfl_xor_sync(0xffffffffu, best, off));
   return best;
