@@ -312,7 +312,7 @@ struct PairLayout {
   int *count = nullptr;
   unsigned long long *sum = nullptr;
   double *ref_part = nullptr;
-  int *seeds = nullptr;      // refinement: each point's neighbour of its last search,
+  float4 *near = nullptr;    // refinement: each point's neighbour of its last search,
   float4 *certs = nullptr;   // where that was made and how far off every other point is
   float *fpose = nullptr;
   int *fcount = nullptr;
@@ -360,7 +360,7 @@ void plan_pair(Arena &a, int nP, int nQ, bool stP, bool stQ, int64_t H, int leve
   L.count = a.take<int>(L.surv_cap);
   L.sum = a.take<unsigned long long>(L.surv_cap);
   L.ref_part = a.take<double>((size_t)refine_partial_doubles());
-  L.seeds = a.take<int>(nP);
+  L.near = a.take<float4>(nP);
   L.certs = a.take<float4>(nP);
   L.fpose = a.take<float>(12);
   L.fcount = a.take<int>(1);
@@ -672,7 +672,7 @@ cudaError_t build_pair(const float *P, const float *Q, const CloudLayout &Pc, co
 // xyz on the device; (ge, start_e, Xe): Q's eps grid for the finest level.
 cudaError_t enqueue_refine(const float4 *XP, const float *P, int nP, const float *Q, const float *boxQ,
                            const GridParams *ge, const int *start_e, const float4 *Xe, const LevelLayout &V, float eps,
-                           float mu_scale, int iters, RansacState *st, double *part, int *seeds, float4 *certs,
+                           float mu_scale, int iters, RansacState *st, double *part, float4 *near, float4 *certs,
                            const ScratchLayout &sc, cudaStream_t s, bool chain) {
   int L = V.levels;
   LSR_CUDA_TRY(refine_reset_tickets(part, s));
@@ -704,9 +704,9 @@ cudaError_t enqueue_refine(const float4 *XP, const float *P, int nP, const float
     const float4 *xs = Xe;
     if (l + 1 < L) g = V.g[l], st0 = V.start[l], xs = V.Xs[l];
     LSR_CUDA_TRY(launch_refine_level_begin(st, s));
-    LSR_CUDA_TRY(cudaMemsetAsync(seeds, 0xff, sizeof(int) * (size_t)np, s));  // no search yet at this level
+    LSR_CUDA_TRY(cudaMemsetAsync(near, 0xff, sizeof(float4) * (size_t)np, s));  // no search yet at this level
     for (int it = 0; it < iters; ++it)
-      LSR_CUDA_TRY(launch_refine_step(xp, np, g, st0, xs, e, mu, iters, st, part, seeds, certs, chain && it > 0, s));
+      LSR_CUDA_TRY(launch_refine_step(xp, np, g, st0, xs, e, mu, iters, st, part, near, certs, chain && it > 0, s));
   }
   return cudaSuccess;
 }
@@ -870,7 +870,7 @@ int enqueue_pair(lsr_ctx *c, const PairLayout &L, const float *P, const float *Q
   float eps = p.eps_inlier;
   TRY_CUDA(c,
            enqueue_refine(Pc.X, P, nP, Q, Qc.box, Qc.ge, Qc.start_e, Qc.Xe, L.lv, eps, p.mu_scale, p.refine_iters,
-                          L.st, L.ref_part, L.seeds, L.certs, L.sc, s, chain),
+                          L.st, L.ref_part, L.near, L.certs, L.sc, s, chain),
            "refine");
   TRY_CUDA(c, launch_final_pose(L.st, L.fpose, s), "final pose");
   TRY_CUDA(c, cudaMemsetAsync(L.fcount, 0, sizeof(int), s), "memset fcount");
@@ -1909,11 +1909,11 @@ int lsr_stage_refine(lsr_ctx *c, const float *P, int64_t nP, const float *Q, int
     return set_err(c, LSR_E_ARG, "bad argument");
   float *boxP = nullptr;
   double *boxP_part = nullptr;
-  int *seeds = nullptr, *ticketP = nullptr;
-  float4 *certs = nullptr;
+  float4 *near = nullptr, *certs = nullptr;
+  int *ticketP = nullptr;
   auto plan = [&](Arena &a, float *&p, float4 *&XP, CloudLayout &Cq, LevelLayout &V, ScratchLayout &S, double *&part,
                   double *&Td, RansacState *&st) {
-    seeds = a.take<int>(nP);
+    near = a.take<float4>(nP);
     certs = a.take<float4>(nP);
     p = a.take<float>(3 * nP);
     XP = a.take<float4>(nP);
@@ -1960,7 +1960,7 @@ int lsr_stage_refine(lsr_ctx *c, const float *P, int64_t nP, const float *Q, int
   TRY_CUDA(c, launch_refine_init(st, boxP, Td, s), "init");
   TRY_CUDA(c,
            enqueue_refine(XP, p, (int)nP, qsrc, Cq.box, Cq.ge, Cq.start_e, Cq.Xe, V, eps, mu_scale, iters, st,
-                          part, seeds, certs, S, s, true),
+                          part, near, certs, S, s, true),
            "refine");
   RansacState h;
   TRY_CUDA(c, cudaMemcpyAsync(&h, st, sizeof(h), cudaMemcpyDeviceToHost, s), "D2H");

@@ -272,37 +272,16 @@ __device__ __forceinline__ void grid_ranges(const GridParams &g, const int *__re
 // is below eps2, so cells beyond it are skipped; the result is the walk's
 // result without a seed (the nearest point wins either way, ties to the
 // smaller carried index).
-//
-// kApart: *apart also receives a distance that no other point is closer than
-// (no point at all, if bt = -1): the second smallest distance seen, the bound
-// up to which cells were visited (the best so far plus guard) and the distance
-// to the border of the 3 x 3 x 3 block, whichever is least, less a margin of
-// 4e-6 of it (above the FP32 rounding of the distances).
 __device__ __forceinline__ float nn_d2(float4 q, float x, float y, float z) {
   float dx = q.x - x, dy = q.y - y, dz = q.z - z;
   return dx * dx + dy * dy + dz * dz;
 }
 
-// A distance that no point outside the 3 x 3 x 3 block of cells around the cell
-// coordinates (fx, fy, fz) is closer than: at least a cell beyond the query's
-// own; for a query outside the box (where nothing is visited) the distance to it.
-__device__ __forceinline__ float nn_border(const GridParams &g, float fx, float fy, float fz) {
-  const float ux = fx - floorf(fx), uy = fy - floorf(fy), uz = fz - floorf(fz);
-  const float in = fminf(fminf(fminf(ux, 1.f - ux), fminf(uy, 1.f - uy)), fminf(uz, 1.f - uz));
-  const float out = fmaxf(fmaxf(fmaxf(-fx, fx - (float)g.nx), fmaxf(-fy, fy - (float)g.ny)), fmaxf(-fz, fz - (float)g.nz));
-  return fmaxf(1.f + in, out) * g.cell - 4e-4f * g.cell;
-}
-
-template <int G, bool kApart = false>
+template <int G>
 __device__ __forceinline__ void group_nn(const GridParams &g, const int *__restrict__ start,
                                          const float4 *__restrict__ Xe, float x, float y, float z, float eps2,
-                                         float &best, int &bt, int &bidx, int seed = -1, float guard = 0.f,
-                                         float *apart = nullptr) {
+                                         float &best, int &bt, int &bidx, int seed = -1) {
   int sub = threadIdx.x & (G - 1);
-  float m1 = 3e38f, m2 = 3e38f, reach2 = 3e38f, border = 0.f;  // kApart: the two smallest d^2 of the walk
-  auto seen2 = [&](float d2) {
-    if (kApart) m2 = fminf(m2, fmaxf(m1, d2)), m1 = fminf(m1, d2);
-  };
   best = eps2;
   bt = -1;
   bidx = 0x7fffffff;
@@ -329,7 +308,6 @@ __device__ __forceinline__ void group_nn(const GridParams &g, const int *__restr
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
         float d2 = nn_d2(q[k], x, y, z);
-        seen2(d2);
         int qi = __float_as_int(q[k].w);
         if (d2 < best || (d2 == best && qi < bidx)) best = d2, bt = t + k * G, bidx = qi;
       }
@@ -338,18 +316,16 @@ __device__ __forceinline__ void group_nn(const GridParams &g, const int *__restr
       int t = b + next - base;
       float4 q = Xe[t];
       float d2 = nn_d2(q, x, y, z);
-      seen2(d2);
       int qi = __float_as_int(q.w);
       if (d2 < best || (d2 == best && qi < bidx)) best = d2, bt = t, bidx = qi;
     }
     base += len;
   };
   const bool wrapped = (g.wx != g.nx) | (g.wy != g.ny) | (g.wz != g.nz);
-  const float fx = (x - g.ox) * g.inv_cell, fy = (y - g.oy) * g.inv_cell, fz = (z - g.oz) * g.inv_cell;
-  if (kApart) border = nn_border(g, fx, fy, fz);
   if (wrapped) {
     grid_ranges(g, start, x, y, z, scan);
   } else {
+    const float fx = (x - g.ox) * g.inv_cell, fy = (y - g.oy) * g.inv_cell, fz = (z - g.oz) * g.inv_cell;
     bool go = fx >= -1.f && fx < (float)g.nx + 1.f && fy >= -1.f && fy < (float)g.ny + 1.f && fz >= -1.f &&
               fz < (float)g.nz + 1.f;
     const int cx = go ? __float2int_rd(fx) : 0, cy = go ? __float2int_rd(fy) : 0, cz = go ? __float2int_rd(fz) : 0;
@@ -371,13 +347,7 @@ __device__ __forceinline__ void group_nn(const GridParams &g, const int *__restr
       const float gyl = gsq((fy - (float)cy) * g.cell), gyh = gsq(((float)cy + 1.f - fy) * g.cell);
       const float gzl = gsq((fz - (float)cz) * g.cell), gzh = gsq(((float)cz + 1.f - fz) * g.cell);
       constexpr float kShrink = 1.f - 1e-6f;  // the FP32 rounding of d^2 itself
-      // the squared distance up to which cells are visited
-      auto bound = [&](float b) {
-        if (!kApart) return b;
-        const float r = sqrtf(b) + guard;
-        return r * r;
-      };
-      float gb = bound(best);  // eps2, or the seed's distance (the same on every lane of the group)
+      float gb = best;  // eps2, or the seed's distance (the same on every lane of the group)
 #pragma unroll 1
       for (int k = 0; k < 9; ++k) {
         // rows: own, then the four edge neighbours, then the four corners
@@ -398,9 +368,8 @@ __device__ __forceinline__ void group_nn(const GridParams &g, const int *__restr
         float m = best;
 #pragma unroll
         for (int off = G / 2; off > 0; off >>= 1) m = fminf(m, __shfl_xor_sync(gmask, m, off));
-        gb = bound(m);
+        gb = m;
       }
-      reach2 = gb * kShrink;
     }
   }
 #pragma unroll
@@ -409,15 +378,6 @@ __device__ __forceinline__ void group_nn(const GridParams &g, const int *__restr
     int ot = __shfl_xor_sync(0xffffffffu, bt, off);
     int oi = __shfl_xor_sync(0xffffffffu, bidx, off);
     if (ob < best || (ob == best && oi < bidx)) best = ob, bt = ot, bidx = oi;
-    if (kApart) {
-      const float o1 = __shfl_xor_sync(0xffffffffu, m1, off), o2 = __shfl_xor_sync(0xffffffffu, m2, off);
-      m2 = fminf(fmaxf(m1, o1), fminf(m2, o2)), m1 = fminf(m1, o1);
-    }
-  }
-  if (kApart) {
-    // the walk meets the best itself once more when it started as the seed
-    const float other = bt >= 0 && m1 <= best ? m2 : m1;
-    *apart = fminf(sqrtf(fminf(other, reach2)), border) * (1.f - 4e-6f);
   }
 }
 
@@ -686,7 +646,6 @@ struct RansacState {
   double T_hyp[16];
   float pose_f[12];    // FP32 copy of the pose used by consensus-type kernels
   double center[3];    // linearisation centre of the refinement (centroid of Q)
-  double last_step;
 };
 
 int hyp_blocks(int64_t H);
@@ -794,13 +753,13 @@ constexpr int kMaxLevels = 8;
 // Subsampling stride of graduated refinement level l of L for a cloud of n points.
 int gnc_stride(int64_t n, int level, int levels);
 cudaError_t launch_refine_level_begin(RansacState *st, cudaStream_t s);
-// One IRLS step on the points of P against the given grid of Q. seeds (nP ints,
-// set to -1 at the start of a level) and certs (nP): what the last search of
+// One IRLS step on the points of P against the given grid of Q. near (nP, all
+// bits set at the start of a level) and certs (nP): what the last search of
 // each point found and while it stands, read and rewritten.
 // chained: launched as a programmatic dependent of the previous step, which
 // must be the kernel directly before it in s.
 cudaError_t launch_refine_step(const float4 *XP, int nP, const GridParams *ge, const int *start_e, const float4 *Xe,
-                               float eps_r, float mu, int max_iters, RansacState *st, double *partials, int *seeds,
+                               float eps_r, float mu, int max_iters, RansacState *st, double *partials, float4 *near,
                                float4 *certs, bool chained, cudaStream_t s);
 // out[m] = (Q[m * stride], m) for m < ceil(n / stride); Q caller-order xyz.
 cudaError_t launch_subsample(const float *xyz, int n, int stride, float4 *out, cudaStream_t s);

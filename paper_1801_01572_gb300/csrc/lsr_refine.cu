@@ -21,8 +21,10 @@ constexpr int kRefThreads = 256;
 constexpr int kRefG = 4;   // lanes per nearest-neighbour query in refinement (4 measured fastest of 4/8/16)
 constexpr int kRefBlocksPerSm = 4;  // resident refinement blocks per SM (64 registers a thread; 3 measured slower)
 constexpr int kRefMaxBlocks = kSms * kRefBlocksPerSm;  // refine_blocks' cap
-constexpr int kRefGroup = 16;                           // blocks per first-level closing sum
+constexpr int kRefGroup = 16;                           // blocks summed together when a step closes
 constexpr int kRefMaxGroups = (kRefMaxBlocks + kRefGroup - 1) / kRefGroup;
+constexpr int kRefAtOnce = 8;                           // groups summed by the last block alone
+static_assert(kRefAtOnce <= kRefThreads / 17, "a segment per group");
 // 21 (upper triangle of A) + 6 (b) + count + sum w + sum w x (3)
 constexpr int kNAcc = kRefAcc;
 static_assert(kNAcc == 32, "refinement partial layout");
@@ -83,149 +85,148 @@ __device__ __forceinline__ double recip_pos(double x) {
 // With J = [-[xc]_x | I], A = [[M, [s]_x], [[s]_x^T, sw I]] where M is the
 // rotation block, s = sum w xc and sw = sum w. The translation block is a
 // multiple of I, so it is eliminated in closed form (Schur complement):
-//   M' = M - [s]_x [s]_x^T / sw = M - (|s|^2 I - s s^T) / sw,
+//   M' = M - (|s|^2 I - s s^T) / sw,
 //   M' d_w = -b_w + (s x b_v) / sw,   d_v = -(b_v - s x d_w) / sw,
 // and the 3x3 system is solved by its adjugate (one reciprocal). A is
-// positive definite iff sw > 0 and M' is (its leading minors m00, m00 m11 -
-// m01^2 and det M' positive). This is the same solution as a 6x6 Cholesky in
-// exact arithmetic with a far shorter chain of dependent FP64 operations,
-// whose latency is long on this part.
+// positive definite iff sw > 0 and M' is (its leading minors positive).
 //
-// Run by warps 0 and 1 of the closing block (every thread of the block
-// reaches its barrier): the solve, the Exp coefficients and the twelve pose
-// entries (lanes 0..11) on warp 0; the next centre on warp 1 meanwhile, and
-// the step length and the state on warp 1 after the pose. Each value is
-// computed by one lane in a fixed order, so the result is deterministic.
+// Bound by the latency of its chain of FP64 operations (a warp instruction
+// every 16 clocks at best, one lane or all): both sides of the 3x3 system are
+// multiplied by sw (times a power of two that brings it to [1, 2), so that the
+// determinant stays in range) instead of waiting for 1 / sw, the terms of each
+// stage are computed a lane each and exchanged by shuffles, and the series of
+// Exp are Horner chains: about 30 dependent operations; with one lane
+// computing all of it in 47 the solve took 4.9 us (now 2.9). Run by one warp; every value is
+// computed in a fixed order. S[kNSum] is 0.
+__device__ __forceinline__ double lane_of(double v, int src) { return __shfl_sync(0xffffffffu, v, src); }
+__device__ __forceinline__ int field(unsigned long long packed, int lane) { return (int)(packed >> (5 * lane)) & 31; }
+// Nine five-bit fields.
+__host__ __device__ constexpr unsigned long long fields(int a, int b, int c, int d, int e, int f, int g = 0, int h = 0,
+                                                        int i = 0) {
+  const int v[9] = {a, b, c, d, e, f, g, h, i};
+  unsigned long long p = 0;
+  for (int k = 0; k < 9; ++k) p |= (unsigned long long)v[k] << (5 * k);
+  return p;
+}
+
 __device__ void refine_solve(const double *S, const StepState &ss, RansacState *st, int max_iters, double tol) {
-  __shared__ double sd[6], scoef[2], scn[3];
-  __shared__ int spd;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const double *xx = S + 5, *b = S + 11;
-  const double sw = S[1], sx0 = S[2], sx1 = S[3], sx2 = S[4];
-  bool pd = S[0] >= 3.0 && sw > 0.0;
-  if (warp == 1 && lane == 0 && sw > 0.0) {
-    const double iw = recip_pos(sw);
-    const double *c = ss.center;
-    scn[0] = c[0] + sx0 * iw, scn[1] = c[1] + sx1 * iw, scn[2] = c[2] + sx2 * iw;
+  const int lane = threadIdx.x & 31, j = lane < 9 ? lane : 0;
+  const double sw = S[1];
+  if (!(S[0] >= 3.0 && sw > 0.0)) {
+    if (lane == 0) st->active = 0;
+    return;
   }
-  if (warp == 0) {
-    if (lane == 0 && pd) {
-      const double iw = recip_pos(sw);
-      const double ss2 = sx0 * sx0 + sx1 * sx1 + sx2 * sx2;
-      // M' (symmetric; M from the weighted second moments of xc)
-      const double m00 = xx[3] + xx[5] - (ss2 - sx0 * sx0) * iw;
-      const double m11 = xx[0] + xx[5] - (ss2 - sx1 * sx1) * iw;
-      const double m22 = xx[0] + xx[3] - (ss2 - sx2 * sx2) * iw;
-      const double m01 = -xx[1] + sx0 * sx1 * iw;
-      const double m02 = -xx[2] + sx0 * sx2 * iw;
-      const double m12 = -xx[4] + sx1 * sx2 * iw;
-      // right-hand side -b_w + (s x b_v) / sw
-      const double r0 = -b[0] + (sx1 * b[5] - sx2 * b[4]) * iw;
-      const double r1 = -b[1] + (sx2 * b[3] - sx0 * b[5]) * iw;
-      const double r2 = -b[2] + (sx0 * b[4] - sx1 * b[3]) * iw;
-      // adjugate (cofactors) and determinant
-      const double c00 = m11 * m22 - m12 * m12, c01 = m02 * m12 - m01 * m22, c02 = m01 * m12 - m02 * m11;
-      const double c11 = m00 * m22 - m02 * m02, c12 = m01 * m02 - m00 * m12, c22 = m00 * m11 - m01 * m01;
-      const double det = m00 * c00 + m01 * c01 + m02 * c02;
-      pd = m00 > 0.0 && c22 > 0.0 && det > 0.0;
-      if (pd) {
-        const double idet = recip_pos(det);
-        const double w0 = (c00 * r0 + c01 * r1 + c02 * r2) * idet;
-        const double w1 = (c01 * r0 + c11 * r1 + c12 * r2) * idet;
-        const double w2 = (c02 * r0 + c12 * r1 + c22 * r2) * idet;
-        sd[0] = w0, sd[1] = w1, sd[2] = w2;
-        // d_v = -(b_v - s x d_w) / sw
-        sd[3] = -(b[3] - (sx1 * w2 - sx2 * w1)) * iw;
-        sd[4] = -(b[4] - (sx2 * w0 - sx0 * w2)) * iw;
-        sd[5] = -(b[5] - (sx0 * w1 - sx1 * w0)) * iw;
-      }
-    }
-    pd = __shfl_sync(0xffffffffu, pd, 0);
-    __syncwarp();
-    if (pd && lane == 0) {
-      // Exp of the rotation part: the series of sin(t)/t and (1 - cos t)/t^2 to
-      // the t^8 term below t = 0.01 (the next term is below 1e-21; the
-      // coefficients' reciprocals are FP64 constants), else sin/cos
-      const double th2 = sd[0] * sd[0] + sd[1] * sd[1] + sd[2] * sd[2];
-      if (th2 < 1e-4) {
-        scoef[0] = 1.0 - th2 * (1.0 / 6.0) * (1.0 - th2 * (1.0 / 20.0) * (1.0 - th2 * (1.0 / 42.0) * (1.0 - th2 * (1.0 / 72.0))));
-        scoef[1] = 0.5 * (1.0 - th2 * (1.0 / 12.0) * (1.0 - th2 * (1.0 / 30.0) * (1.0 - th2 * (1.0 / 56.0) * (1.0 - th2 * (1.0 / 90.0)))));
-      } else {
-        const double th = sqrt(th2);
-        scoef[0] = sin(th) / th;
-        scoef[1] = (1.0 - cos(th)) / th2;
-      }
-    }
-    if (lane == 0) spd = pd;
-    __syncwarp();
+  // lanes 0..5: M' (00 01 02 11 12 22), 6..8: the right-hand side, times sw f:
+  // sw f (base) + f (S S + S S)
+  constexpr int Z = kNSum;  // S[Z] = 0
+  constexpr unsigned long long kBase = fields(8, 6, 7, 5, 9, 5, 11, 12, 13), kMore = fields(10, Z, Z, 10, Z, 8, Z, Z, Z);
+  constexpr unsigned long long kP = fields(3, 2, 2, 2, 3, 2, 3, 4, 2), kQ = fields(3, 3, 4, 2, 4, 2, 16, 14, 15);
+  constexpr unsigned long long kU = fields(4, Z, Z, 4, Z, 3, 4, 2, 3), kV = fields(4, Z, Z, 4, Z, 3, 15, 16, 14);
+  const bool diag = j == 0 || j == 3 || j == 5;
+  // f = 2^-e for sw in [2^e, 2^(e + 1))
+  const double f = __longlong_as_double((long long)(2046 - ((__double_as_longlong(sw) >> 52) & 2047)) << 52);
+  const double base = S[field(kBase, j)] + S[field(kMore, j)];
+  const double P = S[field(kP, j)] * (diag ? -f : f), U = S[field(kU, j)] * -f;
+  const double e = fma(diag ? base : -base, sw * f, fma(P, S[field(kQ, j)], U * S[field(kV, j)]));
+  const double iw = recip_pos(sw);
+  // lanes 0..5: cofactors (00 01 02 11 12 22)
+  constexpr unsigned long long kA = fields(3, 2, 1, 0, 1, 0), kB = fields(5, 4, 4, 5, 2, 3);
+  constexpr unsigned long long kC = fields(4, 1, 2, 2, 0, 1), kD4 = fields(4, 5, 3, 2, 4, 1);
+  const double cof = fma(lane_of(e, field(kA, j)), lane_of(e, field(kB, j)), -(lane_of(e, field(kC, j)) * lane_of(e, field(kD4, j))));
+  // lanes 0..2: rows of the adjugate times the right-hand side; 3: the determinant
+  constexpr unsigned long long kR0 = fields(0, 1, 2, 0, 0, 0), kR1 = fields(1, 3, 4, 1, 0, 0), kR2 = fields(2, 4, 5, 2, 0, 0);
+  const int v = j == 3 ? 0 : 6;  // what the row meets: M' or the right-hand side
+  const double num = fma(lane_of(cof, field(kR2, j)), lane_of(e, v + 2),
+                         fma(lane_of(cof, field(kR1, j)), lane_of(e, v + 1), lane_of(cof, field(kR0, j)) * lane_of(e, v)));
+  const double det = lane_of(num, 3);
+  if (!(lane_of(e, 0) > 0.0 && lane_of(cof, 5) > 0.0 && det > 0.0)) {
+    if (lane == 0) st->active = 0;
+    return;
   }
-  __syncthreads();  // spd, sd, scoef (warp 0) and scn (warp 1)
-  pd = spd != 0;
-  if (warp == 1 && lane == 0) {
-    if (!pd) {
-      st->active = 0;
-      return;
-    }
-    if (sw > 0.0)
-      for (int r = 0; r < 3; ++r) st->center[r] = scn[r];
-    double nd2 = 0.0;
-    for (int i = 0; i < 6; ++i) nd2 += sd[i] * sd[i];
-    st->last_step = sqrt(nd2);
+  const double wl = num * recip_pos(det);
+  const double w0 = lane_of(wl, 0), w1 = lane_of(wl, 1), w2 = lane_of(wl, 2);
+  // Exp of the rotation part: the series of sin(t)/t and (1 - cos t)/t^2 to
+  // the t^8 term below t = 0.01 (the next term is below 1e-21), else sin/cos
+  const double t2 = fma(w2, w2, fma(w1, w1, w0 * w0));
+  double ea, eb;
+  if (t2 < 1e-4) {
+    ea = fma(t2, fma(t2, fma(t2, fma(t2, 1.0 / 362880.0, -1.0 / 5040.0), 1.0 / 120.0), -1.0 / 6.0), 1.0);
+    eb = fma(t2, fma(t2, fma(t2, fma(t2, 1.0 / 3628800.0, -1.0 / 40320.0), 1.0 / 720.0), -1.0 / 24.0), 0.5);
+  } else {
+    const double th = sqrt(t2);
+    ea = sin(th) / th;
+    eb = (1.0 - cos(th)) / t2;
+  }
+  // lane 4 r + q < 12: pose entry (r, q); p, o: the two axes after r
+  const int r = lane < 12 ? lane >> 2 : 0, q = lane & 3, p = r == 2 ? 0 : r + 1, o = p == 2 ? 0 : p + 1;
+  const double wr = r == 0 ? w0 : r == 1 ? w1 : w2, wp = r == 0 ? w1 : r == 1 ? w2 : w0, wo = r == 0 ? w2 : r == 1 ? w0 : w1;
+  // row r of Rd = I + a [w]_x + b [w]_x^2, and of d_v
+  const double Rr = fma(-eb, fma(wp, wp, wo * wo), 1.0), Rp = fma(eb, wr * wp, -(ea * wo)), Ro = fma(eb, wr * wo, ea * wp);
+  const double dv = -(S[14 + r] - (S[2 + p] * wo - S[2 + o] * wp)) * iw;
+  const double *c = ss.center;
+  const double vr = c[r] - fma(Ro, c[o], fma(Rp, c[p], Rr * c[r])) + dv;
+  if (lane < 12) st->T[lane] = fma(Ro, ss.T[4 * o + q], fma(Rp, ss.T[4 * p + q], fma(Rr, ss.T[4 * r + q], q == 3 ? vr : 0.0)));
+  if (lane < 12 && q == 0) st->center[r] = fma(S[2 + r], iw, c[r]);
+  const double dv1 = lane_of(dv, 4), dv2 = lane_of(dv, 8);
+  if (lane == 0) {
+    const double nd2 = t2 + fma(dv2, dv2, fma(dv1, dv1, dv * dv));
     st->iters_done = ss.iters_done + 1;
     st->level_iters = ss.level_iters + 1;
     if (nd2 < tol * tol || ss.level_iters + 1 >= max_iters) st->active = 0;
   }
-  if (warp != 0 || !pd) return;
-  if (lane < 12) {
-    // pose entry (r, q): row r of Rd (its three entries), then row r of Rd T
-    const int r = lane >> 2, q = lane & 3;
-    const double *d = sd;
-    const double a = scoef[0], bb = scoef[1];
-    const double K[9] = {0, -d[2], d[1], d[2], 0, -d[0], -d[1], d[0], 0};
-    double Rd[3];
-    for (int cc = 0; cc < 3; ++cc) {
-      const double k2 = K[3 * r] * K[cc] + K[3 * r + 1] * K[3 + cc] + K[3 * r + 2] * K[6 + cc];
-      Rd[cc] = (r == cc ? 1.0 : 0.0) + a * K[3 * r + cc] + bb * k2;
-    }
-    const double *c = ss.center;
-    const double vr = c[r] - (Rd[0] * c[0] + Rd[1] * c[1] + Rd[2] * c[2]) + d[3 + r];
-    st->T[lane] = Rd[0] * ss.T[q] + Rd[1] * ss.T[4 + q] + Rd[2] * ss.T[8 + q] + (q == 3 ? vr : 0.0);
-  }
 }
 
-// group_nn<kRefG, true> for few queries (grids without wrapped storage): half a
-// warp a query, its lanes read the nine rows' ranges at once and then walk the
-// candidates of all of them together, so that a search is three or four
-// dependent loads long instead of two or more for each row.
+// A distance that no point outside the 3 x 3 x 3 block of cells around the cell
+// coordinates (fx, fy, fz) is closer than: at least a cell beyond the query's
+// own; for a query outside the box (where nothing is visited) the distance to it.
+__device__ __forceinline__ float nn_border(const GridParams &g, float fx, float fy, float fz) {
+  const float ux = fx - floorf(fx), uy = fy - floorf(fy), uz = fz - floorf(fz);
+  const float in = fminf(fminf(fminf(ux, 1.f - ux), fminf(uy, 1.f - uy)), fminf(uz, 1.f - uz));
+  const float out = fmaxf(fmaxf(fmaxf(-fx, fx - (float)g.nx), fmaxf(-fy, fy - (float)g.ny)), fmaxf(-fz, fz - (float)g.nz));
+  return fmaxf(1.f + in, out) * g.cell - 4e-4f * g.cell;
+}
+
+// The result of group_nn (at: the position in Xe, -1 if none), and a distance
+// that no other point is closer than (no point at all, if at = -1): the second
+// smallest distance seen, the bound up to which cells were visited (the seed's
+// or eps plus guard) and the distance to the border of the 3 x 3 x 3 block,
+// whichever is least, less a margin of 4e-6 of it (above the FP32 rounding of
+// the distances).
+struct Found {
+  int at;
+  float apart;
+};
+
+// Half a warp a query (grids without wrapped storage). Its lanes read the mask
+// and the nine rows' ranges at once and then walk the candidates of all rows
+// together, four a lane in flight, so a search is two to four dependent loads
+// long (1.5 us) instead of two or more for each row. seed2: the squared distance
+// of the seed (below eps2), which the walk meets again; none: eps2 and -1. Not
+// inlined: the registers that the caller holds for its point were spilled
+// around the loads, and a search took 9 us.
 constexpr int kRefH = 16;
-__device__ __forceinline__ void half_nn(const GridParams &g, const int *__restrict__ start,
-                                        const float4 *__restrict__ Xe, float x, float y, float z, float eps2,
-                                        int seed, float guard, int &bt, float &apart) {
+__device__ __noinline__ Found half_nn(const GridParams &g, const int *__restrict__ start,
+                                      const float4 *__restrict__ Xe, float x, float y, float z, float seed2, int seed,
+                                      float guard) {
   const int sub = threadIdx.x & (kRefH - 1);
-  float best = eps2, m1 = 3e38f, m2 = 3e38f, reach2 = 3e38f;
-  int bidx = 0x7fffffff;
-  bt = -1;
-  if (seed >= 0 && LSR_IN_BOUNDS(seed, g.npts, kSiteGridPoint)) {
-    const float4 q = Xe[seed];
-    const float d2 = nn_d2(q, x, y, z);
-    if (d2 < eps2) best = d2, bt = seed, bidx = __float_as_int(q.w);
-  }
+  float best = seed2, m1 = 3e38f, m2 = 3e38f, reach2 = 3e38f;
+  int bidx = 0x7fffffff, bt = seed;
   const float fx = (x - g.ox) * g.inv_cell, fy = (y - g.oy) * g.inv_cell, fz = (z - g.oz) * g.inv_cell;
   bool go = fx >= -1.f && fx < (float)g.nx + 1.f && fy >= -1.f && fy < (float)g.ny + 1.f && fz >= -1.f &&
             fz < (float)g.nz + 1.f;
   const int cx = go ? __float2int_rd(fx) : 0, cy = go ? __float2int_rd(fy) : 0, cz = go ? __float2int_rd(fz) : 0;
   const int x0 = cx - 1 < 0 ? 0 : cx - 1, x1 = cx + 1 > g.nx - 1 ? g.nx - 1 : cx + 1;
   go = go && x0 <= x1;
+  unsigned mask = 0xffffffffu;
   if (go && g.nbmask && cx >= 0 && cx < g.nx && cy >= 0 && cy < g.ny && cz >= 0 && cz < g.nz) {
     const int slot = (cz * g.wy + cy) * g.wx + cx;
-    go = (__ldg(g.nbmask + (slot >> 5)) >> (slot & 31)) & 1u;
+    mask = __ldg(g.nbmask + (slot >> 5)) >> (slot & 31);
   }
   constexpr float kShrink = 1.f - 1e-6f;  // the FP32 rounding of d^2 itself
+  // lane sub < 9: a row of cells and the part of it within reach
   int b = 0, len = 0;
   if (go) {
     const float r = sqrtf(best) + guard, gb = r * r;
-    reach2 = gb * kShrink;
-    // lane sub < 9: a row of cells and the part of it within reach
     const int dy = sub % 3 - 1, dz = sub / 3 - 1, iy = cy + dy, iz = cz + dz;
     if (sub < 9 && iy >= 0 && iy < g.ny && iz >= 0 && iz < g.nz) {
       const float mg = 2e-4f * g.cell;
@@ -247,8 +248,10 @@ __device__ __forceinline__ void half_nn(const GridParams &g, const int *__restri
           len = 0;
       }
     }
+    if (mask & 1u) reach2 = gb * kShrink;
+    else len = 0;  // nothing in the block
   }
-  // the rows' candidates numbered through: row k's begin at its first
+  // the rows' candidates numbered through: row k's end at its lane's end
   int end = len;
 #pragma unroll
   for (int off = 1; off < kRefH; off <<= 1) {
@@ -257,17 +260,29 @@ __device__ __forceinline__ void half_nn(const GridParams &g, const int *__restri
   }
   const int total = __shfl_sync(0xffffffffu, end, kRefH - 1, kRefH), shift = b - (end - len);
   const int most = max(total, __shfl_xor_sync(0xffffffffu, total, kRefH));
-  for (int t = sub; t - sub < most; t += kRefH) {
-    int row = 0;
+  int ends[8];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) row += t >= __shfl_sync(0xffffffffu, end, k, kRefH);
-    const int at = t + __shfl_sync(0xffffffffu, shift, row, kRefH);
-    if (t < total) {
-      const float4 q = Xe[at];
-      const float d2 = nn_d2(q, x, y, z);
+  for (int k = 0; k < 8; ++k) ends[k] = __shfl_sync(0xffffffffu, end, k, kRefH);
+#pragma unroll 1
+  for (int t0 = sub; t0 - sub < most; t0 += 4 * kRefH) {
+    int at[4];
+    float4 q[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int t = t0 + u * kRefH;
+      int row = 0;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) row += t >= ends[k];
+      at[u] = t + __shfl_sync(0xffffffffu, shift, row, kRefH);
+      q[u] = make_float4(3e18f, 0.f, 0.f, 0.f);  // out of everyone's reach
+      if (t < total) q[u] = Xe[at[u]];
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const float d2 = nn_d2(q[u], x, y, z);
       m2 = fminf(m2, fmaxf(m1, d2)), m1 = fminf(m1, d2);
-      const int qi = __float_as_int(q.w);
-      if (d2 < best || (d2 == best && qi < bidx)) best = d2, bt = at, bidx = qi;
+      const int qi = __float_as_int(q[u].w);
+      if (d2 < best || (d2 == best && qi < bidx)) best = d2, bt = at[u], bidx = qi;
     }
   }
 #pragma unroll
@@ -279,9 +294,18 @@ __device__ __forceinline__ void half_nn(const GridParams &g, const int *__restri
     const float o1 = __shfl_xor_sync(0xffffffffu, m1, off), o2 = __shfl_xor_sync(0xffffffffu, m2, off);
     m2 = fminf(fmaxf(m1, o1), fminf(m2, o2)), m1 = fminf(m1, o1);
   }
-  // (as group_nn)
-  const float other = bt >= 0 && m1 <= best ? m2 : m1;
-  apart = fminf(sqrtf(fminf(other, reach2)), nn_border(g, fx, fy, fz)) * (1.f - 4e-6f);
+  const float other = bt >= 0 && m1 <= best ? m2 : m1;  // (m1 is the best itself)
+  return {bt, fminf(sqrtf(fminf(other, reach2)), nn_border(g, fx, fy, fz)) * (1.f - 4e-6f)};
+}
+
+// Wrapped storage: the general walk, which vouches for nothing.
+__device__ __noinline__ Found group_nn_wrapped(const GridParams &g, const int *__restrict__ start,
+                                               const float4 *__restrict__ Xe, float x, float y, float z, float eps2,
+                                               int seed) {
+  float best;
+  int bt, bidx;
+  group_nn<kRefH>(g, start, Xe, x, y, z, eps2, best, bt, bidx, seed);
+  return {bt, 0.f};
 }
 
 // One IRLS step. Every block accumulates its points; the last block to
@@ -290,27 +314,30 @@ __device__ __forceinline__ void half_nn(const GridParams &g, const int *__restri
 // Most steps move the points by far less than the gap between their nearest
 // and second nearest Q point, so most searches would find what the last one
 // found. A search therefore also leaves where it was made and a distance that
-// no other point is closer than (group_nn, kApart); by the triangle inequality
+// no other point is closer than (Found); by the triangle inequality
 // the neighbour stands while its distance now is below that distance less the
 // way moved since, and there is still none while eps is. A block first decides
 // that with a point per thread, lists the points that need a search, searches
-// those with kRefG lanes each, and a point per thread then lays out the values
+// those with half a warp each, and a point per thread then lays out the values
 // whose products the sums take. The neighbours are those of a search of every
 // point. With a search of every point each step was bound by the latency of
 // the grid walks (42 us of 55 at 150k points).
-// seeds[i]: the neighbour, kSeedNone or kSeedFresh (no search yet at this level).
+// Bound by a chain of latencies now, whatever the points: a settled step of 50k
+// takes 17.5 us from its first load (pose and values 2.5, searches 3.5, sums 1.5,
+// the two tickets 3, closing sums 2.7, solve 2.9; 12.6 for 4k points).
+// near[i]: the neighbour and its position in Xe, or kSeedNone or kSeedFresh (no
+// search yet at this level) there; certs[i]: where the search was made and the
+// distance. Neither needs a gather, and the loads of a point's values do not
+// wait for the pose.
 //
 // A block's points are the runs of kRefSlots points numbered blockIdx.x,
 // + gridDim.x, ..., kRefRuns of them at a time; the 17 sums of each slot go
 // through the runs in order (four lanes a slot, every fourth sum each), then
 // over the slots.
 constexpr int kSeedFresh = -1, kSeedNone = -2;
-// Cells are visited up to this part of eps beyond the nearest point (a refinement
-// of 50k points took 3.31 ms with 0.06, 3.26 with 0.125, 3.47 with 0.25).
+// Cells are visited up to this part of eps beyond the nearest point (half of it or
+// twice it: 2 and 6% slower at 50k points).
 constexpr float kRefGuard = 0.125f;
-// Up to this many searches of a block take half a warp each (a refinement of 50k
-// points: 3.64 ms with none, 3.26 with 64, 3.28 with all).
-constexpr int kRefFew = 64;
 constexpr int kRefSlots = 64, kRefRuns = kRefThreads / kRefSlots;
 // The values of a point: 1, w, w xc (3), xc (3), xc x e (3), e (3), or all 0
 // without a neighbour; sum k takes the products of kTermA[k] and kTermB[k].
@@ -322,54 +349,68 @@ __global__ void __launch_bounds__(kRefThreads, kRefBlocksPerSm) k_refine_step(co
                                                              const GridParams *gep, const int *__restrict__ start,
                                                              const float4 *__restrict__ Xe, float eps, float mu,
                                                              RansacState *st, double *partials, int max_iters,
-                                                             double tol, int *__restrict__ seeds,
+                                                             double tol, float4 *__restrict__ near,
                                                              float4 *__restrict__ certs) {
   __shared__ int s_last, s_need;
-  __shared__ double tot[kNSum];
+  __shared__ double tot[kNSum + 1];  // the last is 0 (refine_solve)
+  __shared__ GridParams s_grid;
+  __shared__ float s_pose[15];  // rotation, centre, translation less the centre
   __shared__ float4 s_query[kRefThreads];  // the points to search: position, thread
   __shared__ int s_found[kRefThreads];     // per thread: its seed, then its neighbour
+  __shared__ float s_seed2[kRefThreads];   // the seed's squared distance
   __shared__ float s_val[kNVal][kRefThreads + 8];
   // the next step may be scheduled now (launched as a programmatic dependent,
   // it waits below for this one to finish); this step reads the pose, the
-  // state and the seeds the previous step wrote
+  // state and the neighbours the previous step wrote
   asm volatile("griddepcontrol.launch_dependents;");
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
   const int run = gridDim.x * kRefSlots;  // points from one run of this block to its next
+  const int own = (threadIdx.x / kRefSlots) * run + (threadIdx.x % kRefSlots);
+  float4 p = make_float4(0.f, 0.f, 0.f, 0.f), at = p, nr = p;
+  int i = blockIdx.x * kRefSlots + own;
+  if (i < nP) p = XP[i];
+  static_assert(sizeof(GridParams) % 4 == 0 && sizeof(GridParams) <= 128, "a lane per word");
+  if (threadIdx.x < sizeof(GridParams) / 4)
+    reinterpret_cast<int *>(&s_grid)[threadIdx.x] = reinterpret_cast<const int *>(gep)[threadIdx.x];
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  if (!st->active) return;
-  const float eps2 = eps * eps;
-  const double *T = st->T;
-  float R[9], tc[3], c[3];
-  for (int r = 0; r < 3; ++r) {
-    for (int k = 0; k < 3; ++k) R[3 * r + k] = (float)T[4 * r + k];
-    c[r] = (float)st->center[r];
-    tc[r] = (float)(T[4 * r + 3] - st->center[r]);
+  if (i < nP) at = certs[i], nr = near[i];
+  // a lane per entry of the pose: the FP64 unit takes a warp instruction every
+  // 16 clocks, and eighteen of them in each of an SM's 32 warps took 4.8 us
+  if (threadIdx.x < 15) {
+    const int k = threadIdx.x, r = k < 9 ? k / 3 : (k - 9) % 3;
+    const double c = __ldcg(st->center + r);
+    s_pose[k] = (float)(k < 9 ? __ldcg(st->T + 4 * r + k % 3) : k < 12 ? c : __ldcg(st->T + 4 * r + 3) - c);
   }
   if (threadIdx.x == 0) s_need = 0;
+  if (!st->active) return;
+  const float eps2 = eps * eps;
+  __syncthreads();
+  const bool wrapped = (s_grid.wx != s_grid.nx) | (s_grid.wy != s_grid.ny) | (s_grid.wz != s_grid.nz);
   // sums lane % 4, + 4, ... of the slot threadIdx.x / 4
   constexpr int kMine = (kNSum + 3) / 4;
   float acc[kMine];
 #pragma unroll
   for (int u = 0; u < kMine; ++u) acc[u] = 0.f;
   for (int r0 = blockIdx.x * kRefSlots; r0 < nP; r0 += kRefRuns * run) {
-    const int i = r0 + (threadIdx.x / kRefSlots) * run + (threadIdx.x % kRefSlots);
+    i = r0 + own;
     const bool valid = i < nP;
     float xc0 = 0.f, xc1 = 0.f, xc2 = 0.f, x = 0.f, y = 0.f, z = 0.f;
     int bt = kSeedNone;
     bool search = false;
+    float seed2 = eps2;
     __syncthreads();  // s_need is 0; the previous round's s_found and s_val have been read
     if (valid) {
-      const float4 p = XP[i], at = certs[i];
-      const int seed = seeds[i];
+      if (r0 >= run) p = XP[i], at = certs[i], nr = near[i];  // (the first round's are here)
+      const float *R = s_pose, *c = s_pose + 9, *tc = s_pose + 12;
       xc0 = fmaf(R[0], p.x, fmaf(R[1], p.y, fmaf(R[2], p.z, tc[0])));
       xc1 = fmaf(R[3], p.x, fmaf(R[4], p.y, fmaf(R[5], p.z, tc[1])));
       xc2 = fmaf(R[6], p.x, fmaf(R[7], p.y, fmaf(R[8], p.z, tc[2])));
       x = xc0 + c[0], y = xc1 + c[1], z = xc2 + c[2];
-      bt = seed;
+      bt = __float_as_int(nr.w);
       search = true;
-      if (seed != kSeedFresh) {
-        float d = eps;
-        if (seed >= 0 && LSR_IN_BOUNDS(seed, gep->npts, kSiteGridPoint)) d = sqrtf(nn_d2(Xe[seed], x, y, z));
+      if (bt != kSeedFresh) {
+        const float d2 = bt >= 0 ? nn_d2(nr, x, y, z) : eps2, d = bt >= 0 ? sqrtf(d2) : eps;
+        if (d2 < eps2) seed2 = d2;
         // (4e-6: above the FP32 rounding of both distances; a NaN searches)
         search = !((d + sqrtf(nn_d2(at, x, y, z))) * (1.f + 4e-6f) < at.w);
       }
@@ -382,40 +423,40 @@ __global__ void __launch_bounds__(kRefThreads, kRefBlocksPerSm) k_refine_step(co
       if (search) {
         s_query[base + __popc(m & ((1u << lane) - 1u))] = make_float4(x, y, z, __int_as_float(threadIdx.x));
         s_found[threadIdx.x] = bt;
+        s_seed2[threadIdx.x] = seed2;
       }
     }
     __syncthreads();
     const int need = s_need;
     if (need) {
       constexpr int kWarps = kRefThreads / 32;
-      const GridParams g = *gep;
-      const bool few = need <= kRefFew && g.wx == g.nx && g.wy == g.ny && g.wz == g.nz;
-      const int G = few ? kRefH : kRefG;  // lanes a query
       // consecutive queries go to different warps; whole warps reach the shuffles
-      for (int q0 = wp; q0 < need; q0 += kRefThreads / G) {
-        const int k = q0 + kWarps * (lane / G);
+      for (int q0 = wp; q0 < need; q0 += kRefThreads / kRefH) {
+        const int k = q0 + kWarps * (lane / kRefH);
         float4 w = make_float4(__int_as_float(0x7fc00000), 0.f, 0.f, 0.f);  // NaN: the query visits no cell
         int thread = 0, seed = -1;
-        if (k < need) w = s_query[k], thread = __float_as_int(w.w), seed = s_found[thread];
-        float best, apart;
-        int nn, bidx;
-        if (few)
-          half_nn(g, start, Xe, w.x, w.y, w.z, eps2, seed, kRefGuard * eps, nn, apart);
-        else
-          group_nn<kRefG, true>(g, start, Xe, w.x, w.y, w.z, eps2, best, nn, bidx, seed, kRefGuard * eps, &apart);
-        if (k < need && (lane & (G - 1)) == 0) {
-          nn = nn < 0 ? kSeedNone : nn;
-          s_found[thread] = nn;
-          const int j = r0 + (thread / kRefSlots) * run + (thread % kRefSlots);
-          seeds[j] = nn;
-          certs[j] = make_float4(w.x, w.y, w.z, apart);
+        float seed2 = eps2;
+        if (k < need) {
+          w = s_query[k], thread = __float_as_int(w.w);
+          if (s_seed2[thread] < eps2) seed = s_found[thread], seed2 = s_seed2[thread];
+        }
+        const Found f = wrapped ? group_nn_wrapped(s_grid, start, Xe, w.x, w.y, w.z, eps2, seed)
+                                : half_nn(s_grid, start, Xe, w.x, w.y, w.z, seed2, seed, kRefGuard * eps);
+        if (k < need && (lane & (kRefH - 1)) == 0) {
+          s_found[thread] = f.at < 0 ? kSeedNone : f.at;
+          certs[r0 + (thread / kRefSlots) * run + (thread % kRefSlots)] = make_float4(w.x, w.y, w.z, f.apart);
         }
       }
       __syncthreads();
       if (threadIdx.x == 0) s_need = 0;
-      if (search) bt = s_found[threadIdx.x];
+      if (search) {
+        bt = s_found[threadIdx.x];
+        if (bt >= 0) nr = Xe[bt];
+        nr.w = __int_as_float(bt);
+        near[i] = nr;
+      }
     }
-    const float4 q = bt >= 0 ? Xe[bt] : make_float4(__int_as_float(0x7fc00000), 0.f, 0.f, 0.f);
+    const float4 q = bt >= 0 ? nr : make_float4(__int_as_float(0x7fc00000), 0.f, 0.f, 0.f);
     float v[kNVal];
 #pragma unroll
     for (int u = 0; u < kNVal; ++u) v[u] = 0.f;
@@ -461,33 +502,42 @@ __global__ void __launch_bounds__(kRefThreads, kRefBlocksPerSm) k_refine_step(co
       partials[(size_t)blockIdx.x * kNAcc + threadIdx.x] = t;
     }
   }
-  // Two-level close: the last block of each group of kRefGroup blocks sums its
-  // group's partials in block order; the last group to close sums the group
-  // sums and solves (fewer dependent loads on the closing path).
+  // The last block to finish sums the partials: those of each kRefGroup blocks in
+  // block order, sum k = t % 17 over the groups t / 17, t / 17 + 15, ..., then
+  // the 15 segments in order (a fixed order: the sums are deterministic). With
+  // more than kRefAtOnce groups the last block of each group sums its group
+  // first: another fence, atomic and load one after the other (1.7 us), but the
+  // 17 x 608 FP64 additions of a full grid alone keep one SM's unit (two lanes a
+  // clock) busy for 2.7 us.
+  const unsigned nb = gridDim.x, ng = (nb + kRefGroup - 1) / kRefGroup;
+  const bool grouped = ng > kRefAtOnce;
   double *gpart = partials + (size_t)kRefMaxBlocks * kNAcc;
-  unsigned *gticket = reinterpret_cast<unsigned *>(gpart + (size_t)kRefMaxGroups * kNAcc);
-  const unsigned cgrp = blockIdx.x / kRefGroup, ng = (gridDim.x + kRefGroup - 1) / kRefGroup;
-  const unsigned g0 = cgrp * kRefGroup, gsz = min((unsigned)kRefGroup, gridDim.x - g0);
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) s_last = atomicAdd(gticket + cgrp, 1u) == gsz - 1;
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  if (threadIdx.x < kNSum) {
+  const auto group_sum = [&](unsigned g, int k) {
+    const unsigned g0 = g * kRefGroup;
     double v[kRefGroup];
 #pragma unroll
-    for (int u = 0; u < kRefGroup; ++u)
-      v[u] = (unsigned)u < gsz ? __ldcg(partials + (size_t)(g0 + u) * kNAcc + threadIdx.x) : 0.0;
+    for (unsigned u = 0; u < kRefGroup; ++u)
+      v[u] = g0 + u < nb ? __ldcg(partials + (size_t)(g0 + u) * kNAcc + k) : 0.0;
     double t = 0.0;
 #pragma unroll
-    for (int u = 0; u < kRefGroup; ++u) t += v[u];
-    gpart[(size_t)cgrp * kNAcc + threadIdx.x] = t;
+    for (unsigned u = 0; u < kRefGroup; ++u) t += v[u];
+    return t;
+  };
+  if (grouped) {
+    unsigned *gticket = reinterpret_cast<unsigned *>(gpart + (size_t)kRefMaxGroups * kNAcc);
+    const unsigned cgrp = blockIdx.x / kRefGroup, gsz = min((unsigned)kRefGroup, nb - cgrp * kRefGroup);
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(gticket + cgrp, 1u) == gsz - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    if (threadIdx.x < kNSum) gpart[(size_t)cgrp * kNAcc + threadIdx.x] = group_sum(cgrp, threadIdx.x);
+    if (threadIdx.x == 0) gticket[cgrp] = 0u;
   }
-  if (threadIdx.x == 0) gticket[cgrp] = 0u;
   __threadfence();
   __syncthreads();
-  if (threadIdx.x == 0) s_last = atomicAdd(&st->ticket, 1u) == ng - 1;
+  if (threadIdx.x == 0) s_last = atomicAdd(&st->ticket, 1u) == (grouped ? ng : nb) - 1;
   __syncthreads();
   if (!s_last) return;
   __threadfence();
@@ -496,15 +546,17 @@ __global__ void __launch_bounds__(kRefThreads, kRefBlocksPerSm) k_refine_step(co
   else if (threadIdx.x < 15) ss.center[threadIdx.x - 12] = __ldcg(st->center + threadIdx.x - 12);
   else if (threadIdx.x == 15) ss.iters_done = __ldcg(&st->iters_done);
   else if (threadIdx.x == 16) ss.level_iters = __ldcg(&st->level_iters);
+  else if (threadIdx.x == 17) tot[kNSum] = 0.0, st->ticket = 0u;
   {
-    // sum k = t % 17 over the groups t / 17, t / 17 + 15, ..., then the 15
-    // segments in order (a fixed order: the sums are deterministic)
     constexpr int kSeg = kRefThreads / kNSum;
     __shared__ double seg[kSeg][kNSum];
     const int k = threadIdx.x % kNSum, sg = threadIdx.x / kNSum;
     if (sg < kSeg) {
       double sum = 0.0;
-      for (unsigned b = sg; b < ng; b += kSeg) sum += __ldcg(gpart + (size_t)b * kNAcc + k);
+      if (grouped)
+        for (unsigned g = sg; g < ng; g += kSeg) sum += __ldcg(gpart + (size_t)g * kNAcc + k);
+      else if (sg < ng)
+        sum += group_sum(sg, k);
       seg[sg][k] = sum;
     }
     __syncthreads();
@@ -513,10 +565,9 @@ __global__ void __launch_bounds__(kRefThreads, kRefBlocksPerSm) k_refine_step(co
       for (int q = 0; q < kSeg; ++q) t += seg[q][threadIdx.x];
       tot[threadIdx.x] = t;
     }
+    __syncwarp();
   }
-  __syncthreads();
-  if (threadIdx.x == 0) st->ticket = 0u;
-  refine_solve(tot, ss, st, max_iters, tol);
+  if (threadIdx.x < 32) refine_solve(tot, ss, st, max_iters, tol);
 }
 
 __global__ void k_refine_level_begin(RansacState *st) {
@@ -742,8 +793,6 @@ __global__ void k_objective_sum(const __grid_constant__ ObjJobs J) {
 
 }  // namespace
 
-// One query per group of kRefG lanes per round; at most two blocks per SM so
-// that the launch-closing block sums few partials.
 int64_t refine_partial_doubles() { return (int64_t)kNAcc * (kRefMaxBlocks + kRefMaxGroups) + kRefMaxGroups; }
 
 cudaError_t refine_reset_tickets(double *partials, cudaStream_t s) {
@@ -782,18 +831,18 @@ cudaError_t launch_subsample(const float *xyz, int n, int stride, float4 *out, c
 }
 
 cudaError_t launch_refine_step(const float4 *XP, int nP, const GridParams *ge, const int *start_e, const float4 *Xe,
-                               float eps_r, float mu, int max_iters, RansacState *st, double *partials, int *seeds,
+                               float eps_r, float mu, int max_iters, RansacState *st, double *partials, float4 *near,
                                float4 *certs, bool chained, cudaStream_t s) {
   const int nb = refine_blocks(nP);
   if (chained) {
     // directly after the previous step: scheduled while it closes
     cudaError_t e = cudaSuccess;
     LSR_LAUNCH(e = pdl_launch(k_refine_step, dim3(nb), dim3(kRefThreads), s, XP, nP, ge, start_e, Xe, eps_r, mu, st,
-                              partials, max_iters, 1e-6, seeds, certs));
+                              partials, max_iters, 1e-6, near, certs));
     LSR_CUDA_TRY(e);
   } else {
     LSR_LAUNCH(k_refine_step<<<nb, kRefThreads, 0, s>>>(XP, nP, ge, start_e, Xe, eps_r, mu, st, partials, max_iters,
-                                                        1e-6, seeds, certs));
+                                                        1e-6, near, certs));
   }
   return cudaGetLastError();
 }
