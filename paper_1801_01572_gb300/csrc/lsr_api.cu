@@ -199,7 +199,7 @@ int cap_cells_for(int n) { return std::max(8 * n, 1 << 20); }
 // Consensus: clouds of P from this size on take the estimate pre-pass (every
 // kConsensusPrepassStride-th point) before the full bounds pass.
 constexpr int kConsensusPrepassMin = 16384;
-constexpr int kConsensusPrepassStride = 16;
+constexpr int kConsensusPrepassStride = 32;
 
 struct CloudLayout {
   int n = 0, cap_f = 0, cap_n = 0, cap_e = 0;
@@ -329,6 +329,7 @@ struct PairLayout {
   int *count2 = nullptr;     // exact counts of the reaching hypotheses
   int *tie_list = nullptr;   // the survivor slots tied at the top
   unsigned long long *prog = nullptr;  // per survivor: bounds progress (points done << 32 | IN + undecided)
+  Groups far;                // groups of P that a hypothesis moves far from Q (large P)
   int *c0 = nullptr;         // an exact count reached by some survivor (the bounds pass's bar)
   // single-cell lattice of Q (lsr_params.nn_mode = LSR_NN_SINGLE_CELL)
   int cap_s = 0;
@@ -378,6 +379,14 @@ void plan_pair(Arena &a, int nP, int nQ, bool stP, bool stQ, int64_t H, int leve
   L.tie_list = a.take<int>(L.surv_cap);
   L.prog = a.take<unsigned long long>(L.surv_cap);
   L.c0 = a.take<int>(1);
+  if (nP >= kConsensusPrepassMin) {
+    L.far.p = a.take<GroupParams>(1);
+    L.far.grp = a.take<float4>(nP);
+    L.far.first = a.take<int>(nP);
+    L.far.words = a.take<unsigned>(2 * (size_t)kGrpCapWords);
+    L.far.up = a.take<int>(L.surv_cap);
+    L.far.ok = a.take<uint8_t>(L.surv_cap);
+  }
   L.tc_ws = a.take<char>(precision != LSR_MATCH_FP32 ? tc_workspace_bytes(nP, nQ, precision == LSR_MATCH_BF16)
                                                       : fp32_workspace_bytes(nP, nQ));
   L.cap_s = L.Q.cap_e;
@@ -824,7 +833,7 @@ int enqueue_pair(lsr_ctx *c, const PairLayout &L, const float *P, const float *Q
     if (prepass) {
       TRY_CUDA(c,
                launch_consensus_bounds(Pc.Xn, nP, kConsensusPrepassStride, L.cls, L.in_bits, L.near_bits, L.pose, L.ok,
-                                       &L.st->n_surv, L.count, L.amb, nullptr, nullptr, s),
+                                       &L.st->n_surv, L.count, L.amb, s),
                "consensus estimate");
       TRY_CUDA(c, launch_top_upper(L.count, L.amb, L.ok, &L.st->n_surv, 32, L.sel, s), "top");
       TRY_CUDA(c,
@@ -835,11 +844,19 @@ int enqueue_pair(lsr_ctx *c, const PairLayout &L, const float *P, const float *Q
       TRY_CUDA(c, cudaMemsetAsync(L.count, 0, sizeof(int) * L.surv_cap, s), "memset count");
       TRY_CUDA(c, cudaMemsetAsync(L.amb, 0, sizeof(int) * L.surv_cap, s), "memset count");
       TRY_CUDA(c, cudaMemsetAsync(L.prog, 0, sizeof(unsigned long long) * L.surv_cap, s), "memset count");
+      TRY_CUDA(c,
+               launch_group_build(Pc.Xn, nP, Pc.gn, Pc.start_n, p.r_normal, Qc.box, p.eps_inlier, Qc.X, nQ, L.far, s),
+               "groups");
+      TRY_CUDA(c,
+               launch_group_bounds(L.far, Pc.Xn, nP, L.cls, L.in_bits, L.near_bits, L.pose, L.ok, &L.st->n_surv, L.count,
+                                   L.amb, L.c0, L.prog, s),
+               "consensus bounds");
+    } else {
+      TRY_CUDA(c,
+               launch_consensus_bounds(Pc.Xn, nP, 1, L.cls, L.in_bits, L.near_bits, L.pose, L.ok, &L.st->n_surv,
+                                       L.count, L.amb, s),
+               "consensus bounds");
     }
-    TRY_CUDA(c,
-             launch_consensus_bounds(Pc.Xn, nP, 1, L.cls, L.in_bits, L.near_bits, L.pose, L.ok, &L.st->n_surv, L.count,
-                                     L.amb, prepass ? L.c0 : nullptr, prepass ? L.prog : nullptr, s),
-             "consensus bounds");
     if (!prepass) {
       TRY_CUDA(c, launch_top_upper(L.count, L.amb, L.ok, &L.st->n_surv, 32, L.sel, s), "top");
       TRY_CUDA(c,
@@ -851,11 +868,17 @@ int enqueue_pair(lsr_ctx *c, const PairLayout &L, const float *P, const float *Q
     TRY_CUDA(c, launch_reach_rest(L.count, L.amb, L.count2, L.sel, L.ok, &L.st->n_surv, L.rest, L.reach, s), "reach");
     // the others that may reach c0, each given up on once it no longer can
     TRY_CUDA(c, cudaMemsetAsync(L.prog, 0, sizeof(unsigned long long) * L.surv_cap, s), "memset count");
-    TRY_CUDA(c,
-             launch_consensus_count_bar(Pc.Xn, nP, L.cls, L.in_bits, L.near_bits, Qc.ge, Qc.start_e, Qc.Xe, L.pose,
-                                        L.rest, &L.st->n_surv, p.eps_inlier, L.count2, L.c0, L.count, L.amb, L.prog,
-                                        s),
-             "consensus reach");
+    if (prepass)
+      TRY_CUDA(c,
+               launch_group_count_bar(L.far, Pc.Xn, nP, L.cls, L.in_bits, L.near_bits, Qc.ge, Qc.start_e, Qc.Xe, L.pose,
+                                      L.rest, &L.st->n_surv, p.eps_inlier, L.count2, L.c0, L.count, L.amb, L.prog, s),
+               "consensus reach");
+    else
+      TRY_CUDA(c,
+               launch_consensus_count_bar(Pc.Xn, nP, L.cls, L.in_bits, L.near_bits, Qc.ge, Qc.start_e, Qc.Xe, L.pose,
+                                          L.rest, &L.st->n_surv, p.eps_inlier, L.count2, L.c0, L.count, L.amb, L.prog,
+                                          s),
+               "consensus reach");
     TRY_CUDA(c, launch_reach_mask(L.count2, nullptr, L.reach, &L.st->n_surv, L.tie, &L.st->n_tie, L.tie_list, s),
              "ties");
     // (the exact kernel adds its counts too: into amb, no longer needed)

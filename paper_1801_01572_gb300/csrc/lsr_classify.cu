@@ -224,16 +224,9 @@ __device__ __forceinline__ bool warp_any_within(const GridParams &g, const int *
 // Otherwise the undecided lanes are resolved by the whole warp, one at a time,
 // and count receives the exact inlier count. The points are XP[v * stride]
 // for v < ceil(nP / stride).
-// Bounds with c0 (a device count no larger than the winning count, e.g. the
-// exact count of some hypothesis): items run chunk-major, so each hypothesis's
-// chunks come in order, and prog[s] accumulates (points done << 32 | IN +
-// undecided) in one 64-bit word, read as one consistent pair. A chunk whose
-// hypothesis already has IN + undecided + points not yet done < c0 is left
-// out: that upper bound only falls as chunks finish, so the hypothesis can
-// neither win nor tie. (k_bounds_finish then adds the points left out to amb,
-// keeping IN + amb an upper bound.)
-// Exact counts with c0 and the upper bounds ub_lo + ub_extra of a bounds pass:
-// items run chunk-major too, prog[s] accumulates (IN + undecided of the chunks
+// Exact counts with c0 (a device count no larger than the winning count, e.g. the
+// exact count of some hypothesis) and the upper bounds ub_lo + ub_extra of a
+// bounds pass: items run chunk-major, so each hypothesis's chunks come in order, prog[s] accumulates (IN + undecided of the chunks
 // done << 32 | their exact count), and a chunk whose hypothesis has exact so
 // far + (its upper bound - the upper bound of the chunks done) < c0 is left
 // out: its count can no longer reach c0, so it can neither win nor tie (its
@@ -272,8 +265,7 @@ __global__ void __launch_bounds__(kClsThreads, kClsMinBlocks) k_consensus_count(
       if (threadIdx.x == 0) {
         const unsigned long long pv = __ldcg(prog + s);
         const long long lo32 = (long long)(unsigned)pv, hi32 = (long long)(pv >> 32);
-        s_skip = kBounds ? lo32 + ((long long)nP - hi32) < (long long)cbar
-                         : lo32 + ((long long)ub_lo[s] + (long long)ub_extra[s] - hi32) < (long long)cbar;
+        s_skip = lo32 + ((long long)ub_lo[s] + (long long)ub_extra[s] - hi32) < (long long)cbar;
       }
       __syncthreads();
       const bool skip = s_skip != 0;
@@ -329,23 +321,303 @@ __global__ void __launch_bounds__(kClsThreads, kClsMinBlocks) k_consensus_count(
       for (int k = 0; k < kClsThreads / 32; ++k) tc += s_cnt[k], ta += s_amb[k], ti += s_in[k];
       if (tc) atomicAdd(&count[s], tc);
       if (kBounds && ta) atomicAdd(&amb_count[s], ta);
-      if (abandon)
-        atomicAdd(prog + s, kBounds ? ((unsigned long long)(i1 - i0) << 32) | (unsigned)(tc + ta)
-                                    : ((unsigned long long)(ti + ta) << 32) | (unsigned)tc);
+      if (abandon) atomicAdd(prog + s, ((unsigned long long)(ti + ta) << 32) | (unsigned)tc);
     }
     __syncthreads();
   }
 }
 
-// After bounds with abandonment: amb[s] += the points of s left out, so that
-// IN + amb stays an upper bound of the count (below c0 for those left out).
+// ---------------------------------------------------------------- far groups
+// Most points of a wrong hypothesis lie far from Q, and so do their neighbours
+// in P: the points of P's normal-grid cells (some 25 of them, runs of at most
+// kGrpMost) are bounded by a sphere each, and one lookup of the moved centre in
+// a coarse bit-set (the voxels within eps + rmax of Q, by dilating Q's occupied
+// voxels) leaves out the whole group. The points of the groups that are left
+// bound the count from above; hypotheses whose bound is below a count that
+// some hypothesis reaches need no look at their points.
+constexpr int kGrpMost = 32;
+
+__global__ void k_group_params(const float *boxQ, float eps, float r_normal, GroupParams *gp) {
+  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+  GroupParams g{};
+  // flat neighbourhoods of a cell of edge r fit in 0.71 r; corners may not
+  g.rmax = 0.75f * r_normal;
+  const float h = 0.25f * (eps + g.rmax);
+  float ext = 0.f, mag = 0.f;
+  for (int d = 0; d < 3; ++d) {
+    ext = fmaxf(ext, boxQ[3 + d] - boxQ[d]);
+    mag = fmaxf(mag, fmaxf(fabsf(boxQ[d]), fabsf(boxQ[3 + d])));
+  }
+  if (boxQ[6] == 0.f && ext >= 0.f && isfinite(ext) && isfinite(mag)) {
+    // rounding of the voxel coordinates and of the moved points near Q
+    const float m = 4e-6f * (ext + mag + eps + g.rmax);
+    const float reach = (eps + g.rmax + m) * (1.f + 1e-4f);
+    // between voxel centres: half a diagonal more at either end
+    const float r = reach / h + 1.7321f * (1.f + 1e-3f);
+    g.r2 = r * r;
+    const float pad = reach + 2.f * h;
+    long long n[3];
+    bool fits = r < 30.f;
+    for (int d = 0; d < 3; ++d) {
+      const float e = (boxQ[3 + d] - boxQ[d] + 2.f * pad) / h;
+      fits = fits && e < 1e6f;
+      n[d] = fits ? (long long)e + 2 : 0;
+    }
+    const long long wx = (n[0] + 31) / 32;
+    if (fits && wx * n[1] * n[2] <= kGrpCapWords) {
+      g.ox = boxQ[0] - pad, g.oy = boxQ[1] - pad, g.oz = boxQ[2] - pad;
+      g.inv_h = 1.f / h;
+      g.nx = (int)n[0], g.ny = (int)n[1], g.nz = (int)n[2], g.wx = (int)wx;
+      g.usable = 1;
+    }
+  }
+  *gp = g;
+}
+
+// A thread per cell of P: its runs of points as (centre, number) and first point;
+// the number is negative if they do not fit in rmax (with the rounding of the
+// moved points) or there is no bit-set: such a group is never far.
+__global__ void k_group_cells(const float4 *__restrict__ Xn, const GridParams *gn, const int *__restrict__ start,
+                              GroupParams *gp, float4 *__restrict__ grp, int *__restrict__ first) {
+  const float rmax = gp->usable ? gp->rmax : -1.f;
+  const int ncells = gn->ncells;
+  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < ncells; c += gridDim.x * blockDim.x) {
+    const int b = start[c], e = start[c + 1];
+    for (int b0 = b; b0 < e; b0 += kGrpMost) {
+      const int m = min(kGrpMost, e - b0);
+      float lo[3] = {3e38f, 3e38f, 3e38f}, hi[3] = {-3e38f, -3e38f, -3e38f};
+      for (int t = b0; t < b0 + m; ++t) {
+        const float4 p = Xn[t];
+        lo[0] = fminf(lo[0], p.x), lo[1] = fminf(lo[1], p.y), lo[2] = fminf(lo[2], p.z);
+        hi[0] = fmaxf(hi[0], p.x), hi[1] = fmaxf(hi[1], p.y), hi[2] = fmaxf(hi[2], p.z);
+      }
+      float4 c4 = make_float4(0.5f * lo[0] + 0.5f * hi[0], 0.5f * lo[1] + 0.5f * hi[1],
+                                    0.5f * lo[2] + 0.5f * hi[2], __int_as_float(m));
+      float r2 = 0.f;
+      for (int t = b0; t < b0 + m; ++t) r2 = fmaxf(r2, dist2(Xn[t], c4.x, c4.y, c4.z));
+      const float r = sqrtf(r2) * (1.f + 1e-4f) + 4e-6f * (fabsf(c4.x) + fabsf(c4.y) + fabsf(c4.z));
+      if (!(r <= rmax)) c4.w = __int_as_float(-m);
+      const int k = atomicAdd(&gp->n, 1);
+      grp[k] = c4;
+      first[k] = b0;
+    }
+  }
+}
+
+__global__ void k_group_mark(const float4 *__restrict__ XQ, int nQ, const GroupParams *gp, unsigned *__restrict__ occ) {
+  if (!gp->usable) return;
+  const GroupParams g = *gp;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nQ; i += gridDim.x * blockDim.x) {
+    const float4 q = XQ[i];
+    const int x = min(max((int)((q.x - g.ox) * g.inv_h), 0), g.nx - 1), y = min(max((int)((q.y - g.oy) * g.inv_h), 0), g.ny - 1),
+              z = min(max((int)((q.z - g.oz) * g.inv_h), 0), g.nz - 1);
+    atomicOr(occ + (size_t)(z * g.ny + y) * g.wx + (x >> 5), 1u << (x & 31));
+  }
+}
+
+// A thread per word: the voxels within the reach of an occupied one, row by row.
+__global__ void __launch_bounds__(256) k_group_dilate(const GroupParams *gp, const unsigned *__restrict__ occ,
+                                                      unsigned *__restrict__ out) {
+  if (!gp->usable) return;
+  const GroupParams g = *gp;
+  const int total = g.wx * g.ny * g.nz, R = (int)sqrtf(g.r2);
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
+    const int xw = t % g.wx, y = t / g.wx % g.ny, z = t / g.wx / g.ny;
+    unsigned acc = 0u;
+    for (int dz = max(-R, -z); dz <= min(R, g.nz - 1 - z); ++dz)
+      for (int dy = max(-R, -y); dy <= min(R, g.ny - 1 - y); ++dy) {
+        const float rem = g.r2 - (float)(dy * dy + dz * dz);
+        if (rem < 0.f) continue;
+        const unsigned *row = occ + (size_t)t + (dz * g.ny + dy) * g.wx;
+        const unsigned cur = row[0], prev = xw > 0 ? row[-1] : 0u, next = xw + 1 < g.wx ? row[1] : 0u;
+        if (!(cur | prev | next)) continue;
+        // or of the shifts by 0 .. w to either side, doubling
+        unsigned long long a = cur | (unsigned long long)next << 32, b = prev | (unsigned long long)cur << 32;
+        int left = (int)sqrtf(rem);
+        for (int k = 1; left > 0; left -= k, k <<= 1) {
+          k = min(k, left);
+          a |= a >> k, b |= b << k;
+        }
+        acc |= (unsigned)a | (unsigned)(b >> 32);
+      }
+    out[t] = acc;
+  }
+}
+
+// The points of group k under T that may be inliers: all or none.
+__device__ __forceinline__ int group_points(const GroupParams &g, const unsigned *__restrict__ near, float4 c,
+                                            const Rigid12 &T) {
+  const int m = __float_as_int(c.w);
+  if (m < 0) return -m;
+  float x, y, z;
+  T.apply(c, x, y, z);
+  const float fx = (x - g.ox) * g.inv_h, fy = (y - g.oy) * g.inv_h, fz = (z - g.oz) * g.inv_h;
+  if (!(fx >= 0.f && fx < (float)g.nx && fy >= 0.f && fy < (float)g.ny && fz >= 0.f && fz < (float)g.nz)) return 0;
+  const int ix = (int)fx;
+  return (__ldg(near + (size_t)((int)fz * g.ny + (int)fy) * g.wx + (ix >> 5)) >> (ix & 31)) & 1u ? m : 0;
+}
+
+// A block per hypothesis, a thread per group at a time: up[s] = the points of
+// its groups that are not far. ok2: those whose up reaches c0; the others get
+// it in amb.
+__global__ void __launch_bounds__(256) k_group_bounds(const GroupParams *gp, const float4 *__restrict__ grp,
+                                                      const unsigned *__restrict__ near, const float *__restrict__ pose,
+                                                      const uint8_t *__restrict__ ok, const int *n_dev, const int *c0,
+                                                      int *__restrict__ amb, uint8_t *__restrict__ ok2,
+                                                      int *__restrict__ up) {
+  const GroupParams g = *gp;
+  const int nh = *n_dev, bar = *c0;
+  __shared__ int s_sum[8];
+  for (int s = blockIdx.x; s < nh; s += gridDim.x) {
+    if (!ok[s]) {
+      if (threadIdx.x == 0) ok2[s] = 0;
+      continue;
+    }
+    Rigid12 T;
+    T.load(pose + (size_t)s * 12);
+    int sum = 0;
+#pragma unroll 4
+    for (int k = threadIdx.x; k < g.n; k += 256) sum += group_points(g, near, grp[k], T);
+    sum = warp_sum(sum);
+    if ((threadIdx.x & 31) == 0) s_sum[threadIdx.x >> 5] = sum;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      int all = 0;
+      for (int k = 0; k < 8; ++k) all += s_sum[k];
+      up[s] = all;
+      ok2[s] = all >= bar;
+      if (all < bar) amb[s] = all;
+    }
+    __syncthreads();
+  }
+}
+
+// k_consensus_count over the points of the groups that are not far, with c0 and
+// prog: items (hypothesis, run of groups) in the order of the runs. What is
+// left of a hypothesis is bounded by up (the bounds pass; ub_lo + ub_extra for
+// the exact counts) less that of the runs done (prog's high word), so it is
+// given up on after a fraction of its points: with whole chunks and nP for up
+// nine in ten points of 9k hypotheses were read (3.5 ms for 200k points).
+constexpr int kGrpBatch = 128;  // groups whose points are listed at once
+template <bool kBounds>
+__global__ void __launch_bounds__(kClsThreads, 6) k_group_count(
+    const float4 *__restrict__ XP, int nP, const GroupParams *__restrict__ gp, const float4 *__restrict__ grp,
+    const int *__restrict__ first, const unsigned *__restrict__ far_bits, const ClsParams *__restrict__ cpp,
+    const unsigned *__restrict__ in_bits, const unsigned *__restrict__ near_bits, const GridParams *__restrict__ gep,
+    const int *__restrict__ start, const float4 *__restrict__ Xe, const float *__restrict__ pose,
+    const uint8_t *__restrict__ ok, const int *n_dev, float eps2, int *__restrict__ count, int *__restrict__ amb_count,
+    const int *c0, unsigned long long *prog, const int *__restrict__ ub_lo, const int *__restrict__ ub_extra) {
+  __shared__ int s_pts[kGrpBatch * kGrpMost];
+  __shared__ int s_cnt[kClsThreads / 32], s_amb[kClsThreads / 32], s_in[kClsThreads / 32], s_skip, s_n;
+  const ClsParams c = *cpp;
+  const GroupParams gr = *gp;
+  const GridParams g = kBounds ? GridParams{} : *gep;
+  const int nh = *n_dev, cbar = *c0;
+  // runs of about kClsChunk points
+  const int run = max(1, min(16, (int)((long long)kClsChunk * gr.n / nP / kGrpBatch))) * kGrpBatch;
+  const int runs = (gr.n + run - 1) / run;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if (nh <= 0) return;
+  const int64_t items = (int64_t)nh * runs;
+  int64_t major = (int64_t)blockIdx.x / nh, minor = (int64_t)blockIdx.x % nh;
+  const int64_t step_major = (int64_t)gridDim.x / nh, step_minor = (int64_t)gridDim.x % nh;
+  for (int64_t item = blockIdx.x; item < items; item += gridDim.x) {
+    const int s = (int)minor, k0 = (int)major * run;
+    major += step_major, minor += step_minor;
+    if (minor >= nh) minor -= nh, ++major;
+    if (!ok[s]) continue;
+    // (one thread reads the pair, so the whole block takes one decision)
+    if (threadIdx.x == 0) {
+      const unsigned long long pv = __ldcg(prog + s);
+      const long long lo32 = (long long)(unsigned)pv, hi32 = (long long)(pv >> 32);
+      const long long up = kBounds ? (long long)ub_lo[s] : (long long)ub_lo[s] + (long long)ub_extra[s];
+      s_skip = lo32 + (up - hi32) < (long long)cbar;
+      s_n = 0;
+    }
+    __syncthreads();
+    const bool skip = s_skip != 0;
+    __syncthreads();
+    if (skip) continue;
+    Rigid12 T;
+    T.load(pose + (size_t)s * 12);
+    int cnt = 0, namb = 0, nin = 0, left = 0;
+    for (int b0 = k0; b0 < min(gr.n, k0 + run); b0 += kGrpBatch) {
+      // the points of the batch's groups that are not far
+      const int k = b0 + threadIdx.x;
+      if (threadIdx.x < kGrpBatch && k < gr.n) {
+        const int m = group_points(gr, far_bits, grp[k], T);
+        if (m > 0) {
+          const int at = atomicAdd(&s_n, m), f = first[k];
+          for (int u = 0; u < m; ++u) s_pts[at + u] = f + u;
+        }
+      }
+      __syncthreads();
+      const int np = s_n;
+      left += np;
+      for (int r = 0; r < np; r += kClsThreads) {
+        bool in = false, amb = false;
+        float x = 0.f, y = 0.f, z = 0.f;
+        if (r + (int)threadIdx.x < np) {
+          T.apply(XP[s_pts[r + threadIdx.x]], x, y, z);
+          if (c.all_amb) {
+            amb = true;
+          } else {
+            const float fx = (x - c.ox) * c.inv_h, fy = (y - c.oy) * c.inv_h, fz = (z - c.oz) * c.inv_h;
+            if (fx >= 0.f && fx < (float)c.nx && fy >= 0.f && fy < (float)c.ny && fz >= 0.f && fz < (float)c.nz) {
+              const int ix = (int)fx, iy = (int)fy, iz = (int)fz;
+              const size_t word = cls_word(c, ix, iy, iz);
+              const unsigned bit = 1u << cls_bit(ix, iy, iz);
+              if (__ldg(in_bits + word) & bit)
+                in = true;
+              else
+                amb = (__ldg(near_bits + word) & bit) != 0u;
+            }
+          }
+        }
+        cnt += in;
+        nin += in;
+        namb += amb;
+        if (kBounds) continue;
+        unsigned pend = __ballot_sync(0xffffffffu, amb);
+        while (pend) {
+          const int src = __ffs(pend) - 1;
+          pend &= pend - 1;
+          const float qx = __shfl_sync(0xffffffffu, x, src), qy = __shfl_sync(0xffffffffu, y, src),
+                      qz = __shfl_sync(0xffffffffu, z, src);
+          const bool hit = warp_any_within(g, start, Xe, qx, qy, qz, eps2);
+          if (lane == src) cnt += hit;
+        }
+      }
+      __syncthreads();
+      if (threadIdx.x == 0) s_n = 0;
+      __syncthreads();
+    }
+    cnt = warp_sum(cnt);
+    namb = warp_sum(namb);
+    if (!kBounds) nin = warp_sum(nin);
+    if (lane == 0) s_cnt[w] = cnt, s_amb[w] = namb, s_in[w] = nin;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      int tc = 0, ta = 0, ti = 0;
+      for (int k = 0; k < kClsThreads / 32; ++k) tc += s_cnt[k], ta += s_amb[k], ti += s_in[k];
+      if (tc) atomicAdd(&count[s], tc);
+      if (kBounds && ta) atomicAdd(&amb_count[s], ta);
+      atomicAdd(prog + s, kBounds ? ((unsigned long long)left << 32) | (unsigned)(tc + ta)
+                                  : ((unsigned long long)(ti + ta) << 32) | (unsigned)tc);
+    }
+    __syncthreads();
+  }
+}
+
+// After the bounds pass: amb[s] += the points of s left out, so that IN + amb
+// stays an upper bound of the count (below c0 for those left out).
 __global__ void k_bounds_finish(const unsigned long long *__restrict__ prog, const uint8_t *__restrict__ ok,
-                                const int *n_dev, int nP, int *__restrict__ amb) {
+                                const int *n_dev, const int *__restrict__ up, int *__restrict__ amb) {
   const int n = *n_dev;
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
-    if (ok && !ok[k]) continue;
+    if (!ok[k]) continue;
     const int done = (int)(prog[k] >> 32);
-    if (done < nP) amb[k] += nP - done;
+    if (done < up[k]) amb[k] += up[k] - done;
   }
 }
 
@@ -525,11 +797,49 @@ cudaError_t launch_consensus_count_bar(const float4 *XP, int nP, const ClsParams
 cudaError_t launch_consensus_bounds(const float4 *XP, int nP, int stride, const ClsParams *cp,
                                     const unsigned *in_bits, const unsigned *near_bits, const float *pose,
                                     const uint8_t *ok, const int *n_dev, int *in_count, int *amb_count,
-                                    const int *c0, unsigned long long *prog, cudaStream_t s) {
+                                    cudaStream_t s) {
   LSR_LAUNCH(k_consensus_count<true><<<kSms * 8, kClsThreads, 0, s>>>(XP, nP, stride, cp, in_bits, near_bits, nullptr,
                                                                       nullptr, nullptr, pose, ok, n_dev, 0, 0.f,
-                                                                      in_count, amb_count, c0, prog, nullptr, nullptr));
-  if (c0) LSR_LAUNCH(k_bounds_finish<<<kSms * 2, 256, 0, s>>>(prog, ok, n_dev, nP, amb_count));
+                                                                      in_count, amb_count, nullptr, nullptr, nullptr,
+                                                                      nullptr));
+  return cudaGetLastError();
+}
+
+cudaError_t launch_group_build(const float4 *Xn, int nP, const GridParams *gn, const int *start_n, float r_normal,
+                               const float *boxQ, float eps, const float4 *XQ, int nQ, const Groups &G,
+                               cudaStream_t s) {
+  LSR_CUDA_TRY(cudaMemsetAsync(G.words, 0, sizeof(unsigned) * (size_t)kGrpCapWords, s));
+  LSR_LAUNCH(k_group_params<<<1, 32, 0, s>>>(boxQ, eps, r_normal, G.p));
+  const int64_t nb = lsr_div_up(nP, 64), nq = lsr_div_up(nQ, 256);
+  LSR_LAUNCH(k_group_cells<<<(int)(nb < kSms * 8 ? nb : kSms * 8), 256, 0, s>>>(Xn, gn, start_n, G.p, G.grp, G.first));
+  LSR_LAUNCH(k_group_mark<<<(int)(nq < kSms * 8 ? nq : kSms * 8), 256, 0, s>>>(XQ, nQ, G.p, G.words));
+  LSR_LAUNCH(k_group_dilate<<<kSms * 8, 256, 0, s>>>(G.p, G.words, G.words + kGrpCapWords));
+  return cudaGetLastError();
+}
+
+cudaError_t launch_group_bounds(const Groups &G, const float4 *Xn, int nP, const ClsParams *cp, const unsigned *in_bits,
+                                const unsigned *near_bits, const float *pose, const uint8_t *ok, const int *n_dev,
+                                int *in_count, int *amb_count, const int *c0, unsigned long long *prog,
+                                cudaStream_t s) {
+  const unsigned *far_bits = G.words + kGrpCapWords;
+  LSR_LAUNCH(k_group_bounds<<<kSms * 8, 256, 0, s>>>(G.p, G.grp, far_bits, pose, ok, n_dev, c0, amb_count, G.ok, G.up));
+  LSR_LAUNCH(k_group_count<true><<<kSms * 6, kClsThreads, 0, s>>>(Xn, nP, G.p, G.grp, G.first, far_bits, cp, in_bits,
+                                                                  near_bits, nullptr, nullptr, nullptr, pose, G.ok,
+                                                                  n_dev, 0.f, in_count, amb_count, c0, prog, G.up,
+                                                                  nullptr));
+  LSR_LAUNCH(k_bounds_finish<<<kSms * 2, 256, 0, s>>>(prog, G.ok, n_dev, G.up, amb_count));
+  return cudaGetLastError();
+}
+
+cudaError_t launch_group_count_bar(const Groups &G, const float4 *Xn, int nP, const ClsParams *cp,
+                                   const unsigned *in_bits, const unsigned *near_bits, const GridParams *ge,
+                                   const int *start_e, const float4 *Xe, const float *pose, const uint8_t *ok,
+                                   const int *n_dev, float eps, int *count, const int *c0, const int *ub_lo,
+                                   const int *ub_extra, unsigned long long *prog, cudaStream_t s) {
+  LSR_LAUNCH(k_group_count<false><<<kSms * 6, kClsThreads, 0, s>>>(Xn, nP, G.p, G.grp, G.first, G.words + kGrpCapWords,
+                                                                   cp, in_bits, near_bits, ge, start_e, Xe, pose, ok,
+                                                                   n_dev, eps * eps, count, nullptr, c0, prog, ub_lo,
+                                                                   ub_extra));
   return cudaGetLastError();
 }
 

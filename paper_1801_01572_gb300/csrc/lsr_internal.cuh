@@ -696,6 +696,22 @@ __host__ __device__ inline size_t cls_word(const ClsParams &c, int x, int y, int
 }
 __host__ __device__ inline int cls_bit(int x, int y, int z) { return (x & 3) | ((y & 3) << 2) | ((z & 1) << 4); }
 constexpr int kClsCapWords = 1 << 23;  // words per bit-set (32 MB)
+// Far groups: groups of nearby P points, and a coarse bit-set of the voxels
+// within a group's reach of Q.
+struct GroupParams {
+  float ox, oy, oz, inv_h, rmax, r2;  // rmax: largest group radius; r2: the reach squared, in voxels
+  int nx, ny, nz, wx;                 // voxels, words of a row
+  int usable, n;                      // n: the groups
+};
+constexpr int kGrpCapWords = 1 << 20;
+struct Groups {
+  GroupParams *p = nullptr;
+  float4 *grp = nullptr;      // nP: centre, number of points (negative: never far)
+  int *first = nullptr;       // nP: its first point
+  unsigned *words = nullptr;  // 2 kGrpCapWords: Q's voxels, those within reach
+  int *up = nullptr;          // per hypothesis: the points of the groups that are not far
+  uint8_t *ok = nullptr;      // those whose up reaches c0
+};
 cudaError_t launch_cls_build(const float *boxQ, float eps, const float4 *XQ, int nQ, ClsParams *cp, unsigned *in_bits,
                              unsigned *near_bits, cudaStream_t s);
 // Inlier counts (as launch_consensus, without the distance sums).
@@ -705,14 +721,11 @@ cudaError_t launch_consensus_count(const float4 *XP, int nP, const ClsParams *cp
                                    int n_host, float eps, int *count, cudaStream_t s);
 // Bounds without exact tests over the points XP[v * stride]: in_count =
 // points in IN voxels (a lower bound of the inlier count), amb_count = points
-// in undecided voxels. With c0 (device; a count some hypothesis reaches) and
-// prog (device, one zeroed 64-bit word per hypothesis): a hypothesis whose
-// upper bound falls below c0 part-way is left out, its remaining points added
-// to amb_count (stride must be 1).
+// in undecided voxels.
 cudaError_t launch_consensus_bounds(const float4 *XP, int nP, int stride, const ClsParams *cp,
                                     const unsigned *in_bits, const unsigned *near_bits, const float *pose,
                                     const uint8_t *ok, const int *n_dev, int *in_count, int *amb_count,
-                                    const int *c0, unsigned long long *prog, cudaStream_t s);
+                                    cudaStream_t s);
 // Exact counts (count += ...) that give up on a hypothesis as soon as its
 // count can no longer reach c0 (device), from the upper bounds ub_lo + ub_extra
 // of a bounds pass; prog: one zeroed 64-bit word per hypothesis. A count given
@@ -722,6 +735,23 @@ cudaError_t launch_consensus_count_bar(const float4 *XP, int nP, const ClsParams
                                        const float4 *Xe, const float *pose, const uint8_t *ok, const int *n_dev,
                                        float eps, int *count, const int *c0, const int *ub_lo, const int *ub_extra,
                                        unsigned long long *prog, cudaStream_t s);
+// The groups of P (its normal grid) and the bit-set of Q.
+cudaError_t launch_group_build(const float4 *Xn, int nP, const GridParams *gn, const int *start_n, float r_normal,
+                               const float *boxQ, float eps, const float4 *XQ, int nQ, const Groups &G, cudaStream_t s);
+// Bounds over the points of the groups that are not far, with c0 (device; a
+// count some hypothesis reaches) and prog (one zeroed 64-bit word per
+// hypothesis): a hypothesis whose upper bound is below c0, from its groups or
+// part-way, is left out, what remained added to amb_count.
+cudaError_t launch_group_bounds(const Groups &G, const float4 *Xn, int nP, const ClsParams *cp, const unsigned *in_bits,
+                                const unsigned *near_bits, const float *pose, const uint8_t *ok, const int *n_dev,
+                                int *in_count, int *amb_count, const int *c0, unsigned long long *prog, cudaStream_t s);
+// launch_consensus_count_bar after launch_group_bounds (whose upper bounds leave
+// out the far groups, so the exact counts have to as well).
+cudaError_t launch_group_count_bar(const Groups &G, const float4 *Xn, int nP, const ClsParams *cp,
+                                   const unsigned *in_bits, const unsigned *near_bits, const GridParams *ge,
+                                   const int *start_e, const float4 *Xe, const float *pose, const uint8_t *ok,
+                                   const int *n_dev, float eps, int *count, const int *c0, const int *ub_lo,
+                                   const int *ub_extra, unsigned long long *prog, cudaStream_t s);
 // out (device) = max over sel of exact.
 cudaError_t launch_sel_max(const int *exact, const uint8_t *sel, const int *n_dev, int *out, cudaStream_t s);
 // sel: the K ok hypotheses with the largest lo + extra (ties to the smaller id).
