@@ -322,7 +322,10 @@ struct PairLayout {
   ClsParams *cls = nullptr;  // consensus voxel classification of Q
   unsigned *in_bits = nullptr, *near_bits = nullptr;
   uint8_t *sel = nullptr;    // the hypotheses with the largest count upper bounds
-  uint8_t *rest = nullptr;   // the others whose upper bound reaches their best count
+  int *sel_list = nullptr;   // (listed, and their number)
+  int *n_sel = nullptr;
+  int *rest = nullptr;       // the others whose upper bound reaches their best count, listed
+  int *n_rest = nullptr;
   uint8_t *reach = nullptr;  // sel | rest: the hypotheses counted exactly
   uint8_t *tie = nullptr;    // those tied at the maximum exact count
   int *amb = nullptr;        // points in undecided voxels per hypothesis
@@ -371,7 +374,10 @@ void plan_pair(Arena &a, int nP, int nQ, bool stP, bool stQ, int64_t H, int leve
   L.in_bits = a.take<unsigned>(kClsCapWords);
   L.near_bits = a.take<unsigned>(kClsCapWords);
   L.sel = a.take<uint8_t>(L.surv_cap);
-  L.rest = a.take<uint8_t>(L.surv_cap);
+  L.sel_list = a.take<int>(L.surv_cap);
+  L.n_sel = a.take<int>(1);
+  L.rest = a.take<int>(L.surv_cap);
+  L.n_rest = a.take<int>(1);
   L.reach = a.take<uint8_t>(L.surv_cap);
   L.tie = a.take<uint8_t>(L.surv_cap);
   L.amb = a.take<int>(L.surv_cap);
@@ -385,7 +391,7 @@ void plan_pair(Arena &a, int nP, int nQ, bool stP, bool stQ, int64_t H, int leve
     L.far.first = a.take<int>(nP);
     L.far.words = a.take<unsigned>(2 * (size_t)kGrpCapWords);
     L.far.up = a.take<int>(L.surv_cap);
-    L.far.ok = a.take<uint8_t>(L.surv_cap);
+    L.far.list = a.take<int>(L.surv_cap);
   }
   L.tc_ws = a.take<char>(precision != LSR_MATCH_FP32 ? tc_workspace_bytes(nP, nQ, precision == LSR_MATCH_BF16)
                                                       : fp32_workspace_bytes(nP, nQ));
@@ -835,12 +841,12 @@ int enqueue_pair(lsr_ctx *c, const PairLayout &L, const float *P, const float *Q
                launch_consensus_bounds(Pc.Xn, nP, kConsensusPrepassStride, L.cls, L.in_bits, L.near_bits, L.pose, L.ok,
                                        &L.st->n_surv, L.count, L.amb, s),
                "consensus estimate");
-      TRY_CUDA(c, launch_top_upper(L.count, L.amb, L.ok, &L.st->n_surv, 32, L.sel, s), "top");
+      TRY_CUDA(c, launch_top_upper(L.count, L.amb, L.ok, &L.st->n_surv, 32, L.sel, L.sel_list, L.n_sel, s), "top");
       TRY_CUDA(c,
                launch_consensus_count(Pc.Xn, nP, L.cls, L.in_bits, L.near_bits, Qc.ge, Qc.start_e, Qc.Xe, L.pose,
-                                      L.sel, &L.st->n_surv, 0, p.eps_inlier, L.count2, s),
+                                      L.sel_list, L.n_sel, p.eps_inlier, L.count2, nullptr, nullptr, nullptr, nullptr, s),
                "consensus top");
-      TRY_CUDA(c, launch_sel_max(L.count2, L.sel, &L.st->n_surv, L.c0, s), "consensus bar");
+      TRY_CUDA(c, launch_sel_max(L.count2, L.sel_list, L.n_sel, L.c0, s), "consensus bar");
       TRY_CUDA(c, cudaMemsetAsync(L.count, 0, sizeof(int) * L.surv_cap, s), "memset count");
       TRY_CUDA(c, cudaMemsetAsync(L.amb, 0, sizeof(int) * L.surv_cap, s), "memset count");
       TRY_CUDA(c, cudaMemsetAsync(L.prog, 0, sizeof(unsigned long long) * L.surv_cap, s), "memset count");
@@ -858,26 +864,25 @@ int enqueue_pair(lsr_ctx *c, const PairLayout &L, const float *P, const float *Q
                "consensus bounds");
     }
     if (!prepass) {
-      TRY_CUDA(c, launch_top_upper(L.count, L.amb, L.ok, &L.st->n_surv, 32, L.sel, s), "top");
+      TRY_CUDA(c, launch_top_upper(L.count, L.amb, L.ok, &L.st->n_surv, 32, L.sel, L.sel_list, L.n_sel, s), "top");
       TRY_CUDA(c,
                launch_consensus_count(Pc.Xn, nP, L.cls, L.in_bits, L.near_bits, Qc.ge, Qc.start_e, Qc.Xe, L.pose,
-                                      L.sel, &L.st->n_surv, 0, p.eps_inlier, L.count2, s),
+                                      L.sel_list, L.n_sel, p.eps_inlier, L.count2, nullptr, nullptr, nullptr, nullptr, s),
                "consensus top");
-      TRY_CUDA(c, launch_sel_max(L.count2, L.sel, &L.st->n_surv, L.c0, s), "consensus bar");
+      TRY_CUDA(c, launch_sel_max(L.count2, L.sel_list, L.n_sel, L.c0, s), "consensus bar");
     }
-    TRY_CUDA(c, launch_reach_rest(L.count, L.amb, L.count2, L.sel, L.ok, &L.st->n_surv, L.rest, L.reach, s), "reach");
+    TRY_CUDA(c, launch_reach_rest(L.count, L.amb, L.c0, L.sel, L.ok, &L.st->n_surv, L.reach, L.rest, L.n_rest, s), "reach");
     // the others that may reach c0, each given up on once it no longer can
     TRY_CUDA(c, cudaMemsetAsync(L.prog, 0, sizeof(unsigned long long) * L.surv_cap, s), "memset count");
     if (prepass)
       TRY_CUDA(c,
                launch_group_count_bar(L.far, Pc.Xn, nP, L.cls, L.in_bits, L.near_bits, Qc.ge, Qc.start_e, Qc.Xe, L.pose,
-                                      L.rest, &L.st->n_surv, p.eps_inlier, L.count2, L.c0, L.count, L.amb, L.prog, s),
+                                      L.rest, L.n_rest, p.eps_inlier, L.count2, L.c0, L.count, L.amb, L.prog, s),
                "consensus reach");
     else
       TRY_CUDA(c,
-               launch_consensus_count_bar(Pc.Xn, nP, L.cls, L.in_bits, L.near_bits, Qc.ge, Qc.start_e, Qc.Xe, L.pose,
-                                          L.rest, &L.st->n_surv, p.eps_inlier, L.count2, L.c0, L.count, L.amb, L.prog,
-                                          s),
+               launch_consensus_count(Pc.Xn, nP, L.cls, L.in_bits, L.near_bits, Qc.ge, Qc.start_e, Qc.Xe, L.pose,
+                                      L.rest, L.n_rest, p.eps_inlier, L.count2, L.c0, L.count, L.amb, L.prog, s),
                "consensus reach");
     TRY_CUDA(c, launch_reach_mask(L.count2, nullptr, L.reach, &L.st->n_surv, L.tie, &L.st->n_tie, L.tie_list, s),
              "ties");

@@ -238,12 +238,17 @@ __global__ void __launch_bounds__(kClsThreads, kClsMinBlocks) k_consensus_count(
     const int *__restrict__ start, const float4 *__restrict__ Xe, const float *__restrict__ pose,
     const uint8_t *__restrict__ ok, const int *n_dev, int n_host, float eps2, int *__restrict__ count,
     int *__restrict__ amb_count, const int *c0, unsigned long long *prog, const int *__restrict__ ub_lo,
-    const int *__restrict__ ub_extra) {
+    const int *__restrict__ ub_extra, const int *__restrict__ list) {
   const ClsParams c = *cpp;
   const GridParams g = kBounds ? GridParams{} : *gep;
   const int nh = n_dev ? *n_dev : n_host;
   const int nv = (nP + stride - 1) / stride;
-  const int chunks = (nv + kClsChunk - 1) / kClsChunk;
+  // a listed hypothesis's undecided points wait for each other's searches: short
+  // chunks while there are few
+  int chunk = kClsChunk;
+  if (list)
+    while (chunk > kClsThreads && (int64_t)nh * ((nv + chunk - 1) / chunk) < 8 * (int64_t)gridDim.x) chunk >>= 1;
+  const int chunks = (nv + chunk - 1) / chunk;
   const int64_t items = (int64_t)nh * chunks;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const bool abandon = c0 != nullptr;
@@ -256,7 +261,9 @@ __global__ void __launch_bounds__(kClsThreads, kClsMinBlocks) k_consensus_count(
   int64_t major = (int64_t)blockIdx.x / inner, minor = (int64_t)blockIdx.x % inner;
   const int64_t step_major = (int64_t)gridDim.x / inner, step_minor = (int64_t)gridDim.x % inner;
   for (int64_t item = blockIdx.x; item < items; item += gridDim.x) {
-    const int s = (int)(abandon ? minor : major), ch = (int)(abandon ? major : minor);
+    int s = (int)(abandon ? minor : major);
+    const int ch = (int)(abandon ? major : minor);
+    if (list) s = list[s];
     major += step_major, minor += step_minor;
     if (minor >= inner) minor -= inner, ++major;
     if (ok && !ok[s]) continue;
@@ -274,7 +281,7 @@ __global__ void __launch_bounds__(kClsThreads, kClsMinBlocks) k_consensus_count(
     }
     Rigid12 T;
     T.load(pose + (size_t)s * 12);
-    const int i0 = ch * kClsChunk, i1 = min(nv, (ch + 1) * kClsChunk);
+    const int i0 = ch * chunk, i1 = min(nv, (ch + 1) * chunk);
     int cnt = 0, namb = 0, nin = 0;
     for (int r = i0; r < i1; r += kClsThreads) {
       const int i = r + threadIdx.x;
@@ -458,21 +465,18 @@ __device__ __forceinline__ int group_points(const GroupParams &g, const unsigned
 }
 
 // A block per hypothesis, a thread per group at a time: up[s] = the points of
-// its groups that are not far. ok2: those whose up reaches c0; the others get
-// it in amb.
+// its groups that are not far. Those whose up reaches c0 are listed (in no
+// particular order); the others get it in amb.
 __global__ void __launch_bounds__(256) k_group_bounds(const GroupParams *gp, const float4 *__restrict__ grp,
                                                       const unsigned *__restrict__ near, const float *__restrict__ pose,
                                                       const uint8_t *__restrict__ ok, const int *n_dev, const int *c0,
-                                                      int *__restrict__ amb, uint8_t *__restrict__ ok2,
-                                                      int *__restrict__ up) {
+                                                      int *__restrict__ amb, int *__restrict__ up,
+                                                      int *__restrict__ list, int *__restrict__ n_list) {
   const GroupParams g = *gp;
   const int nh = *n_dev, bar = *c0;
   __shared__ int s_sum[8];
   for (int s = blockIdx.x; s < nh; s += gridDim.x) {
-    if (!ok[s]) {
-      if (threadIdx.x == 0) ok2[s] = 0;
-      continue;
-    }
+    if (!ok[s]) continue;
     Rigid12 T;
     T.load(pose + (size_t)s * 12);
     int sum = 0;
@@ -485,19 +489,22 @@ __global__ void __launch_bounds__(256) k_group_bounds(const GroupParams *gp, con
       int all = 0;
       for (int k = 0; k < 8; ++k) all += s_sum[k];
       up[s] = all;
-      ok2[s] = all >= bar;
       if (all < bar) amb[s] = all;
+      else list[atomicAdd(n_list, 1)] = s;
     }
     __syncthreads();
   }
 }
 
-// k_consensus_count over the points of the groups that are not far, with c0 and
-// prog: items (hypothesis, run of groups) in the order of the runs. What is
-// left of a hypothesis is bounded by up (the bounds pass; ub_lo + ub_extra for
-// the exact counts) less that of the runs done (prog's high word), so it is
-// given up on after a fraction of its points: with whole chunks and nP for up
-// nine in ten points of 9k hypotheses were read (3.5 ms for 200k points).
+// Counts over the points of the groups that are not far (as k_consensus_count),
+// of the listed hypotheses. A hypothesis's groups are split into as many
+// stretches as give every block about two items; a block takes a stretch in runs
+// of about kClsChunk points and adds each to prog[s] (up of the runs done << 32 |
+// their count), until what is left of the hypothesis, bounded by up (the bounds
+// pass; ub_lo + ub_extra for the exact counts) less that of the runs done, can no
+// longer reach c0. With items of one chunk over all survivors most of the time
+// went into deciding to skip them, and with nP for up nine in ten points of 9k
+// hypotheses were read (3.5 ms for 200k points).
 constexpr int kGrpBatch = 128;  // groups whose points are listed at once
 template <bool kBounds>
 __global__ void __launch_bounds__(kClsThreads, 6) k_group_count(
@@ -505,46 +512,40 @@ __global__ void __launch_bounds__(kClsThreads, 6) k_group_count(
     const int *__restrict__ first, const unsigned *__restrict__ far_bits, const ClsParams *__restrict__ cpp,
     const unsigned *__restrict__ in_bits, const unsigned *__restrict__ near_bits, const GridParams *__restrict__ gep,
     const int *__restrict__ start, const float4 *__restrict__ Xe, const float *__restrict__ pose,
-    const uint8_t *__restrict__ ok, const int *n_dev, float eps2, int *__restrict__ count, int *__restrict__ amb_count,
+    const int *__restrict__ list, const int *n_list, float eps2, int *__restrict__ count, int *__restrict__ amb_count,
     const int *c0, unsigned long long *prog, const int *__restrict__ ub_lo, const int *__restrict__ ub_extra) {
   __shared__ int s_pts[kGrpBatch * kGrpMost];
   __shared__ int s_cnt[kClsThreads / 32], s_amb[kClsThreads / 32], s_in[kClsThreads / 32], s_skip, s_n;
   const ClsParams c = *cpp;
   const GroupParams gr = *gp;
   const GridParams g = kBounds ? GridParams{} : *gep;
-  const int nh = *n_dev, cbar = *c0;
-  // runs of about kClsChunk points
+  const int nh = *n_list;
+  const long long cbar = *c0;
+  if (nh <= 0 || gr.n <= 0) return;
   const int run = max(1, min(16, (int)((long long)kClsChunk * gr.n / nP / kGrpBatch))) * kGrpBatch;
   const int runs = (gr.n + run - 1) / run;
+  const int parts = max(1, min(runs, (int)(2 * (int64_t)gridDim.x / nh)));
+  const int stretch = (runs + parts - 1) / parts * run;  // groups
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  if (nh <= 0) return;
-  const int64_t items = (int64_t)nh * runs;
-  int64_t major = (int64_t)blockIdx.x / nh, minor = (int64_t)blockIdx.x % nh;
-  const int64_t step_major = (int64_t)gridDim.x / nh, step_minor = (int64_t)gridDim.x % nh;
+  const int64_t items = (int64_t)nh * parts;
   for (int64_t item = blockIdx.x; item < items; item += gridDim.x) {
-    const int s = (int)minor, k0 = (int)major * run;
-    major += step_major, minor += step_minor;
-    if (minor >= nh) minor -= nh, ++major;
-    if (!ok[s]) continue;
+    const int s = list[item % nh], s0 = (int)(item / nh) * stretch, s1 = min(gr.n, s0 + stretch);
+    const long long up = kBounds ? (long long)ub_lo[s] : (long long)ub_lo[s] + (long long)ub_extra[s];
     // (one thread reads the pair, so the whole block takes one decision)
     if (threadIdx.x == 0) {
       const unsigned long long pv = __ldcg(prog + s);
-      const long long lo32 = (long long)(unsigned)pv, hi32 = (long long)(pv >> 32);
-      const long long up = kBounds ? (long long)ub_lo[s] : (long long)ub_lo[s] + (long long)ub_extra[s];
-      s_skip = lo32 + (up - hi32) < (long long)cbar;
+      s_skip = (long long)(unsigned)pv + (up - (long long)(pv >> 32)) < cbar;
       s_n = 0;
     }
     __syncthreads();
-    const bool skip = s_skip != 0;
-    __syncthreads();
-    if (skip) continue;
     Rigid12 T;
     T.load(pose + (size_t)s * 12);
+    for (int k0 = s0; k0 < s1 && !s_skip; k0 += run) {
     int cnt = 0, namb = 0, nin = 0, left = 0;
-    for (int b0 = k0; b0 < min(gr.n, k0 + run); b0 += kGrpBatch) {
+    for (int b0 = k0; b0 < min(s1, k0 + run); b0 += kGrpBatch) {
       // the points of the batch's groups that are not far
       const int k = b0 + threadIdx.x;
-      if (threadIdx.x < kGrpBatch && k < gr.n) {
+      if (threadIdx.x < kGrpBatch && k < s1) {
         const int m = group_points(gr, far_bits, grp[k], T);
         if (m > 0) {
           const int at = atomicAdd(&s_n, m), f = first[k];
@@ -602,42 +603,37 @@ __global__ void __launch_bounds__(kClsThreads, 6) k_group_count(
       for (int k = 0; k < kClsThreads / 32; ++k) tc += s_cnt[k], ta += s_amb[k], ti += s_in[k];
       if (tc) atomicAdd(&count[s], tc);
       if (kBounds && ta) atomicAdd(&amb_count[s], ta);
-      atomicAdd(prog + s, kBounds ? ((unsigned long long)left << 32) | (unsigned)(tc + ta)
-                                  : ((unsigned long long)(ti + ta) << 32) | (unsigned)tc);
+      const unsigned long long add = kBounds ? ((unsigned long long)left << 32) | (unsigned)(tc + ta)
+                                             : ((unsigned long long)(ti + ta) << 32) | (unsigned)tc;
+      const unsigned long long pv = atomicAdd(prog + s, add) + add;
+      s_skip = (long long)(unsigned)pv + (up - (long long)(pv >> 32)) < cbar;
     }
     __syncthreads();
+    }
+    __syncthreads();  // s_skip has been read
   }
 }
 
 // After the bounds pass: amb[s] += the points of s left out, so that IN + amb
 // stays an upper bound of the count (below c0 for those left out).
-__global__ void k_bounds_finish(const unsigned long long *__restrict__ prog, const uint8_t *__restrict__ ok,
-                                const int *n_dev, const int *__restrict__ up, int *__restrict__ amb) {
-  const int n = *n_dev;
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
-    if (!ok[k]) continue;
+__global__ void k_bounds_finish(const unsigned long long *__restrict__ prog, const int *__restrict__ list,
+                                const int *n_list, const int *__restrict__ up, int *__restrict__ amb) {
+  const int n = *n_list;
+  for (int u = blockIdx.x * blockDim.x + threadIdx.x; u < n; u += gridDim.x * blockDim.x) {
+    const int k = list[u];
     const int done = (int)(prog[k] >> 32);
     if (done < up[k]) amb[k] += up[k] - done;
   }
 }
 
-// out = the largest exact[k] over sel[k] (0 if none): a count some hypothesis
-// reaches, so no smaller upper bound can win.
-__global__ void __launch_bounds__(1024) k_sel_max(const int *__restrict__ exact, const uint8_t *__restrict__ sel,
-                                                  const int *n_dev, int *out) {
-  __shared__ int s_max[32];
-  const int n = *n_dev;
+// out = the largest exact[k] over the listed k (0 if none): a count some
+// hypothesis reaches, so no smaller upper bound can win.
+__global__ void k_sel_max(const int *__restrict__ exact, const int *__restrict__ list, const int *n_list, int *out) {
+  const int n = *n_list;
   int mx = 0;
-  for (int k = threadIdx.x; k < n; k += blockDim.x)
-    if (sel[k]) mx = max(mx, exact[k]);
-  for (int off = 16; off > 0; off >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-  if ((threadIdx.x & 31) == 0) s_max[threadIdx.x >> 5] = mx;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int m = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) m = max(m, s_max[w]);
-    *out = m;
-  }
+  for (int k = threadIdx.x; k < n; k += 32) mx = max(mx, exact[list[k]]);
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  if (threadIdx.x == 0) *out = mx;
 }
 
 // One block: L = the maximum of lo over the ok hypotheses, then
@@ -649,8 +645,11 @@ __global__ void __launch_bounds__(1024) k_reach_mask(const int *__restrict__ lo,
   __shared__ int s_max[32];
   const int n = *n_dev;
   int mx = 0;
-  for (int k = threadIdx.x; k < n; k += blockDim.x)
-    if (!ok || ok[k]) mx = max(mx, lo[k]);
+#pragma unroll 4
+  for (int k = threadIdx.x; k < n; k += blockDim.x) {
+    const int v = lo[k];
+    mx = max(mx, !ok || ok[k] ? v : 0);
+  }
   for (int off = 16; off > 0; off >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, off));
   if ((threadIdx.x & 31) == 0) s_max[threadIdx.x >> 5] = mx;
   __syncthreads();
@@ -682,83 +681,118 @@ __global__ void __launch_bounds__(1024) k_reach_mask(const int *__restrict__ lo,
 }
 
 // One block: the K ok hypotheses with the largest lo + extra (ties to the
-// smaller index), marked in sel (cleared first), by K rounds of block argmax.
+// smaller index), marked in sel and listed. The K-th largest key is found by
+// radix selection, eight bits at a time from the top; bytes that all keys share
+// are skipped (half of them: their one bin took every thread's atomic add in
+// turn), and the bins are counted in copies and scanned by a warp.
 __global__ void __launch_bounds__(1024) k_top_upper(const int *__restrict__ lo, const int *__restrict__ extra,
                                                     const uint8_t *__restrict__ ok, const int *n_dev, int K,
-                                                    uint8_t *__restrict__ sel) {
+                                                    uint8_t *__restrict__ sel, int *__restrict__ list,
+                                                    int *__restrict__ n_list) {
   // key: upper bound in the high word, complemented index in the low word,
-  // so keys are distinct and a larger key wins (ties to the smaller index).
-  // The K-th largest key T is found by radix selection, eight bits at a time
-  // from the top; the K keys >= T are then marked.
-  __shared__ unsigned hist[256];
-  __shared__ unsigned long long s_prefix, s_mask;
+  // so keys are distinct and a larger key wins (ties to the smaller index)
+  constexpr int kCopies = 8;
+  __shared__ unsigned hist[kCopies][256];
+  __shared__ unsigned long long s_prefix, s_and, s_or;
   __shared__ unsigned s_need, s_nok;
-  const int n = *n_dev;
+  __shared__ int s_list;
+  const int n = *n_dev, lane = threadIdx.x & 31;
   auto key_of = [&](int k) {
     return ((unsigned long long)(unsigned)(lo[k] + extra[k]) << 32) | (unsigned)(0x7fffffff - k);
   };
-  if (threadIdx.x == 0) s_nok = 0, s_prefix = 0ull, s_mask = 0ull, s_need = (unsigned)K;
+  if (threadIdx.x == 0) s_nok = 0, s_prefix = 0ull, s_and = ~0ull, s_or = 0ull, s_need = (unsigned)K, s_list = 0;
   __syncthreads();
   unsigned mine = 0;
-  for (int k = threadIdx.x; k < n; k += blockDim.x) mine += (!ok || ok[k]) ? 1u : 0u;
-  atomicAdd(&s_nok, mine);
-  __syncthreads();
-  if (s_nok <= (unsigned)K) {  // every candidate is selected
-    for (int k = threadIdx.x; k < n; k += blockDim.x) sel[k] = (!ok || ok[k]) ? 1 : 0;
-    return;
+  unsigned long long both = ~0ull, any = 0ull;
+#pragma unroll 4
+  for (int k = threadIdx.x; k < n; k += blockDim.x) {
+    const unsigned long long key = key_of(k);
+    const bool o = !ok || ok[k];
+    mine += o ? 1u : 0u;
+    both &= o ? key : ~0ull, any |= o ? key : 0ull;
   }
-  for (int shift = 56; shift >= 0; shift -= 8) {
-    for (int d = threadIdx.x; d < 256; d += blockDim.x) hist[d] = 0u;
+  if (mine) {
+    atomicAdd(&s_nok, mine);
+    atomicAnd(&s_and, both);
+    atomicOr(&s_or, any);
+  }
+  __syncthreads();
+  const bool all = s_nok <= (unsigned)K;  // every candidate is selected
+  unsigned long long mask = 0ull;
+  const unsigned long long common = s_and, differ = s_and ^ s_or;
+  for (int shift = 56; shift >= 0 && !all; shift -= 8) {
+    const unsigned long long prefix = s_prefix;
+    if (!((differ >> shift) & 255u)) {
+      __syncthreads();
+      if (threadIdx.x == 0) s_prefix = prefix | (common & (255ull << shift));
+      mask |= 255ull << shift;
+      __syncthreads();
+      continue;
+    }
+    for (int d = threadIdx.x; d < kCopies * 256; d += blockDim.x) hist[0][d] = 0u;
     __syncthreads();
-    const unsigned long long prefix = s_prefix, mask = s_mask;
+    unsigned *h = hist[(threadIdx.x >> 5) % kCopies];
+#pragma unroll 4
     for (int k = threadIdx.x; k < n; k += blockDim.x) {
-      if (ok && !ok[k]) continue;
       const unsigned long long key = key_of(k);
-      if ((key & mask) == prefix) atomicAdd(&hist[(key >> shift) & 255u], 1u);
+      const bool o = !ok || ok[k];
+      if (o && (key & mask) == prefix) atomicAdd(h + ((key >> shift) & 255u), 1u);
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-      unsigned need = s_need, above = 0u;
-      int d = 255;
-      for (; d > 0; --d) {
-        if (above + hist[d] >= need) break;
-        above += hist[d];
+    if (threadIdx.x < 32) {
+      // lane: bins 8 (31 - lane) .. + 7, so that the larger come first
+      unsigned c[8], sum = 0u;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        c[u] = 0u;
+        for (int r = 0; r < kCopies; ++r) c[u] += hist[r][8 * (31 - lane) + 7 - u];
+        sum += c[u];
       }
-      s_need = need - above;
-      s_prefix = prefix | ((unsigned long long)d << shift);
-      s_mask = mask | (255ull << shift);
+      unsigned end = sum;
+#pragma unroll
+      for (int off = 1; off < 32; off <<= 1) {
+        const unsigned o = __shfl_up_sync(0xffffffffu, end, off);
+        if (lane >= off) end += o;
+      }
+      unsigned above = end - sum;
+      const unsigned need = s_need;
+      __syncwarp();
+      if (above < need && need <= end) {
+        for (int u = 0; u < 8; ++u) {
+          if (need <= above + c[u]) {
+            s_need = need - above;
+            s_prefix = prefix | ((unsigned long long)(8 * (31 - lane) + 7 - u) << shift);
+            break;
+          }
+          above += c[u];
+        }
+      }
     }
+    mask |= 255ull << shift;
     __syncthreads();
   }
   const unsigned long long T = s_prefix;
-  for (int k = threadIdx.x; k < n; k += blockDim.x) sel[k] = ((!ok || ok[k]) && key_of(k) >= T) ? 1 : 0;
-}
-
-// One block: C = the maximum exact count among sel; then
-// rest[k] = ok[k] && !sel[k] && lo[k] + extra[k] >= C and all[k] = sel[k] | rest[k].
-__global__ void __launch_bounds__(1024) k_reach_rest(const int *__restrict__ lo, const int *__restrict__ extra,
-                                                     const int *__restrict__ exact, const uint8_t *__restrict__ sel,
-                                                     const uint8_t *__restrict__ ok, const int *n_dev,
-                                                     uint8_t *__restrict__ rest, uint8_t *__restrict__ all) {
-  __shared__ int s_max[32];
-  const int n = *n_dev;
-  int mx = 0;
-  for (int k = threadIdx.x; k < n; k += blockDim.x)
-    if (sel[k]) mx = max(mx, exact[k]);
-  for (int off = 16; off > 0; off >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-  if ((threadIdx.x & 31) == 0) s_max[threadIdx.x >> 5] = mx;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int m = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) m = max(m, s_max[w]);
-    s_max[0] = m;
+#pragma unroll 4
+  for (int k = threadIdx.x; k < n; k += blockDim.x) {
+    const bool in = (!ok || ok[k]) && (all || key_of(k) >= T);
+    sel[k] = in ? 1 : 0;
+    if (in) list[atomicAdd(&s_list, 1)] = k;
   }
   __syncthreads();
-  mx = s_max[0];
-  for (int k = threadIdx.x; k < n; k += blockDim.x) {
-    const bool r = (!ok || ok[k]) && !sel[k] && lo[k] + extra[k] >= mx;
-    rest[k] = r ? 1 : 0;
-    all[k] = (r || sel[k]) ? 1 : 0;
+  if (threadIdx.x == 0) *n_list = s_list;
+}
+
+// rest: the ok hypotheses outside sel with lo + extra >= *c0, listed;
+// all[k] = k is in sel or rest.
+__global__ void k_reach_rest(const int *__restrict__ lo, const int *__restrict__ extra, const int *c0,
+                             const uint8_t *__restrict__ sel, const uint8_t *__restrict__ ok, const int *n_dev,
+                             uint8_t *__restrict__ all, int *__restrict__ list, int *__restrict__ n_list) {
+  const int n = *n_dev, mx = *c0;
+  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+    const int up = lo[k] + extra[k];
+    const bool top = sel[k] != 0, r = (!ok || ok[k]) && !top && up >= mx;
+    if (r) list[atomicAdd(n_list, 1)] = k;
+    all[k] = (r || top) ? 1 : 0;
   }
 }
 
@@ -775,22 +809,12 @@ cudaError_t launch_cls_build(const float *boxQ, float eps, const float4 *XQ, int
 
 cudaError_t launch_consensus_count(const float4 *XP, int nP, const ClsParams *cp, const unsigned *in_bits,
                                    const unsigned *near_bits, const GridParams *ge, const int *start_e,
-                                   const float4 *Xe, const float *pose, const uint8_t *ok, const int *n_dev,
-                                   int n_host, float eps, int *count, cudaStream_t s) {
+                                   const float4 *Xe, const float *pose, const int *list, const int *n_list, float eps,
+                                   int *count, const int *c0, const int *ub_lo, const int *ub_extra,
+                                   unsigned long long *prog, cudaStream_t s) {
   LSR_LAUNCH(k_consensus_count<false><<<kSms * 8, kClsThreads, 0, s>>>(XP, nP, 1, cp, in_bits, near_bits, ge, start_e,
-                                                                       Xe, pose, ok, n_dev, n_host, eps * eps, count,
-                                                                       nullptr, nullptr, nullptr, nullptr, nullptr));
-  return cudaGetLastError();
-}
-
-cudaError_t launch_consensus_count_bar(const float4 *XP, int nP, const ClsParams *cp, const unsigned *in_bits,
-                                       const unsigned *near_bits, const GridParams *ge, const int *start_e,
-                                       const float4 *Xe, const float *pose, const uint8_t *ok, const int *n_dev,
-                                       float eps, int *count, const int *c0, const int *ub_lo, const int *ub_extra,
-                                       unsigned long long *prog, cudaStream_t s) {
-  LSR_LAUNCH(k_consensus_count<false><<<kSms * 8, kClsThreads, 0, s>>>(XP, nP, 1, cp, in_bits, near_bits, ge, start_e,
-                                                                       Xe, pose, ok, n_dev, 0, eps * eps, count,
-                                                                       nullptr, c0, prog, ub_lo, ub_extra));
+                                                                       Xe, pose, nullptr, n_list, 0, eps * eps, count,
+                                                                       nullptr, c0, prog, ub_lo, ub_extra, list));
   return cudaGetLastError();
 }
 
@@ -801,7 +825,7 @@ cudaError_t launch_consensus_bounds(const float4 *XP, int nP, int stride, const 
   LSR_LAUNCH(k_consensus_count<true><<<kSms * 8, kClsThreads, 0, s>>>(XP, nP, stride, cp, in_bits, near_bits, nullptr,
                                                                       nullptr, nullptr, pose, ok, n_dev, 0, 0.f,
                                                                       in_count, amb_count, nullptr, nullptr, nullptr,
-                                                                      nullptr));
+                                                                      nullptr, nullptr));
   return cudaGetLastError();
 }
 
@@ -822,41 +846,43 @@ cudaError_t launch_group_bounds(const Groups &G, const float4 *Xn, int nP, const
                                 int *in_count, int *amb_count, const int *c0, unsigned long long *prog,
                                 cudaStream_t s) {
   const unsigned *far_bits = G.words + kGrpCapWords;
-  LSR_LAUNCH(k_group_bounds<<<kSms * 8, 256, 0, s>>>(G.p, G.grp, far_bits, pose, ok, n_dev, c0, amb_count, G.ok, G.up));
+  LSR_LAUNCH(k_group_bounds<<<kSms * 8, 256, 0, s>>>(G.p, G.grp, far_bits, pose, ok, n_dev, c0, amb_count, G.up, G.list,
+                                                     &G.p->left));
   LSR_LAUNCH(k_group_count<true><<<kSms * 6, kClsThreads, 0, s>>>(Xn, nP, G.p, G.grp, G.first, far_bits, cp, in_bits,
-                                                                  near_bits, nullptr, nullptr, nullptr, pose, G.ok,
-                                                                  n_dev, 0.f, in_count, amb_count, c0, prog, G.up,
+                                                                  near_bits, nullptr, nullptr, nullptr, pose, G.list,
+                                                                  &G.p->left, 0.f, in_count, amb_count, c0, prog, G.up,
                                                                   nullptr));
-  LSR_LAUNCH(k_bounds_finish<<<kSms * 2, 256, 0, s>>>(prog, G.ok, n_dev, G.up, amb_count));
+  LSR_LAUNCH(k_bounds_finish<<<kSms * 2, 256, 0, s>>>(prog, G.list, &G.p->left, G.up, amb_count));
   return cudaGetLastError();
 }
 
 cudaError_t launch_group_count_bar(const Groups &G, const float4 *Xn, int nP, const ClsParams *cp,
                                    const unsigned *in_bits, const unsigned *near_bits, const GridParams *ge,
-                                   const int *start_e, const float4 *Xe, const float *pose, const uint8_t *ok,
-                                   const int *n_dev, float eps, int *count, const int *c0, const int *ub_lo,
+                                   const int *start_e, const float4 *Xe, const float *pose, const int *list,
+                                   const int *n_list, float eps, int *count, const int *c0, const int *ub_lo,
                                    const int *ub_extra, unsigned long long *prog, cudaStream_t s) {
   LSR_LAUNCH(k_group_count<false><<<kSms * 6, kClsThreads, 0, s>>>(Xn, nP, G.p, G.grp, G.first, G.words + kGrpCapWords,
-                                                                   cp, in_bits, near_bits, ge, start_e, Xe, pose, ok,
-                                                                   n_dev, eps * eps, count, nullptr, c0, prog, ub_lo,
+                                                                   cp, in_bits, near_bits, ge, start_e, Xe, pose, list,
+                                                                   n_list, eps * eps, count, nullptr, c0, prog, ub_lo,
                                                                    ub_extra));
   return cudaGetLastError();
 }
 
-cudaError_t launch_sel_max(const int *exact, const uint8_t *sel, const int *n_dev, int *out, cudaStream_t s) {
-  LSR_LAUNCH(k_sel_max<<<1, 1024, 0, s>>>(exact, sel, n_dev, out));
+cudaError_t launch_sel_max(const int *exact, const int *list, const int *n_list, int *out, cudaStream_t s) {
+  LSR_LAUNCH(k_sel_max<<<1, 32, 0, s>>>(exact, list, n_list, out));
   return cudaGetLastError();
 }
 
 cudaError_t launch_top_upper(const int *lo, const int *extra, const uint8_t *ok, const int *n_dev, int K,
-                             uint8_t *sel, cudaStream_t s) {
-  LSR_LAUNCH(k_top_upper<<<1, 1024, 0, s>>>(lo, extra, ok, n_dev, K, sel));
+                             uint8_t *sel, int *list, int *n_list, cudaStream_t s) {
+  LSR_LAUNCH(k_top_upper<<<1, 1024, 0, s>>>(lo, extra, ok, n_dev, K, sel, list, n_list));
   return cudaGetLastError();
 }
 
-cudaError_t launch_reach_rest(const int *lo, const int *extra, const int *exact, const uint8_t *sel, const uint8_t *ok,
-                              const int *n_dev, uint8_t *rest, uint8_t *all, cudaStream_t s) {
-  LSR_LAUNCH(k_reach_rest<<<1, 1024, 0, s>>>(lo, extra, exact, sel, ok, n_dev, rest, all));
+cudaError_t launch_reach_rest(const int *lo, const int *extra, const int *c0, const uint8_t *sel, const uint8_t *ok,
+                              const int *n_dev, uint8_t *all, int *list, int *n_list, cudaStream_t s) {
+  LSR_CUDA_TRY(cudaMemsetAsync(n_list, 0, sizeof(int), s));
+  LSR_LAUNCH(k_reach_rest<<<kSms, 256, 0, s>>>(lo, extra, c0, sel, ok, n_dev, all, list, n_list));
   return cudaGetLastError();
 }
 

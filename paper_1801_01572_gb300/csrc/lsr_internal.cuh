@@ -701,7 +701,7 @@ constexpr int kClsCapWords = 1 << 23;  // words per bit-set (32 MB)
 struct GroupParams {
   float ox, oy, oz, inv_h, rmax, r2;  // rmax: largest group radius; r2: the reach squared, in voxels
   int nx, ny, nz, wx;                 // voxels, words of a row
-  int usable, n;                      // n: the groups
+  int usable, n, left;                // n: the groups; left: the hypotheses listed
 };
 constexpr int kGrpCapWords = 1 << 20;
 struct Groups {
@@ -710,15 +710,20 @@ struct Groups {
   int *first = nullptr;       // nP: its first point
   unsigned *words = nullptr;  // 2 kGrpCapWords: Q's voxels, those within reach
   int *up = nullptr;          // per hypothesis: the points of the groups that are not far
-  uint8_t *ok = nullptr;      // those whose up reaches c0
+  int *list = nullptr;        // those whose up reaches c0
 };
 cudaError_t launch_cls_build(const float *boxQ, float eps, const float4 *XQ, int nQ, ClsParams *cp, unsigned *in_bits,
                              unsigned *near_bits, cudaStream_t s);
-// Inlier counts (as launch_consensus, without the distance sums).
+// Inlier counts (as launch_consensus, without the distance sums) of the
+// hypotheses list[0 .. *n_list), count += ...; with c0 (device; else null) it
+// gives up on a hypothesis as soon as its count can no longer reach *c0, from
+// the upper bounds ub_lo + ub_extra of a bounds pass (prog: one zeroed 64-bit word
+// per hypothesis). A count given up on stays partial and below c0.
 cudaError_t launch_consensus_count(const float4 *XP, int nP, const ClsParams *cp, const unsigned *in_bits,
                                    const unsigned *near_bits, const GridParams *ge, const int *start_e,
-                                   const float4 *Xe, const float *pose, const uint8_t *ok, const int *n_dev,
-                                   int n_host, float eps, int *count, cudaStream_t s);
+                                   const float4 *Xe, const float *pose, const int *list, const int *n_list, float eps,
+                                   int *count, const int *c0, const int *ub_lo, const int *ub_extra,
+                                   unsigned long long *prog, cudaStream_t s);
 // Bounds without exact tests over the points XP[v * stride]: in_count =
 // points in IN voxels (a lower bound of the inlier count), amb_count = points
 // in undecided voxels.
@@ -726,15 +731,6 @@ cudaError_t launch_consensus_bounds(const float4 *XP, int nP, int stride, const 
                                     const unsigned *in_bits, const unsigned *near_bits, const float *pose,
                                     const uint8_t *ok, const int *n_dev, int *in_count, int *amb_count,
                                     cudaStream_t s);
-// Exact counts (count += ...) that give up on a hypothesis as soon as its
-// count can no longer reach c0 (device), from the upper bounds ub_lo + ub_extra
-// of a bounds pass; prog: one zeroed 64-bit word per hypothesis. A count given
-// up on stays partial and below c0.
-cudaError_t launch_consensus_count_bar(const float4 *XP, int nP, const ClsParams *cp, const unsigned *in_bits,
-                                       const unsigned *near_bits, const GridParams *ge, const int *start_e,
-                                       const float4 *Xe, const float *pose, const uint8_t *ok, const int *n_dev,
-                                       float eps, int *count, const int *c0, const int *ub_lo, const int *ub_extra,
-                                       unsigned long long *prog, cudaStream_t s);
 // The groups of P (its normal grid) and the bit-set of Q.
 cudaError_t launch_group_build(const float4 *Xn, int nP, const GridParams *gn, const int *start_n, float r_normal,
                                const float *boxQ, float eps, const float4 *XQ, int nQ, const Groups &G, cudaStream_t s);
@@ -745,22 +741,21 @@ cudaError_t launch_group_build(const float4 *Xn, int nP, const GridParams *gn, c
 cudaError_t launch_group_bounds(const Groups &G, const float4 *Xn, int nP, const ClsParams *cp, const unsigned *in_bits,
                                 const unsigned *near_bits, const float *pose, const uint8_t *ok, const int *n_dev,
                                 int *in_count, int *amb_count, const int *c0, unsigned long long *prog, cudaStream_t s);
-// launch_consensus_count_bar after launch_group_bounds (whose upper bounds leave
+// launch_consensus_count with c0 after launch_group_bounds (whose upper bounds leave
 // out the far groups, so the exact counts have to as well).
 cudaError_t launch_group_count_bar(const Groups &G, const float4 *Xn, int nP, const ClsParams *cp,
                                    const unsigned *in_bits, const unsigned *near_bits, const GridParams *ge,
-                                   const int *start_e, const float4 *Xe, const float *pose, const uint8_t *ok,
-                                   const int *n_dev, float eps, int *count, const int *c0, const int *ub_lo,
+                                   const int *start_e, const float4 *Xe, const float *pose, const int *list,
+                                   const int *n_list, float eps, int *count, const int *c0, const int *ub_lo,
                                    const int *ub_extra, unsigned long long *prog, cudaStream_t s);
-// out (device) = max over sel of exact.
-cudaError_t launch_sel_max(const int *exact, const uint8_t *sel, const int *n_dev, int *out, cudaStream_t s);
-// sel: the K ok hypotheses with the largest lo + extra (ties to the smaller id).
+// out (device) = max over the list of exact.
+cudaError_t launch_sel_max(const int *exact, const int *list, const int *n_list, int *out, cudaStream_t s);
+// sel, list: the K ok hypotheses with the largest lo + extra (ties to the smaller id).
 cudaError_t launch_top_upper(const int *lo, const int *extra, const uint8_t *ok, const int *n_dev, int K,
-                             uint8_t *sel, cudaStream_t s);
-// With C = max over sel of exact: rest = ok && !sel && lo + extra >= C, and
-// all = sel | rest.
-cudaError_t launch_reach_rest(const int *lo, const int *extra, const int *exact, const uint8_t *sel, const uint8_t *ok,
-                              const int *n_dev, uint8_t *rest, uint8_t *all, cudaStream_t s);
+                             uint8_t *sel, int *list, int *n_list, cudaStream_t s);
+// list: the ok hypotheses outside sel with lo + extra >= *c0; all: those and sel.
+cudaError_t launch_reach_rest(const int *lo, const int *extra, const int *c0, const uint8_t *sel, const uint8_t *ok,
+                              const int *n_dev, uint8_t *all, int *list, int *n_list, cudaStream_t s);
 // With L = max over ok of lo: mask[k] = ok[k] && lo[k] + extra[k] >= L. If L is
 // 0: every ok hypothesis when extra is given, none otherwise.
 // n_mask, list (optional, device): the number of set entries and their indices.
