@@ -332,6 +332,7 @@ struct PairLayout {
   int *count2 = nullptr;     // exact counts of the reaching hypotheses
   int *tie_list = nullptr;   // the survivor slots tied at the top
   unsigned long long *prog = nullptr;  // per survivor: bounds progress (points done << 32 | IN + undecided)
+  float4 *sample = nullptr;  // every kConsensusPrepassStride-th point of P (large P)
   Groups far;                // groups of P that a hypothesis moves far from Q (large P)
   int *c0 = nullptr;         // an exact count reached by some survivor (the bounds pass's bar)
   // single-cell lattice of Q (lsr_params.nn_mode = LSR_NN_SINGLE_CELL)
@@ -386,6 +387,7 @@ void plan_pair(Arena &a, int nP, int nQ, bool stP, bool stQ, int64_t H, int leve
   L.prog = a.take<unsigned long long>(L.surv_cap);
   L.c0 = a.take<int>(1);
   if (nP >= kConsensusPrepassMin) {
+    L.sample = a.take<float4>((size_t)lsr_div_up(nP, kConsensusPrepassStride));
     L.far.p = a.take<GroupParams>(1);
     L.far.grp = a.take<float4>(nP);
     L.far.first = a.take<int>(nP);
@@ -837,9 +839,10 @@ int enqueue_pair(lsr_ctx *c, const PairLayout &L, const float *P, const float *Q
     // below c0 part-way (it can neither win nor tie).
     const bool prepass = nP >= kConsensusPrepassMin;
     if (prepass) {
+      TRY_CUDA(c, launch_point_sample(Pc.Xn, nP, kConsensusPrepassStride, L.sample, s), "sample");
       TRY_CUDA(c,
-               launch_consensus_bounds(Pc.Xn, nP, kConsensusPrepassStride, L.cls, L.in_bits, L.near_bits, L.pose, L.ok,
-                                       &L.st->n_surv, L.count, L.amb, s),
+               launch_consensus_bounds(L.sample, (int)lsr_div_up(nP, kConsensusPrepassStride), L.cls, L.in_bits,
+                                       L.near_bits, L.pose, L.ok, &L.st->n_surv, L.count, L.amb, s),
                "consensus estimate");
       TRY_CUDA(c, launch_top_upper(L.count, L.amb, L.ok, &L.st->n_surv, 32, L.sel, L.sel_list, L.n_sel, s), "top");
       TRY_CUDA(c,
@@ -859,7 +862,7 @@ int enqueue_pair(lsr_ctx *c, const PairLayout &L, const float *P, const float *Q
                "consensus bounds");
     } else {
       TRY_CUDA(c,
-               launch_consensus_bounds(Pc.Xn, nP, 1, L.cls, L.in_bits, L.near_bits, L.pose, L.ok, &L.st->n_surv,
+               launch_consensus_bounds(Pc.Xn, nP, L.cls, L.in_bits, L.near_bits, L.pose, L.ok, &L.st->n_surv,
                                        L.count, L.amb, s),
                "consensus bounds");
     }

@@ -222,8 +222,7 @@ __device__ __forceinline__ bool warp_any_within(const GridParams &g, const int *
 // One thread block per (hypothesis, chunk of P), as the exact kernel; a lane
 // per point. kBounds: count IN points into count and undecided ones into amb.
 // Otherwise the undecided lanes are resolved by the whole warp, one at a time,
-// and count receives the exact inlier count. The points are XP[v * stride]
-// for v < ceil(nP / stride).
+// and count receives the exact inlier count.
 // Exact counts with c0 (a device count no larger than the winning count, e.g. the
 // exact count of some hypothesis) and the upper bounds ub_lo + ub_extra of a
 // bounds pass: items run chunk-major, so each hypothesis's chunks come in order, prog[s] accumulates (IN + undecided of the chunks
@@ -233,7 +232,7 @@ __device__ __forceinline__ bool warp_any_within(const GridParams &g, const int *
 // count stays partial, below c0).
 template <bool kBounds>
 __global__ void __launch_bounds__(kClsThreads, kClsMinBlocks) k_consensus_count(
-    const float4 *__restrict__ XP, int nP, int stride, const ClsParams *__restrict__ cpp,
+    const float4 *__restrict__ XP, int nP, const ClsParams *__restrict__ cpp,
     const unsigned *__restrict__ in_bits, const unsigned *__restrict__ near_bits, const GridParams *__restrict__ gep,
     const int *__restrict__ start, const float4 *__restrict__ Xe, const float *__restrict__ pose,
     const uint8_t *__restrict__ ok, const int *n_dev, int n_host, float eps2, int *__restrict__ count,
@@ -242,13 +241,12 @@ __global__ void __launch_bounds__(kClsThreads, kClsMinBlocks) k_consensus_count(
   const ClsParams c = *cpp;
   const GridParams g = kBounds ? GridParams{} : *gep;
   const int nh = n_dev ? *n_dev : n_host;
-  const int nv = (nP + stride - 1) / stride;
   // a listed hypothesis's undecided points wait for each other's searches: short
   // chunks while there are few
   int chunk = kClsChunk;
   if (list)
-    while (chunk > kClsThreads && (int64_t)nh * ((nv + chunk - 1) / chunk) < 8 * (int64_t)gridDim.x) chunk >>= 1;
-  const int chunks = (nv + chunk - 1) / chunk;
+    while (chunk > kClsThreads && (int64_t)nh * ((nP + chunk - 1) / chunk) < 8 * (int64_t)gridDim.x) chunk >>= 1;
+  const int chunks = (nP + chunk - 1) / chunk;
   const int64_t items = (int64_t)nh * chunks;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const bool abandon = c0 != nullptr;
@@ -281,14 +279,14 @@ __global__ void __launch_bounds__(kClsThreads, kClsMinBlocks) k_consensus_count(
     }
     Rigid12 T;
     T.load(pose + (size_t)s * 12);
-    const int i0 = ch * chunk, i1 = min(nv, (ch + 1) * chunk);
+    const int i0 = ch * chunk, i1 = min(nP, (ch + 1) * chunk);
     int cnt = 0, namb = 0, nin = 0;
     for (int r = i0; r < i1; r += kClsThreads) {
       const int i = r + threadIdx.x;
       bool in = false, amb = false;
       float x = 0.f, y = 0.f, z = 0.f;
       if (i < i1) {
-        T.apply(XP[(size_t)i * stride], x, y, z);
+        T.apply(XP[i], x, y, z);
         if (c.all_amb) {
           amb = true;
         } else {
@@ -332,6 +330,12 @@ __global__ void __launch_bounds__(kClsThreads, kClsMinBlocks) k_consensus_count(
     }
     __syncthreads();
   }
+}
+
+// out[v] = XP[v * stride]: points read strided by every hypothesis took a sector each.
+__global__ void k_point_sample(const float4 *__restrict__ XP, int n, int stride, float4 *__restrict__ out) {
+  const int v = blockIdx.x * blockDim.x + threadIdx.x;
+  if (v < n) out[v] = XP[(size_t)v * stride];
 }
 
 // ---------------------------------------------------------------- far groups
@@ -497,69 +501,73 @@ __global__ void __launch_bounds__(256) k_group_bounds(const GroupParams *gp, con
 }
 
 // Counts over the points of the groups that are not far (as k_consensus_count),
-// of the listed hypotheses. A hypothesis's groups are split into as many
-// stretches as give every block about two items; a block takes a stretch in runs
-// of about kClsChunk points and adds each to prog[s] (up of the runs done << 32 |
-// their count), until what is left of the hypothesis, bounded by up (the bounds
-// pass; ub_lo + ub_extra for the exact counts) less that of the runs done, can no
-// longer reach c0. With items of one chunk over all survivors most of the time
-// went into deciding to skip them, and with nP for up nine in ten points of 9k
-// hypotheses were read (3.5 ms for 200k points).
-constexpr int kGrpBatch = 128;  // groups whose points are listed at once
+// of the listed hypotheses. An item is a hypothesis and a stretch of groups, all
+// first stretches before all second ones; a warp takes an item, looks 32 groups
+// up at a time, lists their points and tests those 32 at a time. What is left of
+// a hypothesis is bounded by its up (the bounds pass; ub_lo + ub_extra for the
+// exact counts) less that of what is done (prog[s]: up done << 32 | count, read
+// when the item begins, plus the warp's own), and the warp stops as soon as that
+// can no longer reach c0. Bound by the latency of the lookups. A block an item
+// spent most of its time at its barriers and on the way to prog and back (2.0 ms
+// for 9k hypotheses of 200k points); whole chunks over all survivors, with nP
+// for up, read nine in ten points (3.5 ms).
+constexpr int kGrpStretch = 256;  // groups of a stretch, or fewer
 template <bool kBounds>
 __global__ void __launch_bounds__(kClsThreads, 6) k_group_count(
-    const float4 *__restrict__ XP, int nP, const GroupParams *__restrict__ gp, const float4 *__restrict__ grp,
+    const float4 *__restrict__ XP, const GroupParams *__restrict__ gp, const float4 *__restrict__ grp,
     const int *__restrict__ first, const unsigned *__restrict__ far_bits, const ClsParams *__restrict__ cpp,
     const unsigned *__restrict__ in_bits, const unsigned *__restrict__ near_bits, const GridParams *__restrict__ gep,
     const int *__restrict__ start, const float4 *__restrict__ Xe, const float *__restrict__ pose,
     const int *__restrict__ list, const int *n_list, float eps2, int *__restrict__ count, int *__restrict__ amb_count,
     const int *c0, unsigned long long *prog, const int *__restrict__ ub_lo, const int *__restrict__ ub_extra) {
-  __shared__ int s_pts[kGrpBatch * kGrpMost];
-  __shared__ int s_cnt[kClsThreads / 32], s_amb[kClsThreads / 32], s_in[kClsThreads / 32], s_skip, s_n;
+  __shared__ int s_pts[kClsThreads / 32][32 * kGrpMost];
   const ClsParams c = *cpp;
   const GroupParams gr = *gp;
   const GridParams g = kBounds ? GridParams{} : *gep;
   const int nh = *n_list;
   const long long cbar = *c0;
   if (nh <= 0 || gr.n <= 0) return;
-  const int run = max(1, min(16, (int)((long long)kClsChunk * gr.n / nP / kGrpBatch))) * kGrpBatch;
-  const int runs = (gr.n + run - 1) / run;
-  const int parts = max(1, min(runs, (int)(2 * (int64_t)gridDim.x / nh)));
-  const int stretch = (runs + parts - 1) / parts * run;  // groups
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int64_t items = (int64_t)nh * parts;
-  for (int64_t item = blockIdx.x; item < items; item += gridDim.x) {
+  const int lane = threadIdx.x & 31;
+  int *pts = s_pts[threadIdx.x >> 5];
+  const int64_t warps = (int64_t)gridDim.x * (kClsThreads / 32);
+  // shorter stretches while there are few items a warp; the undecided points of
+  // an exact count wait for each other's searches, so those go down to four groups
+  // (32: 354 us for the 200k pair's, a block an item 103)
+  int stretch = kGrpStretch;
+  while (stretch > (kBounds ? 32 : 4) && (int64_t)nh * ((gr.n + stretch - 1) / stretch) < (kBounds ? 16 : 64) * warps)
+    stretch >>= 1;
+  const int64_t items = (int64_t)nh * ((gr.n + stretch - 1) / stretch);
+  for (int64_t item = (int64_t)blockIdx.x * (kClsThreads / 32) + (threadIdx.x >> 5); item < items; item += warps) {
     const int s = list[item % nh], s0 = (int)(item / nh) * stretch, s1 = min(gr.n, s0 + stretch);
+    const unsigned long long pv = __ldcg(prog + s);
     const long long up = kBounds ? (long long)ub_lo[s] : (long long)ub_lo[s] + (long long)ub_extra[s];
-    // (one thread reads the pair, so the whole block takes one decision)
-    if (threadIdx.x == 0) {
-      const unsigned long long pv = __ldcg(prog + s);
-      s_skip = (long long)(unsigned)pv + (up - (long long)(pv >> 32)) < cbar;
-      s_n = 0;
-    }
-    __syncthreads();
+    // the count so far and what the rest may add
+    const long long bound = (long long)(unsigned)pv + (up - (long long)(pv >> 32));
+    if (bound < cbar) continue;
     Rigid12 T;
     T.load(pose + (size_t)s * 12);
-    for (int k0 = s0; k0 < s1 && !s_skip; k0 += run) {
-    int cnt = 0, namb = 0, nin = 0, left = 0;
-    for (int b0 = k0; b0 < min(s1, k0 + run); b0 += kGrpBatch) {
-      // the points of the batch's groups that are not far
-      const int k = b0 + threadIdx.x;
-      if (threadIdx.x < kGrpBatch && k < s1) {
-        const int m = group_points(gr, far_bits, grp[k], T);
-        if (m > 0) {
-          const int at = atomicAdd(&s_n, m), f = first[k];
-          for (int u = 0; u < m; ++u) s_pts[at + u] = f + u;
-        }
+    int tin = 0, tamb = 0, hits = 0, left = 0;  // (the same on every lane)
+    for (int k0 = s0; k0 < s1; k0 += 32) {
+      const int k = k0 + lane;
+      const int m = k < s1 ? group_points(gr, far_bits, grp[k], T) : 0;
+      int end = m;
+#pragma unroll
+      for (int off = 1; off < 32; off <<= 1) {
+        const int o = __shfl_up_sync(0xffffffffu, end, off);
+        if (lane >= off) end += o;
       }
-      __syncthreads();
-      const int np = s_n;
+      const int np = __shfl_sync(0xffffffffu, end, 31);
+      if (m > 0) {
+        const int f = first[k];
+        for (int u = 0; u < m; ++u) pts[end - m + u] = f + u;
+      }
+      __syncwarp();
       left += np;
-      for (int r = 0; r < np; r += kClsThreads) {
+      for (int r = 0; r < np; r += 32) {
         bool in = false, amb = false;
         float x = 0.f, y = 0.f, z = 0.f;
-        if (r + (int)threadIdx.x < np) {
-          T.apply(XP[s_pts[r + threadIdx.x]], x, y, z);
+        if (r + lane < np) {
+          T.apply(XP[pts[r + lane]], x, y, z);
           if (c.all_amb) {
             amb = true;
           } else {
@@ -575,42 +583,28 @@ __global__ void __launch_bounds__(kClsThreads, 6) k_group_count(
             }
           }
         }
-        cnt += in;
-        nin += in;
-        namb += amb;
-        if (kBounds) continue;
         unsigned pend = __ballot_sync(0xffffffffu, amb);
+        tin += __popc(__ballot_sync(0xffffffffu, in));
+        tamb += __popc(pend);
+        if (kBounds) continue;
         while (pend) {
           const int src = __ffs(pend) - 1;
           pend &= pend - 1;
           const float qx = __shfl_sync(0xffffffffu, x, src), qy = __shfl_sync(0xffffffffu, y, src),
                       qz = __shfl_sync(0xffffffffu, z, src);
-          const bool hit = warp_any_within(g, start, Xe, qx, qy, qz, eps2);
-          if (lane == src) cnt += hit;
+          hits += warp_any_within(g, start, Xe, qx, qy, qz, eps2) ? 1 : 0;
         }
       }
-      __syncthreads();
-      if (threadIdx.x == 0) s_n = 0;
-      __syncthreads();
+      __syncwarp();  // pts is written again
+      if (bound - (kBounds ? left - tin - tamb : tamb - hits) < cbar) break;
     }
-    cnt = warp_sum(cnt);
-    namb = warp_sum(namb);
-    if (!kBounds) nin = warp_sum(nin);
-    if (lane == 0) s_cnt[w] = cnt, s_amb[w] = namb, s_in[w] = nin;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      int tc = 0, ta = 0, ti = 0;
-      for (int k = 0; k < kClsThreads / 32; ++k) tc += s_cnt[k], ta += s_amb[k], ti += s_in[k];
+    if (lane == 0) {
+      const int tc = tin + hits;
       if (tc) atomicAdd(&count[s], tc);
-      if (kBounds && ta) atomicAdd(&amb_count[s], ta);
-      const unsigned long long add = kBounds ? ((unsigned long long)left << 32) | (unsigned)(tc + ta)
-                                             : ((unsigned long long)(ti + ta) << 32) | (unsigned)tc;
-      const unsigned long long pv = atomicAdd(prog + s, add) + add;
-      s_skip = (long long)(unsigned)pv + (up - (long long)(pv >> 32)) < cbar;
+      if (kBounds && tamb) atomicAdd(&amb_count[s], tamb);
+      atomicAdd(prog + s, kBounds ? ((unsigned long long)left << 32) | (unsigned)(tin + tamb)
+                                  : ((unsigned long long)(tin + tamb) << 32) | (unsigned)tc);
     }
-    __syncthreads();
-    }
-    __syncthreads();  // s_skip has been read
   }
 }
 
@@ -812,17 +806,22 @@ cudaError_t launch_consensus_count(const float4 *XP, int nP, const ClsParams *cp
                                    const float4 *Xe, const float *pose, const int *list, const int *n_list, float eps,
                                    int *count, const int *c0, const int *ub_lo, const int *ub_extra,
                                    unsigned long long *prog, cudaStream_t s) {
-  LSR_LAUNCH(k_consensus_count<false><<<kSms * 8, kClsThreads, 0, s>>>(XP, nP, 1, cp, in_bits, near_bits, ge, start_e,
+  LSR_LAUNCH(k_consensus_count<false><<<kSms * 8, kClsThreads, 0, s>>>(XP, nP, cp, in_bits, near_bits, ge, start_e,
                                                                        Xe, pose, nullptr, n_list, 0, eps * eps, count,
                                                                        nullptr, c0, prog, ub_lo, ub_extra, list));
   return cudaGetLastError();
 }
 
-cudaError_t launch_consensus_bounds(const float4 *XP, int nP, int stride, const ClsParams *cp,
-                                    const unsigned *in_bits, const unsigned *near_bits, const float *pose,
-                                    const uint8_t *ok, const int *n_dev, int *in_count, int *amb_count,
-                                    cudaStream_t s) {
-  LSR_LAUNCH(k_consensus_count<true><<<kSms * 8, kClsThreads, 0, s>>>(XP, nP, stride, cp, in_bits, near_bits, nullptr,
+cudaError_t launch_point_sample(const float4 *XP, int nP, int stride, float4 *out, cudaStream_t s) {
+  const int n = (nP + stride - 1) / stride;
+  LSR_LAUNCH(k_point_sample<<<(int)lsr_div_up(n, 256), 256, 0, s>>>(XP, n, stride, out));
+  return cudaGetLastError();
+}
+
+cudaError_t launch_consensus_bounds(const float4 *XP, int nP, const ClsParams *cp, const unsigned *in_bits,
+                                    const unsigned *near_bits, const float *pose, const uint8_t *ok, const int *n_dev,
+                                    int *in_count, int *amb_count, cudaStream_t s) {
+  LSR_LAUNCH(k_consensus_count<true><<<kSms * 8, kClsThreads, 0, s>>>(XP, nP, cp, in_bits, near_bits, nullptr,
                                                                       nullptr, nullptr, pose, ok, n_dev, 0, 0.f,
                                                                       in_count, amb_count, nullptr, nullptr, nullptr,
                                                                       nullptr, nullptr));
@@ -848,7 +847,7 @@ cudaError_t launch_group_bounds(const Groups &G, const float4 *Xn, int nP, const
   const unsigned *far_bits = G.words + kGrpCapWords;
   LSR_LAUNCH(k_group_bounds<<<kSms * 8, 256, 0, s>>>(G.p, G.grp, far_bits, pose, ok, n_dev, c0, amb_count, G.up, G.list,
                                                      &G.p->left));
-  LSR_LAUNCH(k_group_count<true><<<kSms * 6, kClsThreads, 0, s>>>(Xn, nP, G.p, G.grp, G.first, far_bits, cp, in_bits,
+  LSR_LAUNCH(k_group_count<true><<<kSms * 6, kClsThreads, 0, s>>>(Xn, G.p, G.grp, G.first, far_bits, cp, in_bits,
                                                                   near_bits, nullptr, nullptr, nullptr, pose, G.list,
                                                                   &G.p->left, 0.f, in_count, amb_count, c0, prog, G.up,
                                                                   nullptr));
@@ -861,7 +860,7 @@ cudaError_t launch_group_count_bar(const Groups &G, const float4 *Xn, int nP, co
                                    const int *start_e, const float4 *Xe, const float *pose, const int *list,
                                    const int *n_list, float eps, int *count, const int *c0, const int *ub_lo,
                                    const int *ub_extra, unsigned long long *prog, cudaStream_t s) {
-  LSR_LAUNCH(k_group_count<false><<<kSms * 6, kClsThreads, 0, s>>>(Xn, nP, G.p, G.grp, G.first, G.words + kGrpCapWords,
+  LSR_LAUNCH(k_group_count<false><<<kSms * 6, kClsThreads, 0, s>>>(Xn, G.p, G.grp, G.first, G.words + kGrpCapWords,
                                                                    cp, in_bits, near_bits, ge, start_e, Xe, pose, list,
                                                                    n_list, eps * eps, count, nullptr, c0, prog, ub_lo,
                                                                    ub_extra));

@@ -724,13 +724,13 @@ cudaError_t launch_consensus_count(const float4 *XP, int nP, const ClsParams *cp
                                    const float4 *Xe, const float *pose, const int *list, const int *n_list, float eps,
                                    int *count, const int *c0, const int *ub_lo, const int *ub_extra,
                                    unsigned long long *prog, cudaStream_t s);
-// Bounds without exact tests over the points XP[v * stride]: in_count =
-// points in IN voxels (a lower bound of the inlier count), amb_count = points
-// in undecided voxels.
-cudaError_t launch_consensus_bounds(const float4 *XP, int nP, int stride, const ClsParams *cp,
-                                    const unsigned *in_bits, const unsigned *near_bits, const float *pose,
-                                    const uint8_t *ok, const int *n_dev, int *in_count, int *amb_count,
-                                    cudaStream_t s);
+// Bounds without exact tests: in_count = points in IN voxels (a lower bound of
+// the inlier count), amb_count = points in undecided voxels.
+cudaError_t launch_consensus_bounds(const float4 *XP, int nP, const ClsParams *cp, const unsigned *in_bits,
+                                    const unsigned *near_bits, const float *pose, const uint8_t *ok, const int *n_dev,
+                                    int *in_count, int *amb_count, cudaStream_t s);
+// out[v] = XP[v * stride] for v < ceil(nP / stride).
+cudaError_t launch_point_sample(const float4 *XP, int nP, int stride, float4 *out, cudaStream_t s);
 // The groups of P (its normal grid) and the bit-set of Q.
 cudaError_t launch_group_build(const float4 *Xn, int nP, const GridParams *gn, const int *start_n, float r_normal,
                                const float *boxQ, float eps, const float4 *XQ, int nQ, const Groups &G, cudaStream_t s);
