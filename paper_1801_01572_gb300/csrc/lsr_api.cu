@@ -197,9 +197,11 @@ struct Arena {
 int cap_cells_for(int n) { return std::max(8 * n, 1 << 20); }
 
 // Consensus: clouds of P from this size on take the estimate pre-pass (every
-// kConsensusPrepassStride-th point) before the full bounds pass.
+// kConsensusPrepassStride-th point; every 16th and 64th chose as well) before
+// the full bounds pass.
 constexpr int kConsensusPrepassMin = 16384;
 constexpr int kConsensusPrepassStride = 32;
+constexpr int kConsensusTop = 32;  // hypotheses counted exactly first
 
 struct CloudLayout {
   int n = 0, cap_f = 0, cap_n = 0, cap_e = 0;
@@ -375,7 +377,7 @@ void plan_pair(Arena &a, int nP, int nQ, bool stP, bool stQ, int64_t H, int leve
   L.in_bits = a.take<unsigned>(kClsCapWords);
   L.near_bits = a.take<unsigned>(kClsCapWords);
   L.sel = a.take<uint8_t>(L.surv_cap);
-  L.sel_list = a.take<int>(L.surv_cap);
+  L.sel_list = a.take<int>(kConsensusTop);
   L.n_sel = a.take<int>(1);
   L.rest = a.take<int>(L.surv_cap);
   L.n_rest = a.take<int>(1);
@@ -833,10 +835,11 @@ int enqueue_pair(lsr_ctx *c, const PairLayout &L, const float *P, const float *Q
     TRY_CUDA(c, cudaMemsetAsync(L.amb, 0, sizeof(int) * L.surv_cap, s), "memset count");
     TRY_CUDA(c, cudaMemsetAsync(L.count2, 0, sizeof(int) * L.surv_cap, s), "memset count");
     TRY_CUDA(c, cudaMemsetAsync(L.sum, 0, sizeof(unsigned long long) * L.surv_cap, s), "memset sum");
-    // Large P: the 32 largest upper bounds on every 16th point pick the
+    // Large P: the 32 largest upper bounds on every 32nd point pick the
     // hypotheses counted exactly first; their best count c0 then lets the
-    // full bounds pass leave out every hypothesis whose upper bound falls
-    // below c0 part-way (it can neither win nor tie).
+    // full bounds pass, over the groups of P that are not far from Q, leave out
+    // every hypothesis whose upper bound falls below c0 (it can neither win nor
+    // tie).
     const bool prepass = nP >= kConsensusPrepassMin;
     if (prepass) {
       TRY_CUDA(c, launch_point_sample(Pc.Xn, nP, kConsensusPrepassStride, L.sample, s), "sample");
@@ -844,7 +847,7 @@ int enqueue_pair(lsr_ctx *c, const PairLayout &L, const float *P, const float *Q
                launch_consensus_bounds(L.sample, (int)lsr_div_up(nP, kConsensusPrepassStride), L.cls, L.in_bits,
                                        L.near_bits, L.pose, L.ok, &L.st->n_surv, L.count, L.amb, s),
                "consensus estimate");
-      TRY_CUDA(c, launch_top_upper(L.count, L.amb, L.ok, &L.st->n_surv, 32, L.sel, L.sel_list, L.n_sel, s), "top");
+      TRY_CUDA(c, launch_top_upper(L.count, L.amb, L.ok, &L.st->n_surv, kConsensusTop, L.sel, L.sel_list, L.n_sel, s), "top");
       TRY_CUDA(c,
                launch_consensus_count(Pc.Xn, nP, L.cls, L.in_bits, L.near_bits, Qc.ge, Qc.start_e, Qc.Xe, L.pose,
                                       L.sel_list, L.n_sel, p.eps_inlier, L.count2, nullptr, nullptr, nullptr, nullptr, s),
@@ -867,7 +870,7 @@ int enqueue_pair(lsr_ctx *c, const PairLayout &L, const float *P, const float *Q
                "consensus bounds");
     }
     if (!prepass) {
-      TRY_CUDA(c, launch_top_upper(L.count, L.amb, L.ok, &L.st->n_surv, 32, L.sel, L.sel_list, L.n_sel, s), "top");
+      TRY_CUDA(c, launch_top_upper(L.count, L.amb, L.ok, &L.st->n_surv, kConsensusTop, L.sel, L.sel_list, L.n_sel, s), "top");
       TRY_CUDA(c,
                launch_consensus_count(Pc.Xn, nP, L.cls, L.in_bits, L.near_bits, Qc.ge, Qc.start_e, Qc.Xe, L.pose,
                                       L.sel_list, L.n_sel, p.eps_inlier, L.count2, nullptr, nullptr, nullptr, nullptr, s),
