@@ -656,9 +656,9 @@ def roofline(info):
     peak = fp32_alu_peak(sm_mhz)
     ach = terms * 3 / (avg * 1e-3) / 1e12
     # traffic: dram__bytes_read.sum + dram__bytes_write.sum of one full-size
-    # launch of this kernel on the room pair, from an ncu capture (the two
+    # launch of this kernel on a room pair of this size, from an ncu capture (the two
     # descriptor tables read once; the tiles' rows re-read from L2)
-    traffic = 47619328 + 600832 if (nP, nQ) == (150000, 150000) else None
+    traffic = 50922240 + 524544 if (nP, nQ) == (150000, 150000) else None
     return {"kernel": "k_match_win", "bound": "alu", "achieved": ach, "peak": peak, "unit": "TFLOP/s",
             "frac": ach / peak, "traffic": traffic, "launch_ms": avg, "launches_timed": n,
             "algorithmic_bytes": 144.0 * (nP + nQ) + 8.0 * nP,
