@@ -2470,27 +2470,28 @@ static int objective_impl(lsr_ctx *c, int32_t n, const float *const *P, const in
     nn = a.take<int>(nP[i]);
   };
   constexpr size_t kChunkBytes = (size_t)1 << 30;
-  const size_t out_bytes = sizeof(double) * 7 * (size_t)n + kAlign;
+  const size_t out_bytes = sizeof(double) * 7 * (size_t)n;
   std::vector<int> first{0};  // chunks of consecutive pairs
-  size_t most = 0;
+  size_t most = 0;            // end of the longest chunk, each placed after the results
   {
     Arena m(nullptr);
+    m.off = out_bytes;
     for (int i = 0; i < n; ++i) {
       CloudLayout q1;
       ScratchLayout q2;
       double *q3;
       int *q4;
-      const size_t before = m.off;
       plan(m, i, q1, q2, q3, q4);
-      if (i > first.back() && (i - first.back() == kPoseJobs || m.off > kChunkBytes)) {
+      if (i > first.back() && (i - first.back() == kPoseJobs || m.off - out_bytes > kChunkBytes)) {
         first.push_back(i);
-        m.off = m.off - before + kAlign;
+        m.off = out_bytes;
+        plan(m, i, q1, q2, q3, q4);
       }
       most = std::max(most, m.off);
     }
     first.push_back(n);
   }
-  if ((rc = ensure_ws(c, out_bytes + most))) return rc;
+  if ((rc = ensure_ws(c, most))) return rc;
   double *out7 = reinterpret_cast<double *>(c->ws);
   cudaStream_t s = c->stream;
   std::vector<double> host7((size_t)7 * n);
@@ -2533,6 +2534,7 @@ static int objective_impl(lsr_ctx *c, int32_t n, const float *const *P, const in
       o.partials = part, o.out = out7 + 7 * i;
       o.dP = grad ? dP[i] : nullptr, o.dQ = grad ? dQ[i] : nullptr;
     }
+    if (a.off > c->ws_cap) return set_err(c, LSR_E_STATE, "objective workspace outgrew its measure");
     TRY_CUDA(c, build_grids(gj, m, s), "grids");
     TRY_CUDA(c, launch_pose_nn(nj, m, s), "neighbours");
     TRY_CUDA(c, launch_objective(oj, m, grad ? 1 : 0, s), "objective");

@@ -48,3 +48,45 @@ def test_objective_batches_equal_single_pairs(sizes):
             assert np.array_equal(dx1[0], dxi[k])
             assert torch.equal(dP1[0], dP[k])
             assert torch.allclose(dQ1[0], dQ[k], rtol=1e-6, atol=1e-6 * float(dQ[k].abs().max()) + 1e-12)
+
+
+@gpu
+@pytest.mark.parametrize("n", [1, 3, 8, 9])
+def test_objective_in_a_workspace_that_just_suffices(n):
+    """The largest pair that an earlier call's workspace still holds: its plan
+    ends inside that workspace (a plan that does not is refused), and the
+    energy is that of a workspace of its own."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1801_01572_gb300 as lsr
+    rng = np.random.default_rng(n)
+    q = torch.from_numpy(rng.uniform(0, 0.4, (500, 3)).astype(np.float32)).cuda()
+    big = torch.from_numpy(rng.uniform(0, 0.4, (4_000_000, 3)).astype(np.float32)).cuda()
+    last = min(n, 8) - 1  # the last pair of a full chunk grows
+    xi, T0 = np.zeros((n, 6)), np.tile(np.eye(4), (n, 1, 1))
+
+    def clouds(points):
+        return [big[:points if k == last else 1000] for k in range(n)], [q] * n
+
+    def held(points):
+        """(whether the workspace of 1000 points held this many, the energies)"""
+        with lsr.Context(0) as ctx:
+            ctx.objective_fwd(*clouds(1000), xi, T0, EPS)
+            had = ctx.workspace_bytes()
+            E = ctx.objective_fwd(*clouds(points), xi, T0, EPS)
+            return ctx.workspace_bytes() == had, E
+
+    lo, hi = 1000, len(big)
+    assert held(lo)[0] and not held(hi)[0]
+    while hi - lo > 1:
+        mid = (lo + hi) // 2
+        if held(mid)[0]:
+            lo = mid
+        else:
+            hi = mid
+    for points in (lo, lo - 1, lo - 13, lo - 50):
+        same, E = held(points)
+        assert same
+        with lsr.Context(0) as ctx:
+            assert np.array_equal(E, ctx.objective_fwd(*clouds(points), xi, T0, EPS))
