@@ -251,7 +251,10 @@ cudaError_t launch_surfel_correct(int64_t n, const float *pos, const float *nrm,
     const int64_t tiles = lsr_div_up(n, big ? 1024 : 512);
     const int grid = (int)(tiles < kSms * 3 ? tiles : kSms * 3);
     auto kern = big ? k_surfel_tile<2> : k_surfel_tile<1>;
-    LSR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    // the limit belongs to the function on the device, which contexts on other
+    // threads launch too: always the one for the largest table, never the call's own
+    const size_t limit = big ? surfel_tile_smem<2>(kSurfTileKf) : surfel_tile_smem<1>(kSurfTileKf);
+    LSR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit));
     LSR_LAUNCH(kern<<<grid, kSurfTileThreads, smem, s>>>(n, pos, nrm, t0, tu, m, kf, t_kf, cam, pos_out, nrm_out, keep,
                                                          n_keep));
     return cudaGetLastError();

@@ -95,3 +95,74 @@ def test_small_keyframe_tables_equal_the_general_kernel(ctx, n, m):
     assert a[3] == b[3]
     for x, y in zip(a[:3], b[:3]):
         assert np.array_equal(x, y)
+
+
+_THREADS_C = r"""
+#include <pthread.h>
+#include <stdio.h>
+#include <stdlib.h>
+
+#include "lsr.h"
+
+enum { kThreads = 8, kSurfels = 64, kCalls = 3000 };
+
+/* A context of its own and a table of 600 or of 1 keyframes; returns the calls that failed. */
+static void *work(void *arg) {
+  const int m = (long)arg % 2 ? 600 : 1;
+  lsr_ctx *ctx = NULL;
+  if (lsr_create(&ctx, NULL, 0, NULL) != LSR_OK) return (void *)(long)kCalls;
+  float *pos = calloc(3 * kSurfels, 4), *nrm = calloc(3 * kSurfels, 4), *t0 = calloc(kSurfels, 4);
+  float *tu = calloc(kSurfels, 4), *po = calloc(3 * kSurfels, 4), *no = calloc(3 * kSurfels, 4);
+  uint8_t *keep = calloc(kSurfels, 1);
+  double *T = calloc(16 * (size_t)m, 8);
+  float *tk = calloc(m, 4);
+  const float cam[7] = {500, 500, 320, 240, 640, 480, 5};
+  for (int f = 0; f < m; ++f) {
+    for (int k = 0; k < 16; k += 5) T[16 * f + k] = 1;
+    tk[f] = (float)(f + 1);
+  }
+  for (int i = 0; i < kSurfels; ++i) pos[3 * i + 2] = nrm[3 * i + 2] = 1, tu[i] = 1e6f;
+  long bad = 0;
+  for (int c = 0; c < kCalls; ++c) {
+    int64_t kept = 0;
+    const int rc = lsr_surfel_correct(ctx, kSurfels, pos, nrm, t0, tu, m, T, T, tk, cam, po, no, keep, &kept);
+    bad += rc != LSR_OK || kept != kSurfels;
+  }
+  lsr_destroy(ctx);
+  return (void *)bad;
+}
+
+int main(void) {
+  pthread_t t[kThreads];
+  long bad = 0;
+  for (long k = 0; k < kThreads; ++k) pthread_create(t + k, NULL, work, (void *)k);
+  for (int k = 0; k < kThreads; ++k) {
+    void *r;
+    pthread_join(t[k], &r);
+    bad += (long)r;
+  }
+  printf("%ld\n", bad);
+  return 0;
+}
+"""
+
+
+@gpu
+def test_threads_with_tables_of_different_sizes(tmp_path):
+    """Contexts on eight threads, half with 600 keyframes and half with one:
+    the kernel's limit of shared memory is the device's, not the call's, so no
+    call may narrow it between another's setting and launch. Every call
+    succeeds. (In C: with an interpreter between the calls hardly any meet.)"""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import os
+    import subprocess
+
+    from paper_1801_01572_gb300 import _build
+    src, exe = tmp_path / "threads.c", tmp_path / "threads"
+    src.write_text(_THREADS_C)
+    subprocess.run(["gcc", "-O1", "-I", os.path.join(_build.ROOT, "include"), str(src), _build.LIB, "-o", str(exe),
+                    "-lpthread", "-Wl,-rpath," + _build.OUT], check=True)
+    out = subprocess.run([str(exe)], capture_output=True, text=True, timeout=120, check=True)
+    assert int(out.stdout) == 0
