@@ -152,7 +152,7 @@ __device__ void grid_params(const float *box, float radius, int npts, int cap, c
   q.wx = (int)wx, q.wy = (int)wy, q.wz = (int)wz;
   q.ncells = (int)(wx * wy * wz);
   q.npts = npts;
-  q.pad_ = 0;
+  q.margin = grid_margin(q.cell, q.nx, q.ny, q.nz);
   q.nbmask = mask;
   *g = q;
 }

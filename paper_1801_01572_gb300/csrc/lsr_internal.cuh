@@ -52,8 +52,22 @@ struct GridParams {
   int wx, wy, wz;    // stored extents (<= n*, equal unless wrapped)
   int ncells;        // wx * wy * wz
   int npts;
-  int pad_;
+  // What a distance to a face of the query's own cell, taken from its FP32 cell
+  // coordinates, may exceed the true distance to a point behind that face by:
+  // the searches that leave cells out subtract it (grid_margin).
+  float margin;
 };
+
+// The coordinates (x - origin) / cell of a query and of a point of a box F
+// cells long are off by 2^-24 F cells each for the subtraction and as much for
+// the product; twice that, and at least 2e-4 cells, which covers boxes of up
+// to 418. (With 2e-4 for all, 3% of the queries just beyond a face of a box of
+// 26,000 cells missed a nearer point behind it.)
+__host__ __device__ inline float grid_margin(float cell, int nx, int ny, int nz) {
+  const int most = nx > ny ? (nx > nz ? nx : nz) : (ny > nz ? ny : nz);
+  const float cells = 8.f * 5.9604645e-8f * ((float)most + 1.f);
+  return cell * (cells > 2e-4f ? cells : 2e-4f);
+}
 
 // Device view of one cloud after packing and grid building. "Internal order"
 // is the order of the feature-radius grid (points sorted by cell, then by
@@ -261,8 +275,8 @@ __device__ __forceinline__ void grid_ranges(const GridParams &g, const int *__re
 //
 // The query's own row of cells is searched first; each of the other eight
 // rows, and the x-neighbour cells of every row, is visited only if its
-// distance from the query (less a margin of 2e-4 cells, above the FP32
-// rounding of cell coordinates) can still reach the group's best so far. A
+// distance from the query (less the grid's margin, above the FP32 rounding of
+// cell coordinates) can still reach the group's best so far. A
 // skipped cell holds no point at or below that best, so the result is the
 // one of the full walk. (Grids with wrapped storage walk all cells.)
 //
@@ -337,7 +351,7 @@ __device__ __forceinline__ void group_nn(const GridParams &g, const int *__restr
     }
     if (go) {
       const unsigned gmask = G == 32 ? 0xffffffffu : (((1u << G) - 1u) << ((threadIdx.x & 31) & ~(G - 1)));
-      const float mg = 2e-4f * g.cell;
+      const float mg = g.margin;
       auto gsq = [&](float d) {
         const float t = fmaxf(d - mg, 0.f);
         return t * t;

@@ -69,7 +69,7 @@ __global__ void k_cell_grid_params(const float *box, float cell, int npts, int c
   q.wx = (int)wx, q.wy = (int)wy, q.wz = (int)wz;
   q.ncells = (int)(wx * wy * wz);
   q.npts = npts;
-  q.pad_ = 0;
+  q.margin = grid_margin(q.cell, q.nx, q.ny, q.nz);
   q.nbmask = nullptr;
   *g = q;
 }

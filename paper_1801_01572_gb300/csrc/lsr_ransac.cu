@@ -354,10 +354,12 @@ constexpr int kConsChunk = 2048;
 // Minimum squared distance below eps2 by a group of G lanes (no index needed).
 // The query's own row of cells first; a row of cells, and the x-neighbour
 // cells of a row, that the best so far does not reach is left out (as in
-// group_nn, with its margins).
+// group_nn, with its margin, here the address of the grid's: kept in a register
+// it cost spills, 863 us instead of 851 for 256 poses of 50k points).
 template <int G>
-__device__ __forceinline__ float group_min_d2(const GridParams &g, const int *__restrict__ start,
-                                              const float4 *__restrict__ Xe, float x, float y, float z, float eps2) {
+__device__ __forceinline__ float group_min_d2(const GridParams &g, const float *__restrict__ margin,
+                                              const int *__restrict__ start, const float4 *__restrict__ Xe, float x,
+                                              float y, float z, float eps2) {
   const int sub = threadIdx.x & (G - 1);
   float best = eps2;
   int next = sub, base = 0;
@@ -388,7 +390,7 @@ __device__ __forceinline__ float group_min_d2(const GridParams &g, const int *__
     }
     if (go) {
       const unsigned gmask = ((1u << G) - 1u) << ((threadIdx.x & 31) & ~(G - 1));
-      const float mg = 2e-4f * g.cell;
+      const float mg = __ldg(margin);
       auto gsq = [&](float d) {
         const float t = fmaxf(d - mg, 0.f);
         return t * t;
@@ -468,7 +470,7 @@ __global__ void __launch_bounds__(kConsThreads) k_consensus(const float4 *__rest
       float4 p = valid ? XP[i] : make_float4(__int_as_float(0x7fc00000), 0.f, 0.f, 0.f);
       float x, y, z;
       T.apply(p, x, y, z);
-      float best = group_min_d2<G>(g, start, Xe, x, y, z, eps2);
+      float best = group_min_d2<G>(g, &gep->margin, start, Xe, x, y, z, eps2);
       if (valid && sub == 0 && best < eps2) {
         ++cnt;
         acc += (unsigned long long)__double2ll_rn((double)best * kFixScale);

@@ -183,7 +183,7 @@ __device__ __forceinline__ float nn_border(const GridParams &g, float fx, float 
   const float ux = fx - floorf(fx), uy = fy - floorf(fy), uz = fz - floorf(fz);
   const float in = fminf(fminf(fminf(ux, 1.f - ux), fminf(uy, 1.f - uy)), fminf(uz, 1.f - uz));
   const float out = fmaxf(fmaxf(fmaxf(-fx, fx - (float)g.nx), fmaxf(-fy, fy - (float)g.ny)), fmaxf(-fz, fz - (float)g.nz));
-  return fmaxf(1.f + in, out) * g.cell - 4e-4f * g.cell;
+  return fmaxf(1.f + in, out) * g.cell - 2.f * g.margin;
 }
 
 // The result of group_nn (at: the position in Xe, -1 if none), and a distance
@@ -229,7 +229,7 @@ __device__ __noinline__ Found half_nn(const GridParams &g, const int *__restrict
     const float r = sqrtf(best) + guard, gb = r * r;
     const int dy = sub % 3 - 1, dz = sub / 3 - 1, iy = cy + dy, iz = cz + dz;
     if (sub < 9 && iy >= 0 && iy < g.ny && iz >= 0 && iz < g.nz) {
-      const float mg = 2e-4f * g.cell;
+      const float mg = g.margin;
       auto gsq = [&](float d) {
         const float t = fmaxf(d - mg, 0.f);
         return t * t;
