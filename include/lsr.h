@@ -145,7 +145,8 @@ LSR_API int lsr_set_params(lsr_ctx *ctx, const lsr_params *params);
 LSR_API int lsr_get_params(const lsr_ctx *ctx, lsr_params *params);
 
 /* Test hooks: make failures happen without faulting or hanging a GPU, so
- * that the error paths can be exercised. (The paper has no counterpart.)
+ * that the error paths can be exercised, and take paths that sizes choose at
+ * sizes that do not. (The paper has no counterpart.)
  *  LSR_INJECT_ALLOC: the next `count` device workspace allocations of this
  *    context fail as if the device were out of memory (no cudaMalloc is made);
  *    the call returns LSR_E_OOM and the context stays usable.
@@ -158,13 +159,18 @@ LSR_API int lsr_get_params(const lsr_ctx *ctx, lsr_params *params);
  *    next hypothesis-count kernel on the context's stream asks the bounds
  *    checks about one out-of-range index (no memory access follows), so that
  *    call returns LSR_E_CHECK through the same path a real violation takes.
- *  LSR_INJECT_NONE: clear the first two.
+ *  LSR_INJECT_MATCH_LIST: the next `count` calls of lsr_stage_match with a
+ *    BF16 precision contract only the database tiles within reach, listed from
+ *    the descriptor order, at any size (without it: from 2^29 pairs of rows
+ *    on). The same results.
+ *  LSR_INJECT_NONE: clear all but LSR_INJECT_CHECK.
  * Returns LSR_OK, LSR_E_ARG (unknown kind, count outside [0, 10^6]) or
  * LSR_E_STATE (NULL context). */
 #define LSR_INJECT_NONE 0
 #define LSR_INJECT_ALLOC 1
 #define LSR_INJECT_MATCH_STALL 2
 #define LSR_INJECT_CHECK 3
+#define LSR_INJECT_MATCH_LIST 4
 LSR_API int lsr_debug_inject(lsr_ctx *ctx, int32_t kind, int32_t count);
 
 /* 1 if this library is the checked build (compiled with LSR_CHECKED: device

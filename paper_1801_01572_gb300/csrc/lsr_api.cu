@@ -172,6 +172,7 @@ struct lsr_ctx {
   // allocations to fail, tensor-core matcher launches to stall
   int inject_alloc = 0;
   int inject_stall = 0;
+  int inject_list = 0;  // descriptor matches (lsr_stage_match) through the item list whatever their size
   // per-kernel event timing (lsr_set_kernel_timing); null when off
   KernelTimer *ktimer = nullptr;
 };
@@ -1375,9 +1376,10 @@ int lsr_debug_inject(lsr_ctx *c, int32_t kind, int32_t count) {
   if (!c) return LSR_E_STATE;
   if (count < 0 || count > 1000000) return set_err(c, LSR_E_ARG, "bad injection count");
   switch (kind) {
-    case LSR_INJECT_NONE: c->inject_alloc = c->inject_stall = 0; return LSR_OK;
+    case LSR_INJECT_NONE: c->inject_alloc = c->inject_stall = c->inject_list = 0; return LSR_OK;
     case LSR_INJECT_ALLOC: c->inject_alloc = count; return LSR_OK;
     case LSR_INJECT_MATCH_STALL: c->inject_stall = count; return LSR_OK;
+    case LSR_INJECT_MATCH_LIST: c->inject_list = count; return LSR_OK;
     case LSR_INJECT_CHECK: {
       if (!lsr_checked_build()) return set_err(c, LSR_E_ARG, "LSR_INJECT_CHECK needs the checked build");
       if (count == 0) return LSR_OK;
@@ -1689,6 +1691,8 @@ int lsr_stage_match(lsr_ctx *c, const float *FP, int64_t nP, const float *FQ, in
     return set_err(c, LSR_E_ARG, "bad argument");
   if (!valid_precision(precision)) return set_err(c, LSR_E_ARG, "bad precision");
   const bool tc = precision != LSR_MATCH_FP32, split = precision == LSR_MATCH_BF16;
+  const bool list = tc && c->inject_list > 0;
+  if (list) --c->inject_list;
   auto plan = [&](Arena &a, float *&fp, float *&fq, float *&FPi, float *&FQi, int *&dn, float *&dd, int *&flags,
                   char *&tws) {
     fp = a.take<float>(kD * nP);
@@ -1698,7 +1702,7 @@ int lsr_stage_match(lsr_ctx *c, const float *FP, int64_t nP, const float *FQ, in
     dn = a.take<int>(nP);
     dd = a.take<float>(nP);
     flags = a.take<int>(2);
-    tws = a.take<char>(tc ? tc_workspace_bytes((int)nP, (int)nQ, split) : fp32_workspace_bytes((int)nP, (int)nQ));
+    tws = a.take<char>(tc ? tc_workspace_bytes((int)nP, (int)nQ, split, list) : fp32_workspace_bytes((int)nP, (int)nQ));
   };
   Arena m(nullptr);
   float *x1, *x2, *x3, *x4, *x6;
@@ -1716,9 +1720,11 @@ int lsr_stage_match(lsr_ctx *c, const float *FP, int64_t nP, const float *FQ, in
   TRY_CUDA(c, cudaMemcpyAsync(fq, FQ, sizeof(float) * kD * nQ, cudaMemcpyDefault, s), "copy FQ");
   LSR_LAUNCH(k_gather_rows<<<nblk(nP * kDS), 256, 0, s>>>(fp, kD, nullptr, (int)nP, FPi));
   LSR_LAUNCH(k_gather_rows<<<nblk(nQ * kDS), 256, 0, s>>>(fq, kD, nullptr, (int)nQ, FQi));
+  TcFault fault = tc ? take_tc_fault(c) : TcFault();
+  fault.list = list;
   if (tc)
     TRY_CUDA(c, launch_match_bf16(FPi, (int)nP, FQi, (int)nQ, split, match_tile_for(c, (int)nP), tws, dn, dd, flags, flags + 1,
-                                  nullptr, s, take_tc_fault(c)),
+                                  nullptr, s, fault),
              "match");
   else
     TRY_CUDA(c, launch_match_fp32(FPi, (int)nP, FQi, (int)nQ, tws, dn, dd, s), "match");

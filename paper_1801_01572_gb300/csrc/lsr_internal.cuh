@@ -624,12 +624,14 @@ cudaError_t launch_match_fp32_rows(const float *FP, int nP, const float *FQ, int
 // qt: query tiles of 128 per CTA work unit (1 or 2; 0 = tc_default_tile(nP)).
 // f: the limit of the pipeline's waits (0 = 2 s) and the test-only stall
 // (the producer issues no copy or MMA, so the epilogue's first wait runs out
-// and err is set; see lsr_debug_inject).
+// and err is set), and the test-only item list at any size (ws: measured with
+// list); see lsr_debug_inject.
 struct TcFault {
   unsigned long long wait_ns = 0;
   int stall = 0;
+  int list = 0;
 };
-size_t tc_workspace_bytes(int nP, int nQ, bool split);
+size_t tc_workspace_bytes(int nP, int nQ, bool split, bool list = false);
 int tc_score_cols(int nQ);
 int tc_default_tile(int nP);
 cudaError_t launch_match_bf16(const float *FP, int nP, const float *FQ, int nQ, bool split, int qt, char *ws, int *nn,

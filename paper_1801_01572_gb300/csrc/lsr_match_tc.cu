@@ -779,8 +779,8 @@ struct TcLayout {
 // Above 2^22 items (about 2M x 2M rows) the list would outgrow its use of memory.
 constexpr int64_t kWindowPairs = (int64_t)1 << 29;
 constexpr int64_t kMaxItems = (int64_t)1 << 22;
-int item_cap_for(int nP, int nQ) {
-  if ((int64_t)nP * nQ < kWindowPairs) return 0;
+int item_cap_for(int nP, int nQ, bool list) {
+  if (!list && (int64_t)nP * nQ < kWindowPairs) return 0;
   const int64_t n = lsr_div_up(nP, kTcM) * lsr_div_up(lsr_div_up(nQ, kTcN), kItemTiles);
   return n <= kMaxItems ? (int)n : 0;
 }
@@ -788,7 +788,7 @@ int item_cap_for(int nP, int nQ) {
 // Query rows are padded to a multiple of 256 (a whole number of units for
 // either tile shape); unit u of shape QT is tiles QT u .. QT u + QT - 1.
 template <int KS>
-TcLayout tc_layout(char *base, int nP, int nQ) {
+TcLayout tc_layout(char *base, int nP, int nQ, bool list) {
   using S = Shape<KS>;
   auto al = [](size_t x) { return (x + 255) / 256 * 256; };
   size_t tilesA = 2 * (size_t)lsr_div_up(nP, 2 * kTcM), nNT = (size_t)lsr_div_up(nQ, kTcN);
@@ -813,7 +813,7 @@ TcLayout tc_layout(char *base, int nP, int nQ) {
   L.fb_rows = reinterpret_cast<int *>(take((size_t)nP * 4));
   L.packed = reinterpret_cast<unsigned long long *>(take((size_t)nP * 8));
   L.fb_packed = reinterpret_cast<unsigned long long *>(take((size_t)nP * 8));
-  L.item_cap = item_cap_for(nP, nQ);
+  L.item_cap = item_cap_for(nP, nQ, list);
   L.items = reinterpret_cast<TcItem *>(take(sizeof(TcItem) * (size_t)L.item_cap * kClasses));
   L.bytes = off;
   return L;
@@ -852,7 +852,7 @@ cudaError_t launch_tc(const TcLayout &L, int nP, int nQ, bool window, int *fb_co
 template <int KS>
 cudaError_t run_tc(const float *FP, int nP, const float *FQ, int nQ, int qt, char *ws, int *nn, float *d1,
                    int *fb_count, int *err, float *d2, const TcFault &f, cudaStream_t s) {
-  TcLayout L = tc_layout<KS>(ws, nP, nQ);
+  TcLayout L = tc_layout<KS>(ws, nP, nQ, f.list != 0);
   const int nNT = (int)lsr_div_up(nQ, kTcN);
   const bool window = L.item_cap > 0 && !d2;
   // the counters, the search's work word and the flags lie one after another
@@ -894,8 +894,8 @@ constexpr int kKsPlain = 3, kKsSplit = 7;
 
 LSR_CHECK_READER(match_tc)
 
-size_t tc_workspace_bytes(int nP, int nQ, bool split) {
-  return split ? tc_layout<kKsSplit>(nullptr, nP, nQ).bytes : tc_layout<kKsPlain>(nullptr, nP, nQ).bytes;
+size_t tc_workspace_bytes(int nP, int nQ, bool split, bool list) {
+  return split ? tc_layout<kKsSplit>(nullptr, nP, nQ, list).bytes : tc_layout<kKsPlain>(nullptr, nP, nQ, list).bytes;
 }
 
 int tc_score_cols(int nQ) { return (int)lsr_div_up(nQ, kTcN) * kTcN; }
