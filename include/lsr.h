@@ -163,6 +163,9 @@ LSR_API int lsr_get_params(const lsr_ctx *ctx, lsr_params *params);
  *    BF16 precision contract only the database tiles within reach, listed from
  *    the descriptor order, at any size (without it: from 2^29 pairs of rows
  *    on). The same results.
+ *  LSR_INJECT_SEARCH_ALL: the next `count` calls of lsr_stage_refine search the
+ *    neighbour of every point at every step instead of keeping those that
+ *    still stand. The same results.
  *  LSR_INJECT_NONE: clear all but LSR_INJECT_CHECK.
  * Returns LSR_OK, LSR_E_ARG (unknown kind, count outside [0, 10^6]) or
  * LSR_E_STATE (NULL context). */
@@ -171,6 +174,7 @@ LSR_API int lsr_get_params(const lsr_ctx *ctx, lsr_params *params);
 #define LSR_INJECT_MATCH_STALL 2
 #define LSR_INJECT_CHECK 3
 #define LSR_INJECT_MATCH_LIST 4
+#define LSR_INJECT_SEARCH_ALL 5
 LSR_API int lsr_debug_inject(lsr_ctx *ctx, int32_t kind, int32_t count);
 
 /* 1 if this library is the checked build (compiled with LSR_CHECKED: device

@@ -172,6 +172,7 @@ struct lsr_ctx {
   // allocations to fail, tensor-core matcher launches to stall
   int inject_alloc = 0;
   int inject_stall = 0;
+  int inject_search = 0;  // refinements (lsr_stage_refine) that keep no neighbour
   int inject_list = 0;  // descriptor matches (lsr_stage_match) through the item list whatever their size
   // per-kernel event timing (lsr_set_kernel_timing); null when off
   KernelTimer *ktimer = nullptr;
@@ -690,10 +691,11 @@ cudaError_t build_pair(const float *P, const float *Q, const CloudLayout &Pc, co
 // Graduated refinement (levels l = 0..L-1, radius eps * 2^(L-1-l)) from the
 // pose in st. XP: P in internal order with caller indices in w; Q: caller-order
 // xyz on the device; (ge, start_e, Xe): Q's eps grid for the finest level.
+// search_all (test hook): every step searches for every point.
 cudaError_t enqueue_refine(const float4 *XP, const float *P, int nP, const float *Q, const float *boxQ,
                            const GridParams *ge, const int *start_e, const float4 *Xe, const LevelLayout &V, float eps,
                            float mu_scale, int iters, RansacState *st, double *part, float4 *near, float4 *certs,
-                           const ScratchLayout &sc, cudaStream_t s, bool chain) {
+                           const ScratchLayout &sc, cudaStream_t s, bool chain, bool search_all = false) {
   int L = V.levels;
   LSR_CUDA_TRY(refine_reset_tickets(part, s));
   // the coarse levels' grids, as many at once as there is scratch for
@@ -725,8 +727,11 @@ cudaError_t enqueue_refine(const float4 *XP, const float *P, int nP, const float
     if (l + 1 < L) g = V.g[l], st0 = V.start[l], xs = V.Xs[l];
     LSR_CUDA_TRY(launch_refine_level_begin(st, s));
     LSR_CUDA_TRY(cudaMemsetAsync(near, 0xff, sizeof(float4) * (size_t)np, s));  // no search yet at this level
-    for (int it = 0; it < iters; ++it)
-      LSR_CUDA_TRY(launch_refine_step(xp, np, g, st0, xs, e, mu, iters, st, part, near, certs, chain && it > 0, s));
+    for (int it = 0; it < iters; ++it) {
+      if (search_all) LSR_CUDA_TRY(cudaMemsetAsync(near, 0xff, sizeof(float4) * (size_t)np, s));
+      LSR_CUDA_TRY(launch_refine_step(xp, np, g, st0, xs, e, mu, iters, st, part, near, certs,
+                                      chain && it > 0 && !search_all, s));
+    }
   }
   return cudaSuccess;
 }
@@ -1376,10 +1381,11 @@ int lsr_debug_inject(lsr_ctx *c, int32_t kind, int32_t count) {
   if (!c) return LSR_E_STATE;
   if (count < 0 || count > 1000000) return set_err(c, LSR_E_ARG, "bad injection count");
   switch (kind) {
-    case LSR_INJECT_NONE: c->inject_alloc = c->inject_stall = c->inject_list = 0; return LSR_OK;
+    case LSR_INJECT_NONE: c->inject_alloc = c->inject_stall = c->inject_list = c->inject_search = 0; return LSR_OK;
     case LSR_INJECT_ALLOC: c->inject_alloc = count; return LSR_OK;
     case LSR_INJECT_MATCH_STALL: c->inject_stall = count; return LSR_OK;
     case LSR_INJECT_MATCH_LIST: c->inject_list = count; return LSR_OK;
+    case LSR_INJECT_SEARCH_ALL: c->inject_search = count; return LSR_OK;
     case LSR_INJECT_CHECK: {
       if (!lsr_checked_build()) return set_err(c, LSR_E_ARG, "LSR_INJECT_CHECK needs the checked build");
       if (count == 0) return LSR_OK;
@@ -1947,6 +1953,8 @@ int lsr_stage_refine(lsr_ctx *c, const float *P, int64_t nP, const float *Q, int
       iters > 10000 || levels < 1 || levels > kMaxLevels || !(eps > 0.f && eps * (float)(1 << (levels - 1)) <= 10.f) ||
       !(mu_scale > 0.f))
     return set_err(c, LSR_E_ARG, "bad argument");
+  const bool search_all = c->inject_search > 0;
+  if (search_all) --c->inject_search;
   float *boxP = nullptr;
   double *boxP_part = nullptr;
   float4 *near = nullptr, *certs = nullptr;
@@ -2000,7 +2008,7 @@ int lsr_stage_refine(lsr_ctx *c, const float *P, int64_t nP, const float *Q, int
   TRY_CUDA(c, launch_refine_init(st, boxP, Td, s), "init");
   TRY_CUDA(c,
            enqueue_refine(XP, p, (int)nP, qsrc, Cq.box, Cq.ge, Cq.start_e, Cq.Xe, V, eps, mu_scale, iters, st,
-                          part, near, certs, S, s, true),
+                          part, near, certs, S, s, true, search_all),
            "refine");
   RansacState h;
   TRY_CUDA(c, cudaMemcpyAsync(&h, st, sizeof(h), cudaMemcpyDeviceToHost, s), "D2H");

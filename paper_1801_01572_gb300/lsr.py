@@ -40,7 +40,8 @@ ABI_FUNCTIONS = (
     "lsr_kernel_timing_entry", "lsr_checked_build", "lsr_pose_implicit_grad", "lsr_stage_nn",
     "lsr_stage_consensus_modes",
 )
-INJECT_NONE, INJECT_ALLOC, INJECT_MATCH_STALL, INJECT_CHECK, INJECT_MATCH_LIST = 0, 1, 2, 3, 4
+INJECT_NONE, INJECT_ALLOC, INJECT_MATCH_STALL, INJECT_CHECK = 0, 1, 2, 3
+INJECT_MATCH_LIST, INJECT_SEARCH_ALL = 4, 5
 LSR_E_CHECK = -7
 
 
@@ -277,8 +278,9 @@ class Context:
         """Test hook (lsr_debug_inject): make the next `count` workspace
         allocations fail (INJECT_ALLOC) or tensor-core matcher launches stall
         into their bounded wait (INJECT_MATCH_STALL), or BF16 stage matches list
-        the tiles within reach at any size (INJECT_MATCH_LIST); INJECT_NONE
-        clears."""
+        the tiles within reach at any size (INJECT_MATCH_LIST), or stage
+        refinements search every point at every step (INJECT_SEARCH_ALL);
+        INJECT_NONE clears."""
         self._check(self._L.lsr_debug_inject(self._h, int(kind), int(count)))
 
     def set_kernel_timing(self, prefix: str | None = ""):

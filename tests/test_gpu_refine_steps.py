@@ -61,3 +61,46 @@ def test_refinement_steps(ctx, n, iters, kind):
     tol = 2e-5 + 2 * EPS * iters ** 0.5 / n
     ang, tr = pose_error(T, ref)
     assert np.radians(ang) < tol and tr < tol * 2.0, (ang, tr, tol)
+
+
+def _moved(rng, kind, n):
+    """(P, Q, starting pose): P is a part of the surface moved by a small pose."""
+    from scipy.spatial.transform import Rotation
+    Q = _surface(rng, 6000)
+    P = _surface(rng, n)
+    P[1::7] += [4.0, -3.0, 2.0]  # no neighbour
+    if kind == "duplicates":
+        Q = np.concatenate([Q, Q[:3000]])
+    elif kind == "wrapped":
+        Q = np.concatenate([Q, rng.uniform(-1, 1, (40, 3)) * [150.0, 120.0, 90.0]])
+    elif kind == "long":  # thousands of cells along an axis, storage not wrapped
+        s = rng.integers(0, 40, len(Q))
+        Q = np.stack([Q[:, 0] + 20.0 * s - 400.0, 0.2 * Q[:, 1], 0.1 * Q[:, 2]], 1)
+        P = Q[rng.integers(0, len(Q), n)] + rng.normal(0, 0.004, (n, 3))
+    elif kind == "offset":
+        Q, P = Q + [900.0, -700.0, 300.0], P + [900.0, -700.0, 300.0]
+    elif kind == "lattice":  # every query between equally near points
+        Q = np.round(Q / 0.01) * 0.01
+        P = np.round(P / 0.01) * 0.01 + 0.005
+    T0 = np.eye(4)
+    T0[:3, :3] = Rotation.from_rotvec([0.006, -0.004, 0.005] if kind not in ("long", "offset") else
+                                      [2e-6, -3e-6, 2e-6]).as_matrix()
+    T0[:3, 3] = [0.004, -0.003, 0.002]
+    return P.astype(np.float32), Q.astype(np.float32), T0
+
+
+@gpu
+@pytest.mark.parametrize("n", [63, 64, 65, 257, 4099, 38913, 155649])
+@pytest.mark.parametrize("kind", ["plain", "duplicates", "wrapped", "long", "offset", "lattice"])
+@pytest.mark.parametrize("levels", [1, 3])
+def test_kept_neighbours_equal_a_search_of_every_point(ctx, n, kind, levels):
+    """The same poses and step counts to the last bit whether neighbours are
+    kept or searched at every step (LSR_INJECT_SEARCH_ALL), step by step."""
+    import paper_1801_01572_gb300 as lsr
+    P, Q, T0 = _moved(np.random.default_rng(n), kind, n)
+    for iters in (2, 5, 40):
+        T, it = ctx.stage_refine(P, Q, T0, EPS, 1.0, levels, iters)
+        ctx.debug_inject(lsr.INJECT_SEARCH_ALL, 1)
+        Ts, its = ctx.stage_refine(P, Q, T0, EPS, 1.0, levels, iters)
+        assert it == its and it >= min(iters, 2)
+        assert np.array_equal(T, Ts)
