@@ -58,6 +58,8 @@ WORKLOADS = {
 }
 BATCH_PAIRS = {2: 256, 3: 64, 4: 32}
 MATCH_MODES = {"fp32": 0, "bf16": 1, "bf16_plain": 2}
+FP32_PASSES = ("k_match_seed", "k_match_win")  # the FP32 matcher's passes over descriptor terms
+MAIN_KERNEL = {"fp32": "k_match_", "bf16": "k_match_tc", "bf16_plain": "k_match_tc"}  # (prefixes)
 FP32_LANES_PER_SM = 128
 N_SM = 152
 
@@ -176,9 +178,10 @@ def run_ours(args, rank, world):
     torch.cuda.synchronize()
     pk, _ = peaks()
     times, stages, last = [], np.zeros(8), None
-    # the dominant kernel is bracketed by two CUDA events on the context stream
-    # in every timed step (its only added work: two event records per step)
-    main_kernel = "k_match_win" if args.match == "fp32" else "k_match_tc"
+    # the dominant kernel (of the FP32 matcher: both passes over its terms) is
+    # bracketed by two CUDA events on the context stream in every timed step
+    # (the only added work: two event records per launch)
+    main_kernel = MAIN_KERNEL[args.match]
     ctx.set_kernel_timing(main_kernel)
     with ClockSampler(dev) as clk:
         l0 = lsr.launch_count()
@@ -296,8 +299,7 @@ def run_ours(args, rank, world):
             vctx.set_profiling(True)
             for _ in range(args.warmup):
                 vctx.register_pair(P, Q, fp.vpP, fp.vpQ)
-            vkern = "k_match_win" if name == "fp32" else "k_match_tc"
-            vctx.set_kernel_timing(vkern)
+            vctx.set_kernel_timing(MAIN_KERNEL[name])
             vt, vst, vl = [], np.zeros(8), None
             for _ in range(args.steps):
                 with torch.cuda.stream(stream):
@@ -623,6 +625,15 @@ def _kernel_avg_ms(times: dict, prefix: str):
     return n, (ms / n if n else None)
 
 
+def _fp32_passes_ms(times: dict):
+    """(matches, average ms of a match) of the FP32 matcher's two passes over
+    descriptor terms, k_match_seed and k_match_win: the library counts the terms
+    of both together."""
+    n, _ = _kernel_avg_ms(times, "k_match_win")
+    ms = sum(v[1] for k, v in times.items() if k.startswith(FP32_PASSES))
+    return n, (ms / n if n else None)
+
+
 def fp32_alu_peak(sm_mhz: float) -> float:
     """Issue peak of the matcher's instruction mix, TFLOP/s: one FADD and one
     FFMA per term (3 flop in 2 issue slots, 1.5 flop per lane per cycle)."""
@@ -636,8 +647,8 @@ def roofline(info):
     pk, src = peaks()
     nP, nQ = info["nP"], info["nQ"]
     sm_mhz = float(pk.get("sm_max_mhz", 2070.0))
-    n, avg = _kernel_avg_ms(info["main_times"], info["main_kernel"])
     if info["main_kernel"] == "k_match_tc":
+        n, avg = _kernel_avg_ms(info["main_times"], info["main_kernel"])
         K = 112 if info["match"] == "bf16" else 48
         flops = 2.0 * float(nP) * float(nQ) * K
         ach = flops / (avg * 1e-3) / 1e12
@@ -648,18 +659,21 @@ def roofline(info):
                 "dense_equivalent": {"achieved": ach, "unit": "TFLOP/s",
                                      "note": f"rate of the definition's 2*nP*nQ*{K} flop; only the tiles within "
                                              "reach are contracted, so it is no roofline fraction"}}
-    # FP32 matcher: the terms it evaluates (counted by the profiled launch; the
-    # count does not depend on timing), one subtract and one fused multiply-add
-    # each, against the issue peak of that mix
+    # FP32 matcher: the terms that its two passes evaluate (counted by the
+    # profiled launches; the second pass's count varies a little from run to run
+    # with the order in which warps share their best distances), one subtract and
+    # one fused multiply-add each, over the time of both, against the issue peak
+    # of that mix
+    n, avg = _fp32_passes_ms(info["main_times"])
     terms = float(info["prof"].match_terms)
     dense = float(nP) * float(nQ) * 33
     peak = fp32_alu_peak(sm_mhz)
     ach = terms * 3 / (avg * 1e-3) / 1e12
     # traffic: dram__bytes_read.sum + dram__bytes_write.sum of one full-size
-    # launch of this kernel on a room pair of this size, from an ncu capture (the two
+    # launch of k_match_win on a room pair of this size, from an ncu capture (the two
     # descriptor tables read once; the tiles' rows re-read from L2)
     traffic = 50922240 + 524544 if (nP, nQ) == (150000, 150000) else None
-    return {"kernel": "k_match_win", "bound": "alu", "achieved": ach, "peak": peak, "unit": "TFLOP/s",
+    return {"kernel": "k_match_seed + k_match_win", "bound": "alu", "achieved": ach, "peak": peak, "unit": "TFLOP/s",
             "frac": ach / peak, "traffic": traffic, "launch_ms": avg, "launches_timed": n,
             "algorithmic_bytes": 144.0 * (nP + nQ) + 8.0 * nP,
             "executed_terms": terms, "executed_share": terms / dense,
@@ -668,7 +682,8 @@ def roofline(info):
                                          "exact early exits skip "
                                          f"{100 * (1 - terms / dense):.1f}% of them, so it is no roofline fraction"},
             "peak_source": f"152 SMs x 128 FP32 lanes x 1.5 flop x {sm_mhz:.0f} MHz (FADD+FFMA issue peak)",
-            "work": "executed terms x 3 flop (subtract + fused multiply-add), terms counted by the profiled launch"}
+            "work": "executed terms x 3 flop (subtract + fused multiply-add) of both passes over the time of both, terms "
+                    "counted by the profiled launches"}
 
 
 def roofline_tc(info):
@@ -700,23 +715,30 @@ def roofline_tc(info):
 # kernel table in the design notes); both clouds together.
 def _kernel_work(name, nP, nQ, res, prm, terms):
     N = nP + nQ
-    S, n_ok, H = res.survivors, res.n_normal_ok, int(prm.n_hypotheses)
+    S, n_ok = res.survivors, res.n_normal_ok
+    sample = -(-nP // 32) if nP >= 16384 else nP  # the estimate pass of a large P
     table = [
-        ("k_match_win", "alu", 3.0 * terms, "flop", "executed terms x 3 flop"),
+        *((p, "alu", 3.0 * terms, "flop", "executed terms x 3 flop of k_match_seed and k_match_win over the time of both")
+          for p in FP32_PASSES),
         ("k_normals", "hbm", 48.0 * N, "B", "16 B point + 16 B grid copy in, 16 B normal out"),
         ("k_spfh", "hbm", 176.0 * N, "B", "16 B point + 16 B normal in, 144 B SPFH row out"),
         ("k_fpfh", "hbm", 320.0 * N, "B", "16 B point + 16 B normal + 144 B SPFH row in, 144 B FPFH row out"),
         ("k_proj", "hbm", 180.0 * N, "B", "144 B FPFH row in, 36 B projections and bound out"),
-        ("k_gather_db", "hbm", 300.0 * nQ, "B", "4 B order + 8 B projection + 144 B row in, 144 B row out "
-                                                "(Q: the database)"),
+        ("k_gather<true>", "hbm", 332.0 * nQ + 368.0 * nP, "B",
+         "4 B order + 36 B projections and bound + 144 B row in, 144 B row + 4 B index out (queries: 36 B more)"),
         ("k_prep_tiles", "hbm", (144.0 + 224.0) * N, "B", "144 B FPFH row in, 224 B BF16 operand row out"),
-        ("k_hyp_count", "hbm", 36.0 * N, "B", "unique bytes of the sampled arrays (points, normals, nn)"),
+        ("k_hyp_records", "hbm", 68.0 * nP + 32.0 * nQ, "B",
+         "16 B point + 16 B normal + 4 B nn in, 32 B record out; Q's points and normals in"),
+        ("k_hyp_count", "hbm", 32.0 * nP, "B", "unique bytes of the sampled records"),
         ("k_hyp_gather", "hbm", 8.0 * S, "B", "4 B per survivor id in, 4 B out"),
         ("k_rigid_survivors", "hbm", 321.0 * S, "B", "per survivor 4 x (P, Q points and normals, nn) in, 49 B out"),
-        ("k_consensus_count<true>", "hbm", 16.0 * nP + 56.0 * n_ok, "B",
-         "16 B per P point, 56 B per normal-checked pose (L1/L2-resident table lookups dominate)"),
+        ("k_consensus_count<true>", "hbm", 16.0 * sample + 56.0 * n_ok, "B",
+         "16 B per P point read (every 32nd from 16,384 points on), 56 B per normal-checked pose (L1/L2-resident "
+         "table lookups dominate)"),
+        ("k_group_count<true>", "hbm", 16.0 * nP + 56.0 * n_ok, "B",
+         "16 B per P point, 56 B per normal-checked pose at most (L1/L2-resident table lookups dominate)"),
         ("k_pack", "hbm", 28.0 * N, "B", "12 B xyz in, 16 B float4 out"),
-        ("k_bbox_partial", "hbm", 12.0 * N, "B", "12 B xyz in"),
+        ("k_grid_bbox", "hbm", 12.0 * N, "B", "12 B xyz in"),
     ]
     for pre, bound, work, unit, what in table:
         if name.startswith(pre):
@@ -740,6 +762,8 @@ def kernel_table(info):
                          float(info["prof"].match_terms))
         if w is not None:
             bound, work, unit, what = w
+            if name.startswith(FP32_PASSES):
+                ms = sum(v[1] for k, v in kt.items() if k.startswith(FP32_PASSES))
             per_step_s = ms / steps * 1e-3
             if unit == "B":
                 ach = work / per_step_s / 1e9
