@@ -117,7 +117,9 @@ typedef struct {
   int64_t survivors;      /* hypotheses left after pre-rejection */
   int64_t n_normal_ok;    /* survivors that also pass the normal check */
   int64_t best_h;         /* id of the selected hypothesis, -1 if none */
-  int64_t match_fallbacks; /* BF16 matching: queries re-scanned exactly in FP32 */
+  int64_t match_fallbacks; /* BF16 matching: queries without a certificate, re-scanned exactly in FP32. A query is
+                             certified against the best distance that its parts have found so far, so the
+                             number may differ a little between identical calls; the results do not */
   int64_t match_terms;    /* FP32 matching with profiling enabled: descriptor terms (a_k - b_k)^2 evaluated, of
                              nP * nQ * 33 for a scan without early exit; else 0 */
   float fitness;          /* mean squared inlier distance under T (m^2) */
@@ -264,7 +266,8 @@ LSR_API int lsr_stage_fpfh(lsr_ctx *ctx, const float *P, const float *normals, c
  * precision returns the same nn and d1 (the tensor-core modes re-rank their
  * top-8 candidates in FP32 and re-scan, in FP32, every query for which a
  * rounding-error bound cannot prove that the FP32 winner is a candidate).
- * fallbacks (host, may be NULL): queries re-scanned that way. */
+ * fallbacks (host, may be NULL): queries re-scanned that way (see
+ * lsr_result.match_fallbacks). */
 LSR_API int lsr_stage_match(lsr_ctx *ctx, const float *FP, int64_t nP, const float *FQ, int64_t nQ, int32_t precision,
                     int32_t *nn, float *d1, int64_t *fallbacks);
 

@@ -1142,6 +1142,9 @@ __global__ void k_fake_desc(uint64_t seed, int n, float *F) {
 
 // Tensor-core tile shape per size bucket: both shapes timed (CUDA events) on
 // synthetic descriptors of the largest query count of that bucket in the batch.
+// Those rows spread over all bins, so the boxes exclude few tiles and the choice
+// is that for contracting (nearly) all of them, which a scene's descriptors need
+// only below the size from which tiles are listed.
 int tune_tiles(lsr_ctx *c, const BatchIn &b) {
   if (c->prm.match_precision == LSR_MATCH_FP32 || c->prm.match_tile) return LSR_OK;
   const bool split = c->prm.match_precision == LSR_MATCH_BF16;

@@ -93,15 +93,12 @@ __device__ __forceinline__ void stage_ranks(int (&rk)[4]) {
 }
 
 // Scan the m staged rows for the Q queries of this thread (a in
-// desc_order), updating best / bj; row j of the tile is database row ids[j]
-// (base + j when ids is null). A row replaces the best when its distance is
-// smaller, or equal with a smaller index, so the result does not depend on
-// the order in which rows are scanned. kCount: add the terms evaluated per
-// query to terms.
-template <int Q, bool kCount = false>
-__device__ __forceinline__ void scan_tile(const float4 (*tile)[9], int m, int base, const int *ids,
-                                          const float (&a)[Q][kD], float (&best)[Q], int (&bj)[Q],
-                                          unsigned *terms = nullptr) {
+// desc_order), updating best / bj; row j of the tile is database row base + j.
+// A row replaces the best when its distance is smaller, or equal with a smaller
+// index, so the result does not depend on the order in which rows are scanned.
+template <int Q>
+__device__ __forceinline__ void scan_tile(const float4 (*tile)[9], int m, int base, const float (&a)[Q][kD],
+                                          float (&best)[Q], int (&bj)[Q]) {
   for (int j = 0; j < m; ++j) {
     float s[Q];
 #pragma unroll
@@ -115,7 +112,6 @@ __device__ __forceinline__ void scan_tile(const float4 (*tile)[9], int m, int ba
         if (__all_sync(0xffffffffu, past)) break;
       }
       float4 b = tile[j][c];
-      if (kCount) *terms += c == 7 ? 5 : 4;
 #pragma unroll
       for (int u = 0; u < Q; ++u) {
         float t0 = a[u][4 * c] - b.x, t1 = a[u][4 * c + 1] - b.y, t2 = a[u][4 * c + 2] - b.z,
@@ -127,7 +123,7 @@ __device__ __forceinline__ void scan_tile(const float4 (*tile)[9], int m, int ba
       }
       if (c == 7) {
         float b32 = tile[j][8].x;
-        const int id = ids ? ids[j] : base + j;
+        const int id = base + j;
 #pragma unroll
         for (int u = 0; u < Q; ++u) {
           float t = a[u][32] - b32;
@@ -479,7 +475,7 @@ __global__ void k_win_finish(const unsigned long long *__restrict__ packed, cons
 
 // Exact FP32 scan of the queries rows[0..*nrows), split over database chunks
 // (blockIdx.y) so that a short list still fills the GPU. Each block computes
-// the chunk-local minimum exactly as k_match_fp32 does; chunks are combined
+// the chunk-local minimum, ties to the smaller index; chunks are combined
 // with a 64-bit atomicMin on (distance bits << 32 | index), which for the
 // non-negative distances keeps the smallest distance and, among equal
 // distances, the smallest index -- the sequential scan's result.
@@ -513,7 +509,7 @@ __global__ void __launch_bounds__(kMT) k_match_rows_chunked(const float *__restr
       __syncthreads();
       stage_tile(tile, FQ, base, j1, rk);
       __syncthreads();
-      scan_tile<kQR>(tile, j1 - base < kTile ? j1 - base : kTile, base, nullptr, a, best, bj);
+      scan_tile<kQR>(tile, j1 - base < kTile ? j1 - base : kTile, base, a, best, bj);
     }
 #pragma unroll
     for (int u = 0; u < kQR; ++u)

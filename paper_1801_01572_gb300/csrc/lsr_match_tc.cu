@@ -774,8 +774,11 @@ struct TcLayout {
 };
 
 // Whether the order and the item list pay. The order and the first pass cost
-// about 0.15 ms at any size; the contraction over all tiles 0.2 ns a pair of
-// rows, of which the list leaves a tenth to a fifth: they meet near 30k x 30k.
+// about 0.15 ms at any size; the contraction over all tiles 0.2 ps a pair of
+// rows (8.5 ms for 4e10), of which the list leaves a tenth to a fifth. Whole
+// calls on room descriptors, all tiles against listed ones: 8k x 8k 289 and 413
+// us, 16k 350 and 467, 20k 471 and 511, 23k (about where the line lies) 479 and
+// 520, 28k 533 and 525.
 // Above 2^22 items (about 2M x 2M rows) the list would outgrow its use of memory.
 constexpr int64_t kWindowPairs = (int64_t)1 << 29;
 constexpr int64_t kMaxItems = (int64_t)1 << 22;
@@ -901,8 +904,9 @@ size_t tc_workspace_bytes(int nP, int nQ, bool split, bool list) {
 int tc_score_cols(int nQ) { return (int)lsr_div_up(nQ, kTcN) * kTcN; }
 
 // One query tile per CTA (two CTAs per SM) unless the autotuner chose for the
-// size: on the 150k-point room pair it takes 4.58 ms against 5.53 ms with two
-// query tiles per CTA (one CTA per SM).
+// size: on the 150k-point room pair (its listed tiles) it takes 0.64 ms against
+// 0.84 ms with two query tiles per CTA (one CTA per SM); a whole match of 200k x
+// 200k room descriptors 1.93 ms against 2.29.
 int tc_default_tile(int) { return 1; }
 
 cudaError_t launch_match_bf16(const float *FP, int nP, const float *FQ, int nQ, bool split, int qt, char *ws, int *nn,

@@ -6,10 +6,13 @@
 // surfel -- in front of it, no farther than the maximum depth, projecting
 // inside the image --
 //   p' = (1/k) sum_f T_f_new T_f_old^-1 p,   n' = normalize(sum_f R_f_new R_f_old^-1 n),
-// k = |F|; a surfel no keyframe observes is removed. Surfels do not interact:
-// one thread per surfel, the keyframes' two 3 x 4 transforms (precomputed on
-// the host in FP64, stored in FP32) read through the read-only cache, the
-// time window found by binary search over the sorted keyframe stamps.
+// k = |F|; a surfel no keyframe observes is removed. Surfels do not interact.
+// A keyframe's two 3 x 4 transforms are precomputed on the host in FP64 and
+// stored in FP32; the time window is found by binary search over the sorted
+// keyframe stamps. Up to kSurfTileKf keyframes fit in shared memory beside a
+// tile of surfels (k_surfel_tile); with more, a thread per surfel reads the
+// transforms through the read-only cache (k_surfel_correct), half as fast. Both
+// give the same bits.
 #include "lsr_internal.cuh"
 
 namespace lsr {
@@ -83,9 +86,9 @@ __global__ void __launch_bounds__(kSurfThreads) k_surfel_correct(int64_t n, cons
 // kernel above reads 12 to 24 scalars per (surfel, keyframe) through L1 with a
 // different keyframe on every lane (map order says nothing about time), and
 // that gather bound it: 869 us for 2M surfels and 300 keyframes, L1 at 88%,
-// 114 MB of traffic worth 17 us (the whole call 967 us, 412 with this kernel). Here a block takes a tile of surfels, sorts
-// the tile by first keyframe (a counting sort in shared memory), and a warp
-// walks 32 neighbours of that order through the union of their windows one
+// 114 MB of traffic worth 17 us (the whole call 967 us, 412 with this kernel).
+// Here a block takes a tile of surfels, sorts the tile by first keyframe (a
+// counting sort in shared memory), and a warp walks 32 neighbours of that order through the union of their windows one
 // keyframe at a time: the keyframe is the same on every lane, so its rows are
 // broadcasts. A window is 20 keyframes and the union about 50 (the spread of
 // 32 of 1024 first keyframes, and the longest window), so half the lanes idle;
