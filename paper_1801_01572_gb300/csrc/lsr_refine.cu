@@ -211,6 +211,7 @@ __device__ __noinline__ Found half_nn(const GridParams &g, const int *__restrict
   const int sub = threadIdx.x & (kRefH - 1);
   float best = seed2, m1 = 3e38f, m2 = 3e38f, reach2 = 3e38f;
   int bidx = 0x7fffffff, bt = seed;
+  const float mg = g.margin;
   const float fx = (x - g.ox) * g.inv_cell, fy = (y - g.oy) * g.inv_cell, fz = (z - g.oz) * g.inv_cell;
   bool go = fx >= -1.f && fx < (float)g.nx + 1.f && fy >= -1.f && fy < (float)g.ny + 1.f && fz >= -1.f &&
             fz < (float)g.nz + 1.f;
@@ -229,7 +230,6 @@ __device__ __noinline__ Found half_nn(const GridParams &g, const int *__restrict
     const float r = sqrtf(best) + guard, gb = r * r;
     const int dy = sub % 3 - 1, dz = sub / 3 - 1, iy = cy + dy, iz = cz + dz;
     if (sub < 9 && iy >= 0 && iy < g.ny && iz >= 0 && iz < g.nz) {
-      const float mg = g.margin;
       auto gsq = [&](float d) {
         const float t = fmaxf(d - mg, 0.f);
         return t * t;
