@@ -276,9 +276,11 @@ __device__ __forceinline__ void grid_ranges(const GridParams &g, const int *__re
 // The query's own row of cells is searched first; each of the other eight
 // rows, and the x-neighbour cells of every row, is visited only if its
 // distance from the query (less the grid's margin, above the FP32 rounding of
-// cell coordinates) can still reach the group's best so far. A
-// skipped cell holds no point at or below that best, so the result is the
-// one of the full walk. (Grids with wrapped storage walk all cells.)
+// cell coordinates) can still reach the group's best so far. A skipped cell
+// holds no point at or below that best, so the result is the one of the full
+// walk. (Grids with wrapped storage walk all cells.) margin: an address of g's;
+// the grid's own in memory where a register for it costs spills
+// (k_consensus_var).
 //
 // seed (optional, >= 0): an index into Xe known to be a candidate (the
 // previous refinement step's neighbour of the same point). Its distance,
@@ -292,7 +294,7 @@ __device__ __forceinline__ float nn_d2(float4 q, float x, float y, float z) {
 }
 
 template <int G>
-__device__ __forceinline__ void group_nn(const GridParams &g, const int *__restrict__ start,
+__device__ __forceinline__ void group_nn(const GridParams &g, const float *margin, const int *__restrict__ start,
                                          const float4 *__restrict__ Xe, float x, float y, float z, float eps2,
                                          float &best, int &bt, int &bidx, int seed = -1) {
   int sub = threadIdx.x & (G - 1);
@@ -351,7 +353,7 @@ __device__ __forceinline__ void group_nn(const GridParams &g, const int *__restr
     }
     if (go) {
       const unsigned gmask = G == 32 ? 0xffffffffu : (((1u << G) - 1u) << ((threadIdx.x & 31) & ~(G - 1)));
-      const float mg = g.margin;
+      const float mg = *margin;
       auto gsq = [&](float d) {
         const float t = fmaxf(d - mg, 0.f);
         return t * t;

@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(kNnThreads) k_nn_stage(const float *__restrict
       bt = single_cell_nn(g, start, Xs, x, y, z, best);
     } else {
       int bidx;
-      group_nn<G>(g, start, Xs, x, y, z, r2, best, bt, bidx);
+      group_nn<G>(g, &gp->margin, start, Xs, x, y, z, r2, best, bt, bidx);
     }
     if (!valid || sub != 0) continue;
     nn[i] = bt >= 0 ? __float_as_int(Xs[bt].w) : -1;
@@ -171,7 +171,7 @@ __global__ void __launch_bounds__(kNnThreads) k_consensus_var(const float4 *__re
         bt = single_cell_nn(g, start, Xs, x, y, z, best);
       } else {
         int bidx;
-        group_nn<G>(g, start, Xs, x, y, z, eps2, best, bt, bidx);
+        group_nn<G>(g, &gp->margin, start, Xs, x, y, z, eps2, best, bt, bidx);
       }
       if (!valid || sub != 0 || bt < 0 || !(best < eps2)) continue;
       if (kNormals) {

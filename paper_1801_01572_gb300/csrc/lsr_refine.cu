@@ -304,7 +304,7 @@ __device__ __noinline__ Found group_nn_wrapped(const GridParams &g, const int *_
                                                int seed) {
   float best;
   int bt, bidx;
-  group_nn<kRefH>(g, start, Xe, x, y, z, eps2, best, bt, bidx, seed);
+  group_nn<kRefH>(g, &g.margin, start, Xe, x, y, z, eps2, best, bt, bidx, seed);
   return {bt, 0.f};
 }
 
@@ -652,7 +652,7 @@ __global__ void __launch_bounds__(kRefThreads) k_info_sums(const float *__restri
     const float z = fmaf(a.R[6], px, fmaf(a.R[7], py, fmaf(a.R[8], pz, a.t[2])));
     float best;
     int bt, bidx;
-    group_nn<G>(g, start, Xe, x, y, z, a.eps2, best, bt, bidx);
+    group_nn<G>(g, &g.margin, start, Xe, x, y, z, a.eps2, best, bt, bidx);
     if (!valid || bt < 0 || sub != 0) continue;
     const float dx = x - c0, dy = y - c1, dz = z - c2;
     acc[0] += 1.f;
@@ -722,7 +722,7 @@ __global__ void __launch_bounds__(kRefThreads, 5) k_pose_nn(const __grid_constan
   const float z = fmaf(a.R[6], px, fmaf(a.R[7], py, fmaf(a.R[8], pz, a.t[2])));
   float best;
   int bt, bidx;
-  group_nn<kPoseNnG>(g, a.start, a.Xe, x, y, z, a.eps2, best, bt, bidx);
+  group_nn<kPoseNnG>(g, &g.margin, a.start, a.Xe, x, y, z, a.eps2, best, bt, bidx);
   if (valid && (threadIdx.x & (kPoseNnG - 1)) == 0) a.nn[i] = bt;
 }
 
